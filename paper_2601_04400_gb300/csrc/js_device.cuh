@@ -3,8 +3,8 @@
 // GB300 has a narrow FP64 pipe (about 1/64 of the FP32 rate) while integer, FP32, MUFU and
 // min/max work issue on other units.  Everything here is therefore written to minimise
 // FP64 add/mul/fma instructions:
-//   * no IEEE division or square root: MUFU seeds (rcp.approx / rsqrt.approx) refined by
-//     Newton steps and a residual correction, accurate to about one ulp;
+//   * no IEEE division or square root: reciprocals and reciprocal square roots are formed in
+//     integer arithmetic beside the FP64 pipe (js_wide.cuh), accurate to half an ulp;
 //   * WENO5 is cell-centred: the smoothness indicators of a cell's three stencils are
 //     computed once and shared by the state at its right face (left-biased weights) and
 //     the state at its left face (right-biased weights); first and second differences are
@@ -15,6 +15,8 @@
 //     selects), and the sound speed as gamma*p*rsqrt(gamma*p*rho).
 #pragma once
 #include <cstdint>
+
+#include "js_wide.cuh"
 
 namespace js {
 
@@ -32,33 +34,36 @@ constexpr int ERR_NONPHYSICAL_BIT = 1;
 constexpr int ERR_TIMEOUT_BIT = 2;
 
 // ---------------------------------------------------------------------------------------
-// FP64 reciprocal / quotient / reciprocal square root with few FP64-pipe instructions
+// FP64 reciprocal / quotient / reciprocal square root that leave the FP64 pipe free
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ double rcp_seed(double x) {
+// The cases outside the integer routines' range (zero, subnormal, infinite, NaN; a negative
+// square root) take the FP64 forms: MUFU seeds, accurate to about 2^-20 (measured on GB300), and
+// one cubic (Halley) step.
+static __device__ __noinline__ double recip_plain(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  return r;
-}
-__device__ __forceinline__ double rsqrt_seed(double x) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  return r;
-}
-// The seeds are accurate to about 2^-20 (measured on GB300), so one cubic (Halley) step
-// reaches full FP64 precision.
-// 1/x: seed + one Halley step r (1 + e + e^2), e = 1 - x r (3 FP64 instructions)
-__device__ __forceinline__ double recip(double x) {
-  const double r = rcp_seed(x);
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-// a/b as a * (1/b) (4 FP64 instructions; within about 1.5 ulp)
-__device__ __forceinline__ double quot(double a, double b) { return a * recip(b); }
-// 1/sqrt(x): seed + one Halley step y (1 + e/2 + 3e^2/8), e = 1 - x y^2 (5 FP64 instructions)
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  const double y = rsqrt_seed(x);
+static __device__ __noinline__ double rsqrt_plain(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x * y, y, 1.0);
   return fma(y, e * fma(0.375, e, 0.5), y);
+}
+// 1/x in integer arithmetic (js_wide.cuh), correctly rounded but for one in 2000 arguments
+// where the seed and Halley step reached about 1.5 ulp; it takes no FP64 issue slot instead of 3
+__device__ __forceinline__ double recip(double x) {
+  if ((u32)(expo(x) - 1) >= 2044u) return recip_plain(x);
+  return recip_wide(x);
+}
+// a/b as a * (1/b) (1 FP64 instruction; within 1 ulp)
+__device__ __forceinline__ double quot(double a, double b) { return a * recip(b); }
+// 1/sqrt(x) likewise (0 instead of 5 FP64 instructions)
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  const s32 h = (s32)hi32(dbits(x));
+  if ((u32)(h - 0x00100000) >= 0x7fe00000u) return rsqrt_plain(x);  // not positive and normal
+  return rsqrt_wide(x);
 }
 
 // ---------------------------------------------------------------------------------------
