@@ -11,8 +11,8 @@
 //     carried along the line in registers;
 //   * the nonlinear weights use the products of the other stencils' (eps + beta)^2 instead
 //     of 1/(eps + beta)^2, so one division per face state remains;
-//   * HLLC evaluates the star state of the upwind side only (selected with integer
-//     selects), and the sound speed as gamma*p*rsqrt(gamma*p*rho).
+//   * HLLC forms the flux of the upwind side's star state (selected with integer selects),
+//     and the sound speed as gamma*p*rsqrt(gamma*p*rho).
 #pragma once
 #include <cstdint>
 
@@ -209,25 +209,21 @@ struct Win {
 // ---------------------------------------------------------------------------------------
 // HLLC (Sec. 2) in the face-normal frame.  State (rho, un, ut, p) on each side; returns
 // [mass, normal momentum, tangential momentum, energy].  Star-state energy in the
-// standard (Toro) form; sign(s*) = 0 averages both branches.
+// standard (Toro) form.
+//
+// Of the upwind side K of the contact (s* > 0: left), with d = s_K - u, m = rho d and the star
+// pressure p* = p + m (s* - u), the flux F_K + s_K (U*_K - U_K) equals the flux of the star state
+// (the jump relation across s_K), which is formed directly:
+//   G = m s*/(s_K - s*),  F = (G, G s* + p*, G u_t, s*/(s_K - s*) (d E - p u + p* s_K)).
+// A supersonic face (s_K on the far side of zero) has F = F_K, the same expressions with u in
+// the place of s*.  At s* = 0 both sides give (0, p*, 0, 0): the average of the branches that
+// sign(0) = 0 asks for is either of them.  29 FP64 instructions a face (15 at s* = 0, where gas
+// at rest on both sides always lands) where building the star state and its jump took 61.
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ void hllc_branch(double r, double un, double ut, double p, double s, double d,
-                                            double m, double spm, double ss, const Gas& g, double F[4]) {
-  // d = s - un, m = rho (s - un)
-  const double ke = fma(un, un, ut * ut);
-  const double E = fma(0.5 * r, ke, p * g.g1);
-  const double inv = recip(s - ss);
-  const double rs = m * inv;               // rho* = rho (s - u)/(s - s*)
-  const double fac = d * inv;              // (s - u)/(s - s*)
-  const double Us1 = rs * ss;              // rho* s*
-  const double Us2 = rs * ut;              // rho* v
-  const double Es = fma(ss - un, fma(p, inv, Us1), fac * E);
-  const double mom = r * un;
-  F[0] = fma(spm, rs - r, mom);
-  F[1] = fma(spm, Us1 - mom, fma(mom, un, p));
-  F[2] = fma(spm, Us2 - r * ut, mom * ut);
-  F[3] = fma(spm, Es - E, (E + p) * un);
-}
+// signs and positivity from the bits: an FP64 comparison takes an FP64 issue slot
+__device__ __forceinline__ bool sign_clear(double x) { return (s32)hi32(dbits(x)) >= 0; }
+// x > 0 (false for NaN)
+__device__ __forceinline__ bool positive(double x) { return dbits(x) - 1u < 0x7ff0000000000000ull; }
 
 __device__ __forceinline__ void hllc(double rL, double uL, double vL, double pL, double rR, double uR,
                                      double vR, double pR, const Gas& g, double F[4]) {
@@ -240,29 +236,25 @@ __device__ __forceinline__ void hllc(double rL, double uL, double vL, double pL,
   const double mL = rL * dL, mR = rR * dR;
   const double num = fma(-uR, mR, fma(uL, mL, pR - pL));
   const double ss = quot(num, mL - mR);
-  if (ss == 0.0) {
-    if (sL < 0.0 && sR > 0.0) {
-      // With s* = 0 and sL < 0 < sR each branch's star flux F_K + s_K (U*_K - U_K) reduces,
-      // in exact arithmetic, to (0, p_K - m_K u_K, 0, 0): the mass, tangential-momentum and
-      // energy terms cancel identically and the normal momentum is the star pressure.  The
-      // average of the two branches is therefore formed directly (4 instead of ~66 FP64
-      // instructions; quiescent gas, u = 0 on both sides of a face, always lands here).
-      F[0] = 0.0;
-      F[1] = 0.5 * (fma(-mL, uL, pL) + fma(-mR, uR, pR));
-      F[2] = 0.0;
-      F[3] = 0.0;
-      return;
-    }
-    double FL[4], FR[4];
-    hllc_branch(rL, uL, vL, pL, sL, dL, mL, fmin(0.0, sL), ss, g, FL);
-    hllc_branch(rR, uR, vR, pR, sR, dR, mR, fmax(0.0, sR), ss, g, FR);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) F[c] = 0.5 * (FL[c] + FR[c]);
+  const bool left = sign_clear(ss);
+  const double u = left ? uL : uR, ut = left ? vL : vR, p = left ? pL : pR, s = left ? sL : sR,
+               d = left ? dL : dR, m = left ? mL : mR;
+  const bool outside = sign_clear(left ? sL : -sR);  // s_L >= 0, s_R <= 0
+  const double c = outside ? u : ss;
+  const double ps = fma(m, c - u, p);
+  if ((dbits(c) << 1) == 0) {  // gas at rest on both sides: nothing but the pressure
+    F[0] = F[2] = F[3] = 0.0;
+    F[1] = ps;
     return;
   }
-  const bool left = ss > 0.0;
-  hllc_branch(left ? rL : rR, left ? uL : uR, left ? vL : vR, left ? pL : pR, left ? sL : sR,
-              left ? dL : dR, left ? mL : mR, left ? fmin(0.0, sL) : fmax(0.0, sR), ss, g, F);
+  const double w = c * recip(s - c);
+  const double G = m * w;
+  // d E = m (u^2 + u_t^2)/2 + d p/(gamma - 1)
+  const double dE = fma(0.5 * m, fma(u, u, ut * ut), g.g1 * (d * p));
+  F[0] = G;
+  F[1] = fma(G, c, ps);
+  F[2] = G * ut;
+  F[3] = w * fma(ps, s, fma(-p, u, dE));
 }
 
 // ---------------------------------------------------------------------------------------

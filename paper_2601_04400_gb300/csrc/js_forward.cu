@@ -358,10 +358,7 @@ __global__ void __launch_bounds__(TX / LX) stage1d_kernel(StageArgs a0) {
   sweep_line<0, VISC, false, LX>(sq, PS, xs + 3, 1, 0, g, a.vx, [&](int k, const double dF[4]) {
     const int gi = tx0 + xs + k;
     if (gi < a.lay.nx) {
-      double ax[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) ax[c] = a.cx * dF[c];
-      finish_cell<RHS, true>(a, gi, 0, ax, zero, sq[xs + k + 3], sq[3 * PS + xs + k + 3]);
+      finish_cell<RHS>(a, gi, 0, dF, zero, sq[xs + k + 3], sq[3 * PS + xs + k + 3]);
     }
   });
 }

@@ -81,7 +81,7 @@ __device__ __forceinline__ void sweep_line(const double* __restrict__ sq, int ps
 #pragma unroll
       for (int c = 0; c < 4; ++c) { ql[c] = prevL[c]; qr[c] = Rf[c]; }
       if (FI) face(k, ql, qr);
-      if (!(ql[0] > 0.0 && ql[3] > 0.0 && qr[0] > 0.0 && qr[3] > 0.0)) {
+      if (!(positive(ql[0]) && positive(ql[3]) && positive(qr[0]) && positive(qr[3]))) {
         // positivity fallback: first-order (cell) states at this face
 #pragma unroll
         for (int c = 0; c < 4; ++c) { ql[c] = sq[c * ps + cell - st]; qr[c] = sq[c * ps + cell]; }
@@ -130,20 +130,20 @@ __device__ __forceinline__ void sweep_line(const double* __restrict__ sq, int ps
 }
 
 // final combination for one interior cell; returns the value stored in the output
-// dG: raw y-flux differences (scaled here by cy), or already scaled when YSCALED
-template <bool RHS, bool YSCALED = false>
-__device__ __forceinline__ void finish_cell(const StageArgs& a, int gi, int gj, const double acc[4],
+// dF, dG: x and y flux differences (dG zero in 1D)
+template <bool RHS>
+__device__ __forceinline__ void finish_cell(const StageArgs& a, int gi, int gj, const double dF[4],
                                             const double dG[4], double rho, double p) {
   const long long pid = a.lay.idx(gi, gj);
   const bool fluid = (a.tag == nullptr) || (a.tag[(long long)gj * a.lay.nx + gi] == 0);
   double out[4];
   if (fluid) {
-    if (!(rho > 0.0 && p > 0.0)) atomicOr(a.err, ERR_NONPHYSICAL_BIT);
+    if (!(positive(rho) && positive(p))) atomicOr(a.err, ERR_NONPHYSICAL_BIT);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const double* Uc = a.Uin + c * a.lay.plane;
       const double us = RHS ? 0.0 : Uc[pid];
-      double v = YSCALED ? (us - acc[c]) - dG[c] : fma(-a.cy, dG[c], us - acc[c]);
+      double v = fma(-a.cy, dG[c], fma(-a.cx, dF[c], us));
       if (a.has_av) {
         v = fma(a.avx, (Uc[pid + 1] - 2.0 * Uc[pid]) + Uc[pid - 1], v);
         if (a.lay.ny > 1) v = fma(a.avy, (Uc[pid + a.lay.pitch] - 2.0 * Uc[pid]) + Uc[pid - a.lay.pitch], v);
@@ -222,7 +222,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int bx, int by, d
       if (gi < a.lay.nx && gj < a.lay.ny) {
         const long long o = (long long)gj * a.lay.nx + gi;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a.acc[c * ncell + o] = __dmul_rn(a.cx, dF[c]);
+        for (int c = 0; c < 4; ++c) a.acc[c * ncell + o] = dF[c];
       }
     });
   }
@@ -239,11 +239,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int bx, int by, d
         const long long o = (long long)gj * a.lay.nx + gi;
 #pragma unroll
         for (int c = 0; c < 4; ++c) ax[c] = a.acc[c * ncell + o];
-        double ay[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) ay[c] = __dmul_rn(a.cy, dG[c]);  // rounded as when stored
         const int sc = (ty + 3) * S::SP + tx + 3;
-        finish_cell<RHS, true>(a, gi, gj, ax, ay, sq[sc], sq[3 * S::PS + sc]);
+        finish_cell<RHS>(a, gi, gj, ax, dG, sq[sc], sq[3 * S::PS + sc]);
       }
     });
   }
@@ -253,7 +250,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int bx, int by, d
 // ---------------------------------------------------------------------------------------
 // Concurrent-sweep tile: the x sweep (first NX_ITEMS threads) and the y sweep (next
 // NY_ITEMS threads, warp-aligned) run at the same time on the shared primitive tile and
-// write their scaled flux differences to two global accumulators (L2-resident); after a
+// write their flux differences to two global accumulators (L2-resident); after a
 // barrier every thread combines cells of the tile.  Twice the warps per block at the same
 // shared memory: more warps hide the FP64 pipe's latency.
 // ---------------------------------------------------------------------------------------
@@ -400,7 +397,7 @@ __device__ __forceinline__ void stage_tile_c(const StageArgs& a, int bx, int by,
       if (gi < a.lay.nx && gj < a.lay.ny) {
         const long long o = (long long)gj * a.lay.nx + gi;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a.acc[c * ncell + o] = __dmul_rn(a.cx, dF[c]);
+        for (int c = 0; c < 4; ++c) a.acc[c * ncell + o] = dF[c];
       }
     };
     if constexpr (SAVE) {
@@ -426,7 +423,7 @@ __device__ __forceinline__ void stage_tile_c(const StageArgs& a, int bx, int by,
       if (gi < a.lay.nx && gj < a.lay.ny) {
         const long long o = (long long)gj * a.lay.nx + gi;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a.acc2[c * ncell + o] = __dmul_rn(a.cy, dG[c]);
+        for (int c = 0; c < 4; ++c) a.acc2[c * ncell + o] = dG[c];
       }
     };
     if constexpr (SAVE) {
@@ -457,7 +454,7 @@ __device__ __forceinline__ void stage_tile_c(const StageArgs& a, int bx, int by,
       ay[c] = a.acc2[c * ncell + o];
     }
     const int sc = (ty + 3) * S::SP + tx + 3;
-    finish_cell<RHS, true>(a, gi, gj, ax, ay, sq[sc], sq[3 * S::PS + sc]);
+    finish_cell<RHS>(a, gi, gj, ax, ay, sq[sc], sq[3 * S::PS + sc]);
   }
 }
 
