@@ -125,23 +125,8 @@ __device__ __forceinline__ void pass1_body(const AdjArgs& a, int seg_len, long l
     const ViscC& vc = (DIR == 0) ? a.vx : a.vy;
     const int wdir = DIR * 4 * WENO_SAVE;
     auto cell_id = [&](int k) { return (DIR == 0) ? L.idx(k, line) : L.idx(line, k); };
-    // window at cell i = f0 - 1: q_{i-2..i+1}
-    double q0[4], q1[4];
-    Dl d[4];
-    if (!SAVED) {
-      const long long b = cell_id(f0 - 1);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const double* q = a.Q + c * L.plane;
-        const double qm2 = q[b - 2 * st], qm1 = q[b - st], qc = q[b], qp1 = q[b + st];
-        q0[c] = qc;
-        q1[c] = qp1;
-        d[c].m2 = 0.0;
-        d[c].m1 = qm1 - qm2;
-        d[c].p1 = qc - qm1;
-        d[c].p2 = qp1 - qc;
-      }
-    }
+    Win4 w;
+    if (!SAVED) w.init(a.Q + cell_id(f0 - 1), L.plane, st);
     double prevL[4];
 #pragma unroll 1
     for (int i = f0 - 1; i < f1; ++i) {
@@ -158,21 +143,10 @@ __device__ __forceinline__ void pass1_body(const AdjArgs& a, int seg_len, long l
           Rf[c] = fma(sv[5 * a.splane], SIXTH, qc);
         }
       } else {
+        w.template step<true, true, true>(a.Q + ci, L.plane, st, Lf, Rf, [&](int c, const double* sv) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        // slide: d.m2 <- d.m1 ... and bring in q_{i+2}
-        const double q2 = a.Q[c * L.plane + ci + 2 * st];
-        d[c].m2 = d[c].m1;
-        d[c].m1 = d[c].p1;
-        d[c].p1 = d[c].p2;
-        d[c].p2 = q2 - q1[c];
-        double sv[WENO_SAVE];
-        weno_cell_fwd(q0[c], d[c], Lf[c], Rf[c], sv);
-#pragma unroll
-        for (int k = 0; k < WENO_SAVE; ++k) a.wsave[(long long)(wdir + c * WENO_SAVE + k) * a.splane + si] = sv[k];
-        q0[c] = q1[c];
-        q1[c] = q2;
-      }
+          for (int k = 0; k < WENO_SAVE; ++k) a.wsave[(long long)(wdir + c * WENO_SAVE + k) * a.splane + si] = sv[k];
+        });
       }
       if (i >= f0) {
         // face f = i between cells i-1 (state prevL) and i (state Rf)

@@ -5,18 +5,15 @@
 // FP64 add/mul/fma instructions:
 //   * no IEEE division or square root: reciprocals and reciprocal square roots are formed in
 //     integer arithmetic beside the FP64 pipe (js_wide.cuh), accurate to half an ulp;
-//   * WENO5 is cell-centred: the smoothness indicators of a cell's three stencils are
-//     computed once and shared by the state at its right face (left-biased weights) and
-//     the state at its left face (right-biased weights); first and second differences are
-//     carried along the line in registers;
-//   * the nonlinear weights use the products of the other stencils' (eps + beta)^2 instead
-//     of 1/(eps + beta)^2, so one division per face state remains;
+//   * WENO5 runs on the integer pipes (js_weno.cuh) but for three FP64 instructions per cell
+//     and variable; the nonlinear weights use the products of the other stencils'
+//     (eps + beta)^2 instead of 1/(eps + beta)^2, so one division per face state remains;
 //   * HLLC forms the flux of the upwind side's star state (selected with integer selects),
 //     and the sound speed as gamma*p*rsqrt(gamma*p*rho).
 #pragma once
 #include <cstdint>
 
-#include "js_wide.cuh"
+#include "js_weno.cuh"
 
 namespace js {
 
@@ -92,10 +89,10 @@ __device__ __forceinline__ void cons_to_prim(double r, double mx, double my, dou
 //   4 beta_1 = 13/3 D_i^2     + (d_{i-1/2} + d_{i+1/2})^2
 //   4 beta_2 = 13/3 D_{i+1}^2 + (D_{i+1} - 2 d_{i+1/2})^2
 // s_k = 4 beta_k + 4 eps; the weights alpha_k = d_k / s_k^2 are scaled by (s0 s1 s2)^2.
-// Candidate values minus q_i, times 6, are two-term combinations of the d's.
+// Candidate values minus q_i, times 6, are two-term combinations of the d's.  Win evaluates
+// this in integer arithmetic (js_weno.cuh), weno_plain in FP64.
 // ---------------------------------------------------------------------------------------
-constexpr double K13 = 13.0 / 3.0;
-constexpr double EPS4 = 4.0e-6;
+constexpr double EPS12 = 1.2e-5;  // 3 (4 eps)
 constexpr double SIXTH = 1.0 / 6.0;
 
 // Network input of one face (neural flux, Sec. 2.3): the mean of its two WENO5 face states
@@ -119,90 +116,126 @@ __device__ __forceinline__ void face_image(const double wl[4], const double wr[4
   for (int k = 0; k < 4; ++k) m[k] = (m[k] - mean[k]) * inv_sd[k];
 }
 
-struct Win {
-  double q0, q1;          // q_i, q_{i+1}
-  double dm2, dm1, dp1;   // d_{i-3/2}, d_{i-1/2}, d_{i+1/2}
-  double D0, D1;          // D_{i-1}, D_i
-  double cD0, cD1;        // 13/3 D
-  double f5m1, f5p1;      // 5 d_{i-1/2}, 5 d_{i+1/2}
+// the FP64 form of one cell: out[0..1] = the face states at i+1/2 and i-1/2, out[2..8] = the
+// internals of Win::step
+static __device__ __noinline__ void weno_plain(double qm2, double qm1, double q0, double q1, double q2, double out[9]) {
+  const double dm2 = qm1 - qm2, dm1 = q0 - qm1, dp1 = q1 - q0, dp2 = q2 - q1;
+  const double D0 = dm1 - dm2, D1 = dp1 - dm1, D2 = dp2 - dp1;
+  const double t0 = fma(2.0, dm1, D0), t1 = dm1 + dp1, t2 = fma(-2.0, dp1, D2);
+  const double s0 = fma(13.0 * D0, D0, fma(3.0 * t0, t0, EPS12));
+  const double s1 = fma(13.0 * D1, D1, fma(3.0 * t1, t1, EPS12));
+  const double s2 = fma(13.0 * D2, D2, fma(3.0 * t2, t2, EPS12));
+  const double p01 = s0 * s1, p02 = s0 * s2, p12 = s1 * s2;
+  const double w0 = p12 * p12, w1 = p02 * p02, w2 = p01 * p01;  // proportional to 1/s_k^2
+  const double w6 = 6.0 * w1, w2_3 = 3.0 * w2, w0_3 = 3.0 * w0;
+  // left-biased (linear weights 0.1 : 0.6 : 0.3), right-biased (0.3 : 0.6 : 0.1)
+  const double nL = fma(w0, fma(-2.0, dm2, 5.0 * dm1), fma(w6, fma(2.0, dp1, dm1), w2_3 * fma(4.0, dp1, -dp2)));
+  const double nR = fma(w0_3, fma(-4.0, dm1, dm2), fma(w6, fma(-2.0, dm1, -dp1), w2 * fma(2.0, dp2, -5.0 * dp1)));
+  const double rL = recip(w0 + w6 + w2_3), rR = recip(w0_3 + w6 + w2);
+  out[5] = nL * rL;
+  out[6] = rL;
+  out[7] = nR * rR;
+  out[8] = rR;
+  out[0] = fma(out[5], SIXTH, q0);
+  out[1] = fma(out[7], SIXTH, q0);
+  out[2] = s0;
+  out[3] = s1;
+  out[4] = s2;
+}
 
-  // start at cell i from q_{i-2}, q_{i-1}, q_i, q_{i+1}
-  __device__ __forceinline__ void init(double qm2, double qm1, double q, double qp1) {
-    q0 = q;
-    q1 = qp1;
-    dm2 = qm1 - qm2;
-    dm1 = q - qm1;
-    dp1 = qp1 - q;
-    D0 = dm1 - dm2;
-    D1 = dp1 - dm1;
-    cD0 = K13 * D0;
-    cD1 = K13 * D1;
-    f5m1 = 5.0 * dm1;
-    f5p1 = 5.0 * dp1;
+// POS: the variable is positive (density, pressure), see js_weno.cuh on its range
+template <bool POS>
+struct Win {
+  double q0, q1;       // q_i, q_{i+1}
+  Fx dm2, dm1, dp1;    // d_{i-3/2}, d_{i-1/2}, d_{i+1/2}
+  Sm s0, s1, s0n;      // indicators s_0, s_1 of cell i, s_0 of cell i+1
+
+  // start at the cell q points at (neighbours at multiples of st)
+  template <class I>
+  __device__ __forceinline__ void init(const double* q, I st) {
+    q0 = q[0];
+    q1 = q[st];
+    const double qm1 = q[-st];
+    dm2 = fx_of(qm1 - q[-2 * st]);
+    dm1 = fx_of(q0 - qm1);
+    dp1 = fx_of(q1 - q0);
+    Sm unused1, unused2;
+    sm_pair(dm2, dm1, unused1, s0, unused2);
+    sm_pair(dm1, dp1, s1, s0n, unused2);
   }
 
-  // given q_{i+2}: face states at i+1/2 (Lf, left-biased; if NL) and i-1/2 (Rf,
-  // right-biased; if NR), then slide to cell i+1.  With SV the internals the reverse pass
-  // needs go to sv[0..6] = s0, s1, s2, qL, rL, qR, rR (state = q_i + q/6, q = num r, r the
-  // reciprocal of den; zeros for a side not formed).
-  template <bool NL = true, bool NR = true, bool SV = false>
-  __device__ __forceinline__ void step(double q2, double& Lf, double& Rf, double* sv = nullptr) {
-    const double dp2 = q2 - q1;
-    const double D2 = dp2 - dp1;
-    const double cD2 = K13 * D2;
-    const double t0 = fma(2.0, dm1, D0);
-    const double t1 = dm1 + dp1;
-    const double t2 = fma(-2.0, dp1, D2);
-    const double s0 = fma(cD0, D0, fma(t0, t0, EPS4));
-    const double s1 = fma(cD1, D1, fma(t1, t1, EPS4));
-    const double s2 = fma(cD2, D2, fma(t2, t2, EPS4));
-    const double p01 = s0 * s1, p02 = s0 * s2, p12 = s1 * s2;
-    const double w0 = p12 * p12, w1 = p02 * p02, w2 = p01 * p01;  // proportional to 1/s_k^2
-    const double w1_6 = 6.0 * w1;
-    // left-biased (linear weights 0.1 : 0.6 : 0.3)
-    if (NL) {
-      const double w2_3 = 3.0 * w2;
-      const double e0 = fma(-2.0, dm2, f5m1);   // 2q_{i-2} - 7q_{i-1} + 5q_i
-      const double e1 = fma(2.0, dp1, dm1);     // -q_{i-1} - q_i + 2q_{i+1}
-      const double e2 = fma(4.0, dp1, -dp2);    // -4q_i + 5q_{i+1} - q_{i+2}
-      const double num = fma(w0, e0, fma(w1_6, e1, w2_3 * e2));
-      const double den = w0 + w1_6 + w2_3;
-      const double r = recip(den), q = num * r;  // = quot(num, den)
-      Lf = fma(q, SIXTH, q0);
-      if (SV) { sv[3] = q; sv[4] = r; }
-    } else if (SV) {
-      sv[3] = 0.0;
-      sv[4] = 0.0;
+  // cell i, at q: face states at i+1/2 (Lf, left-biased; if NL) and i-1/2 (Rf, right-biased; if
+  // NR), then slide to cell i+1.  With SV the internals the reverse pass needs go to
+  // sv[0..6] = 3 s0, 3 s1, 3 s2, cL, rL, cR, rR (state = q_i + c/6, c = num r, r the reciprocal
+  // of the weights' sum formed from the 3 s_k; zeros for a side not formed).
+  template <bool NL = true, bool NR = true, bool SV = false, class I>
+  __device__ __forceinline__ void step(const double* q, I st, double& Lf, double& Rf, double* sv = nullptr) {
+    const double q2 = q[2 * st];
+    const Fx dp2 = fx_of(q2 - q1);
+    Sm s1n, s0nn, s2;
+    sm_pair(dp1, dp2, s1n, s0nn, s2);
+    const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
+    const int lim = POS ? imin(expo(q0) + 3, 1500) : 1500;
+    double cL = 0.0, cR = 0.0, rL = 0.0, rR = 0.0;
+    if (F > lim && F > (POS ? 0 : 1500)) {
+      double out[9];
+      weno_plain(q[-2 * st], q[-st], q0, q1, q2, out);
+      Lf = out[0];
+      Rf = out[1];
+      if (SV) {
+#pragma unroll
+        for (int m = 0; m < 7; ++m) sv[m] = (m == 3 || m == 4) && !NL ? 0.0 : (m == 5 || m == 6) && !NR ? 0.0 : out[m + 2];
+      }
+    } else {
+      weno_corr<NL, NR, SV>(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR, rL, rR);
+      if (NL) Lf = fma(cL, SIXTH, q0);
+      if (NR) Rf = fma(cR, SIXTH, q0);
+      if (SV) {
+        sv[0] = sm_double(s0);
+        sv[1] = sm_double(s1);
+        sv[2] = sm_double(s2);
+        sv[3] = cL;
+        sv[4] = rL;
+        sv[5] = cR;
+        sv[6] = rR;
+      }
     }
-    // right-biased (linear weights 0.3 : 0.6 : 0.1)
-    const double f5p2 = 5.0 * dp2;
-    if (NR) {
-      const double w0_3 = 3.0 * w0;
-      const double e0 = fma(-4.0, dm1, dm2);    // -q_{i-2} + 5q_{i-1} - 4q_i
-      const double e1 = fma(-2.0, dm1, -dp1);   // 2q_{i-1} - q_i - q_{i+1}
-      const double e2 = fma(2.0, dp2, -f5p1);   // 5q_i - 7q_{i+1} + 2q_{i+2}
-      const double num = fma(w0_3, e0, fma(w1_6, e1, w2 * e2));
-      const double den = w0_3 + w1_6 + w2;
-      const double r = recip(den), q = num * r;  // = quot(num, den)
-      Rf = fma(q, SIXTH, q0);
-      if (SV) { sv[5] = q; sv[6] = r; }
-    } else if (SV) {
-      sv[5] = 0.0;
-      sv[6] = 0.0;
-    }
-    if (SV) { sv[0] = s0; sv[1] = s1; sv[2] = s2; }
     // slide
     q0 = q1;
     q1 = q2;
     dm2 = dm1;
     dm1 = dp1;
     dp1 = dp2;
-    D0 = D1;
-    D1 = D2;
-    cD0 = cD1;
-    cD1 = cD2;
-    f5m1 = f5p1;
-    f5p1 = f5p2;
+    s0 = s0n;
+    s1 = s1n;
+    s0n = s0nn;
+  }
+};
+
+// the windows of the four primitive variables along a line (planes ps apart)
+struct Win4 {
+  Win<true> r;
+  Win<false> u, v;
+  Win<true> p;
+  template <class I, class P>
+  __device__ __forceinline__ void init(const double* q, P ps, I st) {
+    r.init(q, st);
+    u.init(q + ps, st);
+    v.init(q + 2 * ps, st);
+    p.init(q + 3 * ps, st);
+  }
+  // keep(c, sv) receives the internals of variable c (SV)
+  template <bool NL, bool NR, bool SV, class I, class P, class Keep>
+  __device__ __forceinline__ void step(const double* q, P ps, I st, double Lf[4], double Rf[4], Keep&& keep) {
+    double sv[SV ? 7 : 1];
+    r.template step<NL, NR, SV>(q, st, Lf[0], Rf[0], sv);
+    if (SV) keep(0, sv);
+    u.template step<NL, NR, SV>(q + ps, st, Lf[1], Rf[1], sv);
+    if (SV) keep(1, sv);
+    v.template step<NL, NR, SV>(q + 2 * ps, st, Lf[2], Rf[2], sv);
+    if (SV) keep(2, sv);
+    p.template step<NL, NR, SV>(q + 3 * ps, st, Lf[3], Rf[3], sv);
+    if (SV) keep(3, sv);
   }
 };
 

@@ -71,18 +71,13 @@ __device__ __forceinline__ void face_states(const Lay& L, const double* Q, long 
                                             double wl[4], double wr[4]) {
   const long long st = (d == 0) ? 1 : L.pitch;
   const long long cf = (d == 0) ? L.idx(f, h) : L.idx(h, f);
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const double* q = Q + c * qplane + cf;
-    const double qm3 = q[-3 * st], qm2 = q[-2 * st], qm1 = q[-st], q0 = q[0], qp1 = q[st], qp2 = q[2 * st];
-    double dummy;
-    Win a;
-    a.init(qm3, qm2, qm1, q0);
-    a.step<true, false>(qp1, wl[c], dummy);
-    Win b;
-    b.init(qm2, qm1, q0, qp1);
-    b.step<false, true>(qp2, dummy, wr[c]);
-  }
+  const double* q = Q + cf;
+  double dummy[4];
+  auto none = [](int, const double*) {};
+  Win4 w;
+  w.init(q - st, qplane, st);
+  w.template step<true, false, false>(q - st, qplane, st, wl, dummy, none);
+  w.template step<false, true, false>(q, qplane, st, dummy, wr, none);
 }
 
 // the same face states from the stage's stored WENO5 internals: state = q_cell + q/6 with the

@@ -37,43 +37,25 @@ __device__ __forceinline__ void sweep_line(const double* __restrict__ sq, int ps
   constexpr bool FI = !std::is_same<Face, NoFace>::value;
   constexpr int PN = (DIR == 0) ? 1 : 2;  // plane of the face-normal velocity
   constexpr int PT = (DIR == 0) ? 2 : 1;  // plane of the tangential velocity
-  Win w[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const double* q = sq + c * ps;
-    w[c].init(q[base - 3 * st], q[base - 2 * st], q[base - st], q[base]);
-  }
+  Win4 w;
+  w.init(sq + base - st, ps, st);
   double prevL[4], prevF[4];
   {
     // cell -1 of the segment: only its right-face (left-biased) state is needed
     double Rf[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      double sv[SV ? 7 : 1];
-      w[c].template step<true, false, SV>(sq[c * ps + base - st + 2 * st], prevL[c], Rf[c], sv);
-      if (SV) keep(-1, c, sv);
-    }
+    w.template step<true, false, SV>(sq + base - st, ps, st, prevL, Rf, [&](int c, const double* sv) { if constexpr (SV) keep(-1, c, sv); });
   }
 #pragma unroll 1
   for (int k = 0; k <= L; ++k) {
     const int cell = base + k * st;
     double Lf[4], Rf[4];
     if (k < L) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        double sv[SV ? 7 : 1];
-        w[c].template step<true, true, SV>(sq[c * ps + cell + 2 * st], Lf[c], Rf[c], sv);
-        if (SV) keep(k, c, sv);
-      }
+      w.template step<true, true, SV>(sq + cell, ps, st, Lf, Rf, [&](int c, const double* sv) { if constexpr (SV) keep(k, c, sv); });
     } else {
       // cell L (first cell of the next segment): only its left-face state is needed
+      w.template step<false, true, SV>(sq + cell, ps, st, Lf, Rf, [&](int c, const double* sv) { if constexpr (SV) keep(L, c, sv); });
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        double sv[SV ? 7 : 1];
-        w[c].template step<false, true, SV>(sq[c * ps + cell + 2 * st], Lf[c], Rf[c], sv);
-        if (SV) keep(L, c, sv);
-        Lf[c] = 0.0;  // unused
-      }
+      for (int c = 0; c < 4; ++c) Lf[c] = 0.0;  // unused
     }
     {
       // face k - 1/2 between cells k-1 (left state prevL) and k (right state Rf)
