@@ -29,12 +29,10 @@
 
 namespace js {
 
-// the per-grid default tile (variant 0): 32x32 cells, concurrent x/y sweeps
-constexpr int BTX = 32, BTY = 32, BLX = 16, BLY = 16;
-using BStageV = Stage2DC<BTX, BTY, BLX, BLY, true>;
-using BStageE = Stage2DC<BTX, BTY, BLX, BLY, false>;
-constexpr int BNT = BStageV::NT;
-static_assert(BStageV::NT == BStageE::NT && BNT % 32 == 0, "one block shape for both physics");
+// the per-grid tile; the forward launch runs 7 warps a block like the per-grid kernel, the
+// reverse launches 4 (their other phases hold more registers)
+constexpr int BTX = TILE, BTY = TILE;
+constexpr int FNT = 224, BNT = 128;
 
 struct BatchArgs {
   const InstDesc* inst;
@@ -126,7 +124,7 @@ __device__ __forceinline__ double inst_dt(const InstDesc& d, const unsigned long
   return dt;
 }
 
-__global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
+__global__ void __launch_bounds__(FNT, 3) batch_kernel(BatchArgs b) {
   extern __shared__ double smem[];
   const int ntiles = b.tile0[b.count];
   const long long nghost = b.ghost0[b.count], nhalo = b.halo0[b.count];
@@ -140,7 +138,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
     const int t = q - b.tile0[k];
     const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
     const long long n = (long long)d.lay.nx * d.lay.ny;
-    for (int e = tid; e < BTX * BTY; e += BNT) {
+    for (int e = tid; e < BTX * BTY; e += FNT) {
       const int i = i0 + (e % BTX), j = j0 + (e / BTX);
       if (i >= d.lay.nx || j >= d.lay.ny) continue;
       const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
@@ -149,7 +147,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
     }
   }
   if (blockIdx.x == 0)
-    for (int k = tid; k < 2 * b.count; k += BNT) {
+    for (int k = tid; k < 2 * b.count; k += FNT) {
       b.red[2 * k] = 0ULL;
       b.red[2 * k + 1] = 0x7ff0000000000000ULL;
     }
@@ -165,7 +163,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
       const int t = q - b.tile0[k];
       const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
       double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
-      for (int e = tid; e < BTX * BTY; e += BNT) {
+      for (int e = tid; e < BTX * BTY; e += FNT) {
         const int i = i0 + (e % BTX), j = j0 + (e / BTX);
         if (i >= d.lay.nx || j >= d.lay.ny) continue;
         if (d.tag && d.tag[(long long)j * d.lay.nx + i] != 0) continue;
@@ -188,7 +186,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
     if (blockIdx.x == 0) {
       // the other parity was last read in the previous step: reset it for the next one
       unsigned long long* nxt = b.red + 2 * (long long)b.count * (par ^ 1);
-      for (int k = tid; k < b.count; k += BNT) {
+      for (int k = tid; k < b.count; k += FNT) {
         nxt[2 * k] = 0ULL;
         nxt[2 * k + 1] = 0x7ff0000000000000ULL;
         const double dtk = b.dt_in ? b.dt_in[(long long)step * b.count + k] : inst_dt(b.inst[k], red + 2 * k, b.cfl);
@@ -200,7 +198,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
     }
     for (int s = 0; s < 3; ++s) {
       // ---- immersed-boundary ghosts of the stage input
-      for (long long g = (long long)blockIdx.x * BNT + tid; g < nghost; g += (long long)gridDim.x * BNT) {
+      for (long long g = (long long)blockIdx.x * FNT + tid; g < nghost; g += (long long)gridDim.x * FNT) {
         const int k = find_inst64(b.ghost0, b.count, g);
         const InstDesc& d = b.inst[k];
         double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
@@ -208,7 +206,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
       }
       if (!grid_sync(b)) return;
       // ---- domain halos
-      for (long long h = (long long)blockIdx.x * BNT + tid; h < nhalo; h += (long long)gridDim.x * BNT) {
+      for (long long h = (long long)blockIdx.x * FNT + tid; h < nhalo; h += (long long)gridDim.x * FNT) {
         const int k = find_inst64(b.halo0, b.count, h);
         const InstDesc& d = b.inst[k];
         double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
@@ -227,8 +225,6 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
         a.Un = d.N;
         a.Uout = (s == 0) ? d.A : ((s == 1) ? d.B : d.N);
         a.tag = d.tag;
-        a.acc = d.acc;
-        a.acc2 = d.acc2;
         a.dtc = nullptr;
         a.err = b.err;
         a.lay = d.lay;
@@ -245,8 +241,8 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
         a.vy = d.vy;
         a.use_un = (s > 0) ? 1 : 0;
         a.has_av = d.has_av;
-        if (d.visc) stage_tile_c<BTX, BTY, BLX, BLY, true, false>(a, t % d.ntx, t / d.ntx, smem);
-        else stage_tile_c<BTX, BTY, BLX, BLY, false, false>(a, t % d.ntx, t / d.ntx, smem);
+        if (d.visc) stage_tile<true, false>(a, t % d.ntx, t / d.ntx, smem);
+        else stage_tile<false, false>(a, t % d.ntx, t / d.ntx, smem);
         __syncthreads();  // the next tile reuses shared memory
       }
       if (!grid_sync(b)) return;
@@ -266,7 +262,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
         const int t = q - b.tile0[k];
         const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
         const long long n = (long long)d.lay.nx * d.lay.ny;
-        for (int e = tid; e < BTX * BTY; e += BNT) {
+        for (int e = tid; e < BTX * BTY; e += FNT) {
           const int i = i0 + (e % BTX), j = j0 + (e / BTX);
           if (i >= d.lay.nx || j >= d.lay.ny) continue;
           const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
@@ -292,7 +288,7 @@ __global__ void __launch_bounds__(BNT) batch_kernel(BatchArgs b) {
     const int t = q - b.tile0[k];
     const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
     const long long n = (long long)d.lay.nx * d.lay.ny;
-    for (int e = tid; e < BTX * BTY; e += BNT) {
+    for (int e = tid; e < BTX * BTY; e += FNT) {
       const int i = i0 + (e % BTX), j = j0 + (e / BTX);
       if (i >= d.lay.nx || j >= d.lay.ny) continue;
       const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
@@ -508,8 +504,6 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       a.Un = d.N;
       a.Uout = (s == 0) ? d.A : d.B;
       a.tag = d.tag;
-      a.acc = d.acc;
-      a.acc2 = d.acc2;
       a.err = b.err;
       a.lay = d.lay;
       a.gamma = d.gamma;
@@ -529,8 +523,8 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       a.splane = r.a.splane;
       a.tpitch = r.a.tpitch;
       a.dtc = nullptr;
-      if (d.visc) stage_tile_c<BTX, BTY, BLX, BLY, true, false, false, true>(a, t % d.ntx, t / d.ntx, smem);
-      else stage_tile_c<BTX, BTY, BLX, BLY, false, false, false, true>(a, t % d.ntx, t / d.ntx, smem);
+      if (d.visc) stage_tile<true, false, false, true>(a, t % d.ntx, t / d.ntx, smem);
+      else stage_tile<false, false, false, true>(a, t % d.ntx, t / d.ntx, smem);
       __syncthreads();  // the next tile reuses shared memory
     }
   } else if constexpr (PH == RP_SEED) {
@@ -733,7 +727,7 @@ void js_internal_desc(js_ctx* c, js::InstDesc* d);
 int js_internal_rev_desc(js_ctx* c, js::InstRev* d);
 
 namespace {
-size_t batch_smem() { return js::BStageV::SMEM > js::BStageE::SMEM ? js::BStageV::SMEM : js::BStageE::SMEM; }
+size_t batch_smem() { return js::StageTile<true>::SMEM; }
 }  // namespace
 
 namespace {
@@ -956,7 +950,7 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, js::batch_kernel, js::BNT, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, js::batch_kernel, js::FNT, smem);
   if (!coop || per_sm < 1) { js_batch_destroy(b); return JS_ERR_CUDA; }
   b->sms = sms;
   b->per_sm = per_sm;
@@ -1029,7 +1023,7 @@ static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, dou
   cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
   a.budget = (long long)(budget_s * 1e3 * (khz > 0 ? khz : 2000000));
   void* args[] = {&a};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)js::batch_kernel, dim3(b->blocks), dim3(js::BNT), args,
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)js::batch_kernel, dim3(b->blocks), dim3(js::FNT), args,
                                                     batch_smem(), b->stream);
   return e == cudaSuccess ? JS_OK : JS_ERR_CUDA;
 }

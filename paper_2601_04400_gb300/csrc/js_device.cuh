@@ -177,7 +177,7 @@ struct Win {
     const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
     const int lim = POS ? imin(expo(q0) + 3, 1500) : 1500;
     double cL = 0.0, cR = 0.0, rL = 0.0, rR = 0.0;
-    if (F > lim && F > (POS ? 0 : 1500)) {
+    if (F > lim) {
       double out[9];
       weno_plain(q[-2 * st], q[-st], q0, q1, q2, out);
       Lf = out[0];
@@ -211,6 +211,50 @@ struct Win {
     s0n = s0nn;
   }
 };
+
+// The same for one cell per lane: the lanes of a warp hold consecutive cells of a line, q points
+// at the lane's own (q[-st .. st] readable; q[-2 st], q[2 st] too in the inner lanes).  A lane
+// forms the differences on both sides of its cell and the three indicators they determine, and
+// takes its s_0, s_2 and outer differences from its neighbours.  Valid in lanes 1..30 (inner).
+template <bool SV>
+__device__ __forceinline__ void weno_lane(const double* q, int st, bool pos, bool inner, double& Lf, double& Rf,
+                                          double* sv) {
+  const double q0 = q[0];
+  const Fx dm1 = fx_of(q0 - q[-st]), dp1 = fx_of(q[st] - q0);
+  Sm s1, s0n, s2p;
+  sm_pair(dm1, dp1, s1, s0n, s2p);
+  const Sm s0{(u64)__shfl_up_sync(0xffffffffu, (unsigned long long)s0n.m, 1), __shfl_up_sync(0xffffffffu, s0n.x, 1)};
+  const Sm s2{(u64)__shfl_down_sync(0xffffffffu, (unsigned long long)s2p.m, 1),
+              __shfl_down_sync(0xffffffffu, s2p.x, 1)};
+  const Fx dm2{(s64)__shfl_up_sync(0xffffffffu, (long long)dm1.m, 1), __shfl_up_sync(0xffffffffu, dm1.e, 1)};
+  const Fx dp2{(s64)__shfl_down_sync(0xffffffffu, (long long)dp1.m, 1), __shfl_down_sync(0xffffffffu, dp1.e, 1)};
+  const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
+  const int lim = pos ? imin(expo(q0) + 3, 1500) : 1500;
+  if (F > lim && inner) {
+    double out[9];
+    weno_plain(q[-2 * st], q[-st], q0, q[st], q[2 * st], out);
+    Lf = out[0];
+    Rf = out[1];
+    if (SV) {
+#pragma unroll
+      for (int m = 0; m < 7; ++m) sv[m] = out[m + 2];
+    }
+  } else {
+    double cL, cR, rL, rR;
+    weno_corr<true, true, SV>(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR, rL, rR);
+    Lf = fma(cL, SIXTH, q0);
+    Rf = fma(cR, SIXTH, q0);
+    if (SV) {
+      sv[0] = sm_double(s0);
+      sv[1] = sm_double(s1);
+      sv[2] = sm_double(s2);
+      sv[3] = cL;
+      sv[4] = rL;
+      sv[5] = cR;
+      sv[6] = rR;
+    }
+  }
+}
 
 // the windows of the four primitive variables along a line (planes ps apart)
 struct Win4 {

@@ -3,8 +3,8 @@
 //   ib_fill      ghost-cell immersed boundary: slip-wall mirror of the bilinear image-point
 //                interpolation of fluid cells (Sec. 2, Fig. 1(c))
 //   stage2d      one fused kernel per Runge-Kutta stage: conserved tile + halo -> primitives
-//                in shared memory -> x sweep (WENO5, HLLC, viscous flux, divergence) into a
-//                shared accumulator -> y sweep, RK stage combination, store
+//                in shared memory -> fluxes of the x lines, then of the y lines (WENO5, HLLC,
+//                viscous flux, divergence) into a shared accumulator -> RK stage combination
 //   stage1d      the same along a single line (ny == 1)
 //   cfl_reduce   maximum wave speed and minimum density (bit-exact IEEE arithmetic)
 #include <cuda_runtime.h>
@@ -288,62 +288,45 @@ __device__ __forceinline__ bool stage_constants(const StageArgs& a0, StageArgs& 
   return a0.dtc[4] != 0.0;
 }
 
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS>
-__global__ void __launch_bounds__(Stage2D<TX, TY, LX, LY, VISC, RHS>::NT)
-stage2d_kernel(StageArgs a0) {
-  StageArgs a;
-  if (!stage_constants(a0, a)) return;
-  extern __shared__ double smem[];
-  stage_tile<TX, TY, LX, LY, VISC, RHS>(a, blockIdx.x, blockIdx.y, smem);
-}
-
-// persistent concurrent-sweep stage kernel: blocks stride over the tiles; with SAVE the
-// WENO5 internals of the stage go to a.wsave for the reverse pass
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS, bool SAVE, bool IMG = false>
-__global__ void __launch_bounds__(Stage2DC<TX, TY, LX, LY, VISC>::NT, SAVE ? 3 : 1)
-stage2dc_kernel(StageArgs a0, int ntx, int ntiles) {
-  StageArgs a;
-  if (!stage_constants(a0, a)) return;
-  extern __shared__ double smem[];
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    stage_tile_c<TX, TY, LX, LY, VISC, RHS, false, SAVE, IMG>(a, t % ntx, t / ntx, smem);
-    __syncthreads();
-  }
-}
-
-// the same with the tile staged by TMA (tensor map of the stage input as a grid constant)
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS, bool SAVE, bool IMG = false>
-__global__ void __launch_bounds__(Stage2DC<TX, TY, LX, LY, VISC, true>::NT, SAVE ? 3 : 1)
-stage2dc_tma_kernel(StageArgs a0, int ntx, int ntiles, const __grid_constant__ TensorMap128 tmap) {
+// persistent stage kernel of NW warps a block: blocks stride over the tiles, staged by TMA (tensor
+// map of the stage input as a grid constant) or by plain loads; with SAVE the WENO5 internals of
+// the stage go to a.wsave for the reverse pass, with IMG the neural flux's face images to a.img.
+// 7 warps (4 lines each in both directions), 3 blocks an SM: 21 warps at 96 registers.  14 warps
+// for grids of few tiles, where a tile's latency counts.
+template <int NW, bool VISC, bool RHS, bool TMA, bool SAVE, bool IMG>
+__global__ void __launch_bounds__(32 * NW, NW == 7 ? 3 : 1)
+stage2d_kernel(StageArgs a0, int ntx, int ntiles, const __grid_constant__ TensorMap128 tmap) {
   StageArgs a;
   if (!stage_constants(a0, a)) return;
   extern __shared__ __align__(128) double smem[];
   __shared__ __align__(8) unsigned long long bar;
-  if (threadIdx.x == 0) mbar_init(&bar);
-  __syncthreads();
+  if (TMA) {
+    if (threadIdx.x == 0) mbar_init(&bar);
+    __syncthreads();
+  }
   unsigned phase = 0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    stage_tile_c<TX, TY, LX, LY, VISC, RHS, true, SAVE, IMG>(a, t % ntx, t / ntx, smem, &tmap, &bar, &phase);
+    stage_tile<VISC, RHS, TMA, SAVE, IMG>(a, t % ntx, t / ntx, smem, &tmap, &bar, &phase);
     __syncthreads();
   }
 }
 
-template <int TX, int LX, bool VISC, bool RHS>
-__global__ void __launch_bounds__(TX / LX) stage1d_kernel(StageArgs a0) {
+// one line (ny == 1): a warp per 28 cells
+template <bool VISC, bool RHS>
+__global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
   StageArgs a;
   if (!stage_constants(a0, a)) return;
   constexpr int NPL = VISC ? 5 : 4;
-  constexpr int PS = TX + 6;
-  constexpr int NT = TX / LX;
+  constexpr int PS = TILE_B;
   __shared__ double sq[NPL * PS];
   const Gas g{a.gamma, a.gm1, a.g1};
-  const int tx0 = blockIdx.x * TX;
+  const int tx0 = blockIdx.x * TILE, lane = threadIdx.x;
   const int W = a.lay.nx + 6;
-  for (int col = threadIdx.x; col < PS; col += NT) {
-    int gx = tx0 + col;
-    gx = (gx < W) ? gx : W - 1;
-    const double r = a.Uin[gx], mx = a.Uin[a.lay.plane + gx], my = a.Uin[2 * a.lay.plane + gx],
-                 E = a.Uin[3 * a.lay.plane + gx];
+  for (int col = lane; col < PS; col += 32) {
+    const int gx = tx0 + col;
+    const int gc = (gx < W) ? gx : W - 1;
+    const double r = a.Uin[gc], mx = a.Uin[a.lay.plane + gc], my = a.Uin[2 * a.lay.plane + gc],
+                 E = a.Uin[3 * a.lay.plane + gc];
     double u, v, p, T;
     cons_to_prim(r, mx, my, E, g, u, v, p, T);
     sq[col] = r;
@@ -352,124 +335,70 @@ __global__ void __launch_bounds__(TX / LX) stage1d_kernel(StageArgs a0) {
     sq[3 * PS + col] = p;
     if (NPL == 5) sq[4 * PS + col] = T;
   }
-  __syncthreads();
-  const int xs = threadIdx.x * LX;
-  const double zero[4] = {0.0, 0.0, 0.0, 0.0};
-  sweep_line<0, VISC, false, LX>(sq, PS, xs + 3, 1, 0, g, a.vx, [&](int k, const double dF[4]) {
-    const int gi = tx0 + xs + k;
-    if (gi < a.lay.nx) {
-      finish_cell<RHS>(a, gi, 0, dF, zero, sq[xs + k + 3], sq[3 * PS + xs + k + 3]);
-    }
-  });
+  __syncwarp();
+  const int k = lane - 2, gi = tx0 + k;
+  double dF[4], upd[4];
+  line_fluxes<VISC, false>(sq + k + 3, PS, 1, 0, 1, g, a.vx, dF);
+  if (lane < 2 || lane > 29 || gi >= a.lay.nx) return;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) upd[c] = fma(-a.cx, dF[c], RHS ? 0.0 : a.Uin[c * a.lay.plane + a.lay.idx(gi, 0)]);
+  finish_cell<RHS>(a, gi, 0, upd, sq[k + 3], sq[3 * PS + k + 3]);
 }
 
 // =======================================================================================
 // launchers
 // =======================================================================================
 namespace {
-// 1D grids are small (a few hundred cells): short segments, so that more threads share the
-// latency-bound sweep
-constexpr int TX1 = 32, LX1 = 4;
-
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS>
-cudaError_t launch_stage2d(const StageArgs& a, cudaStream_t s) {
-  using S = Stage2D<TX, TY, LX, LY, VISC, RHS>;
-  auto k = stage2d_kernel<TX, TY, LX, LY, VISC, RHS>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  dim3 grid((a.lay.nx + TX - 1) / TX, (a.lay.ny + TY - 1) / TY);
-  k<<<grid, S::NT, S::SMEM, s>>>(a);
-  return cudaGetLastError();
-}
-
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS, bool SAVE = false, bool IMG = false>
-cudaError_t launch_stage2dc(const StageArgs& a, cudaStream_t s) {
-  using S = Stage2DC<TX, TY, LX, LY, VISC>;
-  auto k = stage2dc_kernel<TX, TY, LX, LY, VISC, RHS, SAVE, IMG>;
-  constexpr size_t SM = S::SMEM;
+template <int NW, bool VISC, bool RHS, bool TMA, bool SAVE, bool IMG>
+cudaError_t launch_stage2d_nw(const StageArgs& a, const TensorMap128* tmap, int ntx, int ntiles, cudaStream_t s) {
+  using S = StageTile<VISC>;
+  auto k = stage2d_kernel<NW, VISC, RHS, TMA, SAVE, IMG>;
   static int resident = 0;  // blocks resident on the whole GPU
   if (resident == 0) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, S::NT, SM);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * NW, S::SMEM);
     if (e != cudaSuccess) return e;
     resident = sms * (per_sm > 0 ? per_sm : 1);
   }
-  const int ntx = (a.lay.nx + TX - 1) / TX, nty = (a.lay.ny + TY - 1) / TY;
-  const int ntiles = ntx * nty;
-  k<<<ntiles < resident ? ntiles : resident, S::NT, SM, s>>>(a, ntx, ntiles);
+  static const TensorMap128 none{};
+  k<<<ntiles < resident ? ntiles : resident, 32 * NW, S::SMEM, s>>>(a, ntx, ntiles, TMA ? *tmap : none);
   return cudaGetLastError();
 }
 
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS, bool SAVE = false, bool IMG = false>
-cudaError_t launch_stage2dc_tma(const StageArgs& a, const TensorMap128* tmap, cudaStream_t s) {
-  using S = Stage2DC<TX, TY, LX, LY, VISC, true>;
-  auto k = stage2dc_tma_kernel<TX, TY, LX, LY, VISC, RHS, SAVE, IMG>;
-  constexpr size_t SM = S::SMEM;
-  static int resident = 0;
-  if (resident == 0) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, S::NT, SM);
-    if (e != cudaSuccess) return e;
-    resident = sms * (per_sm > 0 ? per_sm : 1);
+template <bool VISC, bool RHS, bool SAVE = false, bool IMG = false>
+cudaError_t launch_stage2d(const StageArgs& a, int variant, const TensorMap128* tmap, cudaStream_t s) {
+  const int ntx = (a.lay.nx + TILE - 1) / TILE, nty = (a.lay.ny + TILE - 1) / TILE, ntiles = ntx * nty;
+  if constexpr (!SAVE && !IMG) {
+    // blocks of 14 warps take a tile in half the time; worth it while every tile has its SM
+    const bool wide = variant == 2 || variant == 3 || (variant != 1 && variant != 4 && ntiles <= 152);
+    if (wide)
+      return tmap ? launch_stage2d_nw<14, VISC, RHS, true, SAVE, IMG>(a, tmap, ntx, ntiles, s)
+                  : launch_stage2d_nw<14, VISC, RHS, false, SAVE, IMG>(a, tmap, ntx, ntiles, s);
   }
-  const int ntx = (a.lay.nx + TX - 1) / TX, nty = (a.lay.ny + TY - 1) / TY;
-  const int ntiles = ntx * nty;
-  k<<<ntiles < resident ? ntiles : resident, S::NT, SM, s>>>(a, ntx, ntiles, *tmap);
-  return cudaGetLastError();
-}
-
-// tile shapes (TX x TY cells, x / y segment lengths LX / LY) the tuner chooses from:
-// 0 concurrent sweeps with TMA staging, 1-3 concurrent sweeps with plain loads in
-// persistent blocks, 4 sequential sweeps in one warp per tile
-template <bool VISC, bool RHS>
-cudaError_t launch_stage2d_variant(const StageArgs& a, int variant, const TensorMap128* tmap, cudaStream_t s) {
-  switch (variant) {
-    case 1: return launch_stage2dc<32, 32, 16, 16, VISC, RHS>(a, s);
-    case 2: return launch_stage2dc<32, 16, 16, 16, VISC, RHS>(a, s);
-    case 3: return launch_stage2dc<64, 16, 16, 16, VISC, RHS>(a, s);
-    case 4: return launch_stage2d<32, 16, 16, 16, VISC, RHS>(a, s);
-    default:
-      if (tmap == nullptr) return launch_stage2dc<32, 32, 16, 16, VISC, RHS>(a, s);
-      return launch_stage2dc_tma<32, 32, 16, 16, VISC, RHS>(a, tmap, s);
-  }
+  return tmap ? launch_stage2d_nw<7, VISC, RHS, true, SAVE, IMG>(a, tmap, ntx, ntiles, s)
+              : launch_stage2d_nw<7, VISC, RHS, false, SAVE, IMG>(a, tmap, ntx, ntiles, s);
 }
 
 template <bool VISC, bool RHS>
 cudaError_t launch_stage1d(const StageArgs& a, cudaStream_t s) {
-  dim3 grid((a.lay.nx + TX1 - 1) / TX1);
-  stage1d_kernel<TX1, LX1, VISC, RHS><<<grid, TX1 / LX1, 0, s>>>(a);
+  stage1d_kernel<VISC, RHS><<<(a.lay.nx + TILE - 1) / TILE, 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 }  // namespace
 
 cudaError_t launch_stage_save(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s) {
   if (a.lay.ny == 1 || a.wsave == nullptr) return cudaErrorInvalidValue;
-  if (tmap != nullptr)
-    return visc ? launch_stage2dc_tma<32, 32, 16, 16, true, false, true>(a, tmap, s)
-                : launch_stage2dc_tma<32, 32, 16, 16, false, false, true>(a, tmap, s);
-  return visc ? launch_stage2dc<32, 32, 16, 16, true, false, true>(a, s)
-              : launch_stage2dc<32, 32, 16, 16, false, false, true>(a, s);
+  return visc ? launch_stage2d<true, false, true>(a, 0, tmap, s) : launch_stage2d<false, false, true>(a, 0, tmap, s);
 }
 
 cudaError_t launch_stage_img(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s) {
   if (a.lay.ny == 1 || a.img == nullptr) return cudaErrorInvalidValue;
-  if (tmap != nullptr)
-    return visc ? launch_stage2dc_tma<32, 32, 16, 16, true, false, false, true>(a, tmap, s)
-                : launch_stage2dc_tma<32, 32, 16, 16, false, false, false, true>(a, tmap, s);
-  return visc ? launch_stage2dc<32, 32, 16, 16, true, false, false, true>(a, s)
-              : launch_stage2dc<32, 32, 16, 16, false, false, false, true>(a, s);
+  return visc ? launch_stage2d<true, false, false, true>(a, 0, tmap, s)
+              : launch_stage2d<false, false, false, true>(a, 0, tmap, s);
 }
 
 cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, const TensorMap128* tmap,
@@ -479,10 +408,8 @@ cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, c
     return rhs ? launch_stage1d<false, true>(a, s) : launch_stage1d<false, false>(a, s);
   }
   if (visc)
-    return rhs ? launch_stage2d_variant<true, true>(a, variant, tmap, s)
-               : launch_stage2d_variant<true, false>(a, variant, tmap, s);
-  return rhs ? launch_stage2d_variant<false, true>(a, variant, tmap, s)
-             : launch_stage2d_variant<false, false>(a, variant, tmap, s);
+    return rhs ? launch_stage2d<true, true>(a, variant, tmap, s) : launch_stage2d<true, false>(a, variant, tmap, s);
+  return rhs ? launch_stage2d<false, true>(a, variant, tmap, s) : launch_stage2d<false, false>(a, variant, tmap, s);
 }
 
 cudaError_t launch_bc_fill(double* U, const Lay& lay, const BcArgs& bc, cudaStream_t s) {

@@ -28,8 +28,6 @@ struct js_ctx {
   double* N = nullptr;  // padded U^n / step output
   double* A = nullptr;  // padded stage buffers
   double* B = nullptr;
-  double* acc = nullptr;   // stage scratch [4][ny][nx]: x-flux differences
-  double* acc2 = nullptr;  // y-flux differences
   unsigned char* tag = nullptr;       // device [ny][nx] or null (no immersed body)
   std::vector<unsigned char> tag_host;
   int n_ghost = 0;
@@ -286,8 +284,6 @@ StageArgs base_args(const js_ctx* c) {
   StageArgs a;
   std::memset(&a, 0, sizeof(a));
   a.tag = c->tag;
-  a.acc = c->acc;
-  a.acc2 = c->acc2;
   a.err = c->err;
   a.lay = c->lay;
   a.gamma = c->p.gamma;
@@ -331,7 +327,7 @@ EncodeTiledFn encode_tiled() {
 }
 
 // Tensor map of a padded state buffer: 3D (column, row, plane) FP64 tensor, box of the
-// 32x32 tile with its 3-cell halo and all 4 planes; reads past the array return zeros.
+// 28x28 tile with its 3-cell halo and all 4 planes; reads past the array return zeros.
 const js::TensorMap128* stage_tmap(js_ctx* c, const double* buf) {
   if (c->lay.ny == 1) return nullptr;
   for (auto& e : c->tmaps)
@@ -342,7 +338,7 @@ const js::TensorMap128* stage_tmap(js_ctx* c, const double* buf) {
   js::TensorMap128 m;
   const cuuint64_t dims[3] = {(cuuint64_t)c->lay.pitch, (cuuint64_t)c->lay.H, 4};
   const cuuint64_t strides[2] = {(cuuint64_t)c->lay.pitch * sizeof(double), (cuuint64_t)c->lay.plane * sizeof(double)};
-  const cuuint32_t box[3] = {js::TMA_TX + 6, js::TMA_TY + 6, 4};
+  const cuuint32_t box[3] = {js::TMA_BOX, js::TMA_BOX, 4};
   const cuuint32_t estr[3] = {1, 1, 1};
   const CUresult r = enc(reinterpret_cast<CUtensorMap*>(&m), CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)buf, dims,
                          strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -434,7 +430,8 @@ int stage(js_ctx* c, const StageArgs& a, bool visc, bool rhs) {
   if (rc) return rc;
   const bool timed = c->profiling && c->ev_used + 2 <= (int)c->ev.size();
   if (timed) JS_CUDA(cudaEventRecord(c->ev[c->ev_used], c->stream));
-  const js::TensorMap128* tm = (c->variant == 0) ? stage_tmap(c, a.Uin) : nullptr;
+  // tile variants: 0 the library's choice, 1 / 3 plain loads, 2 / 4 TMA; 1, 4: 7 warps a block, 2, 3: 14
+  const js::TensorMap128* tm = (c->variant != 1 && c->variant != 3) ? stage_tmap(c, a.Uin) : nullptr;
   JS_CUDA(js::launch_stage(a, visc, rhs, c->variant, tm, c->stream));
   if (timed) {
     JS_CUDA(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
@@ -463,8 +460,6 @@ void js_internal_desc(js_ctx* c, js::InstDesc* d) {
   d->N = c->N;
   d->A = c->A;
   d->B = c->B;
-  d->acc = c->acc;
-  d->acc2 = c->acc2;
   d->tag = c->tag;
   d->ib = ib_args(c);
   d->bc = c->bc;
@@ -502,7 +497,7 @@ const char* js_strerror(int code) {
 void js_destroy(js_ctx* c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream); else cudaDeviceSynchronize();
-  cudaFree(c->N); cudaFree(c->A); cudaFree(c->B); cudaFree(c->acc); cudaFree(c->acc2);
+  cudaFree(c->N); cudaFree(c->A); cudaFree(c->B);
   cudaFree(c->tag);
   cudaFree(c->ib_dst); cudaFree(c->ib_src); cudaFree(c->ib_w); cudaFree(c->ib_nrm);
   cudaFree(c->err); cudaFree(c->red); cudaFree(c->cfl_bmax); cudaFree(c->dtc);
@@ -560,8 +555,6 @@ int create_ctx(const js_grid* grid, const js_params* params, const js_boundary* 
   const size_t bytes = sizeof(double) * 4 * (size_t)L.plane;
   if (cudaMalloc(&c->N, bytes) != cudaSuccess || cudaMalloc(&c->A, bytes) != cudaSuccess ||
       cudaMalloc(&c->B, bytes) != cudaSuccess || cudaMalloc(&c->err, sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&c->acc, sizeof(double) * 4 * (size_t)grid->nx * grid->ny) != cudaSuccess ||
-      cudaMalloc(&c->acc2, sizeof(double) * 4 * (size_t)grid->nx * grid->ny) != cudaSuccess ||
       cudaMalloc(&c->red, 4 * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMalloc(&c->cfl_bmax, sizeof(double) * js::CFL_MAX_BLOCKS) != cudaSuccess ||
       cudaMalloc(&c->dtc, sizeof(double) * js::DTC_N) != cudaSuccess) {

@@ -11,8 +11,6 @@ struct StageArgs {
   const double* Un;          // padded U^n (RK combination), may alias Uout
   double* Uout;              // padded stage output, or [4][ny][nx] in RHS mode
   const unsigned char* tag;  // [ny][nx] cell tags (0 fluid) or nullptr
-  double* acc;               // [4][ny][nx] scratch: x-flux differences of the stage
-  double* acc2;              // [4][ny][nx] scratch: y-flux differences (concurrent sweeps)
   int* err;                  // device error flag
   Lay lay;
   double gamma, gm1, g1;
@@ -175,8 +173,6 @@ struct InstDesc {
   double* A;
   double* B;
   double* U;                 // user state [4][ny][nx]
-  double* acc;               // stage scratch [4][ny][nx]
-  double* acc2;
   const unsigned char* tag;
   IbArgs ib;
   BcArgs bc;
@@ -213,8 +209,8 @@ struct alignas(64) TensorMap128 {
   unsigned long long opaque[16];
 };
 
-// box of the TMA-staged stage tile (32x32 cells + 3-cell halo, 4 planes)
-constexpr int TMA_TX = 32, TMA_TY = 32;
+// box of the TMA-staged stage tile (28x28 cells + 3-cell halo, 4 planes)
+constexpr int TMA_BOX = 34;
 
 // IEEE-order arithmetic mode (js_ieee.cu): padded primitives Q (4 planes of lay.plane),
 // x-face fluxes F [4][ny][nx+1], y-face fluxes G [4][ny+1][nx]
@@ -233,7 +229,7 @@ constexpr int STAGE_VARIANTS = 5;
 cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, const TensorMap128* tmap,
                          cudaStream_t s);
 // stage update (not RHS mode) that also stores the WENO5 internals to a.wsave (2D only;
-// 32x32 concurrent tile, TMA-staged when tmap is given)
+// TMA-staged when tmap is given)
 cudaError_t launch_stage_save(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s);
 // stage update that also writes the neural flux's face images of its input to a.img (2D)
 cudaError_t launch_stage_img(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s);

@@ -1,9 +1,17 @@
 // Fused stage of the FP64 finite-volume step on one 2D tile (arXiv 2601.04400, Sec. 2):
-// conserved tile + 3-cell halo -> primitives in shared memory -> x sweep (WENO5, HLLC,
-// viscous flux) into a global accumulator (it stays in L2; keeping it out of shared memory
-// lets more blocks share an SM's FP64 pipe) -> y sweep, divergence, artificial viscosity and
-// the SSP-RK3 stage combination.  Used by the per-grid stage kernel and by the persistent
-// batched kernel.
+// conserved tile + 3-cell halo -> primitives in shared memory -> fluxes of the tile's x lines,
+// then of its y lines (WENO5, HLLC, viscous flux) -> divergence, artificial viscosity and the
+// SSP-RK3 stage combination.  Used by the per-grid stage kernels and by the persistent batched
+// kernels.
+//
+// A warp takes one line of the tile, a lane one cell of it: what a cell shares with its
+// neighbours (differences, smoothness indicators, face states, face fluxes) is passed by
+// shuffles.  Of the 32 cells of lanes 0..31 (cells -2 .. 29 of the line's 28 output cells) the
+// differences serve WENO5 of cells -1 .. 28, these the faces -1/2 .. 27 1/2, these the 28 outputs.
+// No state is carried along a line, so a thread holds one cell's values (about 100 registers;
+// sweeping 16 cells with a sliding window in registers took 214 and left 2 warps per SM
+// sub-partition, too few to overlap the integer WENO5 with the FP64 of the fluxes), and a line
+// takes one pass of latency instead of 17.  28 of 32 lanes' work is kept.
 #pragma once
 #include <type_traits>
 
@@ -12,110 +20,113 @@
 
 namespace js {
 
-// =======================================================================================
-// line sweep: WENO5 -> HLLC (+ viscous) -> flux differences, on primitives in shared memory
-// =======================================================================================
-// sq: shared planes rho, u, v, p (and T when VISC), plane stride ps; `base` = index of the
-// first output cell of the segment, `st` = stride along the line, `ts` = stride across it.
-// emit(k, dF) receives F_{k+1/2} - F_{k-1/2} (conserved order) for output cells k = 0..L-1.
-// keep(k, c, sv), when given, receives the WENO5 internals of variable c at cell k for
-// k = -1 (left-biased side only), 0..L-1 (both sides) and L (right-biased side only).
-// face(k, ql, qr), when given, receives the two WENO5 states (before any positivity fallback)
-// of face k - 1/2 for k = 0..L.
+constexpr unsigned FULL = 0xffffffffu;
+__device__ __forceinline__ u64 shfl_up(u64 v) { return (u64)__shfl_up_sync(FULL, (unsigned long long)v, 1); }
+__device__ __forceinline__ u64 shfl_down(u64 v) { return (u64)__shfl_down_sync(FULL, (unsigned long long)v, 1); }
+__device__ __forceinline__ double shfl_up(double v) { return __shfl_up_sync(FULL, v, 1); }
+__device__ __forceinline__ double shfl_down(double v) { return __shfl_down_sync(FULL, v, 1); }
+
 struct NoKeep {
-  __device__ __forceinline__ void operator()(int, int, const double*) const {}
+  __device__ __forceinline__ void operator()(int, const double*) const {}
 };
 struct NoFace {
-  __device__ __forceinline__ void operator()(int, const double*, const double*) const {}
+  __device__ __forceinline__ void operator()(const double*, const double*) const {}
 };
 
-template <int DIR, bool VISC, bool HAS_T, int L, class Emit, class Keep = NoKeep, class Face = NoFace>
-__device__ __forceinline__ void sweep_line(const double* __restrict__ sq, int ps, int base, int st, int ts,
-                                           const Gas& g, const ViscC& vc, Emit&& emit, Keep keep = Keep{},
-                                           Face face = Face{}) {
+// Flux differences F_{i+1/2} - F_{i-1/2} (conserved order) of the cell q points at (planes rho, u,
+// v, p, and T when VISC, `ps` apart; neighbours along the line at multiples of st, across it of
+// ts), valid in lanes 2..29.  pn: plane of the face-normal velocity (1 or 2).  Every lane of the
+// warp calls it, consecutive lanes on consecutive cells; q[-st .. st] is readable for each.
+// keep(c, sv), when given, receives the WENO5 internals of variable c (valid in lanes 1..30);
+// face(ql, qr) the two WENO5 states of face i+1/2 before any positivity fallback (lanes 1..29).
+template <bool VISC, bool HAS_T, class Keep = NoKeep, class Face = NoFace>
+__device__ __forceinline__ void line_fluxes(const double* q, int ps, int st, int ts, int pn, const Gas& g,
+                                            const ViscC& vc, double dF[4], Keep keep = Keep{}, Face face = Face{}) {
   constexpr bool SV = !std::is_same<Keep, NoKeep>::value;
   constexpr bool FI = !std::is_same<Face, NoFace>::value;
-  constexpr int PN = (DIR == 0) ? 1 : 2;  // plane of the face-normal velocity
-  constexpr int PT = (DIR == 0) ? 2 : 1;  // plane of the tangential velocity
-  Win4 w;
-  w.init(sq + base - st, ps, st);
-  double prevL[4], prevF[4];
-  {
-    // cell -1 of the segment: only its right-face (left-biased) state is needed
-    double Rf[4];
-    w.template step<true, false, SV>(sq + base - st, ps, st, prevL, Rf, [&](int c, const double* sv) { if constexpr (SV) keep(-1, c, sv); });
-  }
+  const int lane = threadIdx.x & 31;
+  const bool inner = lane - 1u < 30u;
+  const int pt = 3 - pn;
+  // face states of the cell in the line's frame: rho, normal, tangential velocity, p
+  double L[4], R[4];
 #pragma unroll 1
-  for (int k = 0; k <= L; ++k) {
-    const int cell = base + k * st;
-    double Lf[4], Rf[4];
-    if (k < L) {
-      w.template step<true, true, SV>(sq + cell, ps, st, Lf, Rf, [&](int c, const double* sv) { if constexpr (SV) keep(k, c, sv); });
-    } else {
-      // cell L (first cell of the next segment): only its left-face state is needed
-      w.template step<false, true, SV>(sq + cell, ps, st, Lf, Rf, [&](int c, const double* sv) { if constexpr (SV) keep(L, c, sv); });
+  for (int k = 0; k < 4; ++k) {
+    const int c = (k == 1) ? pn : (k == 2) ? pt : k;
+    double Lf, Rf;
+    double sv[SV ? 7 : 1];
+    weno_lane<SV>(q + c * ps, st, k == 0 || k == 3, inner, Lf, Rf, sv);
+    if (SV) keep(c, sv);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) Lf[c] = 0.0;  // unused
+    for (int m = 0; m < 4; ++m) {
+      L[m] = (k == m) ? Lf : L[m];
+      R[m] = (k == m) ? Rf : R[m];
     }
-    {
-      // face k - 1/2 between cells k-1 (left state prevL) and k (right state Rf)
-      double ql[4], qr[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) { ql[c] = prevL[c]; qr[c] = Rf[c]; }
-      if (FI) face(k, ql, qr);
-      if (!(positive(ql[0]) && positive(ql[3]) && positive(qr[0]) && positive(qr[3]))) {
-        // positivity fallback: first-order (cell) states at this face
-#pragma unroll
-        for (int c = 0; c < 4; ++c) { ql[c] = sq[c * ps + cell - st]; qr[c] = sq[c * ps + cell]; }
-      }
-      double Fn[4];
-      hllc(ql[0], ql[PN], ql[PT], ql[3], qr[0], qr[PN], qr[PT], qr[3], g, Fn);
-      double F[4];
-      F[0] = Fn[0];
-      F[PN] = Fn[1];
-      F[PT] = Fn[2];
-      F[3] = Fn[3];
-      if (VISC) {
-        const int a = cell - st, b = cell;
-        const double* un = sq + PN * ps;
-        const double* ut = sq + PT * ps;
-        const double* Tq = sq + 4 * ps;
-        const double dun = un[b] - un[a], dut = ut[b] - ut[a], dT = Tq[b] - Tq[a];
-        double tnn, tnt;
-        if (HAS_T) {
-          const double sun = (un[a + ts] - un[a - ts]) + (un[b + ts] - un[b - ts]);
-          const double sut = (ut[a + ts] - ut[a - ts]) + (ut[b + ts] - ut[b - ts]);
-          tnn = fma(vc.c43n, dun, -vc.c23t * sut);
-          tnt = fma(vc.cn, dut, vc.ct * sun);
-        } else {
-          tnn = vc.c43n * dun;
-          tnt = vc.cn * dut;
-        }
-        const double sbn = un[a] + un[b], sbt = ut[a] + ut[b];
-        const double e = fma(0.5, fma(sbn, tnn, sbt * tnt), vc.ck * dT);
-        F[PN] -= tnn;
-        F[PT] -= tnt;
-        F[3] -= e;
-      }
-      if (k >= 1) {
-        double dF[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) dF[c] = F[c] - prevF[c];
-        emit(k - 1, dF);
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) prevF[c] = F[c];
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) prevL[c] = Lf[c];
   }
+  // face i+1/2: the cell's left-biased state, its neighbour's right-biased one
+#pragma unroll
+  for (int m = 0; m < 4; ++m) R[m] = shfl_down(R[m]);
+  const double* un = q + pn * ps;
+  const double* ut = q + pt * ps;
+  if (FI) {
+    const double ql[4] = {L[0], pn == 1 ? L[1] : L[2], pn == 1 ? L[2] : L[1], L[3]};
+    const double qr[4] = {R[0], pn == 1 ? R[1] : R[2], pn == 1 ? R[2] : R[1], R[3]};
+    face(ql, qr);
+  }
+  if (!(positive(L[0]) && positive(L[3]) && positive(R[0]) && positive(R[3]))) {
+    // positivity fallback: first-order (cell) states at this face
+    L[0] = q[0], L[1] = un[0], L[2] = ut[0], L[3] = q[3 * ps];
+    R[0] = q[st], R[1] = un[st], R[2] = ut[st], R[3] = q[3 * ps + st];
+  }
+  double F[4];
+  hllc(L[0], L[1], L[2], L[3], R[0], R[1], R[2], R[3], g, F);
+  if (VISC) {
+    const double* Tq = q + 4 * ps;
+    const double ua = un[0], ub = un[st], ta = ut[0], tb = ut[st];
+    const double dun = ub - ua, dut = tb - ta, dT = Tq[st] - Tq[0];
+    double tnn, tnt;
+    if (HAS_T) {
+      const double sun = (un[ts] - un[-ts]) + (un[st + ts] - un[st - ts]);
+      const double sut = (ut[ts] - ut[-ts]) + (ut[st + ts] - ut[st - ts]);
+      tnn = fma(vc.c43n, dun, -vc.c23t * sut);
+      tnt = fma(vc.cn, dut, vc.ct * sun);
+    } else {
+      tnn = vc.c43n * dun;
+      tnt = vc.cn * dut;
+    }
+    const double sbn = ua + ub, sbt = ta + tb;
+    const double e = fma(0.5, fma(sbn, tnn, sbt * tnt), vc.ck * dT);
+    F[1] -= tnn;
+    F[2] -= tnt;
+    F[3] -= e;
+  }
+  double D[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) D[m] = F[m] - shfl_up(F[m]);
+  dF[0] = D[0];
+  dF[1] = pn == 1 ? D[1] : D[2];
+  dF[2] = pn == 1 ? D[2] : D[1];
+  dF[3] = D[3];
 }
 
-// final combination for one interior cell; returns the value stored in the output
-// dF, dG: x and y flux differences (dG zero in 1D)
+// =======================================================================================
+// tiles
+// =======================================================================================
+constexpr int TILE = 28;         // output cells of a tile along x and along y (one warp's lines)
+constexpr int TILE_B = TILE + 6;  // its box with the halo; the TMA copy writes dense rows
+constexpr int TILE_A = TILE + 1;  // row pitch of the accumulator (odd: y lines hit distinct banks)
+
+template <bool VISC>
+struct StageTile {
+  static constexpr int NPL = VISC ? 5 : 4;
+  static constexpr int PS = TILE_B * TILE_B;
+  static constexpr int PA = TILE * TILE_A;
+  static constexpr size_t SMEM = sizeof(double) * (size_t)(NPL * PS + 4 * PA);
+};
+
+// final combination for one interior cell, v = U_s - dt div F (RHS mode: - div F)
 template <bool RHS>
-__device__ __forceinline__ void finish_cell(const StageArgs& a, int gi, int gj, const double dF[4],
-                                            const double dG[4], double rho, double p) {
+__device__ __forceinline__ void finish_cell(const StageArgs& a, int gi, int gj, const double upd[4], double rho,
+                                            double p) {
   const long long pid = a.lay.idx(gi, gj);
   const bool fluid = (a.tag == nullptr) || (a.tag[(long long)gj * a.lay.nx + gi] == 0);
   double out[4];
@@ -124,8 +135,7 @@ __device__ __forceinline__ void finish_cell(const StageArgs& a, int gi, int gj, 
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const double* Uc = a.Uin + c * a.lay.plane;
-      const double us = RHS ? 0.0 : Uc[pid];
-      double v = fma(-a.cy, dG[c], fma(-a.cx, dF[c], us));
+      double v = upd[c];
       if (a.has_av) {
         v = fma(a.avx, (Uc[pid + 1] - 2.0 * Uc[pid]) + Uc[pid - 1], v);
         if (a.lay.ny > 1) v = fma(a.avy, (Uc[pid + a.lay.pitch] - 2.0 * Uc[pid]) + Uc[pid - a.lay.pitch], v);
@@ -148,111 +158,39 @@ __device__ __forceinline__ void finish_cell(const StageArgs& a, int gi, int gj, 
   }
 }
 
-// load the conserved tile with halo and convert to primitives in shared memory
-template <int TX, int TY, int NPL, int NT>
-__device__ __forceinline__ void load_tile(const StageArgs& a, double* sq, int ps, int sp, int ox, int oy,
+// primitives of one cell of the tile box (element e); cells past the array get a uniform state
+// (they feed only cells that are not written)
+template <int NPL>
+__device__ __forceinline__ void put_prims(double* sq, int e, bool in, double r, double mx, double my, double E,
                                           const Gas& g) {
-  constexpr int CW = TX + 6, CH = TY + 6;
+  constexpr int PS = TILE_B * TILE_B;
+  double u = 0.0, v = 0.0, p = 1.0, T = 1.0;
+  if (in) cons_to_prim(r, mx, my, E, g, u, v, p, T);
+  sq[e] = in ? r : 1.0;
+  sq[PS + e] = u;
+  sq[2 * PS + e] = v;
+  sq[3 * PS + e] = p;
+  if (NPL == 5) sq[4 * PS + e] = T;
+}
+
+// load the conserved tile with halo and convert to primitives in shared memory
+template <int NPL>
+__device__ __forceinline__ void load_tile(const StageArgs& a, double* sq, int ox, int oy, const Gas& g) {
   const int W = a.lay.nx + 6;
-  for (int e = threadIdx.x; e < CW * CH; e += NT) {
-    const int row = e / CW, col = e - row * CW;
-    int gx = ox + col, gy = oy + row;  // padded coordinates
-    gx = (gx < W) ? gx : W - 1;
-    gy = (gy < a.lay.H) ? gy : a.lay.H - 1;
-    const long long s = (long long)gy * a.lay.pitch + gx;
-    const double r = a.Uin[s], mx = a.Uin[a.lay.plane + s], my = a.Uin[2 * a.lay.plane + s],
-                 E = a.Uin[3 * a.lay.plane + s];
-    double u, v, p, T;
-    cons_to_prim(r, mx, my, E, g, u, v, p, T);
-    const int d = row * sp + col;
-    sq[d] = r;
-    sq[ps + d] = u;
-    sq[2 * ps + d] = v;
-    sq[3 * ps + d] = p;
-    if (NPL == 5) sq[4 * ps + d] = T;
+  for (int e = threadIdx.x; e < TILE_B * TILE_B; e += blockDim.x) {
+    const int row = e / TILE_B, col = e - row * TILE_B;
+    const int gx = ox + col, gy = oy + row;  // padded coordinates
+    const bool in = gx < W && gy < a.lay.H;
+    const long long s = in ? (long long)gy * a.lay.pitch + gx : 0;
+    put_prims<NPL>(sq, e, in, a.Uin[s], a.Uin[a.lay.plane + s], a.Uin[2 * a.lay.plane + s], a.Uin[3 * a.lay.plane + s],
+                   g);
   }
 }
 
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS>
-struct Stage2D {
-  static constexpr int NPL = VISC ? 5 : 4;
-  static constexpr int SP = TX + 7;  // odd row pitch (in doubles) of the shared tile
-  static constexpr int PS = (TY + 6) * SP;
-  static constexpr int NX_ITEMS = TY * (TX / LX);
-  static constexpr int NY_ITEMS = TX * (TY / LY);
-  static constexpr int NT = (NX_ITEMS > NY_ITEMS) ? NX_ITEMS : NY_ITEMS;
-  static constexpr size_t SMEM = sizeof(double) * (size_t)NPL * PS;
-};
-
-// one tile (bx, by) of one stage; smem holds Stage2D::SMEM bytes; all NT threads take part
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS>
-__device__ __forceinline__ void stage_tile(const StageArgs& a, int bx, int by, double* smem) {
-  using S = Stage2D<TX, TY, LX, LY, VISC, RHS>;
-  double* sq = smem;
-  const long long ncell = (long long)a.lay.nx * a.lay.ny;
-  const Gas g{a.gamma, a.gm1, a.g1};
-  const int tx0 = bx * TX, ty0 = by * TY;  // interior origin of the tile
-  load_tile<TX, TY, S::NPL, S::NT>(a, sq, S::PS, S::SP, tx0, ty0, g);
-  __syncthreads();
-  // x sweep: one thread per (row, segment)
-  for (int it = threadIdx.x; it < S::NX_ITEMS; it += S::NT) {
-    const int ty = it % TY, xs = (it / TY) * LX;
-    const int base = (ty + 3) * S::SP + xs + 3;
-    const int gj = ty0 + ty;
-    sweep_line<0, VISC, true, LX>(sq, S::PS, base, 1, S::SP, g, a.vx, [&](int k, const double dF[4]) {
-      const int gi = tx0 + xs + k;
-      if (gi < a.lay.nx && gj < a.lay.ny) {
-        const long long o = (long long)gj * a.lay.nx + gi;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) a.acc[c * ncell + o] = dF[c];
-      }
-    });
-  }
-  __syncthreads();
-  // y sweep + stage combination: one thread per (column, segment)
-  for (int it = threadIdx.x; it < S::NY_ITEMS; it += S::NT) {
-    const int tx = it % TX, ys = (it / TX) * LY;
-    const int base = (ys + 3) * S::SP + tx + 3;
-    const int gi = tx0 + tx;
-    sweep_line<1, VISC, true, LY>(sq, S::PS, base, S::SP, 1, g, a.vy, [&](int k, const double dG[4]) {
-      const int ty = ys + k, gj = ty0 + ty;
-      if (gi < a.lay.nx && gj < a.lay.ny) {
-        double ax[4];
-        const long long o = (long long)gj * a.lay.nx + gi;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) ax[c] = a.acc[c * ncell + o];
-        const int sc = (ty + 3) * S::SP + tx + 3;
-        finish_cell<RHS>(a, gi, gj, ax, dG, sq[sc], sq[3 * S::PS + sc]);
-      }
-    });
-  }
-}
-
-
 // ---------------------------------------------------------------------------------------
-// Concurrent-sweep tile: the x sweep (first NX_ITEMS threads) and the y sweep (next
-// NY_ITEMS threads, warp-aligned) run at the same time on the shared primitive tile and
-// write their flux differences to two global accumulators (L2-resident); after a
-// barrier every thread combines cells of the tile.  Twice the warps per block at the same
-// shared memory: more warps hide the FP64 pipe's latency.
-// ---------------------------------------------------------------------------------------
-template <int TX, int TY, int LX, int LY, bool VISC, bool TMA = false>
-struct Stage2DC {
-  static constexpr int NPL = VISC ? 5 : 4;
-  static constexpr int SP = TMA ? TX + 6 : TX + 7;  // TMA writes dense box rows
-  static constexpr int PS = (TY + 6) * SP;
-  static constexpr int NX_ITEMS = TY * (TX / LX);
-  static constexpr int NY_ITEMS = TX * (TY / LY);
-  static_assert(NX_ITEMS % 32 == 0 && NY_ITEMS % 32 == 0, "sweep roles must be whole warps");
-  static constexpr int NT = NX_ITEMS + NY_ITEMS;
-  static constexpr size_t SMEM = sizeof(double) * (size_t)NPL * PS;
-};
-
-// ---------------------------------------------------------------------------------------
-// TMA staging: one cp.async.bulk.tensor brings the conserved (TX+6) x (TY+6) x 4 box of the
-// padded state into shared memory ([plane][row][col], row pitch TX+6); an mbarrier tracks
-// completion.  Waits are bounded: on timeout the block records JS_ERR_TIMEOUT, drains its copy
-// (bounded again) and skips the tile.
+// TMA staging: one cp.async.bulk.tensor brings the conserved 34 x 34 x 4 box of the padded state
+// into shared memory ([plane][row][col]); an mbarrier tracks completion.  Waits are bounded: on
+// timeout the block records JS_ERR_TIMEOUT, drains its copy (bounded again) and skips the tile.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
@@ -289,15 +227,16 @@ __device__ __forceinline__ void tma_box3d(void* dst, const void* map, int x, int
 
 // Stage the tile with TMA and convert it to primitives in place (T in plane 4 when VISC).
 // Returns false when the copy did not complete in time (the tile must be skipped).
-template <int TX, int TY, int NPL, int NT>
-__device__ __forceinline__ bool load_tile_tma(const StageArgs& a, const void* tmap, double* sq, int ps, int ox,
-                                              int oy, const Gas& g, unsigned long long* bar, unsigned& phase) {
-  constexpr int CW = TX + 6, CH = TY + 6;
-  constexpr unsigned BYTES = 4u * CW * CH * sizeof(double);
-  static_assert(CW * CH * sizeof(double) % 16 == 0 && CW * sizeof(double) % 16 == 0, "TMA box rows");
+template <int NPL>
+__device__ __forceinline__ bool load_tile_tma(const StageArgs& a, const void* tmap, double* sq, int ox, int oy,
+                                              const Gas& g, unsigned long long* bar, unsigned& phase) {
+  constexpr int PS = TILE_B * TILE_B;
+  constexpr unsigned BYTES = 4u * PS * sizeof(double);
+  static_assert(PS * sizeof(double) % 16 == 0 && TILE_B * sizeof(double) % 16 == 0 && TILE * sizeof(double) % 16 == 0,
+                "TMA box rows and origins");
   __shared__ int s_ok;
   if (threadIdx.x == 0) {
-    // the box origin is the tile origin in padded coordinates: x = ox is a multiple of 32
+    // the box origin is the tile origin in padded coordinates: x = ox is a multiple of 28 cells
     tma_box3d(sq, tmap, ox, oy, 0, bar, BYTES);
     constexpr long long kBudget = 2000000000LL;  // about one second of SM clock
     bool ok = mbar_wait(bar, phase, kBudget);
@@ -310,133 +249,114 @@ __device__ __forceinline__ bool load_tile_tma(const StageArgs& a, const void* tm
   __syncthreads();
   phase ^= 1u;
   if (!s_ok) return false;
-  for (int e = threadIdx.x; e < CW * CH; e += NT) {
-    const double r = sq[e], mx = sq[ps + e], my = sq[2 * ps + e], E = sq[3 * ps + e];
-    double u, v, p, T;
-    cons_to_prim(r, mx, my, E, g, u, v, p, T);
-    sq[ps + e] = u;
-    sq[2 * ps + e] = v;
-    sq[3 * ps + e] = p;
-    if (NPL == 5) sq[4 * ps + e] = T;
+  const int W = a.lay.nx + 6;
+  for (int e = threadIdx.x; e < PS; e += blockDim.x) {
+    const int row = e / TILE_B, col = e - row * TILE_B;
+    put_prims<NPL>(sq, e, ox + col < W && oy + row < a.lay.H, sq[e], sq[PS + e], sq[2 * PS + e], sq[3 * PS + e], g);
   }
   return true;
 }
 
-// Store the WENO5 internals of variable c at cell `k` of line `line` (DIR 0: row, stored
-// transposed; DIR 1: column, padded layout), for the cells -1 .. n the reverse pass reads
-// (n = cells along the line).  `part` is -1 / 0 / +1 for a cell whose left-biased side only /
-// both sides / right-biased side only were formed.  Cell n keeps only its right-biased side,
-// so that every writer of a cell stores the same values.
-template <int DIR>
-__device__ __forceinline__ void keep_internals(const StageArgs& a, int k, int line, int c, const double* sv,
-                                               int part) {
-  const int n = (DIR == 0) ? a.lay.nx : a.lay.ny;
-  const bool store = (part < 0) ? (k == -1) : (part > 0) ? (k == n) : (k >= 0 && k <= n);
-  if (!store) return;
-  const long long si = (DIR == 0) ? (long long)(k + 3) * a.tpitch + (line + a.lay.gy) : a.lay.idx(line, k);
-  double* dst = a.wsave + (long long)(DIR * 28 + c * 7) * a.splane + si;
-  const bool left = k < n;
+// Store the WENO5 internals of variable c at cell k of line `line` (dir 0: row, stored
+// transposed; dir 1: column, padded layout), for the cells -1 .. n the reverse pass reads
+// (n = cells along the line).  Cell -1 keeps only its left-biased side, cell n its right-biased
+// one; `owner`: this lane's cell is one of the tile's outputs.
+__device__ __forceinline__ void keep_internals(const StageArgs& a, int dir, int k, int line, int c, const double* sv,
+                                               bool owner) {
+  const int n = (dir == 0) ? a.lay.nx : a.lay.ny;
+  if (!(k == -1 || k == n || (owner && k >= 0 && k < n))) return;
+  const long long si = (dir == 0) ? (long long)(k + 3) * a.tpitch + (line + a.lay.gy) : a.lay.idx(line, k);
+  double* dst = a.wsave + (long long)(dir * 28 + c * 7) * a.splane + si;
+  const bool left = k < n, right = k >= 0;
 #pragma unroll
-  for (int m = 0; m < 7; ++m) dst[m * a.splane] = (m == 3 || m == 4) && !left ? 0.0 : sv[m];
+  for (int m = 0; m < 7; ++m)
+    dst[m * a.splane] = ((m == 3 || m == 4) && !left) || ((m == 5 || m == 6) && !right) ? 0.0 : sv[m];
 }
 
 // face image of the neural flux (IMG: a.img, FP32 [4][ny][nx+1] for x faces then [4][nx][ny+1]
-// for y faces): face f of a line is written by the segment that holds cell f, the line's last
-// face by the segment that ends there
-template <int DIR>
-__device__ __forceinline__ void put_image(const StageArgs& a, int line, int f, const double* ql, const double* qr) {
+// for y faces): face f of a line
+__device__ __forceinline__ void put_image(const StageArgs& a, int dir, int line, int f, const double* ql,
+                                          const double* qr) {
   const int nx = a.lay.nx, ny = a.lay.ny;
   const long long pix0 = (long long)ny * (nx + 1);
-  const long long pix = (DIR == 0) ? pix0 : (long long)nx * (ny + 1);
-  float* X = a.img + (DIR == 0 ? 0LL : 4 * pix0) + (long long)line * ((DIR == 0 ? nx : ny) + 1) + f;
+  const long long pix = (dir == 0) ? pix0 : (long long)nx * (ny + 1);
+  float* X = a.img + (dir == 0 ? 0LL : 4 * pix0) + (long long)line * ((dir == 0 ? nx : ny) + 1) + f;
+  const double wl[4] = {ql[0], dir == 0 ? ql[1] : ql[2], dir == 0 ? ql[2] : ql[1], ql[3]};
+  const double wr[4] = {qr[0], dir == 0 ? qr[1] : qr[2], dir == 0 ? qr[2] : qr[1], qr[3]};
   float m[4];
-  face_image<float>(ql, qr, DIR == 0 ? 1 : 2, DIR == 0 ? 2 : 1, a.img_g1, a.img_mean, a.img_isd, m);
+  face_image<float>(wl, wr, 1, 2, a.img_g1, a.img_mean, a.img_isd, m);
 #pragma unroll
   for (int k = 0; k < 4; ++k) X[k * pix] = m[k];
 }
 
-template <int TX, int TY, int LX, int LY, bool VISC, bool RHS, bool TMA = false, bool SAVE = false, bool IMG = false>
-__device__ __forceinline__ void stage_tile_c(const StageArgs& a, int bx, int by, double* smem,
-                                             const void* tmap = nullptr, unsigned long long* bar = nullptr,
-                                             unsigned* phase = nullptr) {
-  using S = Stage2DC<TX, TY, LX, LY, VISC, TMA>;
+// one tile (bx, by) of one stage; smem holds StageTile::SMEM bytes; whole warps take part
+template <bool VISC, bool RHS, bool TMA = false, bool SAVE = false, bool IMG = false>
+__device__ __forceinline__ void stage_tile(const StageArgs& a, int bx, int by, double* smem,
+                                           const void* tmap = nullptr, unsigned long long* bar = nullptr,
+                                           unsigned* phase = nullptr) {
+  using S = StageTile<VISC>;
   double* sq = smem;
-  const long long ncell = (long long)a.lay.nx * a.lay.ny;
+  double* acc = smem + S::NPL * S::PS;
   const Gas g{a.gamma, a.gm1, a.g1};
-  const int tx0 = bx * TX, ty0 = by * TY;
+  const int tx0 = bx * TILE, ty0 = by * TILE;
   if (TMA) {
-    if (!load_tile_tma<TX, TY, S::NPL, S::NT>(a, tmap, sq, S::PS, tx0, ty0, g, bar, *phase)) return;
+    if (!load_tile_tma<S::NPL>(a, tmap, sq, tx0, ty0, g, bar, *phase)) return;
   } else {
-    load_tile<TX, TY, S::NPL, S::NT>(a, sq, S::PS, S::SP, tx0, ty0, g);
+    load_tile<S::NPL>(a, sq, tx0, ty0, g);
   }
   __syncthreads();
-  if (threadIdx.x < S::NX_ITEMS) {
-    const int it = threadIdx.x;
-    const int ty = it % TY, xs = (it / TY) * LX;
-    const int gj = ty0 + ty;
-    auto emit = [&](int k, const double dF[4]) {
-      const int gi = tx0 + xs + k;
-      if (gi < a.lay.nx && gj < a.lay.ny) {
-        const long long o = (long long)gj * a.lay.nx + gi;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) a.acc[c * ncell + o] = dF[c];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int k = lane - 2;  // the lane's cell along the line
+  // x lines, then y lines (one copy of the code: the strides and planes differ)
+#pragma unroll 1
+  for (int dir = 0; dir < 2; ++dir) {
+    const int lines = dir == 0 ? min(TILE, a.lay.ny - ty0) : min(TILE, a.lay.nx - tx0);
+    const int ncell = dir == 0 ? min(TILE, a.lay.nx - tx0) : min(TILE, a.lay.ny - ty0);
+    const int st = dir == 0 ? 1 : TILE_B, ts = dir == 0 ? TILE_B : 1;
+    const ViscC vc = dir == 0 ? a.vx : a.vy;
+    const double cn = dir == 0 ? a.cx : a.cy;
+#pragma unroll 1
+    for (int ln = warp; ln < lines; ln += nwarp) {
+      const double* q = sq + (ln + 3) * ts + (k + 3) * st;
+      double dF[4];
+      const int gk = (dir == 0 ? tx0 : ty0) + k, gl = (dir == 0 ? ty0 : tx0) + ln;  // cell and line in the grid
+      const bool owner = lane >= 2 && k < ncell;
+      if constexpr (SAVE) {
+        line_fluxes<VISC, true>(q, S::PS, st, ts, dir + 1, g, vc, dF, [&](int c, const double* sv) {
+          if (lane >= 1 && lane <= 30) keep_internals(a, dir, gk, gl, c, sv, owner && lane < 30);
+        });
+      } else if constexpr (IMG) {
+        line_fluxes<VISC, true>(q, S::PS, st, ts, dir + 1, g, vc, dF, NoKeep{}, [&](const double* ql, const double* qr) {
+          // face gk + 1; the tile's outer face belongs to the next tile unless it is the line's last
+          const int f = gk + 1, n = dir == 0 ? a.lay.nx : a.lay.ny;
+          if (lane >= 1 && f <= n && (lane <= 28 || (lane == 29 && f == n))) put_image(a, dir, gl, f, ql, qr);
+        });
+      } else {
+        line_fluxes<VISC, true>(q, S::PS, st, ts, dir + 1, g, vc, dF);
       }
-    };
-    if constexpr (SAVE) {
-      sweep_line<0, VISC, true, LX>(sq, S::PS, (ty + 3) * S::SP + xs + 3, 1, S::SP, g, a.vx, emit,
-                                    [&](int k, int c, const double* sv) {
-        if (gj < a.lay.ny) keep_internals<0>(a, tx0 + xs + k, gj, c, sv, k < 0 ? -1 : (k == LX ? 1 : 0));
-      });
-    } else if constexpr (IMG) {
-      sweep_line<0, VISC, true, LX>(sq, S::PS, (ty + 3) * S::SP + xs + 3, 1, S::SP, g, a.vx, emit, NoKeep{},
-                                    [&](int k, const double* ql, const double* qr) {
-        const int f = tx0 + xs + k;
-        if (gj < a.lay.ny && f <= a.lay.nx && (k < LX || f == a.lay.nx)) put_image<0>(a, gj, f, ql, qr);
-      });
-    } else {
-      sweep_line<0, VISC, true, LX>(sq, S::PS, (ty + 3) * S::SP + xs + 3, 1, S::SP, g, a.vx, emit);
-    }
-  } else {
-    const int it = threadIdx.x - S::NX_ITEMS;
-    const int tx = it % TX, ys = (it / TX) * LY;
-    const int gi = tx0 + tx;
-    auto emit = [&](int k, const double dG[4]) {
-      const int gj = ty0 + ys + k;
-      if (gi < a.lay.nx && gj < a.lay.ny) {
-        const long long o = (long long)gj * a.lay.nx + gi;
+      if (owner && lane < 30) {
+        const int tx = dir == 0 ? k : ln, ty = dir == 0 ? ln : k;
+        double* t = acc + ty * TILE_A + tx;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a.acc2[c * ncell + o] = dG[c];
+        for (int c = 0; c < 4; ++c) {
+          double base;
+          if (dir == 0) base = RHS ? 0.0 : a.Uin[c * a.lay.plane + a.lay.idx(tx0 + tx, ty0 + ty)];
+          else base = t[c * S::PA];
+          t[c * S::PA] = fma(-cn, dF[c], base);
+        }
       }
-    };
-    if constexpr (SAVE) {
-      sweep_line<1, VISC, true, LY>(sq, S::PS, (ys + 3) * S::SP + tx + 3, S::SP, 1, g, a.vy, emit,
-                                    [&](int k, int c, const double* sv) {
-        if (gi < a.lay.nx) keep_internals<1>(a, ty0 + ys + k, gi, c, sv, k < 0 ? -1 : (k == LY ? 1 : 0));
-      });
-    } else if constexpr (IMG) {
-      sweep_line<1, VISC, true, LY>(sq, S::PS, (ys + 3) * S::SP + tx + 3, S::SP, 1, g, a.vy, emit, NoKeep{},
-                                    [&](int k, const double* ql, const double* qr) {
-        const int f = ty0 + ys + k;
-        if (gi < a.lay.nx && f <= a.lay.ny && (k < LY || f == a.lay.ny)) put_image<1>(a, gi, f, ql, qr);
-      });
-    } else {
-      sweep_line<1, VISC, true, LY>(sq, S::PS, (ys + 3) * S::SP + tx + 3, S::SP, 1, g, a.vy, emit);
     }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < TX * TY; e += S::NT) {
-    const int tx = e % TX, ty = e / TX;
+  for (int e = threadIdx.x; e < TILE * TILE; e += blockDim.x) {
+    const int ty = e / TILE, tx = e - ty * TILE;
     const int gi = tx0 + tx, gj = ty0 + ty;
     if (gi >= a.lay.nx || gj >= a.lay.ny) continue;
-    const long long o = (long long)gj * a.lay.nx + gi;
-    double ax[4], ay[4];
+    double upd[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      ax[c] = a.acc[c * ncell + o];
-      ay[c] = a.acc2[c * ncell + o];
-    }
-    const int sc = (ty + 3) * S::SP + tx + 3;
-    finish_cell<RHS>(a, gi, gj, ax, ay, sq[sc], sq[3 * S::PS + sc]);
+    for (int c = 0; c < 4; ++c) upd[c] = acc[c * S::PA + ty * TILE_A + tx];
+    const int sc = (ty + 3) * TILE_B + tx + 3;
+    finish_cell<RHS>(a, gi, gj, upd, sq[sc], sq[3 * S::PS + sc]);
   }
 }
 
