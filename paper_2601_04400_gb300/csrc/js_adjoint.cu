@@ -3,27 +3,21 @@
 // step of Fig. 1(d)).
 //
 // One stage VJP, given the adjoint of the stage output and the filled stage state X:
-//   seed      lambda' = b dt Ubar_next on fluid cells (0 elsewhere); Ubar(X) gets the
-//             identity and carry terms; Ubar_0 += a Ubar_next on fluid cells
-//   prims     Q = prim(X) on every padded cell (same arithmetic as the forward kernel)
-//   pass 1    per line: WENO5 forward (internals saved to HBM; skipped when the forward
-//             stage kernel already stored them, then the face states are re-formed from the
-//             saved quotients), HLLC + viscous forward and reverse per face with
-//             Fbar = (lambda'_right - lambda'_left)/h; face-state adjoints saved; the adjoints
-//             that go straight to cells (positivity fallback, viscous terms) saved per face
-//   pass 2    per line segment: WENO5 reverse from the saved internals; a 5-cell register
-//             window emits each cell's adjoint into the segment's own output slots
-//   primvjp   per cell, a gather in a fixed order: Qbar = the slots of the (at most three)
-//             segments of its x line and of its y line that reach it + the per-face adjoints
-//             of the faces that touch it; Ubar(X) += (dprim/dX)^T Qbar (+ nu * lap of lambda')
+//   tile      per tile of the padded array: lambda' = b dt Ubar_next on fluid cells (0
+//             elsewhere), identity and carry terms, Ubar_0 += a Ubar_next; primitives; per line
+//             WENO5 forward, HLLC and viscous forward and reverse per face with
+//             Fbar = (lambda'_right - lambda'_left)/h, WENO5 reverse; Ubar(X) = the sum through
+//             (dprim/dX)^T (+ nu * lap of lambda')
 //   bcT       transposed halo fill (y sides, then x sides), written as gathers;
 //             inflow halos accumulate into the inflow-state gradient
 //   ibT       transposed immersed-boundary fill: ghost adjoint -> image-point adjoint ->
 //             gathered onto the fluid source cells (CSR built on the host)
 // Parameter gradients (gamma, mu, Pr, nu, inflow states) are accumulated in pbar.
-// No floating-point atomics: every sum runs in a fixed order (per-block partials of the
-// parameter gradient reduced in block order by one block at the end of the stage), so the
+// No floating-point atomics: every sum runs in a fixed order (per-warp partials of the
+// parameter gradient reduced in a fixed order by one block at the end of the stage), so the
 // reverse pass gives the same bits on every run.
+// With the neural flux on, its reverse runs first, on primitives and lambda' in memory, and the
+// tiles add its face-state adjoints to their own.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,42 +28,38 @@
 namespace js {
 
 // =======================================================================================
-// per-grid launches: one thread per element (or line segment) of each phase
+// per-grid launches
 // =======================================================================================
-__global__ void adj_seed_kernel(AdjArgs a, const double* __restrict__ Unext, double* __restrict__ Uacc, double ra,
-                                double rb, double dt, int rhs_mode) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < a.lay.plane) adj_seed_one(a, t, Unext, Uacc, ra, rb, dt, rhs_mode);
-}
-
-__global__ void adj_prims_kernel(AdjArgs a) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < a.lay.plane) adj_prims_one(a, t);
-}
-
-// x lines in blocks [0, bx), y lines (2D) in the blocks after them: one launch, both directions
-template <bool VISC, bool HAS_T, bool SAVED>
-__global__ void __launch_bounds__(64) adj_pass1_kernel(AdjArgs a, int seg_len, int bx) {
-  if ((int)blockIdx.x < bx)
-    pass1_body<0, VISC, HAS_T, SAVED>(a, seg_len, (long long)blockIdx.x * blockDim.x + threadIdx.x, 0);
-  else
-    pass1_body<1, VISC, HAS_T, SAVED>(a, seg_len, (long long)(blockIdx.x - bx) * blockDim.x + threadIdx.x,
-                                      ((long long)bx * blockDim.x) >> 5);
-}
-
-__global__ void __launch_bounds__(64) adj_pass2_kernel(AdjArgs a, int seg_len, int bx) {
-  if ((int)blockIdx.x < bx)
-    pass2_body<0>(a, seg_len, (long long)blockIdx.x * blockDim.x + threadIdx.x);
-  else
-    pass2_body<1>(a, seg_len, (long long)(blockIdx.x - bx) * blockDim.x + threadIdx.x);
-}
-
+// A block of 8 warps per tile (3 lines a warp in each direction), two blocks an SM by shared memory.
+// Bound by the FP64 pipe (about 190 FP64 instructions per line cell, 24 of 32 lanes kept) with the
+// integer WENO5 forward and reverse beside it.
 template <bool VISC>
-__global__ void adj_primvjp_kernel(AdjArgs a, int seg_len) {
+__global__ void __launch_bounds__(32 * ADJ_WARPS, 2)
+adj_tile_kernel(AdjArgs a, const double* __restrict__ Unext, double* __restrict__ Uacc, double ra, double rb, double dt,
+                int rhs_mode) {
+  extern __shared__ double smem[];
+  adj_tile<VISC>(a, Unext, Uacc, ra, rb, dt, rhs_mode, blockIdx.x, blockIdx.y, smem,
+                 ((long long)blockIdx.y * gridDim.x + blockIdx.x) * ADJ_WARPS);
+}
+
+// primitives of every padded cell and lambda' = bdt Unext on fluid cells (the neural flux's reverse)
+__global__ void adj_nn_seed_kernel(AdjArgs a, double* __restrict__ Q, const double* __restrict__ Unext, double bdt) {
+  const Lay& L = a.lay;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double gb = 0.0, nb = 0.0;
-  adj_primvjp_one<VISC>(a, t, seg_len, gb, nb);
-  warp_partials(a.pp, global_warp(), gb, 0.0, 0.0, nb);
+  if (t >= L.plane) return;
+  const int col = (int)(t % L.pitch), row = (int)(t / L.pitch);
+  if (col >= L.nx + 6 || row >= L.H) return;
+  double u, v, p, T;
+  const double r = a.X[t];
+  cons_to_prim(r, a.X[L.plane + t], a.X[2 * L.plane + t], a.X[3 * L.plane + t], a.gas, u, v, p, T);
+  Q[t] = r;
+  Q[L.plane + t] = u;
+  Q[2 * L.plane + t] = v;
+  Q[3 * L.plane + t] = p;
+  const int i = col - 3, j = row - L.gy;
+  const bool fluid = i >= 0 && i < L.nx && j >= 0 && j < L.ny && (a.tag == nullptr || a.tag[(long long)j * L.nx + i] == 0);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) a.lam[c * L.plane + t] = fluid ? bdt * Unext[c * L.plane + t] : 0.0;
 }
 
 __global__ void adj_bcT_kernel(AdjArgs a, BcArgs bc, int phase_y, double* inflow_part, int tmax) {
@@ -109,84 +99,28 @@ __global__ void adj_unpack_add_kernel(const double* __restrict__ P, const double
 // launchers
 // =======================================================================================
 namespace {
-// short segments and small blocks: enough blocks to fill every SM (one line per thread
-// would leave most of the GPU idle); pass 1 pays one extra WENO cell per segment, except
-// when the forward stored the internals: then a segment costs almost nothing to start and
-// shorter ones split the work into finer waves
-constexpr int kSeg1 = 16, kSeg1Saved = 8, kSeg1D = 4, kBlk = 64;
-
 unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
-
-long long line_items(const AdjArgs& a, int dir, int extra, int seg) {
-  const int nline = (dir == 0) ? a.lay.ny : a.lay.nx;
-  const int ncell = (dir == 0) ? a.lay.nx : a.lay.ny;
-  return (long long)nline * ((ncell + extra + seg - 1) / seg);
-}
-
-// blocks of pass 1 for the x lines (bx) and the y lines (by); seg = segment length
-void pass1_shape(const AdjArgs& a, bool two_d, int& seg, int& bx, int& by) {
-  if (a.weno_saved) {
-    seg = kSeg1Saved;
-  } else {
-    seg = two_d ? kSeg1 : kSeg1D;  // a 1D grid is one line: short segments give it more threads
-  }
-  bx = (int)blocks_for(line_items(a, 0, 1, seg), kBlk);
-  by = two_d ? (int)blocks_for(line_items(a, 1, 1, seg), kBlk) : 0;
-}
-
-cudaError_t pass1(const AdjArgs& a, bool visc, bool two_d, cudaStream_t s) {
-  int seg, bx, by;
-  pass1_shape(a, two_d, seg, bx, by);
-  if (a.weno_saved) {
-    if (!two_d) return cudaErrorInvalidValue;  // the forward saves exist for 2D grids only
-    if (visc) adj_pass1_kernel<true, true, true><<<bx + by, kBlk, 0, s>>>(a, seg, bx);
-    else adj_pass1_kernel<false, false, true><<<bx + by, kBlk, 0, s>>>(a, seg, bx);
-    return cudaGetLastError();
-  }
-  if (visc) {
-    if (two_d) adj_pass1_kernel<true, true, false><<<bx + by, kBlk, 0, s>>>(a, seg, bx);
-    else adj_pass1_kernel<true, false, false><<<bx + by, kBlk, 0, s>>>(a, seg, bx);
-  } else {
-    adj_pass1_kernel<false, false, false><<<bx + by, kBlk, 0, s>>>(a, seg, bx);
-  }
-  return cudaGetLastError();
-}
-
-int seg2_of(const Lay& L) { return L.ny > 1 ? ADJ_SEG2 : ADJ_SEG2_1D; }
-
-cudaError_t pass2(const AdjArgs& a, bool two_d, cudaStream_t s) {
-  const int seg = seg2_of(a.lay);
-  const int bx = (int)blocks_for(line_items(a, 0, 2, seg), kBlk);
-  const int by = two_d ? (int)blocks_for(line_items(a, 1, 2, seg), kBlk) : 0;
-  adj_pass2_kernel<<<bx + by, kBlk, 0, s>>>(a, seg, bx);
-  return cudaGetLastError();
-}
-
 unsigned ib_blocks(int n) { return n > 0 ? blocks_for(n, 128) : 0; }
+
+template <bool VISC>
+cudaError_t launch_tiles(const AdjArgs& a, const double* Unext, double* Uacc, double ra, double rb, double dt,
+                         bool rhs_mode, cudaStream_t s) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    const cudaError_t e = cudaFuncSetAttribute(adj_tile_kernel<VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)adj_smem<VISC>());
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
+  const dim3 grid(adj_tiles_x(a.lay), adj_tiles_y(a.lay));
+  adj_tile_kernel<VISC><<<grid, 32 * ADJ_WARPS, adj_smem<VISC>(), s>>>(a, Unext, Uacc, ra, rb, dt, rhs_mode ? 1 : 0);
+  return cudaGetLastError();
+}
 }  // namespace
 
-long long adj_wrev_doubles(const Lay& L) {
-  const int seg = seg2_of(L);
-  long long n = 4LL * ((L.nx + 2 + seg - 1) / seg) * (seg + 4) * L.ny;
-  if (L.ny > 1) n += 4LL * ((L.ny + 2 + seg - 1) / seg) * (seg + 4) * L.nx;
-  return n;
-}
-
 long long adj_ppart_doubles(const Lay& L, int n_ghost, int n_src, long long nn_blocks) {
-  // pass 1 takes the most blocks with the shortest segments (saved internals)
-  AdjArgs a;
-  a.lay = L;
-  const bool two_d = L.ny > 1;
-  long long b1 = 0;
-  for (int saved = 0; saved < 2; ++saved) {
-    if (saved && !two_d) continue;
-    a.weno_saved = saved;
-    int seg, bx, by;
-    pass1_shape(a, two_d, seg, bx, by);
-    b1 = std::max(b1, (long long)bx + by);
-  }
-  // warps: pass 1 (64-thread blocks), the neural image reverse and primvjp (256), IB (128)
-  const long long warps = 2 * b1 + 8 * nn_blocks + 8 * (long long)blocks_for(L.plane, 256) +
+  // warps: the tiles, the neural image reverse (256 threads a block), IB (128)
+  const long long warps = (long long)ADJ_WARPS * adj_tiles_x(L) * adj_tiles_y(L) + 8 * nn_blocks +
                           4 * (long long)(ib_blocks(n_ghost) + ib_blocks(n_src));
   return 4 * warps;
 }
@@ -197,8 +131,8 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
                              long long* launches, const NnArgs* nn) {
   AdjArgs a = a0;
   const Lay& L = a.lay;
-  const unsigned gp = blocks_for(L.plane, 256);
   long long n = 0;
+  cudaError_t e;
   // warp partials of pbar[0..3]: consecutive slices for the launches that produce them
   double* const pp0 = a0.pbar ? a0.pp : nullptr;
   long long used = 0;
@@ -207,32 +141,22 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
     used += warps;
     return p;
   };
-  a.pp = nullptr;
-  adj_seed_kernel<<<gp, 256, 0, s>>>(a, Unext, Uacc, ra, rb, dt, rhs_mode ? 1 : 0);
-  adj_prims_kernel<<<gp, 256, 0, s>>>(a);
-  n += 2;
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const bool two_d = L.ny > 1;
-  {
-    int seg, bx, by;
-    pass1_shape(a, two_d, seg, bx, by);
-    a.pp = slice(2LL * (bx + by));
-    if ((e = pass1(a, a.visc != 0, two_d, s)) != cudaSuccess) return e;
-  }
   if (nn) {
     // the neural flux: its face-state adjoints join the HLLC ones before the WENO5 reverse
+    adj_nn_seed_kernel<<<blocks_for(L.plane, 256), 256, 0, s>>>(a, const_cast<double*>(a.Q), Unext,
+                                                                 rhs_mode ? 1.0 : rb * dt);
     a.pp = slice(8 * nn_image_vjp_blocks(L));
     if ((e = nn_reverse(*nn, a, s)) != cudaSuccess) return e;
-    n += nn->w_bar ? 13 : 9;
+    n += nn->w_bar ? 14 : 10;
+  } else {
+    a.fadj = nullptr;
   }
-  a.pp = nullptr;
-  if ((e = pass2(a, two_d, s)) != cudaSuccess) return e;
-  n += 2;
-  a.pp = slice(8LL * gp);
-  if (a.visc) adj_primvjp_kernel<true><<<gp, 256, 0, s>>>(a, seg2_of(L));
-  else adj_primvjp_kernel<false><<<gp, 256, 0, s>>>(a, seg2_of(L));
+  a.pp = slice((long long)ADJ_WARPS * adj_tiles_x(L) * adj_tiles_y(L));
+  e = a.visc ? launch_tiles<true>(a, Unext, Uacc, ra, rb, dt, rhs_mode, s)
+             : launch_tiles<false>(a, Unext, Uacc, ra, rb, dt, rhs_mode, s);
+  if (e != cudaSuccess) return e;
   ++n;
+  const bool two_d = L.ny > 1;
   a.pp = nullptr;
   const int tmax = std::max(L.nx + 6, L.ny);
   if (two_d) {

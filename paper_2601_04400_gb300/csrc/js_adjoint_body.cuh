@@ -1,6 +1,6 @@
 // Device bodies of the reverse-mode stage (gradient chain rule of Sec. 2 applied to the
 // discrete operator), shared by the per-grid launches of js_adjoint.cu and the persistent
-// batched reverse kernel of js_batch.cu: one element, line segment or block of each phase.
+// batched reverse kernel of js_batch.cu: one tile, element or block of each phase.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -8,7 +8,6 @@
 #include "js_internal.h"
 
 namespace js {
-
 
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -39,372 +38,312 @@ __device__ __forceinline__ long long global_warp() {
   return ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
 }
 
-__device__ __forceinline__ bool valid_padded(const Lay& L, long long t, int& i, int& j) {
-  const int col = (int)(t % L.pitch);
-  const int row = (int)(t / L.pitch);
-  if (col >= L.nx + 6 || row >= L.H) return false;
-  i = col - 3;
-  j = row - L.gy;
-  return true;
-}
-
-// Position of cell k of line `line` in the saved arrays: y lines use the padded layout
-// (lanes = consecutive columns); x lines are stored transposed so that the lanes of a warp
-// (consecutive rows) also write consecutive addresses.
-template <int DIR>
-__device__ __forceinline__ long long save_id(const AdjArgs& a, int k, int line) {
-  return (DIR == 0) ? (long long)(k + 3) * a.tpitch + (line + a.lay.gy) : a.lay.idx(line, k);
+// Position of face k of line `line` in the planes of the neural flux's face-state adjoints: y lines
+// use the padded layout, x lines are stored transposed (its kernel runs lanes across the lines in
+// both directions).
+__device__ __forceinline__ long long face_id(const AdjArgs& a, int dir, int k, int line) {
+  return dir == 0 ? (long long)(k + 3) * a.tpitch + (line + a.lay.gy) : a.lay.idx(line, k);
 }
 
 // =======================================================================================
-// seed + prims
+// Reverse of one stage on one tile of the padded array: given the adjoint Unext of the stage
+// output and the filled stage state X,
+//   lambda' = b dt Unext on fluid cells (0 elsewhere), U^n part Uacc += a Unext,
+//   Ub(X) = identity and carry terms + (dprim/dX)^T (reverse of the x and y fluxes) + nu lap(lambda')
+// in one pass: primitives and lambda' of the tile and its halo in shared memory, then per line
+// (a warp each, a lane per cell, as in the stage kernel) WENO5 forward, HLLC and viscous forward and
+// reverse per face, WENO5 reverse.  Of the 32 cells of lanes 0..31 the differences serve WENO5 of
+// lanes 1..30, these the faces at i+1/2 of lanes 1..29, these the WENO5 reverse of lanes 2..29 and
+// these the primitive adjoints of lanes 4..27: the 24 outputs.  Nothing is stored between: the
+// WENO5 internals, face adjoints and segment sums that separate passes kept in memory (1.3 KB a
+// cell) are recomputed in integer arithmetic beside the FP64 pipe or passed by shuffles.
+// Every sum has a fixed order, so the reverse pass gives the same bits on every run.
 // =======================================================================================
-__device__ __forceinline__ void adj_seed_one(const AdjArgs& a, long long t, const double* __restrict__ Unext,
-                                             double* __restrict__ Uacc, double ra, double rb, double dt,
-                                             int rhs_mode) {
-  const Lay& L = a.lay;
-  if (t >= L.plane) return;
-  int i, j;
-  if (!valid_padded(L, t, i, j)) return;
-  const bool interior = i >= 0 && i < L.nx && j >= 0 && j < L.ny;
-  const bool fluid = interior && (a.tag == nullptr || a.tag[(long long)j * L.nx + i] == 0);
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const long long o = c * L.plane + t;
-    const double un = interior ? Unext[o] : 0.0;
-    double lam, ub;
-    if (rhs_mode) {
-      lam = fluid ? un : 0.0;
-      ub = 0.0;
-    } else {
-      lam = fluid ? rb * dt * un : 0.0;
-      ub = fluid ? rb * un : un;  // identity on fluid cells, carry on solid and ghost cells
-      if (fluid && ra != 0.0) Uacc[o] += ra * un;
-    }
-    a.lam[o] = lam;
-    a.Ub[o] = ub;
-  }
-}
-
-__device__ __forceinline__ void adj_prims_one(const AdjArgs& a, long long t) {
-  const Lay& L = a.lay;
-  if (t >= L.plane) return;
-  int i, j;
-  if (!valid_padded(L, t, i, j)) return;
-  double u, v, p, T;
-  const double r = a.X[t];
-  cons_to_prim(r, a.X[L.plane + t], a.X[2 * L.plane + t], a.X[3 * L.plane + t], a.gas, u, v, p, T);
-  a.Q[t] = r;
-  a.Q[L.plane + t] = u;
-  a.Q[2 * L.plane + t] = v;
-  a.Q[3 * L.plane + t] = p;
-  a.Q[4 * L.plane + t] = T;
-}
-
-// =======================================================================================
-// pass 1: WENO forward (saved), HLLC + viscous forward and reverse per face
-// =======================================================================================
-// DIR 0: lines are rows, faces f in [0, nx] (face f between cells f-1 and f).
-// DIR 1: lines are columns, faces f in [0, ny].
-template <int DIR, bool VISC, bool HAS_T, bool SAVED>
-__device__ __forceinline__ void pass1_body(const AdjArgs& a, int seg_len, long long item, long long wbase) {
-  const Lay& L = a.lay;
-  const int nline = (DIR == 0) ? L.ny : L.nx;
-  const int ncell = (DIR == 0) ? L.nx : L.ny;
-  const int nseg = (ncell + 1 + seg_len - 1) / seg_len;
-  const bool active = item < (long long)nline * nseg;
-  double gb = 0.0, mub = 0.0, prb = 0.0;
-  if (active) {
-    const int line = (int)(item % nline), seg = (int)(item / nline);
-    const int f0 = seg * seg_len;
-    const int f1 = min(f0 + seg_len, ncell + 1);
-    const long long st = (DIR == 0) ? 1 : L.pitch;   // stride along the line
-    const long long ts = (DIR == 0) ? L.pitch : 1;   // stride across it
-    constexpr int PN = (DIR == 0) ? 1 : 2, PT = (DIR == 0) ? 2 : 1;
-    const double invh = (DIR == 0) ? a.inv_dx : a.inv_dy;
-    const ViscC& vc = (DIR == 0) ? a.vx : a.vy;
-    const int wdir = DIR * 4 * WENO_SAVE;
-    auto cell_id = [&](int k) { return (DIR == 0) ? L.idx(k, line) : L.idx(line, k); };
-    Win4 w;
-    if (!SAVED) w.init(a.Q + cell_id(f0 - 1), L.plane, st);
-    double prevL[4];
-#pragma unroll 1
-    for (int i = f0 - 1; i < f1; ++i) {
-      const long long ci = cell_id(i);
-      const long long si = save_id<DIR>(a, i, line);
-      double Lf[4], Rf[4];
-      if (SAVED) {
-        // face states of cell i from the quotients the forward stage stored
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const double qc = a.Q[c * L.plane + ci];
-          const double* sv = a.wsave + (long long)(wdir + c * WENO_SAVE) * a.splane + si;
-          Lf[c] = fma(sv[3 * a.splane], SIXTH, qc);
-          Rf[c] = fma(sv[5 * a.splane], SIXTH, qc);
-        }
-      } else {
-        w.template step<true, true, true>(a.Q + ci, L.plane, st, Lf, Rf, [&](int c, const double* sv) {
-#pragma unroll
-          for (int k = 0; k < WENO_SAVE; ++k) a.wsave[(long long)(wdir + c * WENO_SAVE + k) * a.splane + si] = sv[k];
-        });
-      }
-      if (i >= f0) {
-        // face f = i between cells i-1 (state prevL) and i (state Rf)
-        const long long ca = ci - st, cb = ci;
-        double ql[4], qr[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) { ql[c] = prevL[c]; qr[c] = Rf[c]; }
-        const bool fallback = !(ql[0] > 0.0 && ql[3] > 0.0 && qr[0] > 0.0 && qr[3] > 0.0);
-        if (fallback) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) { ql[c] = a.Q[c * L.plane + ca]; qr[c] = a.Q[c * L.plane + cb]; }
-        }
-        double Fb[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) Fb[c] = (a.lam[c * L.plane + cb] - a.lam[c * L.plane + ca]) * invh;
-        const Face4 FL{ql[0], ql[PN], ql[PT], ql[3]}, FR{qr[0], qr[PN], qr[PT], qr[3]};
-        Face4 bL{0.0, 0.0, 0.0, 0.0}, bR{0.0, 0.0, 0.0, 0.0};
-        const double Fbn[4] = {Fb[0], Fb[PN], Fb[PT], Fb[3]};
-        hllc_vjp(FL, FR, a.gas, Fbn, bL, bR, gb);
-        double bql[4], bqr[4];
-        bql[0] = bL.r; bql[PN] = bL.un; bql[PT] = bL.ut; bql[3] = bL.p;
-        bqr[0] = bR.r; bqr[PN] = bR.un; bqr[PT] = bR.ut; bqr[3] = bR.p;
-        const int fdir = DIR * 8;
-        // adjoints that go straight to the face's cells ca (left) and cb (right): rho, u, v, p, T
-        double dca[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, dcb[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        if (fallback) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            dca[c] = bql[c];
-            dcb[c] = bqr[c];
-            a.fadj[(long long)(fdir + c) * a.splane + si] = 0.0;
-            a.fadj[(long long)(fdir + 4 + c) * a.splane + si] = 0.0;
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            a.fadj[(long long)(fdir + c) * a.splane + si] = bql[c];      // left state of face
-            a.fadj[(long long)(fdir + 4 + c) * a.splane + si] = bqr[c];  // right state of face
-          }
-        }
-        double* fc = a.fcell + (long long)(DIR * 12) * a.splane + si;
-        if (VISC) {
-          // F[n] -= tnn; F[t] -= tnt; F[3] -= 0.5 (sbn tnn + sbt tnt) + ck dT
-          const double* un = a.Q + PN * L.plane;
-          const double* ut = a.Q + PT * L.plane;
-          const double* Tq = a.Q + 4 * L.plane;
-          const double dun = un[cb] - un[ca], dut = ut[cb] - ut[ca], dT = Tq[cb] - Tq[ca];
-          double sun = 0.0, sut = 0.0, tnn, tnt;
-          if (HAS_T) {
-            sun = (un[ca + ts] - un[ca - ts]) + (un[cb + ts] - un[cb - ts]);
-            sut = (ut[ca + ts] - ut[ca - ts]) + (ut[cb + ts] - ut[cb - ts]);
-            tnn = fma(vc.c43n, dun, -vc.c23t * sut);
-            tnt = fma(vc.cn, dut, vc.ct * sun);
-          } else {
-            tnn = vc.c43n * dun;
-            tnt = vc.cn * dut;
-          }
-          const double sbn = un[ca] + un[cb], sbt = ut[ca] + ut[cb];
-          const double btnn = -Fb[PN] - 0.5 * Fb[3] * sbn;
-          const double btnt = -Fb[PT] - 0.5 * Fb[3] * sbt;
-          const double bsbn = -0.5 * Fb[3] * tnn, bsbt = -0.5 * Fb[3] * tnt;
-          const double bck = -Fb[3] * dT;
-          const double bdT = -Fb[3] * vc.ck;
-          const double bdun = vc.c43n * btnn, bdut = vc.cn * btnt;
-          dca[PN] += bsbn - bdun;
-          dcb[PN] += bsbn + bdun;
-          dca[PT] += bsbt - bdut;
-          dcb[PT] += bsbt + bdut;
-          dca[4] = -bdT;
-          dcb[4] = bdT;
-          // tangential differences: +(bsun, bsut) to the cells ca + ts and cb + ts, minus to
-          // ca - ts and cb - ts (gathered by those cells)
-          fc[10 * a.splane] = HAS_T ? vc.ct * btnt : 0.0;
-          fc[11 * a.splane] = HAS_T ? -vc.c23t * btnn : 0.0;
-          const double ckck = bck * vc.ck;
-          mub += a.inv_mu * fma(btnn, tnn, fma(btnt, tnt, ckck));
-          gb += a.kg * ckck;
-          prb += a.kp * ckck;
-        }
-#pragma unroll
-        for (int c = 0; c < (VISC ? 5 : 4); ++c) {
-          fc[c * a.splane] = dca[c];
-          fc[(5 + c) * a.splane] = dcb[c];
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) prevL[c] = Lf[c];
-    }
-  }
-  warp_partials(a.pp, wbase + (item >> 5), gb, mub, prb, 0.0);
-}
-
-// =======================================================================================
-// pass 2: WENO reverse from the saved internals, along line segments.  Segment `seg` of a
-// line runs cells c0 = -1 + seg * L .. c1 - 1 and emits the adjoints of cells c0 - 2 .. c1 + 1
-// (its whole reach) into its own slots; a cell's total is gathered later from the (at most
-// three) segments that reach it, in segment order.
-// =======================================================================================
-// slot k of segment seg, variable c, in direction DIR's part of wrev (lines fastest)
-template <int DIR>
-__device__ __forceinline__ long long wrev_slot(const Lay& L, int seg_len, int c, int seg, int k, int line) {
-  const int nline = (DIR == 0) ? L.ny : L.nx;
-  const int ncell = (DIR == 0) ? L.nx : L.ny;
-  const long long nseg = (ncell + 2 + seg_len - 1) / seg_len;
-  const long long base = (DIR == 0) ? 0 : 4LL * ((L.nx + 2 + seg_len - 1) / seg_len) * (seg_len + 4) * L.ny;
-  return base + ((c * nseg + seg) * (seg_len + 4) + k) * nline + line;
-}
-
-template <int DIR>
-__device__ __forceinline__ void pass2_body(const AdjArgs& a, int seg_len, long long item) {
-  const Lay& L = a.lay;
-  const int nline = (DIR == 0) ? L.ny : L.nx;
-  const int ncell = (DIR == 0) ? L.nx : L.ny;
-  const int nseg = (ncell + 2 + seg_len - 1) / seg_len;  // cells -1 .. ncell
-  if (item >= (long long)nline * nseg) return;
-  const int line = (int)(item % nline), seg = (int)(item / nline);
-  const int c0 = -1 + seg * seg_len;
-  const int c1 = min(c0 + seg_len, ncell + 1);
-  const long long st = (DIR == 0) ? 1 : L.pitch;
-  const int wdir = DIR * 4 * WENO_SAVE;
-  const int fdir = DIR * 8;
-  auto cell_id = [&](int k) { return (DIR == 0) ? L.idx(k, line) : L.idx(line, k); };
-  for (int c = 0; c < 4; ++c) {
-    // one variable at a time keeps the register window small
-    const double* q = a.Q + c * L.plane;
-    double* out = a.wrev + wrev_slot<DIR>(L, seg_len, c, seg, 0, line);
-    long long ci = cell_id(c0);
-    const long long sst = (DIR == 0) ? a.tpitch : L.pitch;  // stride along the line in saved arrays
-    long long si = save_id<DIR>(a, c0, line);
-    WenoRev w;
-    w.init(q[ci - 2 * st], q[ci - st], q[ci], q[ci + st]);
-    int k = 0;  // slot of cell c0 - 2 + k
-#pragma unroll 1
-    for (int i = c0; i < c1; ++i, ci += st, si += sst, ++k) {
-      double sv[WENO_SAVE];
-#pragma unroll
-      for (int m = 0; m < WENO_SAVE; ++m) sv[m] = a.wsave[(long long)(wdir + c * WENO_SAVE + m) * a.splane + si];
-      const double Lb = a.fadj[(long long)(fdir + c) * a.splane + si + sst];  // left state of face i+1/2
-      const double Rb = a.fadj[(long long)(fdir + 4 + c) * a.splane + si];    // right state of face i-1/2
-      // cell i-2: this segment's contribution is complete
-      out[(long long)k * nline] = w.step(q[ci + 2 * st], sv, Lb, Rb);
-    }
-    // cells c1-2 .. c1+1
-    double rest[4];
-    w.flush(rest);
-    for (int m = 0; m < 4; ++m) out[(long long)(k + m) * nline] = rest[m];
-  }
-}
-
-// sum of the pass-2 slots of the segments of a DIR line that reach cell m (-3 <= m <= ncell + 2),
-// in segment order
-template <int DIR>
-__device__ __forceinline__ double wrev_gather(const AdjArgs& a, int seg_len, int c, int m, int line) {
-  const Lay& L = a.lay;
-  const int ncell = (DIR == 0) ? L.nx : L.ny;
-  const int nseg = (ncell + 2 + seg_len - 1) / seg_len;
-  int s = (m + 1 >= 0) ? (m + 1) / seg_len : 0;
-  s = min(s, nseg - 1);
-  double t = 0.0;
-  for (int q = s - 1; q <= s + 1; ++q) {
-    if (q < 0 || q >= nseg) continue;
-    const int c0 = -1 + q * seg_len;
-    const int c1 = min(c0 + seg_len, ncell + 1);
-    if (m < c0 - 2 || m >= c1 + 2) continue;
-    t += a.wrev[wrev_slot<DIR>(L, seg_len, c, q, m - (c0 - 2), line)];
-  }
-  return t;
-}
-
-// =======================================================================================
-// prim reverse (+ artificial viscosity), after gathering each cell's primitive adjoint
-// =======================================================================================
-// per-face adjoints of direction DIR that reach padded cell (i, j), added to qb in a fixed
-// order: the face to its low side (the cell is its right cell), the face to its high side,
-// then (viscous, 2D) the tangential-difference terms of the faces of the two neighbouring
-// lines: + from the line below, - from the line above
-template <int DIR, bool VISC>
-__device__ __forceinline__ void face_gather(const AdjArgs& a, int i, int j, double qb[5]) {
-  const Lay& L = a.lay;
-  const int m = (DIR == 0) ? i : j, line = (DIR == 0) ? j : i;
-  const int nline = (DIR == 0) ? L.ny : L.nx, ncell = (DIR == 0) ? L.nx : L.ny;
-  constexpr int PN = (DIR == 0) ? 1 : 2, PT = (DIR == 0) ? 2 : 1, NC = VISC ? 5 : 4;
-  const long long sp = a.splane;
-  const double* fc = a.fcell + (long long)(DIR * 12) * sp;
-  if (line >= 0 && line < nline) {
-    if (m >= 0 && m <= ncell) {
-      const long long f = save_id<DIR>(a, m, line);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) qb[c] += fc[(5 + c) * sp + f];
-    }
-    if (m + 1 >= 0 && m + 1 <= ncell) {
-      const long long f = save_id<DIR>(a, m + 1, line);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) qb[c] += fc[c * sp + f];
-    }
-  }
-  if (VISC && a.two_d) {
-#pragma unroll
-    for (int dl = -1; dl <= 1; dl += 2) {
-      const int ln = line + dl;
-      if (ln < 0 || ln >= nline) continue;
-      for (int f = m; f <= m + 1; ++f) {
-        if (f < 0 || f > ncell) continue;
-        const long long id = save_id<DIR>(a, f, ln);
-        if (dl < 0) {
-          qb[PN] += fc[10 * sp + id];
-          qb[PT] += fc[11 * sp + id];
-        } else {
-          qb[PN] -= fc[10 * sp + id];
-          qb[PT] -= fc[11 * sp + id];
-        }
-      }
-    }
-  }
-}
-
-// padded cell t; the gamma and nu parameter-gradient contributions are added to gb, nb
+constexpr int AB = 34;              // box of the tile: outputs at 5 .. 28
+constexpr int AP = AB * AB;
+constexpr int AQ = ADJ_TILE + 1;    // row pitch of the accumulator planes
+constexpr int AA = ADJ_TILE * AQ;
+constexpr int AS = (ADJ_TILE + 2) * AQ;  // tangential terms: lines -1 .. 24
+// doubles of shared memory: 4 planes of primitives, 4 of lambda', accumulators (5 viscous), 2 planes
+// of tangential terms (viscous)
 template <bool VISC>
-__device__ __forceinline__ void adj_primvjp_one(const AdjArgs& a, long long t, int seg_len, double& gb, double& nb) {
+__host__ __device__ constexpr size_t adj_smem() {
+  return sizeof(double) * (size_t)(8 * AP + (VISC ? 5 * AA + 2 * AS : 4 * AA));
+}
+
+// the reverse of one line at the lane's cell (q: primitives, l: lambda'; neighbours at multiples of
+// st, across the line of ts).  f: number of the face at i+1/2 (faces 0 .. n exist), own: the lane's
+// face counts for the parameter gradient, out(c, v) receives the adjoint of primitive c (lanes
+// 4..27), tang(n, t) the cell's tangential terms of its two faces (VISC, 2D).
+template <bool VISC, bool HAS_T, class Nn, class Out, class Tang>
+__device__ __forceinline__ void adj_line(const double* q, const double* l, int st, int ts, int pn, int f, int n,
+                                         const Gas& g, const ViscC& vc, double invh, bool own, double& gs1,
+                                         double& gs2, double& vmu, double& vk, Nn nn, Out out, Tang tang) {
+  const int lane = threadIdx.x & 31;
+  const bool inner = lane - 1u < 30u;
+  const int pt = 3 - pn;
+  const bool face = lane >= 1 && lane <= 29 && f >= 0 && f <= n;
+  double L[4], R[4];
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) {
+    const int c = (k == 1) ? pn : (k == 2) ? pt : k;
+    double Lf, Rf;
+    weno_lane(q + c * AP, st, k == 0 || k == 3, inner, Lf, Rf);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      L[m] = (k == m) ? Lf : L[m];
+      R[m] = (k == m) ? Rf : R[m];
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) R[m] = __shfl_down_sync(0xffffffffu, R[m], 1);
+  const double* un = q + pn * AP;
+  const double* ut = q + pt * AP;
+  const bool fallback = !(positive(L[0]) && positive(L[3]) && positive(R[0]) && positive(R[3]));
+  if (fallback) {
+    L[0] = q[0], L[1] = un[0], L[2] = ut[0], L[3] = q[3 * AP];
+    R[0] = q[st], R[1] = un[st], R[2] = ut[st], R[3] = q[3 * AP + st];
+  }
+  double Fb[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const double* lm = l + (m == 1 ? pn : m == 2 ? pt : m) * AP;
+    Fb[m] = (lm[st] - lm[0]) * invh;
+  }
+  double bL[4], bR[4], s1 = 0.0, s2 = 0.0;
+  hllc_vjp(L, R, g, Fb, bL, bR, s1, s2);
+  if (own && face) {
+    gs1 += s1;
+    gs2 += s2;
+  }
+  // adjoints that go straight to the face's cells: its left cell (dl) and its right cell (dr)
+  double dl[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, dr[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    dl[m] = fallback && face ? bL[m] : 0.0;
+    dr[m] = fallback && face ? bR[m] : 0.0;
+    bL[m] = fallback || !face ? 0.0 : bL[m];
+    bR[m] = fallback || !face ? 0.0 : bR[m];
+  }
+  nn(face, bL, bR);
+  bool straight = __any_sync(0xffffffffu, fallback && face);
+  if (VISC) {
+    // F[n] -= tnn; F[t] -= tnt; F[3] -= 0.5 (sbn tnn + sbt tnt) + ck dT
+    const double Tc = q[3 * AP] * recip(q[0]);
+    const double dT = __shfl_down_sync(0xffffffffu, Tc, 1) - Tc;
+    const double ua = un[0], ub = un[st], ta = ut[0], tb = ut[st];
+    const double dun = ub - ua, dut = tb - ta;
+    double tnn, tnt;
+    if (HAS_T) {
+      const double sun = (un[ts] - un[-ts]) + (un[st + ts] - un[st - ts]);
+      const double sut = (ut[ts] - ut[-ts]) + (ut[st + ts] - ut[st - ts]);
+      tnn = fma(vc.c43n, dun, -vc.c23t * sut);
+      tnt = fma(vc.cn, dut, vc.ct * sun);
+    } else {
+      tnn = vc.c43n * dun;
+      tnt = vc.cn * dut;
+    }
+    const double h3 = 0.5 * Fb[3];
+    const double btnn = fma(-h3, ua + ub, -Fb[1]), btnt = fma(-h3, ta + tb, -Fb[2]);
+    const double bck = -Fb[3] * dT, bdT = -Fb[3] * vc.ck;
+    const double bn = -h3 * tnn, bt = -h3 * tnt, bdun = vc.c43n * btnn, bdut = vc.cn * btnt;
+    if (face) {
+      dl[1] += bn - bdun;
+      dr[1] += bn + bdun;
+      dl[2] += bt - bdut;
+      dr[2] += bt + bdut;
+      dl[4] = -bdT;
+      dr[4] = bdT;
+      if (own) {
+        vmu += fma(btnn, tnn, fma(btnt, tnt, bck * vc.ck));
+        vk += bck * vc.ck;
+      }
+    }
+    if (HAS_T) {
+      // tangential differences: + to the cells one line up, minus to those one line down
+      const double xn = face ? vc.ct * btnt : 0.0, xt = face ? -vc.c23t * btnn : 0.0;
+      tang(xn + __shfl_up_sync(0xffffffffu, xn, 1), xt + __shfl_up_sync(0xffffffffu, xt, 1));
+    }
+    straight = true;
+  }
+  if (straight) {
+#pragma unroll
+    for (int m = 0; m < (VISC ? 5 : 4); ++m)
+      out((m == 1) ? pn : (m == 2) ? pt : m, dl[m] + __shfl_up_sync(0xffffffffu, dr[m], 1));
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) bR[m] = __shfl_up_sync(0xffffffffu, bR[m], 1);  // of the face at i-1/2
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) {
+    const int c = (k == 1) ? pn : (k == 2) ? pt : k;
+    const double Lb = (k == 0) ? bL[0] : (k == 1) ? bL[1] : (k == 2) ? bL[2] : bL[3];
+    const double Rb = (k == 0) ? bR[0] : (k == 1) ? bR[1] : (k == 2) ? bR[2] : bR[3];
+    double w[4];
+    weno_grad_lane(q + c * AP, st, k == 0 || k == 3, inner, Lb, Rb, w);
+    // adjoint of d_{i+1/2}: its share in the cells i-1 .. i+2
+    const double t = (w[2] + __shfl_up_sync(0xffffffffu, w[3], 1)) +
+                     (__shfl_down_sync(0xffffffffu, w[1], 1) + __shfl_down_sync(0xffffffffu, w[0], 2));
+    out(c, fma(SIXTH, __shfl_up_sync(0xffffffffu, t, 1) - t, Lb + Rb));
+  }
+}
+
+// tile (bx, by) of the padded array; slot0: warp slot of the tile's partials of pbar[0..3]
+template <bool VISC>
+__device__ __forceinline__ void adj_tile(const AdjArgs& a, const double* __restrict__ Unext, double* __restrict__ Uacc,
+                                         double ra, double rb, double dt, int rhs_mode, int bx, int by, double* smem,
+                                         long long slot0) {
   const Lay& L = a.lay;
-  int i = 0, j = 0;
-  if (t < L.plane && valid_padded(L, t, i, j)) {
-    // primitive adjoint: WENO5 reverse of the cell's x line and y line, then the faces
-    double qb[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    if (j >= 0 && j < L.ny) {
+  double* sq = smem;
+  double* sl = smem + 4 * AP;
+  double* acc = smem + 8 * AP;
+  double* tan = acc + 5 * AA;  // VISC
+  const Gas g = a.gas;
+  const int W = L.nx + 6;
+  const int ox = bx * ADJ_TILE, oy = by * ADJ_TILE;  // padded coordinates of the first output
+  const double bdt = rhs_mode ? 1.0 : rb * dt;
+  for (int e = threadIdx.x; e < AP; e += blockDim.x) {
+    const int row = e / AB, col = e - row * AB;
+    const int gx = ox - 5 + col, gy = oy - 5 + row;
+    const bool in = gx >= 0 && gx < W && gy >= 0 && gy < L.H;
+    const long long t = in ? (long long)gy * L.pitch + gx : 0;
+    const double r = a.X[t], mx = a.X[L.plane + t], my = a.X[2 * L.plane + t], E = a.X[3 * L.plane + t];
+    double u = 0.0, v = 0.0, p = 1.0, T;
+    if (in) cons_to_prim(r, mx, my, E, g, u, v, p, T);
+    sq[e] = in ? r : 1.0;
+    sq[AP + e] = u;
+    sq[2 * AP + e] = v;
+    sq[3 * AP + e] = p;
+    const int i = gx - 3, j = gy - L.gy;
+    const bool fluid = i >= 0 && i < L.nx && j >= 0 && j < L.ny && (a.tag == nullptr || a.tag[(long long)j * L.nx + i] == 0);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) qb[c] += wrev_gather<0>(a, seg_len, c, i, j);
-    }
-    if (a.two_d && i >= 0 && i < L.nx) {
+    for (int c = 0; c < 4; ++c) sl[c * AP + e] = fluid ? bdt * Unext[c * L.plane + t] : 0.0;
+  }
+  for (int e = threadIdx.x; e < (VISC ? 5 : 4) * AA; e += blockDim.x) acc[e] = 0.0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int k = lane - 4;  // the lane's cell: output k of the line
+  const bool own = k >= 0 && k < ADJ_TILE;
+  double gs1 = 0.0, gs2 = 0.0, vmu = 0.0, vk = 0.0, gb = 0.0, nb = 0.0;
+#pragma unroll 1
+  for (int dir = 0; dir < (a.two_d ? 2 : 1); ++dir) {
+    const int st = dir == 0 ? 1 : AB, ts = dir == 0 ? AB : 1;
+    const int k0 = (dir == 0 ? ox - 3 : oy - L.gy), l0 = (dir == 0 ? oy - L.gy : ox - 3);  // grid cell of output 0
+    const int nline = dir == 0 ? L.ny : L.nx, ncell = dir == 0 ? L.nx : L.ny;
+    const ViscC vc = dir == 0 ? a.vx : a.vy;
+    const double invh = dir == 0 ? a.inv_dx : a.inv_dy;
+    const int pn = dir + 1;
+    // with tangential terms the lines next to the tile are needed for those alone
+    const int edge = VISC && a.two_d ? 1 : 0;
+#pragma unroll 1
+    for (int ln = warp - edge; ln < ADJ_TILE + edge; ln += nwarp) {
+      const double* q = sq + (ln + 5) * ts + (k + 5) * st;
+      const double* lm = sl + (ln + 5) * ts + (k + 5) * st;
+      const int line = l0 + ln, f = k0 + k + 1;
+      if (VISC && a.two_d && (ln < 0 || ln >= ADJ_TILE || line < 0 || line >= nline)) {
+        // tangential terms only (zero past the grid's lines)
+        double xn = 0.0, xt = 0.0;
+        if (line >= 0 && line < nline && lane >= 1 && lane <= 29 && f >= 0 && f <= ncell) {
+          const double* un = q + pn * AP;
+          const double* ut = q + (3 - pn) * AP;
+          const double h3 = 0.5 * ((lm[3 * AP + st] - lm[3 * AP]) * invh);
+          const double Fn = (lm[pn * AP + st] - lm[pn * AP]) * invh, Ft = (lm[(3 - pn) * AP + st] - lm[(3 - pn) * AP]) * invh;
+          xn = vc.ct * fma(-h3, ut[0] + ut[st], -Ft);
+          xt = -vc.c23t * fma(-h3, un[0] + un[st], -Fn);
+        }
+        const double xn1 = __shfl_up_sync(0xffffffffu, xn, 1), xt1 = __shfl_up_sync(0xffffffffu, xt, 1);
+        if (own) {
+          tan[(ln + 1) * AQ + k] = xn + xn1;
+          tan[AS + (ln + 1) * AQ + k] = xt + xt1;
+        }
+        continue;
+      }
+      if (line < 0 || line >= nline) continue;
+      double* o = acc + (dir == 0 ? ln * AQ + k : k * AQ + ln);
+      auto nn = [&](bool face, double bL[4], double bR[4]) {
+        if (a.fadj == nullptr || !face) return;
+        const long long si = face_id(a, dir, f, line);
+        const double* fa = a.fadj + (long long)(dir * 8) * a.splane + si;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) qb[c] += wrev_gather<1>(a, seg_len, c, j, i);
+        for (int m = 0; m < 4; ++m) {
+          const int c = (m == 1) ? pn : (m == 2) ? 3 - pn : m;
+          bL[m] += fa[c * a.splane];
+          bR[m] += fa[(4 + c) * a.splane];
+        }
+      };
+      auto out = [&](int c, double v) {
+        if (own) o[c * AA] += v;
+      };
+      auto tang = [&](double xn, double xt) {
+        if (own) {
+          tan[(ln + 1) * AQ + k] = xn;
+          tan[AS + (ln + 1) * AQ + k] = xt;
+        }
+      };
+      if (a.two_d) adj_line<VISC, true>(q, lm, st, ts, pn, f, ncell, g, vc, invh, own, gs1, gs2, vmu, vk, nn, out, tang);
+      else adj_line<VISC, false>(q, lm, st, ts, pn, f, ncell, g, vc, invh, own, gs1, gs2, vmu, vk, nn, out, tang);
     }
-    face_gather<0, VISC>(a, i, j, qb);
-    if (a.two_d) face_gather<1, VISC>(a, i, j, qb);
-    double ub[4];
-    prim_vjp(a.X[t], a.X[L.plane + t], a.X[2 * L.plane + t], a.X[3 * L.plane + t], a.gas, qb, ub, gb);
+    __syncthreads();
+    if (VISC && a.two_d) {
+      // tangential terms: from the line below and, negative, from the line above
+      for (int e = threadIdx.x; e < ADJ_TILE * ADJ_TILE; e += blockDim.x) {
+        const int ln = e / ADJ_TILE, kk = e - ln * ADJ_TILE;
+        double* o = acc + (dir == 0 ? ln * AQ + kk : kk * AQ + ln);
+        o[pn * AA] += tan[ln * AQ + kk] - tan[(ln + 2) * AQ + kk];
+        o[(3 - pn) * AA] += tan[AS + ln * AQ + kk] - tan[AS + (ln + 2) * AQ + kk];
+      }
+      __syncthreads();
+    }
+  }
+  // primitive reverse, artificial viscosity, identity terms
+  for (int e = threadIdx.x; e < ADJ_TILE * ADJ_TILE; e += blockDim.x) {
+    const int ty = e / ADJ_TILE, tx = e - ty * ADJ_TILE;
+    const int gx = ox + tx, gy = oy + ty;
+    if (gx >= W || gy >= L.H) continue;
+    const int i = gx - 3, j = gy - L.gy;
+    const long long t = (long long)gy * L.pitch + gx;
+    const int b = (ty + 5) * AB + tx + 5;
+    double qb[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, ub[4];
+#pragma unroll
+    for (int c = 0; c < (VISC ? 5 : 4); ++c) qb[c] = acc[c * AA + ty * AQ + tx];
+    prim_vjp(sq[b], sq[AP + b], sq[2 * AP + b], sq[3 * AP + b], g, qb, ub, gb);
+    const bool interior = i >= 0 && i < L.nx && j >= 0 && j < L.ny;
     if (a.has_av) {
       const bool near = i >= -1 && i <= L.nx && j >= (a.two_d ? -1 : 0) && j <= (a.two_d ? L.ny : 0);
-      const bool interior = i >= 0 && i < L.nx && j >= 0 && j < L.ny;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const double* lam = a.lam + c * L.plane;
+        const double* lam = sl + c * AP + b;
         if (near) {
-          double add = a.nu_x * ((lam[t - 1] - 2.0 * lam[t]) + lam[t + 1]);
-          if (a.two_d) add += a.nu_y * ((lam[t - L.pitch] - 2.0 * lam[t]) + lam[t + L.pitch]);
+          double add = a.nu_x * ((lam[-1] - 2.0 * lam[0]) + lam[1]);
+          if (a.two_d) add += a.nu_y * ((lam[-AB] - 2.0 * lam[0]) + lam[AB]);
           ub[c] += add;
         }
-        if (interior && lam[t] != 0.0) {
+        if (interior && lam[0] != 0.0) {
           const double* X = a.X + c * L.plane;
           double lap = a.nu_x1 * ((X[t - 1] - 2.0 * X[t]) + X[t + 1]);
           if (a.two_d) lap += a.nu_y1 * ((X[t - L.pitch] - 2.0 * X[t]) + X[t + L.pitch]);
-          nb += lam[t] * lap;
+          nb += lam[0] * lap;
         }
       }
     }
+    const bool fluid = interior && (a.tag == nullptr || a.tag[(long long)j * L.nx + i] == 0);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) a.Ub[c * L.plane + t] += ub[c];
+    for (int c = 0; c < 4; ++c) {
+      const long long o = c * L.plane + t;
+      if (interior && !rhs_mode) {
+        const double un = Unext[o];
+        ub[c] += fluid ? rb * un : un;  // identity on fluid cells, carry on solid and ghost cells
+        if (fluid && ra != 0.0) Uacc[o] += ra * un;
+      }
+      a.Ub[o] = ub[c];
+    }
   }
+  gb += gs2 / g.gamma - gs1 * g.g1 * g.g1;
+  if (VISC) {
+    gb += a.kg * vk;
+    vmu *= a.inv_mu;
+    vk *= a.kp;
+  }
+  warp_partials(a.pp, slot0 + warp, gb, vmu, vk, nb);
 }
 
 // =======================================================================================
@@ -479,9 +418,9 @@ __device__ __forceinline__ void adj_bcT_one(const AdjArgs& a, const BcArgs& bc, 
 __device__ __forceinline__ void adj_inflow_block(const AdjArgs& a, const BcArgs& bc, const double* inflow_part,
                                                  int tmax, const double* inflow_prim) {
   __shared__ double S[4][4];
-  const int side = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int side = threadIdx.x >> 5, lane = threadIdx.x & 31;  // (at least four warps)
   const Lay& L = a.lay;
-  if (bc.kind[side] == 3 && a.pbar != nullptr) {
+  if (side < 4 && bc.kind[side] == 3 && a.pbar != nullptr) {
     const int ntan = (side < 2) ? L.ny : L.nx + 6;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     for (int k = lane; k < ntan; k += 32)
@@ -608,7 +547,10 @@ __device__ __forceinline__ void adj_ib_src_one(const AdjArgs& a, const IbTArgs& 
     const long long id = tb.cell[s];
     // the fill used IEEE-rounded primitives; their derivative is the same map
     double ub[4];
-    prim_vjp(a.X[id], a.X[L.plane + id], a.X[2 * L.plane + id], a.X[3 * L.plane + id], a.gas, S, ub, gb);
+    double u, v, p, T;
+    const double r = a.X[id];
+    cons_to_prim(r, a.X[L.plane + id], a.X[2 * L.plane + id], a.X[3 * L.plane + id], a.gas, u, v, p, T);
+    prim_vjp(r, u, v, p, a.gas, S, ub, gb);
 #pragma unroll
     for (int c = 0; c < 4; ++c) a.Ub[c * L.plane + id] += ub[c];
   }

@@ -29,10 +29,10 @@
 
 namespace js {
 
-// the per-grid tile; the forward launch runs 7 warps a block like the per-grid kernel, the
-// reverse launches 4 (their other phases hold more registers)
+// the per-grid tiles; the forward launch runs 7 warps a block, the reverse launches 8, like the
+// per-grid kernels
 constexpr int BTX = TILE, BTY = TILE;
-constexpr int FNT = 224, BNT = 128;
+constexpr int FNT = 224, BNT = 32 * ADJ_WARPS;
 
 struct BatchArgs {
   const InstDesc* inst;
@@ -124,7 +124,7 @@ __device__ __forceinline__ double inst_dt(const InstDesc& d, const unsigned long
   return dt;
 }
 
-__global__ void __launch_bounds__(FNT, 3) batch_kernel(BatchArgs b) {
+__global__ void __launch_bounds__(FNT, 2) batch_kernel(BatchArgs b) {
   extern __shared__ double smem[];
   const int ntiles = b.tile0[b.count];
   const long long nghost = b.ghost0[b.count], nhalo = b.halo0[b.count];
@@ -303,19 +303,18 @@ __global__ void __launch_bounds__(FNT, 3) batch_kernel(BatchArgs b) {
 // gradient chain rule of Sec. 2 per instance) -- the per-grid js_step_vjp's phases, each run
 // over the work items of all instances, separated by grid barriers:
 //   pack U_n, lambda_{n+1}; zero Uacc
-//   forward recompute, stages 0 and 1: IB fill | halo fill | stage tiles (storing their WENO5
-//   internals); IB and halo fill of the stage-2 input
-//   reverse, stages 2, 1, 0: seed + primitives (+ the previous stage's parameter-gradient
-//   reduction) | pass 1 | pass 2 | primitive reverse | transposed y halos | transposed x halos |
-//   inflow gradient + transposed IB ghosts | transposed IB sources
+//   forward recompute, stages 0 and 1: IB fill | halo fill | stage tiles; IB and halo fill of
+//   the stage-2 input
+//   reverse, stages 2, 1, 0: reverse tiles | transposed y halos (+ the previous stage's part of
+//   the parameter gradient is reduced before the tiles) | transposed x halos | inflow gradient +
+//   transposed IB ghosts | transposed IB sources
 //   unpack lambda_n (+ the last reduction)
 // The device bodies are those of the per-grid launches (js_adjoint_body.cuh, js_stage.cuh,
-// js_fill.cuh) on the same elements in the same order, so lambda_n equals js_step_vjp's bit for
-// bit; the parameter gradient is reduced in a fixed order too (its partial sums are grouped
-// by 128-thread blocks here, so it agrees with js_step_vjp's to rounding).
-// Work items of every instance are padded to whole warps, so a warp never spans two instances.
+// js_fill.cuh) on the same elements in the same order; the parameter gradient is reduced in a
+// fixed order too.  Work items of every instance are padded to whole warps, so a warp never spans
+// two instances.
 // =======================================================================================
-enum RevKind { RK_PLANE = 0, RK_USER4, RK_GHOST, RK_HALO, RK_P1RE, RK_P1SV, RK_P2, RK_BCTY, RK_BCTX, RK_SRC, RK_N };
+enum RevKind { RK_PLANE = 0, RK_USER4, RK_GHOST, RK_HALO, RK_BCTY, RK_BCTX, RK_SRC, RK_N };
 
 struct RevCall {
   const double* const* Un;    // [count] user states U_n
@@ -324,7 +323,7 @@ struct RevCall {
   double* const* pbar;        // [count] parameter gradients (entries may be null) or null
   const double* dt;           // [count] step sizes
   // [count] the step's stage states U1, U2 (user layout, e.g. kept by a rollout's forward), or
-  // null: the reverse recomputes them (storing their WENO5 internals for pass 1 of stages 1, 0)
+  // null: the reverse recomputes them
   const double* const* U1;
   const double* const* U2;
 };
@@ -335,6 +334,7 @@ struct BatchRevArgs {
   int count;
   const long long* pre;       // [RK_N][count + 1] prefix sums of the padded item counts
   const int* tile0;
+  const int* rtile0;          // prefix sums (count + 1) of the reverse tiles
   RevCall call;
   unsigned* bar;
   int* err;
@@ -359,10 +359,6 @@ __device__ __forceinline__ void rev_items(const BatchRevArgs& b, int kind, F f) 
   }
 }
 
-// pass 1 of reverse stage s reads the WENO5 internals stored by the forward recompute (stages
-// 1, 0 when the reverse recomputes the stage states) or recomputes them
-__device__ __forceinline__ bool rev_saved(const RevCall& call, int s) { return s < 2 && call.U1 == nullptr; }
-
 __device__ __forceinline__ AdjArgs rev_adj(const InstRev& r, const InstDesc& d, int s, const RevCall& call, int k,
                                            double* dst, bool with_pbar) {
   AdjArgs a = r.a;
@@ -370,21 +366,15 @@ __device__ __forceinline__ AdjArgs rev_adj(const InstRev& r, const InstDesc& d, 
   a.Ub = dst;
   a.pbar = with_pbar && call.pbar ? call.pbar[k] : nullptr;
   a.pp = a.pbar ? r.ppart : nullptr;
-  if (rev_saved(call, s)) {
-    a.wsave = r.wfwd + (long long)56 * s * r.a.splane;
-    a.weno_saved = 1;
-  } else {
-    a.wsave = r.wsave_own;
-    a.weno_saved = 0;
-  }
+  a.fadj = nullptr;
   return a;
 }
 
-// the parameter-gradient slot ranges of reverse stage s of one instance, summed into its pbar
-__device__ __forceinline__ void rev_reduce(const InstRev& r, bool saved, double* pbar) {
-  const long long off[4] = {0, r.off_prim, r.off_g, r.off_s};
-  const long long cnt[4] = {saved ? r.w1_sv : r.w1_re, r.w_prim, r.w_g, r.w_s};
-  adj_pbar_reduce_block(r.ppart, off, cnt, 4, pbar);
+// the parameter-gradient slot ranges of one reverse stage of one instance, summed into its pbar
+__device__ __forceinline__ void rev_reduce(const InstRev& r, double* pbar) {
+  const long long off[3] = {0, r.off_g, r.off_s};
+  const long long cnt[3] = {r.w_adj, r.w_g, r.w_s};
+  adj_pbar_reduce_block(r.ppart, off, cnt, 3, pbar);
 }
 
 // The phases of one batched reverse step.  Each runs over the work items of all instances with
@@ -395,11 +385,9 @@ enum RevPhase {
   RP_PACK = 0,      // pack U_n, lambda_{n+1} (and given stage states); Uacc = 0
   RP_GHOST,         // IB fill of stage input s
   RP_HALO,          // halo fill of stage input s
-  RP_STAGE,         // forward recompute of stage s (0, 1), storing its WENO5 internals
-  RP_SEED,          // reverse stage s: seed + primitives (+ reduction of stage s+1's partials)
-  RP_PASS1,         // pass 1 (x lines, then y lines)
-  RP_PASS2,         // pass 2
-  RP_PRIMVJP,       // primitive reverse
+  RP_STAGE,         // forward recompute of stage s (0, 1)
+  RP_REDUCE,        // the parameter gradient of reverse stage s+1 (before the tiles reuse its slots)
+  RP_TILES,         // reverse tiles of stage s
   RP_BCTY,          // transposed y halos
   RP_BCTX,          // transposed x halos
   RP_INFLOW_GHOST,  // inflow-state gradient + transposed IB ghosts
@@ -407,48 +395,6 @@ enum RevPhase {
   RP_UNPACK,        // lambda_n = P1 + Uacc; the last stage's parameter gradient
   RP_N
 };
-
-// pass 1 of reverse stage s (x lines, then y lines from the 32-aligned offset xpad).  SVM 0:
-// WENO5 internals stored or recomputed as the call decides (rev_saved), 1: stored, 2:
-// recomputed; VM 0: every instance, 1: the viscous instances only, 2: the inviscid ones only --
-// the split launch fixes both on the host, so that each kernel holds only the pass-1 variant it
-// runs (and its register allocation is that variant's).
-template <int SVM, int VM = 0>
-__device__ __forceinline__ void rev_pass1(const BatchRevArgs& b, int s) {
-  const RevCall& call = b.call;
-  const bool even = (s == 2) || (s == 0);
-  const bool sv = (SVM == 0) ? rev_saved(call, s) : (SVM == 1);
-  rev_items(b, sv ? RK_P1SV : RK_P1RE, [&](int k, long long item) {
-    if (k < 0) return;  // whole warps past the end: nothing to do, no partials
-    const InstDesc& d = b.inst[k];
-    if ((VM == 1 && !d.visc) || (VM == 2 && d.visc)) return;  // the other kernel's instance
-    const InstRev& r = b.rev[k];
-    const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
-    const long long xpad = sv ? r.xpad_sv : r.xpad_re;
-    const int seg = sv ? r.seg1_sv : r.seg1_re;
-    const int dir = item < xpad ? 0 : 1;
-    const long long it = dir == 0 ? item : item - xpad;
-    const long long wofs = dir == 0 ? 0 : (xpad >> 5);
-    const bool visc = (VM == 0) ? d.visc : (VM == 1);
-    if (SVM != 2 && sv) {
-      if (VM != 2 && visc) {
-        if (dir == 0) pass1_body<0, true, true, true>(a, seg, it, wofs);
-        else pass1_body<1, true, true, true>(a, seg, it, wofs);
-      } else if (VM != 1) {
-        if (dir == 0) pass1_body<0, false, false, true>(a, seg, it, wofs);
-        else pass1_body<1, false, false, true>(a, seg, it, wofs);
-      }
-    } else if (SVM != 1) {
-      if (VM != 2 && visc) {
-        if (dir == 0) pass1_body<0, true, true, false>(a, seg, it, wofs);
-        else pass1_body<1, true, true, false>(a, seg, it, wofs);
-      } else if (VM != 1) {
-        if (dir == 0) pass1_body<0, false, false, false>(a, seg, it, wofs);
-        else pass1_body<1, false, false, false>(a, seg, it, wofs);
-      }
-    }
-  });
-}
 
 template <int PH>
 __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* smem) {
@@ -496,7 +442,6 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     for (int it = blockIdx.x; it < b.tile0[b.count]; it += gridDim.x) {
       const int k = find_inst(b.tile0, b.count, it);
       const InstDesc& d = b.inst[k];
-      const InstRev& r = b.rev[k];
       const int t = it - b.tile0[k];
       const double dt = call.dt[k];
       StageArgs a;
@@ -519,52 +464,29 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       a.vy = d.vy;
       a.use_un = (s > 0) ? 1 : 0;
       a.has_av = d.has_av;
-      a.wsave = r.wfwd + (long long)56 * s * r.a.splane;
-      a.splane = r.a.splane;
-      a.tpitch = r.a.tpitch;
       a.dtc = nullptr;
-      if (d.visc) stage_tile<true, false, false, true>(a, t % d.ntx, t / d.ntx, smem);
-      else stage_tile<false, false, false, true>(a, t % d.ntx, t / d.ntx, smem);
+      if (d.visc) stage_tile<true, false>(a, t % d.ntx, t / d.ntx, smem);
+      else stage_tile<false, false>(a, t % d.ntx, t / d.ntx, smem);
       __syncthreads();  // the next tile reuses shared memory
     }
-  } else if constexpr (PH == RP_SEED) {
-    const double ra[3] = {0.0, 0.75, 1.0 / 3.0};
-    const double rb[3] = {1.0, 0.25, 2.0 / 3.0};
-    // seed + primitives; the parameter-gradient partials of stage s+1 are reduced meanwhile
-    rev_items(b, RK_PLANE, [&](int k, long long t) {
-      if (k < 0) return;
-      const InstDesc& d = b.inst[k];
-      const InstRev& r = b.rev[k];
-      if (t >= d.lay.plane) return;
-      const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, false);
-      adj_seed_one(a, t, even ? r.P0 : r.P1, r.Uacc, ra[s], rb[s], call.dt[k], 0);
-      adj_prims_one(a, t);
-    });
+  } else if constexpr (PH == RP_REDUCE) {
     if (s < 2 && call.pbar)
       for (int k = blockIdx.x; k < b.count; k += gridDim.x)
-        if (call.pbar[k]) rev_reduce(b.rev[k], rev_saved(call, s + 1), call.pbar[k]);
-  } else if constexpr (PH == RP_PASS1) {
-    rev_pass1<0>(b, s);
-  } else if constexpr (PH == RP_PASS2) {
-    rev_items(b, RK_P2, [&](int k, long long item) {
-      if (k < 0) return;
-      const InstDesc& d = b.inst[k];
-      const InstRev& r = b.rev[k];
-      const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, false);
-      if (item < r.xpad_p2) pass2_body<0>(a, r.seg2, item);
-      else pass2_body<1>(a, r.seg2, item - r.xpad_p2);
-    });
-  } else if constexpr (PH == RP_PRIMVJP) {
-    rev_items(b, RK_PLANE, [&](int k, long long t) {
-      if (k < 0) return;
+        if (call.pbar[k]) rev_reduce(b.rev[k], call.pbar[k]);
+  } else if constexpr (PH == RP_TILES) {
+    const double ra[3] = {0.0, 0.75, 1.0 / 3.0};
+    const double rb[3] = {1.0, 0.25, 2.0 / 3.0};
+    for (int it = blockIdx.x; it < b.rtile0[b.count]; it += gridDim.x) {
+      const int k = find_inst(b.rtile0, b.count, it);
       const InstDesc& d = b.inst[k];
       const InstRev& r = b.rev[k];
       const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
-      double gb = 0.0, nb = 0.0;
-      if (d.visc) adj_primvjp_one<true>(a, t, r.seg2, gb, nb);
-      else adj_primvjp_one<false>(a, t, r.seg2, gb, nb);
-      warp_partials(a.pp, r.off_prim + (t >> 5), gb, 0.0, 0.0, nb);
-    });
+      const double* src = even ? r.P0 : r.P1;
+      const int t = it - b.rtile0[k], ntx = adj_tiles_x(d.lay);
+      if (d.visc) adj_tile<true>(a, src, r.Uacc, ra[s], rb[s], call.dt[k], 0, t % ntx, t / ntx, smem, (long long)t * ADJ_WARPS);
+      else adj_tile<false>(a, src, r.Uacc, ra[s], rb[s], call.dt[k], 0, t % ntx, t / ntx, smem, (long long)t * ADJ_WARPS);
+      __syncthreads();  // the next tile reuses shared memory
+    }
   } else if constexpr (PH == RP_BCTY || PH == RP_BCTX) {
     rev_items(b, PH == RP_BCTY ? RK_BCTY : RK_BCTX, [&](int k, long long t) {
       if (k < 0) return;
@@ -580,6 +502,7 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       const InstRev& r = b.rev[k];
       const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
       adj_inflow_block(a, d.bc, r.inflow_part, r.tmax, r.inflow_prim);
+      __syncthreads();  // the next instance reuses the block's shared sums
     }
     rev_items(b, RK_GHOST, [&](int k, long long g) {
       if (k < 0) return;
@@ -610,11 +533,11 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     });
     if (call.pbar)
       for (int k = blockIdx.x; k < b.count; k += gridDim.x)
-        if (call.pbar[k]) rev_reduce(b.rev[k], rev_saved(call, 0), call.pbar[k]);
+        if (call.pbar[k]) rev_reduce(b.rev[k], call.pbar[k]);
   }
 }
 
-__global__ void __launch_bounds__(BNT) batch_vjp_kernel(BatchRevArgs b) {
+__global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
   extern __shared__ double smem[];
   rev_phase<RP_PACK>(b, 0, smem);
   if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
@@ -631,13 +554,9 @@ __global__ void __launch_bounds__(BNT) batch_vjp_kernel(BatchRevArgs b) {
   }
   // ---- reverse through the stages 2, 1, 0: P0 -> P1 -> P0 -> P1
   for (int s = 2; s >= 0; --s) {
-    rev_phase<RP_SEED>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_PASS1>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_PASS2>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_PRIMVJP>(b, s, smem);
+    rev_phase<RP_REDUCE>(b, s, smem);
+    if (s < 2 && b.call.pbar && !grid_sync_on(b.bar, b.err, 0, b.budget)) return;
+    rev_phase<RP_TILES>(b, s, smem);
     if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
     rev_phase<RP_BCTY>(b, s, smem);
     if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
@@ -651,16 +570,11 @@ __global__ void __launch_bounds__(BNT) batch_vjp_kernel(BatchRevArgs b) {
   rev_phase<RP_UNPACK>(b, 0, smem);
 }
 
-// one phase of the reverse step as a kernel of its own (split launch); pass 1 has one kernel
-// per WENO5-internals mode
+// one phase of the reverse step as a kernel of its own (split launch)
 template <int PH>
-__global__ void __launch_bounds__(BNT) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
+__global__ void __launch_bounds__(BNT, PH == RP_STAGE || PH == RP_TILES ? 2 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
   extern __shared__ double smem[];
   rev_phase<PH>(b, s, smem);
-}
-template <bool SV, bool VISC>
-__global__ void __launch_bounds__(BNT) batch_vjp_pass1_kernel(BatchRevArgs b, int s) {
-  rev_pass1<SV ? 1 : 2, VISC ? 1 : 2>(b, s);
 }
 
 // one launch copying every instance's state: dst[k][i] = src[k][i], i < pre[k+1] - pre[k]
@@ -708,8 +622,7 @@ struct js_batch {
   int rev_blocks = 0;
   int rev_split = 0;                  // 1: one launch per phase (js_batch_set_reverse_launch)
   int rev_pblocks[js::RP_N] = {};     // grid of each phase kernel of the split launch
-  int rev_p1blocks[2][2] = {};        // grid of its pass-1 kernels [stored internals][viscous]
-  bool has_visc = false, has_inv = false;  // the batch holds viscous / inviscid instances
+  int* d_rtile0 = nullptr;            // prefix sums of the reverse tiles
   void** d_tab = nullptr;       // call table of js_batch_step_vjp: U_n, lam_np1, lam_n, p_bar x count
   double* d_dt = nullptr;       // its step sizes
   // checkpointed rollout reverse (js_batch_rollout_vjp)
@@ -728,18 +641,13 @@ int js_internal_rev_desc(js_ctx* c, js::InstRev* d);
 
 namespace {
 size_t batch_smem() { return js::StageTile<true>::SMEM; }
+size_t rev_smem() { return std::max(batch_smem(), js::adj_smem<true>()); }
+size_t rev_phase_smem(int ph) { return ph == js::RP_STAGE ? batch_smem() : ph == js::RP_TILES ? js::adj_smem<true>() : 0; }
 }  // namespace
 
 namespace {
 
 long long round32(long long n) { return (n + 31) / 32 * 32; }
-
-// line items of pass 1 / pass 2 in one direction (dir 0: rows): lines x segments
-long long line_items_of(const js::Lay& L, int dir, int extra, int seg) {
-  const int nline = (dir == 0) ? L.ny : L.nx;
-  const int ncell = (dir == 0) ? L.nx : L.ny;
-  return (long long)nline * ((ncell + extra + seg - 1) / seg);
-}
 
 // the reverse descriptors and per-kind item prefix sums of the batch (first reverse call:
 // allocates each instance's reverse workspace; call before any stream capture)
@@ -748,36 +656,27 @@ int rev_prepare(js_batch* b) {
   const int n = b->count;
   std::vector<js::InstRev> rev(n);
   std::vector<long long> pre((size_t)js::RK_N * (n + 1), 0);
+  std::vector<int> rtile0(n + 1, 0);
   for (int k = 0; k < n; ++k) {
     js::InstRev& r = rev[k];
     const int rc = js_internal_rev_desc(b->ctx[k], &r);
     if (rc) return rc;
     const js::InstDesc& d = b->desc[k];
     const js::Lay& L = d.lay;
-    r.seg1_re = 16;  // the per-grid pass 1: recomputed WENO5 (2D), stored internals
-    r.seg1_sv = 8;
-    r.seg2 = js::ADJ_SEG2;
-    const long long x_re = line_items_of(L, 0, 1, r.seg1_re), y_re = line_items_of(L, 1, 1, r.seg1_re);
-    const long long x_sv = line_items_of(L, 0, 1, r.seg1_sv), y_sv = line_items_of(L, 1, 1, r.seg1_sv);
-    const long long x_p2 = line_items_of(L, 0, 2, r.seg2), y_p2 = line_items_of(L, 1, 2, r.seg2);
-    r.xpad_re = round32(x_re);
-    r.xpad_sv = round32(x_sv);
-    r.xpad_p2 = round32(x_p2);
-    r.w1_re = (r.xpad_re + round32(y_re)) / 32;
-    r.w1_sv = (r.xpad_sv + round32(y_sv)) / 32;
-    r.off_prim = std::max(r.w1_re, r.w1_sv);
-    r.w_prim = round32(L.plane) / 32;
-    r.off_g = r.off_prim + r.w_prim;
+    r.tile0 = rtile0[k];
+    const int tiles = js::adj_tiles_x(L) * js::adj_tiles_y(L);
+    rtile0[k + 1] = rtile0[k] + tiles;
+    r.w_adj = (long long)tiles * js::ADJ_WARPS;
+    r.off_g = r.w_adj;
     r.w_g = round32(d.ib.n) / 32;
     r.off_s = r.off_g + r.w_g;
     r.w_s = round32(r.ibt.nsrc) / 32;
     const long long cnt[js::RK_N] = {
         round32(L.plane), round32(4LL * L.nx * L.ny), round32(d.ib.n), round32(js::halo_count(L)),
-        r.xpad_re + round32(y_re), r.xpad_sv + round32(y_sv), r.xpad_p2 + round32(y_p2),
         round32(6LL * (L.nx + 6)), round32(6LL * L.ny), round32(r.ibt.nsrc)};
     for (int q = 0; q < js::RK_N; ++q) pre[(size_t)q * (n + 1) + k + 1] = pre[(size_t)q * (n + 1) + k] + cnt[q];
   }
-  const size_t smem = batch_smem();
+  const size_t smem = rev_smem();
   if (cudaFuncSetAttribute(js::batch_vjp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return JS_ERR_CUDA;
@@ -789,43 +688,34 @@ int rev_prepare(js_batch* b) {
   b->rev_blocks = sms * per_sm;
   // the split launch: each phase kernel's own resident blocks per SM
   if (cudaFuncSetAttribute(js::batch_vjp_phase_kernel<js::RP_STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)batch_smem()) != cudaSuccess ||
+      cudaFuncSetAttribute(js::batch_vjp_phase_kernel<js::RP_TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess)
     return JS_ERR_CUDA;
   const void* kern[js::RP_N] = {
       (const void*)js::batch_vjp_phase_kernel<js::RP_PACK>, (const void*)js::batch_vjp_phase_kernel<js::RP_GHOST>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_HALO>, (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE>,
-      (const void*)js::batch_vjp_phase_kernel<js::RP_SEED>, (const void*)js::batch_vjp_phase_kernel<js::RP_PASS1>,
-      (const void*)js::batch_vjp_phase_kernel<js::RP_PASS2>, (const void*)js::batch_vjp_phase_kernel<js::RP_PRIMVJP>,
+      (const void*)js::batch_vjp_phase_kernel<js::RP_REDUCE>, (const void*)js::batch_vjp_phase_kernel<js::RP_TILES>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_BCTY>, (const void*)js::batch_vjp_phase_kernel<js::RP_BCTX>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_INFLOW_GHOST>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_SRC>, (const void*)js::batch_vjp_phase_kernel<js::RP_UNPACK>};
   for (int ph = 0; ph < js::RP_N; ++ph) {
     int ps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern[ph], js::BNT, ph == js::RP_STAGE ? smem : 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern[ph], js::BNT, rev_phase_smem(ph)) !=
             cudaSuccess ||
         ps < 1)
       return JS_ERR_CUDA;
     b->rev_pblocks[ph] = sms * ps;
   }
-  const void* p1[2][2] = {
-      {(const void*)js::batch_vjp_pass1_kernel<false, false>, (const void*)js::batch_vjp_pass1_kernel<false, true>},
-      {(const void*)js::batch_vjp_pass1_kernel<true, false>, (const void*)js::batch_vjp_pass1_kernel<true, true>}};
-  for (int sv = 0; sv < 2; ++sv)
-    for (int v = 0; v < 2; ++v) {
-      int ps = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, p1[sv][v], js::BNT, 0) != cudaSuccess || ps < 1)
-        return JS_ERR_CUDA;
-      b->rev_p1blocks[sv][v] = sms * ps;
-    }
-  b->has_visc = b->has_inv = false;
-  for (int k = 0; k < n; ++k) (b->desc[k].visc ? b->has_visc : b->has_inv) = true;
   if (cudaMalloc(&b->d_rev, sizeof(js::InstRev) * n) != cudaSuccess ||
       cudaMalloc(&b->d_pre, sizeof(long long) * pre.size()) != cudaSuccess ||
+      cudaMalloc(&b->d_rtile0, sizeof(int) * (n + 1)) != cudaSuccess ||
       cudaMalloc(&b->d_tab, sizeof(void*) * 4 * n) != cudaSuccess ||
       cudaMalloc(&b->d_dt, sizeof(double) * n) != cudaSuccess)
     return JS_ERR_NOMEM;
   if (cudaMemcpy(b->d_rev, rev.data(), sizeof(js::InstRev) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_pre, pre.data(), sizeof(long long) * pre.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(b->d_rtile0, rtile0.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess)
     return JS_ERR_CUDA;
   b->rev_ready = true;
@@ -840,6 +730,7 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
   a.count = b->count;
   a.pre = b->d_pre;
   a.tile0 = b->d_tile0;
+  a.rtile0 = b->d_rtile0;
   a.call = call;
   a.bar = b->d_bar;
   a.err = b->d_err;
@@ -853,7 +744,7 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
     bool ok = true;
     auto run = [&](auto kernel, int ph, int s) {
       if (!ok) return;
-      kernel<<<b->rev_pblocks[ph], js::BNT, ph == js::RP_STAGE ? batch_smem() : 0, b->stream>>>(a, s);
+      kernel<<<b->rev_pblocks[ph], js::BNT, rev_phase_smem(ph), b->stream>>>(a, s);
       ok = cudaGetLastError() == cudaSuccess;
     };
     run(js::batch_vjp_phase_kernel<js::RP_PACK>, js::RP_PACK, 0);
@@ -865,24 +756,8 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
       run(js::batch_vjp_phase_kernel<js::RP_STAGE>, js::RP_STAGE, s);
     }
     for (int s = 2; s >= 0; --s) {
-      run(js::batch_vjp_phase_kernel<js::RP_SEED>, js::RP_SEED, s);
-      if (ok) {
-        // pass 1 reads the WENO5 internals stored by the forward recompute of stages 0 and 1
-        // when the stage states were not given (the device's rev_saved)
-        // (one kernel for the viscous instances, one for the inviscid ones)
-        const bool sv = s < 2 && call.U1 == nullptr;
-        cudaStream_t st = b->stream;
-        if (sv) {
-          if (b->has_visc) js::batch_vjp_pass1_kernel<true, true><<<b->rev_p1blocks[1][1], js::BNT, 0, st>>>(a, s);
-          if (b->has_inv) js::batch_vjp_pass1_kernel<true, false><<<b->rev_p1blocks[1][0], js::BNT, 0, st>>>(a, s);
-        } else {
-          if (b->has_visc) js::batch_vjp_pass1_kernel<false, true><<<b->rev_p1blocks[0][1], js::BNT, 0, st>>>(a, s);
-          if (b->has_inv) js::batch_vjp_pass1_kernel<false, false><<<b->rev_p1blocks[0][0], js::BNT, 0, st>>>(a, s);
-        }
-        ok = cudaGetLastError() == cudaSuccess;
-      }
-      run(js::batch_vjp_phase_kernel<js::RP_PASS2>, js::RP_PASS2, s);
-      run(js::batch_vjp_phase_kernel<js::RP_PRIMVJP>, js::RP_PRIMVJP, s);
+      if (s < 2 && call.pbar) run(js::batch_vjp_phase_kernel<js::RP_REDUCE>, js::RP_REDUCE, s);
+      run(js::batch_vjp_phase_kernel<js::RP_TILES>, js::RP_TILES, s);
       run(js::batch_vjp_phase_kernel<js::RP_BCTY>, js::RP_BCTY, s);
       run(js::batch_vjp_phase_kernel<js::RP_BCTX>, js::RP_BCTX, s);
       run(js::batch_vjp_phase_kernel<js::RP_INFLOW_GHOST>, js::RP_INFLOW_GHOST, s);
@@ -893,7 +768,7 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
   }
   void* args[] = {&a};
   if (cudaLaunchCooperativeKernel((void*)js::batch_vjp_kernel, dim3(b->rev_blocks), dim3(js::BNT), args,
-                                  batch_smem(), b->stream) != cudaSuccess)
+                                  rev_smem(), b->stream) != cudaSuccess)
     return JS_ERR_CUDA;
   return JS_OK;
 }
@@ -905,7 +780,7 @@ extern "C" {
 void js_batch_destroy(js_batch* b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream); else cudaDeviceSynchronize();
-  cudaFree(b->d_rev); cudaFree(b->d_pre); cudaFree(b->d_tab); cudaFree(b->d_dt); cudaFree(b->d_order);
+  cudaFree(b->d_rev); cudaFree(b->d_pre); cudaFree(b->d_rtile0); cudaFree(b->d_tab); cudaFree(b->d_dt); cudaFree(b->d_order);
   for (double* p : b->ro_buf) cudaFree(p);
   cudaFree(b->d_ro); cudaFree(b->d_spre);
   for (js_ctx* c : b->ctx) js_destroy(c);

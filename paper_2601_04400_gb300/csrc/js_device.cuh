@@ -89,8 +89,8 @@ __device__ __forceinline__ void cons_to_prim(double r, double mx, double my, dou
 //   4 beta_1 = 13/3 D_i^2     + (d_{i-1/2} + d_{i+1/2})^2
 //   4 beta_2 = 13/3 D_{i+1}^2 + (D_{i+1} - 2 d_{i+1/2})^2
 // s_k = 4 beta_k + 4 eps; the weights alpha_k = d_k / s_k^2 are scaled by (s0 s1 s2)^2.
-// Candidate values minus q_i, times 6, are two-term combinations of the d's.  Win evaluates
-// this in integer arithmetic (js_weno.cuh), weno_plain in FP64.
+// Candidate values minus q_i, times 6, are two-term combinations of the d's.  weno_lane and
+// weno_cell evaluate this in integer arithmetic (js_weno.cuh), weno_plain in FP64.
 // ---------------------------------------------------------------------------------------
 constexpr double EPS12 = 1.2e-5;  // 3 (4 eps)
 constexpr double SIXTH = 1.0 / 6.0;
@@ -116,9 +116,8 @@ __device__ __forceinline__ void face_image(const double wl[4], const double wr[4
   for (int k = 0; k < 4; ++k) m[k] = (m[k] - mean[k]) * inv_sd[k];
 }
 
-// the FP64 form of one cell: out[0..1] = the face states at i+1/2 and i-1/2, out[2..8] = the
-// internals of Win::step
-static __device__ __noinline__ void weno_plain(double qm2, double qm1, double q0, double q1, double q2, double out[9]) {
+// the FP64 form of one cell: its face states at i+1/2 (left-biased) and i-1/2 (right-biased)
+static __device__ __noinline__ double2 weno_plain(double qm2, double qm1, double q0, double q1, double q2) {
   const double dm2 = qm1 - qm2, dm1 = q0 - qm1, dp1 = q1 - q0, dp2 = q2 - q1;
   const double D0 = dm1 - dm2, D1 = dp1 - dm1, D2 = dp2 - dp1;
   const double t0 = fma(2.0, dm1, D0), t1 = dm1 + dp1, t2 = fma(-2.0, dp1, D2);
@@ -131,157 +130,72 @@ static __device__ __noinline__ void weno_plain(double qm2, double qm1, double q0
   // left-biased (linear weights 0.1 : 0.6 : 0.3), right-biased (0.3 : 0.6 : 0.1)
   const double nL = fma(w0, fma(-2.0, dm2, 5.0 * dm1), fma(w6, fma(2.0, dp1, dm1), w2_3 * fma(4.0, dp1, -dp2)));
   const double nR = fma(w0_3, fma(-4.0, dm1, dm2), fma(w6, fma(-2.0, dm1, -dp1), w2 * fma(2.0, dp2, -5.0 * dp1)));
-  const double rL = recip(w0 + w6 + w2_3), rR = recip(w0_3 + w6 + w2);
-  out[5] = nL * rL;
-  out[6] = rL;
-  out[7] = nR * rR;
-  out[8] = rR;
-  out[0] = fma(out[5], SIXTH, q0);
-  out[1] = fma(out[7], SIXTH, q0);
-  out[2] = s0;
-  out[3] = s1;
-  out[4] = s2;
+  return make_double2(fma(quot(nL, w0 + w6 + w2_3), SIXTH, q0), fma(quot(nR, w0_3 + w6 + w2), SIXTH, q0));
 }
 
-// POS: the variable is positive (density, pressure), see js_weno.cuh on its range
-template <bool POS>
-struct Win {
-  double q0, q1;       // q_i, q_{i+1}
-  Fx dm2, dm1, dp1;    // d_{i-3/2}, d_{i-1/2}, d_{i+1/2}
-  Sm s0, s1, s0n;      // indicators s_0, s_1 of cell i, s_0 of cell i+1
+// the largest exponent of a stencil's differences up to which the integer form serves
+// (js_weno.cuh); pos: the variable is positive (density, pressure)
+__device__ __forceinline__ int weno_limit(double q0, bool pos) { return pos ? imin(expo(q0) + 3, 1500) : 1500; }
 
-  // start at the cell q points at (neighbours at multiples of st)
-  template <class I>
-  __device__ __forceinline__ void init(const double* q, I st) {
-    q0 = q[0];
-    q1 = q[st];
-    const double qm1 = q[-st];
-    dm2 = fx_of(qm1 - q[-2 * st]);
-    dm1 = fx_of(q0 - qm1);
-    dp1 = fx_of(q1 - q0);
-    Sm unused1, unused2;
-    sm_pair(dm2, dm1, unused1, s0, unused2);
-    sm_pair(dm1, dp1, s1, s0n, unused2);
-  }
+__device__ __forceinline__ Sm shfl_up(const Sm& s) {
+  return Sm{(u64)__shfl_up_sync(0xffffffffu, (unsigned long long)s.m, 1), __shfl_up_sync(0xffffffffu, s.x, 1)};
+}
+__device__ __forceinline__ Sm shfl_down(const Sm& s) {
+  return Sm{(u64)__shfl_down_sync(0xffffffffu, (unsigned long long)s.m, 1), __shfl_down_sync(0xffffffffu, s.x, 1)};
+}
+__device__ __forceinline__ Fx shfl_up(const Fx& d) {
+  return Fx{(s64)__shfl_up_sync(0xffffffffu, (long long)d.m, 1), __shfl_up_sync(0xffffffffu, d.e, 1)};
+}
+__device__ __forceinline__ Fx shfl_down(const Fx& d) {
+  return Fx{(s64)__shfl_down_sync(0xffffffffu, (long long)d.m, 1), __shfl_down_sync(0xffffffffu, d.e, 1)};
+}
 
-  // cell i, at q: face states at i+1/2 (Lf, left-biased; if NL) and i-1/2 (Rf, right-biased; if
-  // NR), then slide to cell i+1.  With SV the internals the reverse pass needs go to
-  // sv[0..6] = 3 s0, 3 s1, 3 s2, cL, rL, cR, rR (state = q_i + c/6, c = num r, r the reciprocal
-  // of the weights' sum formed from the 3 s_k; zeros for a side not formed).
-  template <bool NL = true, bool NR = true, bool SV = false, class I>
-  __device__ __forceinline__ void step(const double* q, I st, double& Lf, double& Rf, double* sv = nullptr) {
-    const double q2 = q[2 * st];
-    const Fx dp2 = fx_of(q2 - q1);
-    Sm s1n, s0nn, s2;
-    sm_pair(dp1, dp2, s1n, s0nn, s2);
-    const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
-    const int lim = POS ? imin(expo(q0) + 3, 1500) : 1500;
-    double cL = 0.0, cR = 0.0, rL = 0.0, rR = 0.0;
-    if (F > lim) {
-      double out[9];
-      weno_plain(q[-2 * st], q[-st], q0, q1, q2, out);
-      Lf = out[0];
-      Rf = out[1];
-      if (SV) {
-#pragma unroll
-        for (int m = 0; m < 7; ++m) sv[m] = (m == 3 || m == 4) && !NL ? 0.0 : (m == 5 || m == 6) && !NR ? 0.0 : out[m + 2];
-      }
-    } else {
-      weno_corr<NL, NR, SV>(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR, rL, rR);
-      if (NL) Lf = fma(cL, SIXTH, q0);
-      if (NR) Rf = fma(cR, SIXTH, q0);
-      if (SV) {
-        sv[0] = sm_double(s0);
-        sv[1] = sm_double(s1);
-        sv[2] = sm_double(s2);
-        sv[3] = cL;
-        sv[4] = rL;
-        sv[5] = cR;
-        sv[6] = rR;
-      }
-    }
-    // slide
-    q0 = q1;
-    q1 = q2;
-    dm2 = dm1;
-    dm1 = dp1;
-    dp1 = dp2;
-    s0 = s0n;
-    s1 = s1n;
-    s0n = s0nn;
-  }
-};
-
-// The same for one cell per lane: the lanes of a warp hold consecutive cells of a line, q points
-// at the lane's own (q[-st .. st] readable; q[-2 st], q[2 st] too in the inner lanes).  A lane
+// Face states at i+1/2 (Lf, left-biased) and i-1/2 (Rf, right-biased) of one cell per lane: the
+// lanes of a warp hold consecutive cells of a line, q points at the lane's own (q[-st .. st]
+// readable; q[-2 st], q[2 st] too in the inner lanes 1..30, where the result is valid).  A lane
 // forms the differences on both sides of its cell and the three indicators they determine, and
-// takes its s_0, s_2 and outer differences from its neighbours.  Valid in lanes 1..30 (inner).
-template <bool SV>
-__device__ __forceinline__ void weno_lane(const double* q, int st, bool pos, bool inner, double& Lf, double& Rf,
-                                          double* sv) {
+// takes its s_0, s_2 and outer differences from its neighbours.
+__device__ __forceinline__ void weno_lane(const double* q, int st, bool pos, bool inner, double& Lf, double& Rf) {
   const double q0 = q[0];
   const Fx dm1 = fx_of(q0 - q[-st]), dp1 = fx_of(q[st] - q0);
   Sm s1, s0n, s2p;
   sm_pair(dm1, dp1, s1, s0n, s2p);
-  const Sm s0{(u64)__shfl_up_sync(0xffffffffu, (unsigned long long)s0n.m, 1), __shfl_up_sync(0xffffffffu, s0n.x, 1)};
-  const Sm s2{(u64)__shfl_down_sync(0xffffffffu, (unsigned long long)s2p.m, 1),
-              __shfl_down_sync(0xffffffffu, s2p.x, 1)};
-  const Fx dm2{(s64)__shfl_up_sync(0xffffffffu, (long long)dm1.m, 1), __shfl_up_sync(0xffffffffu, dm1.e, 1)};
-  const Fx dp2{(s64)__shfl_down_sync(0xffffffffu, (long long)dp1.m, 1), __shfl_down_sync(0xffffffffu, dp1.e, 1)};
+  const Sm s0 = shfl_up(s0n), s2 = shfl_down(s2p);
+  const Fx dm2 = shfl_up(dm1), dp2 = shfl_down(dp1);
   const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
-  const int lim = pos ? imin(expo(q0) + 3, 1500) : 1500;
-  if (F > lim && inner) {
-    double out[9];
-    weno_plain(q[-2 * st], q[-st], q0, q[st], q[2 * st], out);
-    Lf = out[0];
-    Rf = out[1];
-    if (SV) {
-#pragma unroll
-      for (int m = 0; m < 7; ++m) sv[m] = out[m + 2];
-    }
+  if (F > weno_limit(q0, pos) && inner) {
+    const double2 r = weno_plain(q[-2 * st], q[-st], q0, q[st], q[2 * st]);
+    Lf = r.x;
+    Rf = r.y;
   } else {
-    double cL, cR, rL, rR;
-    weno_corr<true, true, SV>(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR, rL, rR);
+    double cL, cR;
+    weno_corr(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR);
     Lf = fma(cL, SIXTH, q0);
     Rf = fma(cR, SIXTH, q0);
-    if (SV) {
-      sv[0] = sm_double(s0);
-      sv[1] = sm_double(s1);
-      sv[2] = sm_double(s2);
-      sv[3] = cL;
-      sv[4] = rL;
-      sv[5] = cR;
-      sv[6] = rR;
-    }
   }
 }
 
-// the windows of the four primitive variables along a line (planes ps apart)
-struct Win4 {
-  Win<true> r;
-  Win<false> u, v;
-  Win<true> p;
-  template <class I, class P>
-  __device__ __forceinline__ void init(const double* q, P ps, I st) {
-    r.init(q, st);
-    u.init(q + ps, st);
-    v.init(q + 2 * ps, st);
-    p.init(q + 3 * ps, st);
+// the same for a single thread (q[-2 st .. 2 st] readable): the same bits
+template <class I>
+__device__ __forceinline__ void weno_cell(const double* q, I st, bool pos, double& Lf, double& Rf) {
+  const double q0 = q[0];
+  const Fx dm2 = fx_of(q[-st] - q[-2 * st]), dm1 = fx_of(q0 - q[-st]), dp1 = fx_of(q[st] - q0), dp2 = fx_of(q[2 * st] - q[st]);
+  Sm s0, s1, s2, x, y;
+  sm_pair(dm2, dm1, x, s0, y);
+  sm_pair(dp1, dp2, x, y, s2);
+  sm_pair(dm1, dp1, s1, x, y);
+  const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
+  if (F > weno_limit(q0, pos)) {
+    const double2 r = weno_plain(q[-2 * st], q[-st], q0, q[st], q[2 * st]);
+    Lf = r.x;
+    Rf = r.y;
+  } else {
+    double cL, cR;
+    weno_corr(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR);
+    Lf = fma(cL, SIXTH, q0);
+    Rf = fma(cR, SIXTH, q0);
   }
-  // keep(c, sv) receives the internals of variable c (SV)
-  template <bool NL, bool NR, bool SV, class I, class P, class Keep>
-  __device__ __forceinline__ void step(const double* q, P ps, I st, double Lf[4], double Rf[4], Keep&& keep) {
-    double sv[SV ? 7 : 1];
-    r.template step<NL, NR, SV>(q, st, Lf[0], Rf[0], sv);
-    if (SV) keep(0, sv);
-    u.template step<NL, NR, SV>(q + ps, st, Lf[1], Rf[1], sv);
-    if (SV) keep(1, sv);
-    v.template step<NL, NR, SV>(q + 2 * ps, st, Lf[2], Rf[2], sv);
-    if (SV) keep(2, sv);
-    p.template step<NL, NR, SV>(q + 3 * ps, st, Lf[3], Rf[3], sv);
-    if (SV) keep(3, sv);
-  }
-};
+}
 
 // ---------------------------------------------------------------------------------------
 // HLLC (Sec. 2) in the face-normal frame.  State (rho, un, ut, p) on each side; returns
@@ -294,8 +208,8 @@ struct Win4 {
 //   G = m s*/(s_K - s*),  F = (G, G s* + p*, G u_t, s*/(s_K - s*) (d E - p u + p* s_K)).
 // A supersonic face (s_K on the far side of zero) has F = F_K, the same expressions with u in
 // the place of s*.  At s* = 0 both sides give (0, p*, 0, 0): the average of the branches that
-// sign(0) = 0 asks for is either of them.  29 FP64 instructions a face (15 at s* = 0, where gas
-// at rest on both sides always lands) where building the star state and its jump took 61.
+// sign(0) = 0 asks for is either of them.  35 FP64 instructions a face (19 at s* = 0, where gas
+// at rest on both sides always lands) where building the star state and its jump took 69.
 // ---------------------------------------------------------------------------------------
 // signs and positivity from the bits: an FP64 comparison takes an FP64 issue slot
 __device__ __forceinline__ bool sign_clear(double x) { return (s32)hi32(dbits(x)) >= 0; }
@@ -305,14 +219,16 @@ __device__ __forceinline__ bool positive(double x) { return dbits(x) - 1u < 0x7f
 __device__ __forceinline__ void hllc(double rL, double uL, double vL, double pL, double rR, double uR,
                                      double vR, double pR, const Gas& g, double F[4]) {
   const double gpL = g.gamma * pL, gpR = g.gamma * pR;
-  const double aL = gpL * rsqrt_nr(gpL * rL);
-  const double aR = gpR * rsqrt_nr(gpR * rR);
-  const double sL = fmin(uL - aL, uR - aR);
-  const double sR = fmax(uL + aL, uR + aR);
+  // sound speed a = gp y
+  const double yL = rsqrt_nr(gpL * rL), yR = rsqrt_nr(gpR * rR);
+  const double sL = fmin(fma(-gpL, yL, uL), fma(-gpR, yR, uR));
+  const double sR = fmax(fma(gpL, yL, uL), fma(gpR, yR, uR));
+  // (products that a later sum or difference could be contracted with are rounded on their own:
+  // every kernel that inlines this then gives the same bits)
   const double dL = sL - uL, dR = sR - uR;
-  const double mL = rL * dL, mR = rR * dR;
+  const double mL = __dmul_rn(rL, dL), mR = __dmul_rn(rR, dR);
   const double num = fma(-uR, mR, fma(uL, mL, pR - pL));
-  const double ss = quot(num, mL - mR);
+  const double ss = __dmul_rn(num, recip(mL - mR));
   const bool left = sign_clear(ss);
   const double u = left ? uL : uR, ut = left ? vL : vR, p = left ? pL : pR, s = left ? sL : sR,
                d = left ? dL : dR, m = left ? mL : mR;
@@ -324,14 +240,14 @@ __device__ __forceinline__ void hllc(double rL, double uL, double vL, double pL,
     F[1] = ps;
     return;
   }
-  const double w = c * recip(s - c);
-  const double G = m * w;
+  const double w = __dmul_rn(c, recip(s - c));
+  const double G = __dmul_rn(m, w);
   // d E = m (u^2 + u_t^2)/2 + d p/(gamma - 1)
   const double dE = fma(0.5 * m, fma(u, u, ut * ut), g.g1 * (d * p));
   F[0] = G;
   F[1] = fma(G, c, ps);
-  F[2] = G * ut;
-  F[3] = w * fma(ps, s, fma(-p, u, dE));
+  F[2] = __dmul_rn(G, ut);
+  F[3] = __dmul_rn(w, fma(ps, s, fma(-p, u, dE)));
 }
 
 // ---------------------------------------------------------------------------------------

@@ -289,11 +289,11 @@ __device__ __forceinline__ bool stage_constants(const StageArgs& a0, StageArgs& 
 }
 
 // persistent stage kernel of NW warps a block: blocks stride over the tiles, staged by TMA (tensor
-// map of the stage input as a grid constant) or by plain loads; with SAVE the WENO5 internals of
-// the stage go to a.wsave for the reverse pass, with IMG the neural flux's face images to a.img.
+// map of the stage input as a grid constant) or by plain loads; with IMG the neural flux's face
+// images of the stage input go to a.img.
 // 7 warps (4 lines each in both directions), 3 blocks an SM: 21 warps at 96 registers.  14 warps
 // for grids of few tiles, where a tile's latency counts.
-template <int NW, bool VISC, bool RHS, bool TMA, bool SAVE, bool IMG>
+template <int NW, bool VISC, bool RHS, bool TMA, bool IMG>
 __global__ void __launch_bounds__(32 * NW, NW == 7 ? 3 : 1)
 stage2d_kernel(StageArgs a0, int ntx, int ntiles, const __grid_constant__ TensorMap128 tmap) {
   StageArgs a;
@@ -306,7 +306,7 @@ stage2d_kernel(StageArgs a0, int ntx, int ntiles, const __grid_constant__ Tensor
   }
   unsigned phase = 0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    stage_tile<VISC, RHS, TMA, SAVE, IMG>(a, t % ntx, t / ntx, smem, &tmap, &bar, &phase);
+    stage_tile<VISC, RHS, TMA, IMG>(a, t % ntx, t / ntx, smem, &tmap, &bar, &phase);
     __syncthreads();
   }
 }
@@ -349,10 +349,10 @@ __global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
 // launchers
 // =======================================================================================
 namespace {
-template <int NW, bool VISC, bool RHS, bool TMA, bool SAVE, bool IMG>
+template <int NW, bool VISC, bool RHS, bool TMA, bool IMG>
 cudaError_t launch_stage2d_nw(const StageArgs& a, const TensorMap128* tmap, int ntx, int ntiles, cudaStream_t s) {
   using S = StageTile<VISC>;
-  auto k = stage2d_kernel<NW, VISC, RHS, TMA, SAVE, IMG>;
+  auto k = stage2d_kernel<NW, VISC, RHS, TMA, IMG>;
   static int resident = 0;  // blocks resident on the whole GPU
   if (resident == 0) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
@@ -369,18 +369,18 @@ cudaError_t launch_stage2d_nw(const StageArgs& a, const TensorMap128* tmap, int 
   return cudaGetLastError();
 }
 
-template <bool VISC, bool RHS, bool SAVE = false, bool IMG = false>
+template <bool VISC, bool RHS, bool IMG = false>
 cudaError_t launch_stage2d(const StageArgs& a, int variant, const TensorMap128* tmap, cudaStream_t s) {
   const int ntx = (a.lay.nx + TILE - 1) / TILE, nty = (a.lay.ny + TILE - 1) / TILE, ntiles = ntx * nty;
-  if constexpr (!SAVE && !IMG) {
+  if constexpr (!IMG) {
     // blocks of 14 warps take a tile in half the time; worth it while every tile has its SM
     const bool wide = variant == 2 || variant == 3 || (variant != 1 && variant != 4 && ntiles <= 152);
     if (wide)
-      return tmap ? launch_stage2d_nw<14, VISC, RHS, true, SAVE, IMG>(a, tmap, ntx, ntiles, s)
-                  : launch_stage2d_nw<14, VISC, RHS, false, SAVE, IMG>(a, tmap, ntx, ntiles, s);
+      return tmap ? launch_stage2d_nw<14, VISC, RHS, true, IMG>(a, tmap, ntx, ntiles, s)
+                  : launch_stage2d_nw<14, VISC, RHS, false, IMG>(a, tmap, ntx, ntiles, s);
   }
-  return tmap ? launch_stage2d_nw<7, VISC, RHS, true, SAVE, IMG>(a, tmap, ntx, ntiles, s)
-              : launch_stage2d_nw<7, VISC, RHS, false, SAVE, IMG>(a, tmap, ntx, ntiles, s);
+  return tmap ? launch_stage2d_nw<7, VISC, RHS, true, IMG>(a, tmap, ntx, ntiles, s)
+              : launch_stage2d_nw<7, VISC, RHS, false, IMG>(a, tmap, ntx, ntiles, s);
 }
 
 template <bool VISC, bool RHS>
@@ -390,15 +390,10 @@ cudaError_t launch_stage1d(const StageArgs& a, cudaStream_t s) {
 }
 }  // namespace
 
-cudaError_t launch_stage_save(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s) {
-  if (a.lay.ny == 1 || a.wsave == nullptr) return cudaErrorInvalidValue;
-  return visc ? launch_stage2d<true, false, true>(a, 0, tmap, s) : launch_stage2d<false, false, true>(a, 0, tmap, s);
-}
-
 cudaError_t launch_stage_img(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s) {
   if (a.lay.ny == 1 || a.img == nullptr) return cudaErrorInvalidValue;
-  return visc ? launch_stage2d<true, false, false, true>(a, 0, tmap, s)
-              : launch_stage2d<false, false, false, true>(a, 0, tmap, s);
+  return visc ? launch_stage2d<true, false, true>(a, 0, tmap, s)
+              : launch_stage2d<false, false, true>(a, 0, tmap, s);
 }
 
 cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, const TensorMap128* tmap,

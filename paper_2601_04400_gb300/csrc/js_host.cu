@@ -48,17 +48,10 @@ struct js_ctx {
   double* ibt_w = nullptr;
   // adjoint workspace (allocated by the first vjp call)
   bool adj_ready = false;
-  double* Q = nullptr;       // 5 planes
-  double* fcell = nullptr;   // 24 saved planes: per-face adjoints for the cells of the face
-  double* wrev = nullptr;    // pass-2 segment slots (js::adj_wrev_doubles)
   double* ppart = nullptr;   // block partials of the parameter gradient (js::adj_ppart_doubles)
-  double* lam = nullptr;     // 4 planes
   double* P0 = nullptr;      // 4 planes (stage adjoint ping)
   double* P1 = nullptr;      // 4 planes (pong)
   double* Uacc = nullptr;    // 4 planes
-  double* wsave = nullptr;   // 56 planes
-  double* wsave_fwd = nullptr;  // 2 x 56 planes: internals stored by the forward stages 1, 2
-  double* fadj = nullptr;    // 16 planes
   double* inflow_part = nullptr;  // [4 sides][max(nx + 6, ny)][4] inflow halo adjoint partials
   double* inflow_prim = nullptr;  // 16
   double* inflow_host = nullptr;  // 16, pinned
@@ -68,7 +61,8 @@ struct js_ctx {
   bool nn_on = false;
   js::NnArgs nn;
   double* nnQ = nullptr;        // primitives of the stage input (4 planes)
-  double* nn_wsave = nullptr;   // WENO5 internals of the current stage (2D; 56 planes)
+  double* nn_lam = nullptr;     // reverse: lambda' of the stage (4 padded planes)
+  double* nn_fadj = nullptr;    // reverse: face-state adjoints of the network (16 planes)
   void* nn_buf[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   void* nn_bf16[2] = {nullptr, nullptr};  // BF16 pixel-major activations (16 and 32 channels)
   // network input and activations (X, A1, A2, T3: 56 channels) of the forward stages 0 and 1 of
@@ -80,12 +74,8 @@ struct js_ctx {
   int arith = JS_ARITH_FAST;  // js_set_arith
   js::IeeeBufs ieee = {nullptr, nullptr, nullptr};  // workspace of JS_ARITH_IEEE
   std::vector<std::pair<const double*, js::TensorMap128>> tmaps;  // TMA maps of stage inputs
-  // tape: per slot the three filled stage states of one recorded step and, when recording
-  // internals (2D), the WENO5 internals of its three stages
+  // tape: per slot the three filled stage states of one recorded step
   std::vector<double*> tape;
-  std::vector<double*> tape_w;     // 3 per slot (56 planes each) or nullptr
-  std::vector<char> tape_w_ok;     // per slot: internals of the recorded step are present
-  bool tape_weno = false;
   // y slab of a decomposed grid (js_create_slab): local row k is global row
   // (slab_lo + k) mod slab_nyg; rows [slab_own, slab_own + slab_nown) are owned; the y sides
   // in slab_xchg[0] (low) / [1] (high) border a neighbouring slab
@@ -93,7 +83,7 @@ struct js_ctx {
   int slab_nyg = 0, slab_lo = 0, slab_own = 0, slab_nown = 0;
   bool slab_xchg[2] = {false, false};
   int svjp_next = 2;  // stage expected by the next js_step_stage_vjp (2, 1, 0, 2, ...)
-  bool stage_kept[2] = {false, false};  // js_step_stage stored stage 0 / 1 internals in wsave_fwd
+  bool stage_kept[2] = {false, false};  // js_step_stage ran stage 0 / 1 with JS_STAGE_INTERNALS
   // instrumentation
   bool profiling = false;
   std::vector<cudaEvent_t> ev;  // 2 per timed stage launch
@@ -350,16 +340,11 @@ const js::TensorMap128* stage_tmap(js_ctx* c, const double* buf) {
 
 // neural flux of the stage input a.Uin (before the stage kernel) and its divergence
 // subtracted from the stage output (after it)
-// (wsave: the stage's stored WENO5 internals, or nullptr to recompute the face states)
-int nn_before(js_ctx* c, const StageArgs& a, const double* wsave = nullptr, long long splane = 0, int tpitch = 0) {
+int nn_before(js_ctx* c, const StageArgs& a) {
   if (!c->nn_on) return JS_OK;
   c->nn.g1 = 1.0 / (c->p.gamma - 1.0);
-  js::NnArgs n = c->nn;
-  n.wsave = wsave;
-  n.splane = splane;
-  n.tpitch = tpitch;
   JS_CUDA(js::nn_prims(a.Uin, c->nnQ, c->lay, c->p.gamma, c->stream));
-  JS_CUDA(js::nn_forward(n, c->nnQ, c->lay.plane, c->stream));
+  JS_CUDA(js::nn_forward(c->nn, c->nnQ, c->lay.plane, c->stream));
   c->launches += 5;
   return JS_OK;
 }
@@ -370,33 +355,13 @@ int nn_after(js_ctx* c, const StageArgs& a, bool rhs) {
   return JS_OK;
 }
 
-// saved-array layouts: y lines padded (pitch x H), x lines transposed ((nx+6) x tpitch)
+// layouts of the neural flux's face-state adjoints: y lines padded (pitch x H), x lines transposed
+// ((nx+6) x tpitch)
 int transposed_pitch(const js_ctx* c) { return (c->lay.H + 3) / 4 * 4; }
 long long saved_plane(const js_ctx* c) {
   const long long t = (long long)(c->lay.nx + 6) * transposed_pitch(c);
   const long long m = t > c->lay.plane ? t : c->lay.plane;
   return (m + 31) / 32 * 32;
-}
-
-size_t internals_bytes(const js_ctx* c) { return sizeof(double) * 56 * (size_t)saved_plane(c); }
-
-// stage update that also stores its WENO5 internals to `wsave` (2D), bracketed by events
-// while profiling like stage()
-int stage_save(js_ctx* c, StageArgs a, bool visc, double* wsave) {
-  a.wsave = wsave;
-  a.splane = saved_plane(c);
-  a.tpitch = transposed_pitch(c);
-  const bool timed = c->profiling && c->ev_used + 2 <= (int)c->ev.size();
-  if (timed) JS_CUDA(cudaEventRecord(c->ev[c->ev_used], c->stream));
-  JS_CUDA(js::launch_stage_save(a, visc, stage_tmap(c, a.Uin), c->stream));
-  if (timed) {
-    JS_CUDA(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
-    c->ev_used += 2;
-  }
-  ++c->launches;
-  int rc = nn_before(c, a, wsave, a.splane, a.tpitch);
-  if (rc) return rc;
-  return nn_after(c, a, false);
 }
 
 // fused stage kernel, bracketed by events while profiling
@@ -422,10 +387,8 @@ int stage_img(js_ctx* c, StageArgs a, bool visc) {
 }
 
 int stage(js_ctx* c, const StageArgs& a, bool visc, bool rhs) {
-  // with the neural flux on a 2D grid the stage kernel also forms the network's face images
-  // (FP32 and BF16 networks) or stores the WENO5 internals they are formed from (FP64)
+  // with an FP32 or BF16 network on a 2D grid the stage kernel also forms its face images
   if (c->nn_on && !rhs && c->g.ny > 1 && c->nn.fp32) return stage_img(c, a, visc);
-  if (c->nn_on && c->nn_wsave && !rhs) return stage_save(c, a, visc, c->nn_wsave);
   int rc = nn_before(c, a);
   if (rc) return rc;
   const bool timed = c->profiling && c->ev_used + 2 <= (int)c->ev.size();
@@ -503,17 +466,15 @@ void js_destroy(js_ctx* c) {
   cudaFree(c->err); cudaFree(c->red); cudaFree(c->cfl_bmax); cudaFree(c->dtc);
   cudaFree(c->ieee.Q); cudaFree(c->ieee.F); cudaFree(c->ieee.G);
   cudaFree(c->ibt_cell); cudaFree(c->ibt_ptr); cudaFree(c->ibt_ghost); cudaFree(c->ibt_w);
-  cudaFree(c->Q); cudaFree(c->fcell); cudaFree(c->wrev); cudaFree(c->ppart); cudaFree(c->lam); cudaFree(c->P0); cudaFree(c->P1); cudaFree(c->Uacc);
-  cudaFree(c->wsave); cudaFree(c->wsave_fwd); cudaFree(c->fadj);
+  cudaFree(c->ppart); cudaFree(c->P0); cudaFree(c->P1); cudaFree(c->Uacc);
   if (c->inflow_host) cudaFreeHost(c->inflow_host);
-  cudaFree(c->nnQ); cudaFree(c->nn_partial); cudaFree(c->nn_wsave);
+  cudaFree(c->nnQ); cudaFree(c->nn_partial); cudaFree(c->nn_lam); cudaFree(c->nn_fadj);
   for (void* b : c->nn_buf) cudaFree(b);
   for (void* b : c->nn_bf16) cudaFree(b);
   for (void* b : c->nn_keep) cudaFree(b);
   cudaFree(c->inflow_part); cudaFree(c->inflow_prim); cudaFree(c->qIb);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   for (double* t : c->tape) cudaFree(t);
-  for (double* t : c->tape_w) cudaFree(t);
   delete c;
 }
 
@@ -804,12 +765,12 @@ int js_step_stage(js_ctx* c, const double* U_n, const double* U_in, double* U_ou
   const int stage_k = stage_flags & ~JS_STAGE_INTERNALS;
   if (!c || !U_in || !U_out || stage_k < 0 || stage_k > 2 || !(dt > 0.0) || (stage_k > 0 && !U_n))
     return JS_ERR_ARG;
-  // stages 0 and 1 of a 2D grid may store their WENO5 internals for js_step_stage_vjp
+  // stages 0 and 1 of a 2D grid may be marked for js_step_stage_vjp (fast arithmetic; the reverse
+  // recomputes their WENO5 internals, so nothing is stored)
   const bool keep = (stage_flags & JS_STAGE_INTERNALS) && stage_k < 2 && c->g.ny > 1;
   if (keep) {
     const int rc = adj_reserve(c);
     if (rc) return rc;
-    if (!c->wsave_fwd) return JS_ERR_NOMEM;
   }
   double* X = (stage_k == 0) ? c->N : c->A;
   JS_CUDA(js::launch_pack(U_in, X, c->lay, c->stream));
@@ -833,7 +794,7 @@ int js_step_stage(js_ctx* c, const double* U_n, const double* U_in, double* U_ou
   a.rk_a = ra[stage_k];
   a.rk_b = rb[stage_k];
   a.use_un = (stage_k > 0) ? 1 : 0;
-  if (keep) rc = stage_save(c, a, c->p.mu > 0.0, c->wsave_fwd + 56 * (size_t)saved_plane(c) * stage_k);
+  if (keep) rc = stage(c, a, c->p.mu > 0.0, false);
   else rc = stage_fwd(c, a, false, dt, stage_k);
   if (rc) return rc;
   if (stage_k < 2) c->stage_kept[stage_k] = keep;
@@ -848,30 +809,14 @@ int adj_reserve(js_ctx* c) {
   if (c->adj_ready) return JS_OK;
   const size_t pl = sizeof(double) * (size_t)c->lay.plane;
   struct { double** p; size_t planes; } bufs[] = {
-      {&c->Q, 5}, {&c->lam, 4}, {&c->P0, 4}, {&c->P1, 4}, {&c->Uacc, 4}};
+      {&c->P0, 4}, {&c->P1, 4}, {&c->Uacc, 4}};
   for (auto& b : bufs) {
     if (cudaMalloc(b.p, b.planes * pl) != cudaSuccess) return JS_ERR_NOMEM;
     JS_CUDA(cudaMemsetAsync(*b.p, 0, b.planes * pl, c->stream));  // ordered with the caller's work
   }
-  const size_t spl = sizeof(double) * (size_t)saved_plane(c);
-  if (cudaMalloc(&c->wsave, 2 * 4 * 7 * spl) != cudaSuccess || cudaMalloc(&c->fadj, 16 * spl) != cudaSuccess)
-    return JS_ERR_NOMEM;
-  JS_CUDA(cudaMemsetAsync(c->wsave, 0, 2 * 4 * 7 * spl, c->stream));
-  JS_CUDA(cudaMemsetAsync(c->fadj, 0, 16 * spl, c->stream));
-  // internals stored by the forward stages 1, 2 of js_step_vjp (2D)
-  if (c->g.ny > 1) {
-    if (cudaMalloc(&c->wsave_fwd, 2 * 56 * spl) != cudaSuccess) {
-      c->wsave_fwd = nullptr;
-      return JS_ERR_NOMEM;
-    }
-    JS_CUDA(cudaMemsetAsync(c->wsave_fwd, 0, 2 * 56 * spl, c->stream));
-  }
   const size_t tmax = (size_t)std::max(c->g.nx + 6, c->g.ny);
   const size_t npp = (size_t)js::adj_ppart_doubles(c->lay, c->n_ghost, c->n_src, js::nn_image_vjp_blocks(c->lay));
-  if (cudaMalloc(&c->fcell, 24 * spl) != cudaSuccess ||
-      cudaMalloc(&c->wrev, sizeof(double) * (size_t)js::adj_wrev_doubles(c->lay)) != cudaSuccess ||
-      cudaMalloc(&c->ppart, sizeof(double) * npp) != cudaSuccess)
-    return JS_ERR_NOMEM;
+  if (cudaMalloc(&c->ppart, sizeof(double) * npp) != cudaSuccess) return JS_ERR_NOMEM;
   if (cudaMalloc(&c->inflow_part, sizeof(double) * 16 * tmax) != cudaSuccess ||
       cudaMalloc(&c->inflow_prim, 16 * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&c->qIb, sizeof(double) * 4 * (size_t)(c->n_ghost > 0 ? c->n_ghost : 1)) != cudaSuccess)
@@ -885,14 +830,11 @@ js::AdjArgs adj_args(js_ctx* c, const double* X, double* Ub, double* p_bar) {
   std::memset(&a, 0, sizeof(a));
   a.lay = c->lay;
   a.X = X;
-  a.Q = c->Q;
-  a.lam = c->lam;
-  a.fcell = c->fcell;
-  a.wrev = c->wrev;
+  a.Q = c->nnQ;
+  a.lam = c->nn_lam;
   a.pp = c->ppart;
   a.Ub = Ub;
-  a.wsave = c->wsave;
-  a.fadj = c->fadj;
+  a.fadj = c->nn_fadj;
   a.splane = saved_plane(c);
   a.tpitch = transposed_pitch(c);
   a.pbar = p_bar;
@@ -927,15 +869,10 @@ js::IbTArgs ibt_args(const js_ctx* c) {
   return t;
 }
 
-// one stage VJP; `saved` = WENO internals of this stage stored by its forward (or nullptr:
-// pass 1 recomputes them into the context's own buffer)
+// one stage VJP
 int adj_stage(js_ctx* c, const double* X, const double* Unext, double* Ub, double ra, double rb, double dt,
-              bool rhs_mode, double* p_bar, double* saved = nullptr) {
-  js::AdjArgs a = adj_args(c, X, Ub, p_bar);
-  if (saved) {
-    a.wsave = saved;
-    a.weno_saved = 1;
-  }
+              bool rhs_mode, double* p_bar) {
+  const js::AdjArgs a = adj_args(c, X, Ub, p_bar);
   c->nn.g1 = 1.0 / (c->p.gamma - 1.0);
   JS_CUDA(js::launch_adj_stage(a, c->bc, ib_args(c), ibt_args(c), c->p.wall, Unext, c->Uacc, ra, rb, dt, rhs_mode,
                                c->inflow_part, c->inflow_prim, c->qIb, c->stream, &c->launches,
@@ -1015,7 +952,7 @@ js::NnArgs nn_use_kept(js_ctx* c, int s, bool reverse) {
 int js_step_vjp(js_ctx* c, const double* U_n, double dt, const double* lam_np1, double* lam_n, double* p_bar) {
   if (!c || !U_n || !lam_np1 || !lam_n || !(dt > 0.0)) return JS_ERR_ARG;
   c->svjp_next = 2;  // the stage-wise reverse sequence (js_step_stage_vjp) restarts
-  c->stage_kept[0] = c->stage_kept[1] = false;  // wsave_fwd is reused here
+  c->stage_kept[0] = c->stage_kept[1] = false;
   int rc = adj_reserve(c);
   if (rc) return rc;
   if ((rc = upload_inflow(c))) return rc;
@@ -1029,11 +966,6 @@ int js_step_vjp(js_ctx* c, const double* U_n, double dt, const double* lam_np1, 
   a.avx = dt * c->p.nu / (c->g.dx * c->g.dx);
   a.avy = dt * c->p.nu / (c->g.dy * c->g.dy);
   const bool visc = c->p.mu > 0.0;
-  // 2D: the forward stages 1 and 2 also store their WENO internals, so that their reverse
-  // skips the WENO recompute (stage 3 is not run forward; its pass 1 recomputes them)
-  const bool keep = c->g.ny > 1 && c->wsave_fwd != nullptr;
-  double* saved[3] = {keep ? c->wsave_fwd : nullptr,
-                      keep ? c->wsave_fwd + 56 * (size_t)saved_plane(c) : nullptr, nullptr};
   double* in[2] = {c->N, c->A};
   double* outp[2] = {c->A, c->B};
   const double ra[3] = {0.0, 0.75, 1.0 / 3.0};
@@ -1049,7 +981,7 @@ int js_step_vjp(js_ctx* c, const double* U_n, double dt, const double* lam_np1, 
     a.rk_b = rb[s];
     a.use_un = (s > 0) ? 1 : 0;
     const js::NnArgs prev = nnk ? nn_use_kept(c, s, false) : c->nn;
-    rc = keep ? stage_save(c, a, visc, saved[s]) : stage(c, a, visc, false);
+    rc = stage(c, a, visc, false);
     c->nn = prev;
     if (rc) return rc;
   }
@@ -1061,7 +993,7 @@ int js_step_vjp(js_ctx* c, const double* U_n, double dt, const double* lam_np1, 
   double* dst = c->P1;
   for (int s = 2; s >= 0; --s) {
     const js::NnArgs prev = (nnk && s < 2) ? nn_use_kept(c, s, true) : c->nn;
-    rc = adj_stage(c, X[s], src, dst, ra[s], rb[s], dt, false, p_bar, saved[s]);
+    rc = adj_stage(c, X[s], src, dst, ra[s], rb[s], dt, false, p_bar);
     c->nn = prev;
     if (rc) return rc;
     double* t = src;
@@ -1091,8 +1023,7 @@ int js_step_stage_vjp(js_ctx* c, const double* U_in, double dt, int stage_flags,
   if (stage_k == 2) JS_CUDA(cudaMemsetAsync(c->Uacc, 0, sizeof(double) * 4 * (size_t)c->lay.plane, c->stream));
   const double ra[3] = {0.0, 0.75, 1.0 / 3.0};
   const double rb[3] = {1.0, 0.25, 2.0 / 3.0};
-  double* saved = kept ? c->wsave_fwd + 56 * (size_t)saved_plane(c) * stage_k : nullptr;
-  if ((rc = adj_stage(c, c->N, c->P0, c->P1, ra[stage_k], rb[stage_k], dt, false, p_bar, saved))) return rc;
+  if ((rc = adj_stage(c, c->N, c->P0, c->P1, ra[stage_k], rb[stage_k], dt, false, p_bar))) return rc;
   JS_CUDA(js::launch_adj_unpack(c->P1, stage_k == 0 ? c->Uacc : nullptr, lam_in, c->lay, c->stream));
   ++c->launches;
   c->svjp_next = (stage_k == 0) ? 2 : stage_k - 1;
@@ -1104,8 +1035,8 @@ size_t state_bytes(const js_ctx* c) { return sizeof(double) * 4 * (size_t)c->lay
 double* tape_state(js_ctx* c, int slot, int s) { return c->tape[(size_t)slot * 3 + s]; }
 
 // one SSP-RK3 step whose three stage inputs live in X[0..2] (X[0] already holds U^n);
-// the step result goes to `out` (padded); W[s] (if non-null) receives stage s's internals
-int step_through(js_ctx* c, double* const X[3], double* out, double dt, double* const W[3]) {
+// the step result goes to `out` (padded)
+int step_through(js_ctx* c, double* const X[3], double* out, double dt) {
   StageArgs a = base_args(c);
   a.cx = dt / c->g.dx;
   a.cy = dt / c->g.dy;
@@ -1123,7 +1054,7 @@ int step_through(js_ctx* c, double* const X[3], double* out, double dt, double* 
     a.rk_a = ra[s];
     a.rk_b = rb[s];
     a.use_un = (s > 0) ? 1 : 0;
-    rc = W[s] ? stage_save(c, a, visc, W[s]) : stage(c, a, visc, false);
+    rc = stage(c, a, visc, false);
     if (rc) return rc;
   }
   return JS_OK;
@@ -1141,19 +1072,6 @@ int js_tape_reserve_ex(js_ctx* c, int n_slots, int flags) {
     if (cudaMemsetAsync(p, 0, state_bytes(c), c->stream) != cudaSuccess) { cudaFree(p); return JS_ERR_CUDA; }
     c->tape.push_back(p);
   }
-  c->tape_weno = (flags & JS_TAPE_WENO) != 0 && c->g.ny > 1;
-  c->tape_w.resize(c->tape.size(), nullptr);
-  c->tape_w_ok.resize(c->tape.size() / 3, 0);
-  if (c->tape_weno) {
-    for (size_t k = 0; k < need; ++k) {
-      if (c->tape_w[k]) continue;
-      if (cudaMalloc(&c->tape_w[k], internals_bytes(c)) != cudaSuccess) {
-        c->tape_w[k] = nullptr;
-        c->tape_weno = false;
-        return JS_ERR_NOMEM;
-      }
-    }
-  }
   JS_CUDA(cudaStreamSynchronize(c->stream));
   return JS_OK;
 }
@@ -1163,15 +1081,9 @@ int js_tape_reserve(js_ctx* c, int n_slots) { return js_tape_reserve_ex(c, n_slo
 int js_step_taped(js_ctx* c, double* U, double dt, int slot) {
   if (!c || !U || !(dt > 0.0) || slot < 0 || (size_t)(slot + 1) * 3 > c->tape.size()) return JS_ERR_ARG;
   double* X[3] = {tape_state(c, slot, 0), tape_state(c, slot, 1), tape_state(c, slot, 2)};
-  const size_t b = (size_t)slot * 3;
-  const bool keep = c->tape_weno && c->tape_w[b] && c->tape_w[b + 1] && c->tape_w[b + 2];
-  double* W[3] = {keep ? c->tape_w[b] : nullptr, keep ? c->tape_w[b + 1] : nullptr,
-                  keep ? c->tape_w[b + 2] : nullptr};
-  c->tape_w_ok[slot] = 0;
   JS_CUDA(js::launch_pack(U, X[0], c->lay, c->stream));
-  int rc = step_through(c, X, c->N, dt, W);
+  int rc = step_through(c, X, c->N, dt);
   if (rc) return rc;
-  c->tape_w_ok[slot] = keep ? 1 : 0;
   JS_CUDA(js::launch_unpack(c->N, U, c->lay, c->stream));
   c->launches += 2;
   return JS_OK;
@@ -1191,10 +1103,8 @@ int js_step_vjp_taped(js_ctx* c, int slot, double dt, const double* lam_np1, dou
   const double rb[3] = {1.0, 0.25, 2.0 / 3.0};
   double* src = c->P0;
   double* dst = c->P1;
-  const bool saved = c->tape_w_ok[slot] != 0;
   for (int s = 2; s >= 0; --s) {
-    double* w = saved ? c->tape_w[(size_t)slot * 3 + s] : nullptr;
-    if ((rc = adj_stage(c, tape_state(c, slot, s), src, dst, ra[s], rb[s], dt, false, p_bar, w))) return rc;
+    if ((rc = adj_stage(c, tape_state(c, slot, s), src, dst, ra[s], rb[s], dt, false, p_bar))) return rc;
     double* t = src;
     src = dst;
     dst = t;
@@ -1359,13 +1269,19 @@ int js_set_neural(js_ctx* c, const double* w, double* w_bar, const double* norm,
     n.scale[k] = norm[8 + k];
   }
   n.g1 = 1.0 / (c->p.gamma - 1.0);
-  // 2D: the stage kernel stores the WENO5 internals the face images are formed from
-  if (two_d && !c->nn_wsave) {
-    if (cudaMalloc(&c->nn_wsave, internals_bytes(c)) != cudaSuccess) {
-      c->nn_wsave = nullptr;
+  if (!c->nn_lam) {  // reverse workspace
+    const size_t lam = sizeof(double) * 4 * (size_t)c->lay.plane, fa = sizeof(double) * 16 * (size_t)saved_plane(c);
+    if (cudaMalloc(&c->nn_lam, lam) != cudaSuccess) {
+      c->nn_lam = nullptr;
       return JS_ERR_NOMEM;
     }
-    JS_CUDA(cudaMemsetAsync(c->nn_wsave, 0, internals_bytes(c), c->stream));
+    if (cudaMalloc(&c->nn_fadj, fa) != cudaSuccess) {
+      cudaFree(c->nn_lam);
+      c->nn_lam = c->nn_fadj = nullptr;
+      return JS_ERR_NOMEM;
+    }
+    JS_CUDA(cudaMemsetAsync(c->nn_lam, 0, lam, c->stream));
+    JS_CUDA(cudaMemsetAsync(c->nn_fadj, 0, fa, c->stream));
   }
   JS_CUDA(cudaStreamSynchronize(c->stream));
   c->nn_on = true;
@@ -1394,15 +1310,12 @@ int js_internal_rev_desc(js_ctx* c, js::InstRev* d) {
   std::memset(d, 0, sizeof(*d));
   int rc = adj_reserve(c);
   if (rc) return rc;
-  if (!c->wsave_fwd) return JS_ERR_NOMEM;
   if ((rc = upload_inflow(c))) return rc;
   d->a = adj_args(c, nullptr, nullptr, nullptr);
   d->ibt = ibt_args(c);
   d->P0 = c->P0;
   d->P1 = c->P1;
   d->Uacc = c->Uacc;
-  d->wsave_own = c->wsave;
-  d->wfwd = c->wsave_fwd;
   d->inflow_part = c->inflow_part;
   d->inflow_prim = c->inflow_prim;
   d->qIb = c->qIb;

@@ -19,11 +19,6 @@ struct StageArgs {
   double avx, avy;           // (dt) nu / dx^2, (dt) nu / dy^2
   ViscC vx, vy;              // viscous constants of x and y faces
   int use_un, has_av;
-  // WENO5 internals for the reverse pass (kernels instantiated with SAVE): 56 planes of
-  // `splane` doubles, x lines transposed (row pitch tpitch), y lines in the padded layout
-  double* wsave;
-  long long splane;
-  int tpitch;
   // device-resident step size (js_step_cfl): when set, cx, cy, avx, avy are read from
   // dtc[0..3] at kernel start, and dtc[4] == 0 means the step is inactive (skip the stage)
   const double* dtc;
@@ -63,12 +58,12 @@ struct IbTArgs {
 struct AdjArgs {
   Lay lay;
   const double* X;           // padded filled stage state (4 planes)
-  double* Q;                 // padded primitives rho, u, v, p, T (5 planes)
-  double* lam;               // padded lambda' (4 planes), zero outside fluid cells
+  const double* Q;           // padded primitives (4 planes; the neural flux's reverse only)
+  double* lam;               // padded lambda' (4 planes), zero outside fluid cells (likewise)
   double* Ub;                // padded conserved adjoints of X (4 planes)
-  double* wsave;             // WENO internals [dir][var][7] planes of splane doubles
-  double* fadj;              // face-state adjoints [dir][left/right][var] planes of splane
-  long long splane;          // plane size of wsave / fadj (>= both layouts below)
+  double* fadj;              // the neural flux's face-state adjoints [dir][left/right][var] planes
+                             //   of splane, or nullptr without the network
+  long long splane;          // plane size of fadj (>= both layouts below)
   int tpitch;                // x-direction planes are stored transposed: (i+3)*tpitch + j+gy
   double* pbar;              // parameter gradient (JS_NPARAM) or nullptr
   const unsigned char* tag;
@@ -79,21 +74,16 @@ struct AdjArgs {
   ViscC vx, vy;
   double inv_mu, kg, kp;     // 1/mu, -1/(gamma (gamma-1)), -1/Pr
   int visc, has_av, two_d;
-  int weno_saved;            // wsave already holds the stage's WENO internals (forward SAVE)
-  // deterministic reverse (no floating-point atomics: every sum in a fixed order)
-  double* fcell;             // per face [dir][12] planes of splane: adjoints that go straight to
-                             //   the two cells of the face (positivity fallback, viscous terms:
-                             //   left cell rho,u,v,p,T at 0-4, right cell at 5-9, tangential
-                             //   derivative terms at 10-11)
-  double* wrev;              // pass-2 output slots [dir][4][seg][SL][line] (WENO5 reverse)
-  double* pp;                // block partials of pbar[0..3] of the current launch (4 per block)
+  double* pp;                // warp partials of pbar[0..3] of the current launch (4 per warp)
 };
 
-// pass-2 segment length (cells per thread along a line) and slot length of wrev
-constexpr int ADJ_SEG2 = 8, ADJ_SEG2_1D = 4;
-// doubles of the wrev slots of a grid, and of the parameter-gradient block partials of one
-// reverse stage (bounds; nn_blocks = blocks of the neural image reverse, 0 without it)
-long long adj_wrev_doubles(const Lay& lay);
+// the reverse tile kernel: output cells of the padded array per tile and direction, warps a block
+constexpr int ADJ_TILE = 24, ADJ_WARPS = 8;
+// tiles of a grid's padded array along x and y
+inline __host__ __device__ int adj_tiles_x(const Lay& lay) { return (lay.nx + 6 + ADJ_TILE - 1) / ADJ_TILE; }
+inline __host__ __device__ int adj_tiles_y(const Lay& lay) { return (lay.H + ADJ_TILE - 1) / ADJ_TILE; }
+// doubles of the parameter-gradient warp partials of one reverse stage (nn_blocks = blocks of the
+// neural image reverse, 0 without it)
 long long adj_ppart_doubles(const Lay& lay, int n_ghost, int n_src, long long nn_blocks);
 // blocks of the neural image-reverse kernel for a grid (one partial each)
 long long nn_image_vjp_blocks(const Lay& lay);
@@ -125,11 +115,6 @@ struct NnArgs {
   void* G32;                  // 32-channel gradient scratch
   double* partial;            // weight-gradient partial sums [nwblk][NN_NPARAM]
   int nwblk;
-  // WENO5 internals of the stage (2D, layout of StageArgs::wsave) to form the face states
-  // from, or nullptr: the image kernels then recompute WENO5
-  const double* wsave;
-  long long splane;
-  int tpitch;
   int bf16;                   // layers 2 and 3 on the tensor cores (BF16 operands, FP32 accumulate)
   void* A1h;                  // BF16 copies of the activations of layers 1 and 2, pixel-major with
   void* A2h;                  //   the channels contiguous ([image][H][W][C]), tensor-core inputs
@@ -149,7 +134,7 @@ cudaError_t nn_layers(const NnArgs& n, cudaStream_t s);
 // stage output (or RHS) minus the divergence of the neural flux held in T3
 cudaError_t nn_apply(const NnArgs& n, const StageArgs& a, bool rhs, cudaStream_t s);
 // reverse: recompute the network on a.Q, seed with the face-flux adjoints of a.lam, back-
-// propagate (parameter gradient into n.w_bar), add the face-state adjoints to a.fadj
+// propagate (parameter gradient into n.w_bar), write the face-state adjoints to a.fadj
 cudaError_t nn_reverse(const NnArgs& n, const AdjArgs& a, cudaStream_t s);
 // the network alone on one image X[4][H][W] (FP64, device) -> scaled output Y[4][H][W]
 cudaError_t nn_eval(const NnArgs& n, const double* X, int H, int W, double* Y, cudaStream_t s);
@@ -158,7 +143,7 @@ cudaError_t nn_eval_vjp(const NnArgs& n, const double* X, int H, int W, const do
 // out[4][ny/fy][nx/fx] = means of fx x fy blocks of U[4][ny][nx]
 cudaError_t launch_block_average(const double* U, int nx, int ny, int fx, int fy, double* out, cudaStream_t s);
 
-// nn: the neural flux's reverse (run between pass 1 and pass 2) or nullptr
+// nn: the neural flux's reverse (run first: a.Q, a.lam, a.fadj are its workspace) or nullptr
 // inflow_part: [4 sides][max(nx + 6, ny)][4] partial sums of the inflow halo adjoints
 cudaError_t launch_adj_stage(const AdjArgs& a, const BcArgs& bc, const IbArgs& ib, const IbTArgs& ibt, int wall,
                              const double* Unext, double* Uacc, double ra, double rb, double dt, bool rhs_mode,
@@ -184,24 +169,21 @@ struct InstDesc {
 
 // reverse-pass description of one instance for the persistent batched reverse kernel
 // (js_batch.cu): the context's adjoint arguments and workspace (js_internal_rev_desc) and the
-// instance's work-item counts and parameter-gradient slot offsets (set by js_batch.cu)
+// instance's tiles and parameter-gradient slot offsets (set by js_batch.cu)
 struct InstRev {
-  AdjArgs a;                 // X, Ub, pbar, pp, wsave, weno_saved are set per phase
+  AdjArgs a;                 // X, Ub, pbar, pp are set per phase
   IbTArgs ibt;
   double* P0;                // adjoint ping-pong states (4 padded planes each)
   double* P1;
   double* Uacc;              // U^n part of the step's adjoint (4 padded planes)
-  double* wsave_own;         // WENO5 internals recomputed by pass 1 (stage 2)
-  double* wfwd;              // internals stored by the forward stages 0 and 1 (2 x 56 planes)
   double* inflow_part;
   const double* inflow_prim;
   double* qIb;
   double* ppart;             // warp partials of the parameter gradient
   int tmax;                  // max(nx + 6, ny): inflow_part row length
-  int seg1_re, seg1_sv, seg2;  // pass-1 segment lengths (recompute / stored internals), pass 2
-  long long xpad_re, xpad_sv, xpad_p2;  // x-line items of passes 1 and 2, rounded up to 32
-  long long w1_re, w1_sv;    // warp slots of pass 1 (both directions)
-  long long off_prim, w_prim, off_g, w_g, off_s, w_s;  // slots of primvjp, IB ghost, IB source
+  int tile0;                 // the instance's first reverse tile
+  long long w_adj;           // warp slots of its reverse tiles
+  long long off_g, w_g, off_s, w_s;  // slots of IB ghost, IB source
 };
 
 // opaque 128-byte, 64-byte aligned tensor map (CUtensorMap) for TMA copies
@@ -228,9 +210,6 @@ cudaError_t launch_ieee_stage(const StageArgs& a, const IeeeBufs& b, double dt, 
 constexpr int STAGE_VARIANTS = 5;
 cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, const TensorMap128* tmap,
                          cudaStream_t s);
-// stage update (not RHS mode) that also stores the WENO5 internals to a.wsave (2D only;
-// TMA-staged when tmap is given)
-cudaError_t launch_stage_save(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s);
 // stage update that also writes the neural flux's face images of its input to a.img (2D)
 cudaError_t launch_stage_img(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s);
 cudaError_t launch_bc_fill(double* U, const Lay& lay, const BcArgs& bc, cudaStream_t s);

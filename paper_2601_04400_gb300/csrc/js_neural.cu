@@ -70,36 +70,18 @@ __device__ __forceinline__ uint4 pack_bf16x8(const float v[8]) {
 __device__ __forceinline__ void face_states(const Lay& L, const double* Q, long long qplane, int d, int h, int f,
                                             double wl[4], double wr[4]) {
   const long long st = (d == 0) ? 1 : L.pitch;
-  const long long cf = (d == 0) ? L.idx(f, h) : L.idx(h, f);
-  const double* q = Q + cf;
-  double dummy[4];
-  auto none = [](int, const double*) {};
-  Win4 w;
-  w.init(q - st, qplane, st);
-  w.template step<true, false, false>(q - st, qplane, st, wl, dummy, none);
-  w.template step<false, true, false>(q, qplane, st, dummy, wr, none);
-}
-
-// the same face states from the stage's stored WENO5 internals: state = q_cell + q/6 with the
-// quotient q saved for the left-biased state of cell f-1 and the right-biased one of cell f
-__device__ __forceinline__ void face_states_saved(const NnArgs& n, const Lay& L, const double* Q, long long qplane,
-                                                  int d, int h, int f, double wl[4], double wr[4]) {
-  const long long ca = (d == 0) ? L.idx(f - 1, h) : L.idx(h, f - 1);
-  const long long cb = (d == 0) ? L.idx(f, h) : L.idx(h, f);
-  const long long sa = (d == 0) ? (long long)(f + 2) * n.tpitch + (h + L.gy) : ca;
-  const long long sb = (d == 0) ? (long long)(f + 3) * n.tpitch + (h + L.gy) : cb;
-#pragma unroll
+  const double* q = Q + ((d == 0) ? L.idx(f, h) : L.idx(h, f));
+#pragma unroll 1
   for (int c = 0; c < 4; ++c) {
-    const double* sv = n.wsave + (long long)(d * 28 + c * 7) * n.splane;
-    wl[c] = fma(sv[3 * n.splane + sa], SIXTH, Q[c * qplane + ca]);
-    wr[c] = fma(sv[5 * n.splane + sb], SIXTH, Q[c * qplane + cb]);
+    double l, r, unused;
+    weno_cell(q + c * qplane - st, st, c == 0 || c == 3, l, unused);
+    weno_cell(q + c * qplane, st, c == 0 || c == 3, unused, r);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      wl[m] = (c == m) ? l : wl[m];
+      wr[m] = (c == m) ? r : wr[m];
+    }
   }
-}
-
-__device__ __forceinline__ void face_states_any(const NnArgs& n, const Lay& L, const double* Q, long long qplane,
-                                                int d, int h, int f, double wl[4], double wr[4]) {
-  if (n.wsave) face_states_saved(n, L, Q, qplane, d, h, f, wl, wr);
-  else face_states(L, Q, qplane, d, h, f, wl, wr);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -146,7 +128,7 @@ __global__ void __launch_bounds__(256) nn_image_kernel(NnArgs n, const double* _
     if (h >= H || f >= Wd) continue;
     double wl[4], wr[4];
     T m[4];
-    face_states_any(n, n.lay, Q, qplane, d, h, f, wl, wr);
+    face_states(n.lay, Q, qplane, d, h, f, wl, wr);
     face_image<T>(wl, wr, un, ut, (T)n.g1, mean, isd, m);
 #pragma unroll
     for (int k = 0; k < 4; ++k) sx[k][hl][fl] = m[k];
@@ -1547,7 +1529,7 @@ __device__ __forceinline__ double nn_warp_sum(double v) {
   return v;
 }
 
-// image reverse: network-input adjoint -> WENO face-state adjoints (added to a.fadj) and
+// image reverse: network-input adjoint -> WENO face-state adjoints (a.fadj) and
 // d/dgamma of the face energies (added to pbar[0]); 32 x 32 pixel tiles as nn_image_kernel
 template <class T>
 __global__ void __launch_bounds__(256) nn_image_vjp_kernel(NnArgs n, AdjArgs a) {
@@ -1578,7 +1560,7 @@ __global__ void __launch_bounds__(256) nn_image_vjp_kernel(NnArgs n, AdjArgs a) 
     const int h = h0 + hl, f = f0 + fl;
     if (h >= H || f >= Wd) continue;
     double wl[4], wr[4];
-    face_states_any(n, a.lay, a.Q, a.lay.plane, d, h, f, wl, wr);
+    face_states(a.lay, a.Q, a.lay.plane, d, h, f, wl, wr);
     double gk[4];  // adjoint of each side's conserved frame state (the image is their mean)
 #pragma unroll
     for (int k = 0; k < 4; ++k) gk[k] = 0.5 * n.inv_sd[k] * (double)sx[k][hl][fl];
@@ -1593,7 +1575,7 @@ __global__ void __launch_bounds__(256) nn_image_vjp_kernel(NnArgs n, AdjArgs a) 
       b[3] = gk[3] * n.g1;
       gbar -= pr * n.g1 * n.g1 * gk[3];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) a.fadj[(long long)(fdir + 4 * sd + c) * a.splane + si] += b[c];
+      for (int c = 0; c < 4; ++c) a.fadj[(long long)(fdir + 4 * sd + c) * a.splane + si] = b[c];
     }
   }
   gbar = nn_warp_sum(gbar);
@@ -1905,12 +1887,7 @@ long long nn_image_vjp_blocks(const Lay& lay) {
 }
 
 cudaError_t nn_reverse(const NnArgs& n, const AdjArgs& a, cudaStream_t s) {
-  // pass 1 has run: on 2D grids a.wsave holds the stage's WENO5 internals
-  NnArgs m = n;
-  m.wsave = a.two_d ? a.wsave : nullptr;
-  m.splane = a.splane;
-  m.tpitch = a.tpitch;
-  return m.fp32 ? reverse_t<float>(m, a, s) : reverse_t<double>(m, a, s);
+  return n.fp32 ? reverse_t<float>(n, a, s) : reverse_t<double>(n, a, s);
 }
 
 // ---------------------------------------------------------------------------------------

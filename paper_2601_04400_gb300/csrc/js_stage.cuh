@@ -26,9 +26,6 @@ __device__ __forceinline__ u64 shfl_down(u64 v) { return (u64)__shfl_down_sync(F
 __device__ __forceinline__ double shfl_up(double v) { return __shfl_up_sync(FULL, v, 1); }
 __device__ __forceinline__ double shfl_down(double v) { return __shfl_down_sync(FULL, v, 1); }
 
-struct NoKeep {
-  __device__ __forceinline__ void operator()(int, const double*) const {}
-};
 struct NoFace {
   __device__ __forceinline__ void operator()(const double*, const double*) const {}
 };
@@ -37,12 +34,11 @@ struct NoFace {
 // v, p, and T when VISC, `ps` apart; neighbours along the line at multiples of st, across it of
 // ts), valid in lanes 2..29.  pn: plane of the face-normal velocity (1 or 2).  Every lane of the
 // warp calls it, consecutive lanes on consecutive cells; q[-st .. st] is readable for each.
-// keep(c, sv), when given, receives the WENO5 internals of variable c (valid in lanes 1..30);
-// face(ql, qr) the two WENO5 states of face i+1/2 before any positivity fallback (lanes 1..29).
-template <bool VISC, bool HAS_T, class Keep = NoKeep, class Face = NoFace>
+// face(ql, qr), when given, receives the two WENO5 states of face i+1/2 before any positivity
+// fallback (lanes 1..29).
+template <bool VISC, bool HAS_T, class Face = NoFace>
 __device__ __forceinline__ void line_fluxes(const double* q, int ps, int st, int ts, int pn, const Gas& g,
-                                            const ViscC& vc, double dF[4], Keep keep = Keep{}, Face face = Face{}) {
-  constexpr bool SV = !std::is_same<Keep, NoKeep>::value;
+                                            const ViscC& vc, double dF[4], Face face = Face{}) {
   constexpr bool FI = !std::is_same<Face, NoFace>::value;
   const int lane = threadIdx.x & 31;
   const bool inner = lane - 1u < 30u;
@@ -53,9 +49,7 @@ __device__ __forceinline__ void line_fluxes(const double* q, int ps, int st, int
   for (int k = 0; k < 4; ++k) {
     const int c = (k == 1) ? pn : (k == 2) ? pt : k;
     double Lf, Rf;
-    double sv[SV ? 7 : 1];
-    weno_lane<SV>(q + c * ps, st, k == 0 || k == 3, inner, Lf, Rf, sv);
-    if (SV) keep(c, sv);
+    weno_lane(q + c * ps, st, k == 0 || k == 3, inner, Lf, Rf);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       L[m] = (k == m) ? Lf : L[m];
@@ -257,22 +251,6 @@ __device__ __forceinline__ bool load_tile_tma(const StageArgs& a, const void* tm
   return true;
 }
 
-// Store the WENO5 internals of variable c at cell k of line `line` (dir 0: row, stored
-// transposed; dir 1: column, padded layout), for the cells -1 .. n the reverse pass reads
-// (n = cells along the line).  Cell -1 keeps only its left-biased side, cell n its right-biased
-// one; `owner`: this lane's cell is one of the tile's outputs.
-__device__ __forceinline__ void keep_internals(const StageArgs& a, int dir, int k, int line, int c, const double* sv,
-                                               bool owner) {
-  const int n = (dir == 0) ? a.lay.nx : a.lay.ny;
-  if (!(k == -1 || k == n || (owner && k >= 0 && k < n))) return;
-  const long long si = (dir == 0) ? (long long)(k + 3) * a.tpitch + (line + a.lay.gy) : a.lay.idx(line, k);
-  double* dst = a.wsave + (long long)(dir * 28 + c * 7) * a.splane + si;
-  const bool left = k < n, right = k >= 0;
-#pragma unroll
-  for (int m = 0; m < 7; ++m)
-    dst[m * a.splane] = ((m == 3 || m == 4) && !left) || ((m == 5 || m == 6) && !right) ? 0.0 : sv[m];
-}
-
 // face image of the neural flux (IMG: a.img, FP32 [4][ny][nx+1] for x faces then [4][nx][ny+1]
 // for y faces): face f of a line
 __device__ __forceinline__ void put_image(const StageArgs& a, int dir, int line, int f, const double* ql,
@@ -290,7 +268,7 @@ __device__ __forceinline__ void put_image(const StageArgs& a, int dir, int line,
 }
 
 // one tile (bx, by) of one stage; smem holds StageTile::SMEM bytes; whole warps take part
-template <bool VISC, bool RHS, bool TMA = false, bool SAVE = false, bool IMG = false>
+template <bool VISC, bool RHS, bool TMA = false, bool IMG = false>
 __device__ __forceinline__ void stage_tile(const StageArgs& a, int bx, int by, double* smem,
                                            const void* tmap = nullptr, unsigned long long* bar = nullptr,
                                            unsigned* phase = nullptr) {
@@ -321,12 +299,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int bx, int by, d
       double dF[4];
       const int gk = (dir == 0 ? tx0 : ty0) + k, gl = (dir == 0 ? ty0 : tx0) + ln;  // cell and line in the grid
       const bool owner = lane >= 2 && k < ncell;
-      if constexpr (SAVE) {
-        line_fluxes<VISC, true>(q, S::PS, st, ts, dir + 1, g, vc, dF, [&](int c, const double* sv) {
-          if (lane >= 1 && lane <= 30) keep_internals(a, dir, gk, gl, c, sv, owner && lane < 30);
-        });
-      } else if constexpr (IMG) {
-        line_fluxes<VISC, true>(q, S::PS, st, ts, dir + 1, g, vc, dF, NoKeep{}, [&](const double* ql, const double* qr) {
+      if constexpr (IMG) {
+        line_fluxes<VISC, true>(q, S::PS, st, ts, dir + 1, g, vc, dF, [&](const double* ql, const double* qr) {
           // face gk + 1; the tile's outer face belongs to the next tile unless it is the line's last
           const int f = gk + 1, n = dir == 0 ? a.lay.nx : a.lay.ny;
           if (lane >= 1 && f <= n && (lane <= 28 || (lane == 29 && f == n))) put_image(a, dir, gl, f, ql, qr);

@@ -43,7 +43,6 @@ JS_HD Sm sm_norm(u64 s, int x2) {
   const int lz = clz64(s);
   return Sm{s << (lz & 63), x2 - lz};
 }
-JS_HD double sm_double(const Sm& s) { return bitsd(((u64)(u32)(s.x - 1015) << 52) + (s.m >> 11) + ((s.m >> 10) & 1u)); }
 
 // 3 (4 eps) 2^76, and the exponent of d at which the indicators hold it at that scale: pairs of
 // smaller differences keep the scale, larger ones shift it down
@@ -67,52 +66,154 @@ JS_HD void sm_pair(const Fx& a, const Fx& b, Sm& s1, Sm& s0n, Sm& s2p) {
   s2p = sm_norm(g - h12, 2 * E);
 }
 
-// c_L = 6 (q_{i+1/2}^L - q_i) (NL) and c_R = 6 (q_{i-1/2}^R - q_i) (NR) of cell i from its four
-// differences and three indicators.  With SV also r_L, r_R = 1 over the weights' sums on the
-// scale of (3 s_k)^4 (0 where they leave the FP64 range).
-template <bool NL, bool NR, bool SV>
-JS_HD void weno_corr(const Fx& dm2, const Fx& dm1, const Fx& dp1, const Fx& dp2, const Sm& s0, const Sm& s1,
-                     const Sm& s2, int F, double& cL, double& cR, double& rL, double& rR) {
-  // weights w_0 = (s1 s2)^2, w_1 = (s0 s2)^2, w_2 = (s0 s1)^2 (proportional to 1/s_k^2): shifted
-  // so that the weighted sums 3 w_0 + 6 w_1 + 3 w_2 (at most X 2^36) stay below 2^62
+// weights of one cell: W_k 2^-n_k proportional to 1/s_k^2, and w_k = W_k >> (n_k + up) on the
+// scale on which the weighted sum 3 w_0 + 6 w_1 + 3 w_2 (at most X 2^36) has 60 to 62 bits
+struct Wgt {
+  u64 W0, W1, W2;
+  int n0, n1, n2, up;
+  s64 w0, w1, w2;
+};
+JS_HD Wgt weno_weights(const Sm& s0, const Sm& s1, const Sm& s2) {
+  Wgt g;
   const u64 p12 = mul_top(s1.m, s2.m), p02 = mul_top(s0.m, s2.m), p01 = mul_top(s0.m, s1.m);
-  const u64 W0 = sqr_top(p12), W1 = sqr_top(p02), W2 = sqr_top(p01);
+  g.W0 = sqr_top(p12), g.W1 = sqr_top(p02), g.W2 = sqr_top(p01);
   const int xm = imin(imin(s0.x, s1.x), s2.x);
-  const int n0 = 2 * (s0.x - xm), n1 = 2 * (s1.x - xm), n2 = 2 * (s2.x - xm);
-  const u32 X = 3u * (shr32(hi32(W0), n0 + 4) + shr32(hi32(W2), n2 + 4) + 2u * shr32(hi32(W1), n1 + 4) + 4u);
-  const int up = 6 - clz32(X);
-  const s64 w0 = (s64)shr(W0, n0 + up), w1 = (s64)shr(W1, n1 + up), w2 = (s64)shr(W2, n2 + up);
-  const s64 w6 = 6 * w1;
+  g.n0 = 2 * (s0.x - xm), g.n1 = 2 * (s1.x - xm), g.n2 = 2 * (s2.x - xm);
+  const u32 X = 3u * (shr32(hi32(g.W0), g.n0 + 4) + shr32(hi32(g.W2), g.n2 + 4) + 2u * shr32(hi32(g.W1), g.n1 + 4) + 4u);
+  g.up = 6 - clz32(X);
+  g.w0 = (s64)shr(g.W0, g.n0 + g.up), g.w1 = (s64)shr(g.W1, g.n1 + g.up), g.w2 = (s64)shr(g.W2, g.n2 + g.up);
+  return g;
+}
+
+// c_L = 6 (q_{i+1/2}^L - q_i) and c_R = 6 (q_{i-1/2}^R - q_i) of cell i from its four differences
+// (F: the largest's exponent) and three indicators
+JS_HD void weno_corr(const Fx& dm2, const Fx& dm1, const Fx& dp1, const Fx& dp2, const Sm& s0, const Sm& s1,
+                     const Sm& s2, int F, double& cL, double& cR) {
+  const Wgt g = weno_weights(s0, s1, s2);
+  const s64 w6 = 6 * g.w1;
   // differences on the scale of the largest
   const s64 a = sar(dm2.m, F - dm2.e), b = sar(dm1.m, F - dm1.e), c = sar(dp1.m, F - dp1.e), d = sar(dp2.m, F - dp2.e);
   const Limb l6 = limbs(w6);
-  const int K = SV ? 2 * (s0.x + s1.x + s2.x) - 2 * xm + up - 8208 : 0;
-  if (NL) {  // linear weights 1 : 6 : 3
-    const s64 w2_3 = 3 * w2;
-    const u64 den = (u64)(w0 + w6 + w2_3);
-    const s64 num = mul62(limbs(w0), limbs(5 * b - 2 * a)) + mul62(l6, limbs(b + 2 * c)) +
+  {  // linear weights 1 : 6 : 3
+    const s64 w2_3 = 3 * g.w2;
+    const u64 den = (u64)(g.w0 + w6 + w2_3);
+    const s64 num = mul62(limbs(g.w0), limbs(5 * b - 2 * a)) + mul62(l6, limbs(b + 2 * c)) +
                     mul62(limbs(w2_3), limbs(4 * c - d));
-    const int lz = clz64(den);
-    const u64 r = recip_top(den << lz);
-    cL = fix_to_double(mul62(limbs(num), limbs((s64)r)), F + lz + 4);
-    if (SV) {
-      const int be = 959 + lz - K;
-      rL = (be < 1 || be > 2046) ? 0.0 : pack62(r, be);
-    }
+    const int lz = clz32(hi32(den));
+    cL = fix_to_double(mul62(limbs(num), limbs((s64)recip_top(den << lz))), F + lz + 4);
   }
-  if (NR) {  // 3 : 6 : 1
-    const s64 w0_3 = 3 * w0;
-    const u64 den = (u64)(w0_3 + w6 + w2);
+  {  // 3 : 6 : 1
+    const s64 w0_3 = 3 * g.w0;
+    const u64 den = (u64)(w0_3 + w6 + g.w2);
     const s64 num = mul62(limbs(w0_3), limbs(a - 4 * b)) + mul62(l6, limbs(-2 * b - c)) +
-                    mul62(limbs(w2), limbs(2 * d - 5 * c));
-    const int lz = clz64(den);
-    const u64 r = recip_top(den << lz);
-    cR = fix_to_double(mul62(limbs(num), limbs((s64)r)), F + lz + 4);
-    if (SV) {
-      const int be = 959 + lz - K;
-      rR = (be < 1 || be > 2046) ? 0.0 : pack62(r, be);
-    }
+                    mul62(limbs(g.w2), limbs(2 * d - 5 * c));
+    const int lz = clz32(hi32(den));
+    cR = fix_to_double(mul62(limbs(num), limbs((s64)recip_top(den << lz))), F + lz + 4);
   }
+}
+
+// ---------------------------------------------------------------------------------------
+// Derivatives of c_L and c_R with respect to the cell's four differences a, b, c, d.
+// With the normalised weights om_k, the candidates e_k (c = sum om_k e_k) and sigma_k = 3 s_k:
+//   dc/dx = sum_k om_k de_k/dx - 4 sum_k Z_k V_kx,   Z_k = om_k (e_k - c),
+//   V_kx = (dsigma_k/dx) / (2 sigma_k).
+// Z_k is formed from the pairs, Z_0 = om_0 om_1 (e_0 - e_1) + om_0 om_2 (e_0 - e_2) and so on,
+// which keeps it accurate where one weight is nearly 1 and e_k - c nearly 0; the differences of
+// candidates are multiples of the third differences T_0 = a - 2 b + c, T_1 = b - 2 c + d.  Every
+// factor carries its own exponent to the end; the eight results are rounded from a common scale
+// of 2^-56 (they stay below 2^4).  Errors against 128-bit arithmetic: 1e-16 rms, 4 to 6 times below
+// those of the FP64 formulas.
+// ---------------------------------------------------------------------------------------
+// half the logarithmic derivatives of one indicator with respect to its pair: V = m 2^(960 + k)
+struct Lv {
+  s64 a, b;
+  s32 k;
+};
+
+// sm_pair and the derivatives of its three indicators
+JS_HD void sm_pair_grad(const Fx& a, const Fx& b, Sm& s1, Sm& s0n, Sm& s2p, Lv& v1, Lv& v0n, Lv& v2p) {
+  sm_pair(a, b, s1, s0n, s2p);
+  const int E = imax(imax(a.e, b.e), W_EMIN);
+  const s64 p = sar(a.m, E - a.e + 3), q = sar(b.m, E - b.e + 3);
+  const Limb r1 = limbs((s64)recip_top(s1.m)), r0 = limbs((s64)recip_top(s0n.m)), r2 = limbs((s64)recip_top(s2p.m));
+  v1 = Lv{mul62(limbs(8 * p - 5 * q), r1), mul62(limbs(8 * q - 5 * p), r1), E - s1.x};
+  v0n = Lv{mul62(limbs(8 * p - 11 * q), r0), mul62(limbs(20 * q - 11 * p), r0), E - s0n.x};
+  v2p = Lv{mul62(limbs(20 * p - 11 * q), r2), mul62(limbs(8 * q - 11 * p), r2), E - s2p.x};
+}
+
+// x 2^l with 2^60 <= |x 2^l| < 2^61 (two low bits of x dropped)
+struct Nm {
+  s64 m;
+  s32 l;
+};
+JS_HD Nm nm_of(s64 x) {
+  const int l = clz64((u64)(x ^ (x >> 63)) | 1u) - 3;
+  return Nm{(x >> 2) << (l + 2), l};
+}
+// x 2^-n for n of either sign
+JS_HD s64 scale_down(s64 x, int n) { return n >= 0 ? sar(x, n) : (s64)((u64)x << (-n)); }
+
+// what both sides' derivatives share
+struct GradCell {
+  Wgt g;
+  Sm N0, N1, N2;       // W_k normalised
+  s64 T0, T1;          // third differences on the scale 2^(F - 1081)
+  Nm t0, t1;
+  Limb v0a, v0b, v1b, v1c, v2c, v2d;
+  int k0, k1, k2, F;
+};
+JS_HD GradCell grad_cell(const Fx& dm2, const Fx& dm1, const Fx& dp1, const Fx& dp2, const Sm& s0, const Sm& s1,
+                         const Sm& s2, const Lv& v0, const Lv& v1, const Lv& v2, int F) {
+  GradCell q;
+  q.g = weno_weights(s0, s1, s2);
+  const s64 a = sar(dm2.m, F - dm2.e), b = sar(dm1.m, F - dm1.e), c = sar(dp1.m, F - dp1.e), d = sar(dp2.m, F - dp2.e);
+  q.T0 = c - 2 * b + a, q.T1 = d - 2 * c + b;
+  q.t0 = nm_of(q.T0), q.t1 = nm_of(q.T1);
+  q.N0 = sm_norm(q.g.W0, q.g.n0), q.N1 = sm_norm(q.g.W1, q.g.n1), q.N2 = sm_norm(q.g.W2, q.g.n2);
+  q.v0a = limbs(v0.a), q.v0b = limbs(v0.b), q.v1b = limbs(v1.a), q.v1c = limbs(v1.b), q.v2c = limbs(v2.a), q.v2d = limbs(v2.b);
+  q.k0 = v0.k, q.k1 = v1.k, q.k2 = v2.k, q.F = F;
+  return q;
+}
+
+// o[0..3] = dc/d(a, b, c, d) of the right-biased (right) or left-biased side.  One code copy for both
+// (inlined twice and interleaved they take more registers than two blocks an SM leave).
+JS_HD void weno_grad_side(const GradCell& q, bool right, double o[4]) {
+  constexpr int CF = 56;
+  const Wgt& g = q.g;
+  const s64 c0 = (right ? 3 : 1) * g.w0, c1 = 6 * g.w1, c2 = (right ? 1 : 3) * g.w2;
+  const u64 den = (u64)(c0 + c1 + c2);
+  const int lz = clz32(hi32(den));
+  const u64 r = recip_top(den << lz);
+  const Limb rl = limbs((s64)r);
+  // om_k 2^CF
+  const s64 o0 = sar(mul62(limbs(c0), rl), 7 - lz), o1 = sar(mul62(limbs(c1), rl), 7 - lz), o2 = sar(mul62(limbs(c2), rl), 7 - lz);
+  // products of two weights, with their linear weights' product as 3 or 9 times a power of two
+  const u64 r4 = r << 2;
+  const u64 q0 = mul_top(q.N0.m, r4), q1 = mul_top(q.N1.m, r4), q2 = mul_top(q.N2.m, r4);
+  const u64 P01 = mul_top(q0, q1), P02 = mul_top(q0, q2), P12 = mul_top(q1, q2);
+  const s64 K01 = right ? (s64)(9 * (P01 >> 6)) : (s64)(3 * (P01 >> 4)), K02 = (s64)(3 * (P02 >> 4)),
+            K12 = right ? (s64)(3 * (P12 >> 4)) : (s64)(9 * (P12 >> 6));
+  // e_0 - e_1 = -2 T_0 (left), T_0 (right); e_1 - e_2 = T_1, -2 T_1; e_0 - e_2 their sum
+  const Nm t02 = nm_of(right ? q.T0 - 2 * q.T1 : q.T1 - 2 * q.T0);
+  const s64 E01 = right ? q.t0.m : -q.t0.m, E12 = right ? -q.t1.m : q.t1.m;
+  const int m0 = 2 * g.n0 - q.N0.x, m1 = 2 * g.n1 - q.N1.x, m2 = 2 * g.n2 - q.N2.x;  // n_k + lz_k
+  const int f = right ? 1 : 0;
+  const int h01 = m0 + m1 + q.t0.l - (2 + f), h02 = m0 + m2 + t02.l, h12 = m1 + m2 + q.t1.l - (3 - f);
+  const int nu = imin(imin(h01, h02), h12);
+  const s64 z01 = sar(mul62(limbs(K01), limbs(E01)), h01 - nu), z02 = sar(mul62(limbs(K02), limbs(t02.m)), h02 - nu),
+            z12 = sar(mul62(limbs(K12), limbs(E12)), h12 - nu);
+  const Limb Z0 = limbs(z01 + z02), Z1 = limbs(z12 - z01), Z2 = limbs(-z02 - z12);
+  // 4 Z V on the scale 2^-CF: Z 2^(4 + 2 lz - 2 up - nu + F - 1081), V 2^(960 + k), product >> 62
+  const int sh = -(4 + 2 * lz - 2 * g.up - nu + q.F - 1081) - 1024 - CF;
+  const s64 x0a = scale_down(mul62(Z0, q.v0a), sh - q.k0), x0b = scale_down(mul62(Z0, q.v0b), sh - q.k0);
+  const s64 x1b = scale_down(mul62(Z1, q.v1b), sh - q.k1), x1c = scale_down(mul62(Z1, q.v1c), sh - q.k1);
+  const s64 x2c = scale_down(mul62(Z2, q.v2c), sh - q.k2), x2d = scale_down(mul62(Z2, q.v2d), sh - q.k2);
+  const s64 ga = right ? o0 : -2 * o0, gb = right ? -4 * o0 - 2 * o1 : 5 * o0 + o1,
+            gc = right ? -o1 - 5 * o2 : 2 * o1 + 4 * o2, gd = right ? 2 * o2 : -o2;
+  o[0] = fix_to_double(ga - x0a, 1086 - CF);
+  o[1] = fix_to_double(gb - x0b - x1b, 1086 - CF);
+  o[2] = fix_to_double(gc - x1c - x2c, 1086 - CF);
+  o[3] = fix_to_double(gd - x2d, 1086 - CF);
 }
 
 }  // namespace js
