@@ -3,11 +3,11 @@
 // step of Fig. 1(d)).
 //
 // One stage VJP, given the adjoint of the stage output and the filled stage state X:
-//   tile      per tile of the padded array: lambda' = b dt Ubar_next on fluid cells (0
-//             elsewhere), identity and carry terms, Ubar_0 += a Ubar_next; primitives; per line
-//             WENO5 forward, HLLC and viscous forward and reverse per face with
-//             Fbar = (lambda'_right - lambda'_left)/h, WENO5 reverse; Ubar(X) = the sum through
-//             (dprim/dX)^T (+ nu * lap of lambda')
+//   lines     per 28 cells of every x and y line: primitives, WENO5 forward, HLLC and viscous forward
+//             and reverse per face with Fbar = (lambda'_right - lambda'_left)/h, lambda' = b dt
+//             Ubar_next on fluid cells (0 elsewhere), WENO5 reverse: primitive adjoints
+//   cells     Ubar(X) = identity and carry terms + the lines' sum through (dprim/dX)^T (+ nu * lap
+//             of lambda'); Ubar_0 += a Ubar_next
 //   bcT       transposed halo fill (y sides, then x sides), written as gathers;
 //             inflow halos accumulate into the inflow-state gradient
 //   ibT       transposed immersed-boundary fill: ghost adjoint -> image-point adjoint ->
@@ -17,7 +17,7 @@
 // parameter gradient reduced in a fixed order by one block at the end of the stage), so the
 // reverse pass gives the same bits on every run.
 // With the neural flux on, its reverse runs first, on primitives and lambda' in memory, and the
-// tiles add its face-state adjoints to their own.
+// lines add its face-state adjoints to their own.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,16 +30,23 @@ namespace js {
 // =======================================================================================
 // per-grid launches
 // =======================================================================================
-// A block of 8 warps per tile (3 lines a warp in each direction), two blocks an SM by shared memory.
-// Bound by the FP64 pipe (about 190 FP64 instructions per line cell, 24 of 32 lanes kept) with the
-// integer WENO5 forward and reverse beside it.
+// x line blocks, then y line blocks.  Bound by the FP64 pipe (about 200 FP64 instructions per lane
+// and direction) with the integer WENO5 forward and reverse beside it; 16 warps an SM at 128 registers.
 template <bool VISC>
-__global__ void __launch_bounds__(32 * ADJ_WARPS, 2)
-adj_tile_kernel(AdjArgs a, const double* __restrict__ Unext, double* __restrict__ Uacc, double ra, double rb, double dt,
-                int rhs_mode) {
-  extern __shared__ double smem[];
-  adj_tile<VISC>(a, Unext, Uacc, ra, rb, dt, rhs_mode, blockIdx.x, blockIdx.y, smem,
-                 ((long long)blockIdx.y * gridDim.x + blockIdx.x) * ADJ_WARPS);
+__global__ void __launch_bounds__(32 * ADJ_LINES, 2)
+adj_lines_kernel(AdjArgs a, const double* __restrict__ Unext, double bdt, int bx) {
+  __shared__ double smem[8 * AP];
+  const int b = blockIdx.x;
+  adj_lines<VISC>(a, Unext, bdt, b < bx ? 0 : 1, b < bx ? b : b - bx, smem, (long long)b * ADJ_LINES);
+}
+
+template <bool VISC>
+__global__ void __launch_bounds__(256) adj_cells_kernel(AdjArgs a, const double* __restrict__ Unext,
+                                                        double* __restrict__ Uacc, double ra, double rb, double bdt,
+                                                        int rhs_mode) {
+  double gb = 0.0, nb = 0.0;
+  adj_cell<VISC>(a, Unext, Uacc, ra, rb, bdt, rhs_mode, (long long)blockIdx.x * blockDim.x + threadIdx.x, gb, nb);
+  warp_partials(a.pp, global_warp(), gb, 0.0, 0.0, nb);
 }
 
 // primitives of every padded cell and lambda' = bdt Unext on fluid cells (the neural flux's reverse)
@@ -101,26 +108,14 @@ __global__ void adj_unpack_add_kernel(const double* __restrict__ P, const double
 namespace {
 unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 unsigned ib_blocks(int n) { return n > 0 ? blocks_for(n, 128) : 0; }
-
-template <bool VISC>
-cudaError_t launch_tiles(const AdjArgs& a, const double* Unext, double* Uacc, double ra, double rb, double dt,
-                         bool rhs_mode, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(adj_tile_kernel<VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)adj_smem<VISC>());
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  const dim3 grid(adj_tiles_x(a.lay), adj_tiles_y(a.lay));
-  adj_tile_kernel<VISC><<<grid, 32 * ADJ_WARPS, adj_smem<VISC>(), s>>>(a, Unext, Uacc, ra, rb, dt, rhs_mode ? 1 : 0);
-  return cudaGetLastError();
-}
 }  // namespace
 
+long long adj_strip_doubles(const Lay& L) { return strip_size(L, 0) + strip_size(L, 1); }
+
 long long adj_ppart_doubles(const Lay& L, int n_ghost, int n_src, long long nn_blocks) {
-  // warps: the tiles, the neural image reverse (256 threads a block), IB (128)
-  const long long warps = (long long)ADJ_WARPS * adj_tiles_x(L) * adj_tiles_y(L) + 8 * nn_blocks +
+  // warps: the line blocks, the neural image reverse and the cells (256 threads a block), IB (128)
+  const long long warps = (long long)ADJ_LINES * (adj_blocks(L, 0) + adj_blocks(L, 1)) + 8 * nn_blocks +
+                          8 * (long long)blocks_for(L.plane, 256) +
                           4 * (long long)(ib_blocks(n_ghost) + ib_blocks(n_src));
   return 4 * warps;
 }
@@ -151,11 +146,18 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
   } else {
     a.fadj = nullptr;
   }
-  a.pp = slice((long long)ADJ_WARPS * adj_tiles_x(L) * adj_tiles_y(L));
-  e = a.visc ? launch_tiles<true>(a, Unext, Uacc, ra, rb, dt, rhs_mode, s)
-             : launch_tiles<false>(a, Unext, Uacc, ra, rb, dt, rhs_mode, s);
-  if (e != cudaSuccess) return e;
-  ++n;
+  const double bdt = rhs_mode ? 1.0 : rb * dt;
+  const int bx = adj_blocks(L, 0), nb = bx + adj_blocks(L, 1);
+  a.pp = slice((long long)ADJ_LINES * nb);
+  if (a.visc) adj_lines_kernel<true><<<nb, 32 * ADJ_LINES, 0, s>>>(a, Unext, bdt, bx);
+  else adj_lines_kernel<false><<<nb, 32 * ADJ_LINES, 0, s>>>(a, Unext, bdt, bx);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const unsigned gp = blocks_for(L.plane, 256);
+  a.pp = slice(8LL * gp);
+  if (a.visc) adj_cells_kernel<true><<<gp, 256, 0, s>>>(a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
+  else adj_cells_kernel<false><<<gp, 256, 0, s>>>(a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  n += 2;
   const bool two_d = L.ny > 1;
   a.pp = nullptr;
   const int tmax = std::max(L.nx + 6, L.ny);

@@ -46,304 +46,315 @@ __device__ __forceinline__ long long face_id(const AdjArgs& a, int dir, int k, i
 }
 
 // =======================================================================================
-// Reverse of one stage on one tile of the padded array: given the adjoint Unext of the stage
-// output and the filled stage state X,
+// Reverse of one stage, given the adjoint Unext of the stage output and the filled stage state X:
 //   lambda' = b dt Unext on fluid cells (0 elsewhere), U^n part Uacc += a Unext,
 //   Ub(X) = identity and carry terms + (dprim/dX)^T (reverse of the x and y fluxes) + nu lap(lambda')
-// in one pass: primitives and lambda' of the tile and its halo in shared memory, then per line
-// (a warp each, a lane per cell, as in the stage kernel) WENO5 forward, HLLC and viscous forward and
-// reverse per face, WENO5 reverse.  Of the 32 cells of lanes 0..31 the differences serve WENO5 of
-// lanes 1..30, these the faces at i+1/2 of lanes 1..29, these the WENO5 reverse of lanes 2..29 and
-// these the primitive adjoints of lanes 4..27: the 24 outputs.  Nothing is stored between: the
-// WENO5 internals, face adjoints and segment sums that separate passes kept in memory (1.3 KB a
-// cell) are recomputed in integer arithmetic beside the FP64 pipe or passed by shuffles.
+// in two launches: lines (the reverse of the fluxes of every x and y line, to primitive adjoints in
+// memory) and cells (their sum through the primitive map).
+//
+// A warp takes 28 cells of one line, a lane one cell, as in the stage kernel: WENO5 forward, HLLC
+// and viscous forward and reverse per face, WENO5 reverse.  Lanes 0..31 hold the cells i0 - 2 ..
+// i0 + 29; the differences serve WENO5 of lanes 1..30, these the faces at i+1/2 of lanes 1..29,
+// these the WENO5 reverse of lanes 2..29, whose 28 cells send primitive adjoints to all 32: those of
+// the outer two on either side go to strips that the cell launch adds to the neighbouring warps'
+// sums.  28 of 32 lanes' work is kept (24 when a warp formed complete sums alone).
+// Nothing else is stored between forward and reverse: the WENO5 internals, face adjoints and segment
+// sums that separate passes kept in memory (1.3 KB a cell) are recomputed in integer arithmetic
+// beside the FP64 pipe or passed by shuffles.  Lines are independent, so that a grid of a few
+// thousand lines fills the GPU (a 24x24-tile kernel of the same arithmetic took 234 us a stage at
+// 250x190, six lines in turn per warp).
 // Every sum has a fixed order, so the reverse pass gives the same bits on every run.
 // =======================================================================================
-constexpr int AB = 34;              // box of the tile: outputs at 5 .. 28
-constexpr int AP = AB * AB;
-constexpr int AQ = ADJ_TILE + 1;    // row pitch of the accumulator planes
-constexpr int AA = ADJ_TILE * AQ;
-constexpr int AS = (ADJ_TILE + 2) * AQ;  // tangential terms: lines -1 .. 24
-// doubles of shared memory: 4 planes of primitives, 4 of lambda', accumulators (5 viscous), 2 planes
-// of tangential terms (viscous)
-template <bool VISC>
-__host__ __device__ constexpr size_t adj_smem() {
-  return sizeof(double) * (size_t)(8 * AP + (VISC ? 5 * AA + 2 * AS : 4 * AA));
+constexpr int AB = 34;                   // positions of a line's box: lane l at l + 1
+constexpr int AL = ADJ_LINES + 2;        // lines of a block's box: its own and one on either side
+constexpr int AP = AB * AL;              // plane of the box, [line][position] in both directions
+
+// line blocks of a direction: groups of ADJ_LINES lines x chunks of 28 cells (-1 .. n) along them
+__host__ __device__ inline int adj_chunks(int n) { return (n + 2 + ADJ_CHUNK - 1) / ADJ_CHUNK; }
+__host__ __device__ inline int adj_groups(int nline) { return (nline + ADJ_LINES - 1) / ADJ_LINES; }
+__host__ __device__ inline int adj_blocks(const Lay& L, int dir) {
+  return dir == 0 ? adj_groups(L.ny) * adj_chunks(L.nx) : L.ny > 1 ? adj_groups(L.nx) * adj_chunks(L.ny) : 0;
+}
+// strips of a direction: [chunk][variable (5)][4 outer cells][line]
+__host__ __device__ inline long long strip_size(const Lay& L, int dir) {
+  return dir == 0 ? 20LL * adj_chunks(L.nx) * L.ny : L.ny > 1 ? 20LL * adj_chunks(L.ny) * L.nx : 0;
+}
+__device__ __forceinline__ double* strip(const AdjArgs& a, int dir, int chunk, int c, int e, int line) {
+  const int nline = dir == 0 ? a.lay.ny : a.lay.nx;
+  return a.strips + (dir == 0 ? 0 : strip_size(a.lay, 0)) + ((long long)(chunk * 5 + c) * 4 + e) * nline + line;
 }
 
-// the reverse of one line at the lane's cell (q: primitives, l: lambda'; neighbours at multiples of
-// st, across the line of ts).  f: number of the face at i+1/2 (faces 0 .. n exist), own: the lane's
-// face counts for the parameter gradient, out(c, v) receives the adjoint of primitive c (lanes
-// 4..27), tang(n, t) the cell's tangential terms of its two faces (VISC, 2D).
-template <bool VISC, bool HAS_T, class Nn, class Out, class Tang>
-__device__ __forceinline__ void adj_line(const double* q, const double* l, int st, int ts, int pn, int f, int n,
-                                         const Gas& g, const ViscC& vc, double invh, bool own, double& gs1,
-                                         double& gs2, double& vmu, double& vk, Nn nn, Out out, Tang tang) {
-  const int lane = threadIdx.x & 31;
-  const bool inner = lane - 1u < 30u;
-  const int pt = 3 - pn;
-  const bool face = lane >= 1 && lane <= 29 && f >= 0 && f <= n;
-  double L[4], R[4];
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    const int c = (k == 1) ? pn : (k == 2) ? pt : k;
-    double Lf, Rf;
-    weno_lane(q + c * AP, st, k == 0 || k == 3, inner, Lf, Rf);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      L[m] = (k == m) ? Lf : L[m];
-      R[m] = (k == m) ? Rf : R[m];
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < 4; ++m) R[m] = __shfl_down_sync(0xffffffffu, R[m], 1);
-  const double* un = q + pn * AP;
-  const double* ut = q + pt * AP;
-  const bool fallback = !(positive(L[0]) && positive(L[3]) && positive(R[0]) && positive(R[3]));
-  if (fallback) {
-    L[0] = q[0], L[1] = un[0], L[2] = ut[0], L[3] = q[3 * AP];
-    R[0] = q[st], R[1] = un[st], R[2] = ut[st], R[3] = q[3 * AP + st];
-  }
-  double Fb[4];
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const double* lm = l + (m == 1 ? pn : m == 2 ? pt : m) * AP;
-    Fb[m] = (lm[st] - lm[0]) * invh;
-  }
-  double bL[4], bR[4], s1 = 0.0, s2 = 0.0;
-  hllc_vjp(L, R, g, Fb, bL, bR, s1, s2);
-  if (own && face) {
-    gs1 += s1;
-    gs2 += s2;
-  }
-  // adjoints that go straight to the face's cells: its left cell (dl) and its right cell (dr)
-  double dl[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, dr[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    dl[m] = fallback && face ? bL[m] : 0.0;
-    dr[m] = fallback && face ? bR[m] : 0.0;
-    bL[m] = fallback || !face ? 0.0 : bL[m];
-    bR[m] = fallback || !face ? 0.0 : bR[m];
-  }
-  nn(face, bL, bR);
-  bool straight = __any_sync(0xffffffffu, fallback && face);
-  if (VISC) {
-    // F[n] -= tnn; F[t] -= tnt; F[3] -= 0.5 (sbn tnn + sbt tnt) + ck dT
-    const double Tc = q[3 * AP] * recip(q[0]);
-    const double dT = __shfl_down_sync(0xffffffffu, Tc, 1) - Tc;
-    const double ua = un[0], ub = un[st], ta = ut[0], tb = ut[st];
-    const double dun = ub - ua, dut = tb - ta;
-    double tnn, tnt;
-    if (HAS_T) {
-      const double sun = (un[ts] - un[-ts]) + (un[st + ts] - un[st - ts]);
-      const double sut = (ut[ts] - ut[-ts]) + (ut[st + ts] - ut[st - ts]);
-      tnn = fma(vc.c43n, dun, -vc.c23t * sut);
-      tnt = fma(vc.cn, dut, vc.ct * sun);
-    } else {
-      tnn = vc.c43n * dun;
-      tnt = vc.cn * dut;
-    }
-    const double h3 = 0.5 * Fb[3];
-    const double btnn = fma(-h3, ua + ub, -Fb[1]), btnt = fma(-h3, ta + tb, -Fb[2]);
-    const double bck = -Fb[3] * dT, bdT = -Fb[3] * vc.ck;
-    const double bn = -h3 * tnn, bt = -h3 * tnt, bdun = vc.c43n * btnn, bdut = vc.cn * btnt;
-    if (face) {
-      dl[1] += bn - bdun;
-      dr[1] += bn + bdun;
-      dl[2] += bt - bdut;
-      dr[2] += bt + bdut;
-      dl[4] = -bdT;
-      dr[4] = bdT;
-      if (own) {
-        vmu += fma(btnn, tnn, fma(btnt, tnt, bck * vc.ck));
-        vk += bck * vc.ck;
-      }
-    }
-    if (HAS_T) {
-      // tangential differences: + to the cells one line up, minus to those one line down
-      const double xn = face ? vc.ct * btnt : 0.0, xt = face ? -vc.c23t * btnn : 0.0;
-      tang(xn + __shfl_up_sync(0xffffffffu, xn, 1), xt + __shfl_up_sync(0xffffffffu, xt, 1));
-    }
-    straight = true;
-  }
-  if (straight) {
-#pragma unroll
-    for (int m = 0; m < (VISC ? 5 : 4); ++m)
-      out((m == 1) ? pn : (m == 2) ? pt : m, dl[m] + __shfl_up_sync(0xffffffffu, dr[m], 1));
-  }
-#pragma unroll
-  for (int m = 0; m < 4; ++m) bR[m] = __shfl_up_sync(0xffffffffu, bR[m], 1);  // of the face at i-1/2
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    const int c = (k == 1) ? pn : (k == 2) ? pt : k;
-    const double Lb = (k == 0) ? bL[0] : (k == 1) ? bL[1] : (k == 2) ? bL[2] : bL[3];
-    const double Rb = (k == 0) ? bR[0] : (k == 1) ? bR[1] : (k == 2) ? bR[2] : bR[3];
-    double w[4];
-    weno_grad_lane(q + c * AP, st, k == 0 || k == 3, inner, Lb, Rb, w);
-    // adjoint of d_{i+1/2}: its share in the cells i-1 .. i+2
-    const double t = (w[2] + __shfl_up_sync(0xffffffffu, w[3], 1)) +
-                     (__shfl_down_sync(0xffffffffu, w[1], 1) + __shfl_down_sync(0xffffffffu, w[0], 2));
-    out(c, fma(SIXTH, __shfl_up_sync(0xffffffffu, t, 1) - t, Lb + Rb));
-  }
-}
-
-// tile (bx, by) of the padded array; slot0: warp slot of the tile's partials of pbar[0..3]
+// block `item` of direction dir: ADJ_LINES warps, a line each; slot0: warp slot of the block's
+// partials of pbar[0..3]; smem: 8 AP doubles
 template <bool VISC>
-__device__ __forceinline__ void adj_tile(const AdjArgs& a, const double* __restrict__ Unext, double* __restrict__ Uacc,
-                                         double ra, double rb, double dt, int rhs_mode, int bx, int by, double* smem,
-                                         long long slot0) {
+__device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __restrict__ Unext, double bdt, int dir,
+                                          int item, double* smem, long long slot0) {
   const Lay& L = a.lay;
-  double* sq = smem;
-  double* sl = smem + 4 * AP;
-  double* acc = smem + 8 * AP;
-  double* tan = acc + 5 * AA;  // VISC
+  double* sq = smem;           // rho, u, v, p
+  double* sl = smem + 4 * AP;  // Unext on fluid cells
   const Gas g = a.gas;
-  const int W = L.nx + 6;
-  const int ox = bx * ADJ_TILE, oy = by * ADJ_TILE;  // padded coordinates of the first output
-  const double bdt = rhs_mode ? 1.0 : rb * dt;
-  for (int e = threadIdx.x; e < AP; e += blockDim.x) {
-    const int row = e / AB, col = e - row * AB;
-    const int gx = ox - 5 + col, gy = oy - 5 + row;
-    const bool in = gx >= 0 && gx < W && gy >= 0 && gy < L.H;
-    const long long t = in ? (long long)gy * L.pitch + gx : 0;
-    const double r = a.X[t], mx = a.X[L.plane + t], my = a.X[2 * L.plane + t], E = a.X[3 * L.plane + t];
-    double u = 0.0, v = 0.0, p = 1.0, T;
-    if (in) cons_to_prim(r, mx, my, E, g, u, v, p, T);
-    sq[e] = in ? r : 1.0;
-    sq[AP + e] = u;
-    sq[2 * AP + e] = v;
-    sq[3 * AP + e] = p;
-    const int i = gx - 3, j = gy - L.gy;
+  const int nline = dir == 0 ? L.ny : L.nx, ncell = dir == 0 ? L.nx : L.ny;
+  const int nch = adj_chunks(ncell);
+  const int chunk = item % nch, line0 = item / nch * ADJ_LINES;
+  const int i0 = -1 + ADJ_CHUNK * chunk;  // first reversed cell
+  const int gyl = dir == 0 ? L.gy : 3, gyc = dir == 0 ? 3 : L.gy;  // ghost layers across / along the line
+  for (int e = threadIdx.x; e < AP; e += 32 * ADJ_LINES) {
+    // consecutive threads along x in both directions
+    const int ln = dir == 0 ? e / AB : e % AL, pos = dir == 0 ? e % AB : e / AL;
+    const int line = line0 - 1 + ln, cell = i0 - 3 + pos;
+    const bool in = line >= -gyl && line < nline + gyl && cell >= -gyc && cell < ncell + gyc;
+    const int i = dir == 0 ? cell : line, j = dir == 0 ? line : cell;
+    const long long t = in ? L.idx(i, j) : 0;
+    double r = 1.0, u = 0.0, v = 0.0, p = 1.0, T;
+    if (in) {
+      r = a.X[t];
+      cons_to_prim(r, a.X[L.plane + t], a.X[2 * L.plane + t], a.X[3 * L.plane + t], g, u, v, p, T);
+    }
+    const int o = ln * AB + pos;
+    sq[o] = r;
+    sq[AP + o] = u;
+    sq[2 * AP + o] = v;
+    sq[3 * AP + o] = p;
     const bool fluid = i >= 0 && i < L.nx && j >= 0 && j < L.ny && (a.tag == nullptr || a.tag[(long long)j * L.nx + i] == 0);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) sl[c * AP + e] = fluid ? bdt * Unext[c * L.plane + t] : 0.0;
+    for (int c = 0; c < 4; ++c) sl[c * AP + o] = fluid ? Unext[c * L.plane + t] : 0.0;
   }
-  for (int e = threadIdx.x; e < (VISC ? 5 : 4) * AA; e += blockDim.x) acc[e] = 0.0;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  const int k = lane - 4;  // the lane's cell: output k of the line
-  const bool own = k >= 0 && k < ADJ_TILE;
-  double gs1 = 0.0, gs2 = 0.0, vmu = 0.0, vk = 0.0, gb = 0.0, nb = 0.0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int line = line0 + warp;
+  double gs1 = 0.0, gs2 = 0.0, vmu = 0.0, vk = 0.0;
+  if (line < nline) {
+    const ViscC& vc = dir == 0 ? a.vx : a.vy;
+    const double fl = bdt * (dir == 0 ? a.inv_dx : a.inv_dy);  // lambda' differences over h
+    const int pn = dir + 1, pt = 2 - dir;
+    const bool inner = lane - 1u < 30u;
+    const double* q = sq + (warp + 1) * AB + lane + 1;
+    const double* l = sl + (warp + 1) * AB + lane + 1;
+    const double* un = q + pn * AP;
+    const double* ut = q + pt * AP;
+    const int cell = i0 - 2 + lane, f = cell + 1;  // the lane's cell and its face at i+1/2
+    const bool face = inner && lane < 30 && f >= 0 && f <= ncell;
+    const bool own = lane >= 2;  // (with face) the warp's faces: lanes 2..29
+    const bool rev = lane >= 2 && lane < 30;
+    double bL[4], bR[4], dl[VISC ? 5 : 4], dr[VISC ? 5 : 4];
+    bool straight;
+    {
+      double Lq[4], Rq[4];
 #pragma unroll 1
-  for (int dir = 0; dir < (a.two_d ? 2 : 1); ++dir) {
-    const int st = dir == 0 ? 1 : AB, ts = dir == 0 ? AB : 1;
-    const int k0 = (dir == 0 ? ox - 3 : oy - L.gy), l0 = (dir == 0 ? oy - L.gy : ox - 3);  // grid cell of output 0
-    const int nline = dir == 0 ? L.ny : L.nx, ncell = dir == 0 ? L.nx : L.ny;
-    const ViscC vc = dir == 0 ? a.vx : a.vy;
-    const double invh = dir == 0 ? a.inv_dx : a.inv_dy;
-    const int pn = dir + 1;
-    // with tangential terms the lines next to the tile are needed for those alone
-    const int edge = VISC && a.two_d ? 1 : 0;
-#pragma unroll 1
-    for (int ln = warp - edge; ln < ADJ_TILE + edge; ln += nwarp) {
-      const double* q = sq + (ln + 5) * ts + (k + 5) * st;
-      const double* lm = sl + (ln + 5) * ts + (k + 5) * st;
-      const int line = l0 + ln, f = k0 + k + 1;
-      if (VISC && a.two_d && (ln < 0 || ln >= ADJ_TILE || line < 0 || line >= nline)) {
-        // tangential terms only (zero past the grid's lines)
-        double xn = 0.0, xt = 0.0;
-        if (line >= 0 && line < nline && lane >= 1 && lane <= 29 && f >= 0 && f <= ncell) {
-          const double* un = q + pn * AP;
-          const double* ut = q + (3 - pn) * AP;
-          const double h3 = 0.5 * ((lm[3 * AP + st] - lm[3 * AP]) * invh);
-          const double Fn = (lm[pn * AP + st] - lm[pn * AP]) * invh, Ft = (lm[(3 - pn) * AP + st] - lm[(3 - pn) * AP]) * invh;
-          xn = vc.ct * fma(-h3, ut[0] + ut[st], -Ft);
-          xt = -vc.c23t * fma(-h3, un[0] + un[st], -Fn);
-        }
-        const double xn1 = __shfl_up_sync(0xffffffffu, xn, 1), xt1 = __shfl_up_sync(0xffffffffu, xt, 1);
-        if (own) {
-          tan[(ln + 1) * AQ + k] = xn + xn1;
-          tan[AS + (ln + 1) * AQ + k] = xt + xt1;
-        }
-        continue;
-      }
-      if (line < 0 || line >= nline) continue;
-      double* o = acc + (dir == 0 ? ln * AQ + k : k * AQ + ln);
-      auto nn = [&](bool face, double bL[4], double bR[4]) {
-        if (a.fadj == nullptr || !face) return;
-        const long long si = face_id(a, dir, f, line);
-        const double* fa = a.fadj + (long long)(dir * 8) * a.splane + si;
+      for (int k = 0; k < 4; ++k) {
+        const int c = (k == 1) ? pn : (k == 2) ? pt : k;
+        double Lf, Rf;
+        weno_lane(q + c * AP, 1, k == 0 || k == 3, inner, Lf, Rf);
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-          const int c = (m == 1) ? pn : (m == 2) ? 3 - pn : m;
-          bL[m] += fa[c * a.splane];
-          bR[m] += fa[(4 + c) * a.splane];
+          Lq[m] = (k == m) ? Lf : Lq[m];
+          Rq[m] = (k == m) ? Rf : Rq[m];
         }
-      };
-      auto out = [&](int c, double v) {
-        if (own) o[c * AA] += v;
-      };
-      auto tang = [&](double xn, double xt) {
-        if (own) {
-          tan[(ln + 1) * AQ + k] = xn;
-          tan[AS + (ln + 1) * AQ + k] = xt;
-        }
-      };
-      if (a.two_d) adj_line<VISC, true>(q, lm, st, ts, pn, f, ncell, g, vc, invh, own, gs1, gs2, vmu, vk, nn, out, tang);
-      else adj_line<VISC, false>(q, lm, st, ts, pn, f, ncell, g, vc, invh, own, gs1, gs2, vmu, vk, nn, out, tang);
-    }
-    __syncthreads();
-    if (VISC && a.two_d) {
-      // tangential terms: from the line below and, negative, from the line above
-      for (int e = threadIdx.x; e < ADJ_TILE * ADJ_TILE; e += blockDim.x) {
-        const int ln = e / ADJ_TILE, kk = e - ln * ADJ_TILE;
-        double* o = acc + (dir == 0 ? ln * AQ + kk : kk * AQ + ln);
-        o[pn * AA] += tan[ln * AQ + kk] - tan[(ln + 2) * AQ + kk];
-        o[(3 - pn) * AA] += tan[AS + ln * AQ + kk] - tan[AS + (ln + 2) * AQ + kk];
       }
-      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < 4; ++m) Rq[m] = __shfl_down_sync(0xffffffffu, Rq[m], 1);
+      const bool fallback = !(positive(Lq[0]) && positive(Lq[3]) && positive(Rq[0]) && positive(Rq[3]));
+      if (fallback) {
+        Lq[0] = q[0], Lq[1] = un[0], Lq[2] = ut[0], Lq[3] = q[3 * AP];
+        Rq[0] = q[1], Rq[1] = un[1], Rq[2] = ut[1], Rq[3] = q[3 * AP + 1];
+      }
+      double Fb[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const double* lm = l + (m == 1 ? pn : m == 2 ? pt : m) * AP;
+        Fb[m] = (lm[1] - lm[0]) * fl;
+      }
+      double s1 = 0.0, s2 = 0.0;
+      hllc_vjp(Lq, Rq, g, Fb, bL, bR, s1, s2);
+      gs1 = own && face ? s1 : 0.0;
+      gs2 = own && face ? s2 : 0.0;
+      // adjoints that go straight to the cells of the warp's faces: left cell dl, right cell dr
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        dl[m] = fallback && face && own ? bL[m] : 0.0;
+        dr[m] = fallback && face && own ? bR[m] : 0.0;
+        bL[m] = fallback || !face ? 0.0 : bL[m];
+        bR[m] = fallback || !face ? 0.0 : bR[m];
+      }
+      straight = VISC || __any_sync(0xffffffffu, fallback && face);
+      if (VISC) {
+        // F[n] -= tnn; F[t] -= tnt; F[3] -= 0.5 (sbn tnn + sbt tnt) + ck dT
+        const double Tc = q[3 * AP] * recip(q[0]);
+        const double dT = __shfl_down_sync(0xffffffffu, Tc, 1) - Tc;
+        const double ua = un[0], ub = un[1], ta = ut[0], tb = ut[1];
+        const double dun = ub - ua, dut = tb - ta;
+        double tnn, tnt;
+        if (a.two_d) {
+          const double sun = (un[AB] - un[-AB]) + (un[AB + 1] - un[1 - AB]);
+          const double sut = (ut[AB] - ut[-AB]) + (ut[AB + 1] - ut[1 - AB]);
+          tnn = fma(vc.c43n, dun, -vc.c23t * sut);
+          tnt = fma(vc.cn, dut, vc.ct * sun);
+        } else {
+          tnn = vc.c43n * dun;
+          tnt = vc.cn * dut;
+        }
+        const double h3 = 0.5 * Fb[3];
+        const double btnn = fma(-h3, ua + ub, -Fb[1]), btnt = fma(-h3, ta + tb, -Fb[2]);
+        const double bT = Fb[3] * vc.ck, ckk = -bT * dT;
+        const double bdun = vc.c43n * btnn, bdut = vc.cn * btnt;
+        if (own && face) {
+          dl[1] += fma(-h3, tnn, -bdun);
+          dr[1] += fma(-h3, tnn, bdun);
+          dl[2] += fma(-h3, tnt, -bdut);
+          dr[2] += fma(-h3, tnt, bdut);
+          vmu = fma(btnn, tnn, fma(btnt, tnt, ckk));
+          vk = ckk;
+        }
+        dl[VISC ? 4 : 0] = own && face ? bT : 0.0;
+        dr[VISC ? 4 : 0] = own && face ? -bT : 0.0;
+        if (a.two_d) {
+          // tangential differences: + to the cells one line up, minus to those one line down; the
+          // cell's sum over its two faces
+          const double xn = face ? vc.ct * btnt : 0.0, xt = face ? -vc.c23t * btnn : 0.0;
+          const double tn = xn + __shfl_up_sync(0xffffffffu, xn, 1), tt = xt + __shfl_up_sync(0xffffffffu, xt, 1);
+          if (rev && cell <= ncell) {
+            double* o = a.tang + (long long)(2 * dir) * L.plane + (dir == 0 ? L.idx(cell, line) : L.idx(line, cell));
+            o[0] = tn;
+            o[L.plane] = tt;
+          }
+        }
+      }
     }
+    if (a.fadj != nullptr && face) {
+      const double* fa = a.fadj + (long long)(dir * 8) * a.splane + face_id(a, dir, f, line);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int c = (m == 1) ? pn : (m == 2) ? pt : m;
+        bL[m] += fa[c * a.splane];
+        bR[m] += fa[(4 + c) * a.splane];
+      }
+    }
+    // the reversed cells' face states: L at i+1/2, R at i-1/2; right cells' straight terms
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const double up = __shfl_up_sync(0xffffffffu, bR[m], 1);
+      bL[m] = rev ? bL[m] : 0.0;
+      bR[m] = rev ? up : 0.0;
+    }
+    if (straight) {
+#pragma unroll
+      for (int m = 0; m < (VISC ? 5 : 4); ++m) {
+        const double up = __shfl_up_sync(0xffffffffu, dr[m], 1);
+        dl[m] += lane > 0 ? up : 0.0;
+      }
+    }
+    // where the lane's sums go: the cell's place, or a strip of the warp
+    const bool in = cell >= -gyc && cell < ncell + gyc;
+    double* qo = rev ? a.Qb + (long long)(dir * 5) * L.plane + (in ? (dir == 0 ? L.idx(cell, line) : L.idx(line, cell)) : 0)
+                     : strip(a, dir, chunk, 0, lane < 2 ? lane : lane - 28, line);
+    const long long qs = rev ? L.plane : 4LL * nline;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+      const int c = (k == 1) ? pn : (k == 2) ? pt : k;
+      const double Lb = (k == 0) ? bL[0] : (k == 1) ? bL[1] : (k == 2) ? bL[2] : bL[3];
+      const double Rb = (k == 0) ? bR[0] : (k == 1) ? bR[1] : (k == 2) ? bR[2] : bR[3];
+      double w[4];
+      weno_grad_lane(q + c * AP, 1, k == 0 || k == 3, inner, Lb, Rb, w);  // 0 where Lb = Rb = 0
+      // adjoint of d_{i+1/2}: its share in the reversed cells i-1 .. i+2
+      const double u3 = __shfl_up_sync(0xffffffffu, w[3], 1);
+      const double t = (w[2] + (lane > 0 ? u3 : 0.0)) +
+                       (__shfl_down_sync(0xffffffffu, w[1], 1) + __shfl_down_sync(0xffffffffu, w[0], 2));
+      const double tm = __shfl_up_sync(0xffffffffu, t, 1);
+      double v = fma(SIXTH, (lane > 0 ? tm : 0.0) - t, Lb + Rb);
+      if (straight) v += (k == 0) ? dl[0] : (k == 1) ? dl[1] : (k == 2) ? dl[2] : dl[3];
+      if (in) qo[c * qs] = v;
+    }
+    if (VISC && in) qo[4 * qs] = dl[VISC ? 4 : 0];
   }
-  // primitive reverse, artificial viscosity, identity terms
-  for (int e = threadIdx.x; e < ADJ_TILE * ADJ_TILE; e += blockDim.x) {
-    const int ty = e / ADJ_TILE, tx = e - ty * ADJ_TILE;
-    const int gx = ox + tx, gy = oy + ty;
-    if (gx >= W || gy >= L.H) continue;
-    const int i = gx - 3, j = gy - L.gy;
-    const long long t = (long long)gy * L.pitch + gx;
-    const int b = (ty + 5) * AB + tx + 5;
-    double qb[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, ub[4];
-#pragma unroll
-    for (int c = 0; c < (VISC ? 5 : 4); ++c) qb[c] = acc[c * AA + ty * AQ + tx];
-    prim_vjp(sq[b], sq[AP + b], sq[2 * AP + b], sq[3 * AP + b], g, qb, ub, gb);
-    const bool interior = i >= 0 && i < L.nx && j >= 0 && j < L.ny;
-    if (a.has_av) {
-      const bool near = i >= -1 && i <= L.nx && j >= (a.two_d ? -1 : 0) && j <= (a.two_d ? L.ny : 0);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const double* lam = sl + c * AP + b;
-        if (near) {
-          double add = a.nu_x * ((lam[-1] - 2.0 * lam[0]) + lam[1]);
-          if (a.two_d) add += a.nu_y * ((lam[-AB] - 2.0 * lam[0]) + lam[AB]);
-          ub[c] += add;
-        }
-        if (interior && lam[0] != 0.0) {
-          const double* X = a.X + c * L.plane;
-          double lap = a.nu_x1 * ((X[t - 1] - 2.0 * X[t]) + X[t + 1]);
-          if (a.two_d) lap += a.nu_y1 * ((X[t - L.pitch] - 2.0 * X[t]) + X[t + L.pitch]);
-          nb += lam[0] * lap;
-        }
-      }
-    }
-    const bool fluid = interior && (a.tag == nullptr || a.tag[(long long)j * L.nx + i] == 0);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const long long o = c * L.plane + t;
-      if (interior && !rhs_mode) {
-        const double un = Unext[o];
-        ub[c] += fluid ? rb * un : un;  // identity on fluid cells, carry on solid and ghost cells
-        if (fluid && ra != 0.0) Uacc[o] += ra * un;
-      }
-      a.Ub[o] = ub[c];
-    }
-  }
-  gb += gs2 / g.gamma - gs1 * g.g1 * g.g1;
+  double gb = gs2 / g.gamma - gs1 * g.g1 * g.g1;
   if (VISC) {
     gb += a.kg * vk;
     vmu *= a.inv_mu;
     vk *= a.kp;
   }
-  warp_partials(a.pp, slot0 + warp, gb, vmu, vk, nb);
+  warp_partials(a.pp, slot0 + warp, gb, vmu, vk, 0.0);
+}
+
+// the line sums of primitive c at padded cell (i, j)
+template <int DIR>
+__device__ __forceinline__ double line_sum(const AdjArgs& a, int c, int i, int j) {
+  const Lay& L = a.lay;
+  const int m = DIR == 0 ? i : j, line = DIR == 0 ? j : i;
+  const int n = DIR == 0 ? L.nx : L.ny, nch = adj_chunks(n);
+  if (m < -1) return *strip(a, DIR, 0, c, m + 3, line);  // cells -3, -2: the first warp's strip
+  const int ch = (m + 1) / ADJ_CHUNK, pos = (m + 1) % ADJ_CHUNK;
+  double v = ch < nch ? a.Qb[(long long)(DIR * 5 + c) * L.plane + L.idx(i, j)] : 0.0;
+  if (pos < 2 && ch > 0) v += *strip(a, DIR, ch - 1, c, 2 + pos, line);
+  if (pos >= ADJ_CHUNK - 2 && ch + 1 < nch) v += *strip(a, DIR, ch + 1, c, pos - (ADJ_CHUNK - 2), line);
+  return v;
+}
+
+// Ub of padded cell t (all four planes); gamma and nu contributions are added to gb, nb
+template <bool VISC>
+__device__ __forceinline__ void adj_cell(const AdjArgs& a, const double* __restrict__ Unext, double* __restrict__ Uacc,
+                                         double ra, double rb, double bdt, int rhs_mode, long long t, double& gb,
+                                         double& nb) {
+  const Lay& L = a.lay;
+  if (t >= L.plane) return;
+  const int col = (int)(t % L.pitch), row = (int)(t / L.pitch);
+  if (col >= L.nx + 6 || row >= L.H) return;
+  const int i = col - 3, j = row - L.gy;
+  const bool xl = j >= 0 && j < L.ny, yl = a.two_d && i >= 0 && i < L.nx;  // on an x / a y line
+  double qb[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, ub[4];
+#pragma unroll
+  for (int c = 0; c < (VISC ? 5 : 4); ++c) {
+    if (xl) qb[c] += line_sum<0>(a, c, i, j);
+    if (yl) qb[c] += line_sum<1>(a, c, i, j);
+  }
+  if (VISC && a.two_d) {
+    // tangential terms: from the line below and, negative, from the line above (cells -1 .. n of them)
+    const double* tx = a.tang;
+    const double* ty = a.tang + 2 * L.plane;
+    if (i >= -1 && i <= L.nx) {
+      if (j - 1 >= 0 && j - 1 < L.ny) qb[1] += tx[t - L.pitch], qb[2] += tx[L.plane + t - L.pitch];
+      if (j + 1 >= 0 && j + 1 < L.ny) qb[1] -= tx[t + L.pitch], qb[2] -= tx[L.plane + t + L.pitch];
+    }
+    if (j >= -1 && j <= L.ny) {
+      if (i - 1 >= 0 && i - 1 < L.nx) qb[2] += ty[t - 1], qb[1] += ty[L.plane + t - 1];
+      if (i + 1 >= 0 && i + 1 < L.nx) qb[2] -= ty[t + 1], qb[1] -= ty[L.plane + t + 1];
+    }
+  }
+  double u, v, p, T;
+  const double r = a.X[t];
+  cons_to_prim(r, a.X[L.plane + t], a.X[2 * L.plane + t], a.X[3 * L.plane + t], a.gas, u, v, p, T);
+  prim_vjp(r, u, v, p, a.gas, qb, ub, gb);
+  auto fluid_at = [&](int x, int y) {
+    return x >= 0 && x < L.nx && y >= 0 && y < L.ny && (a.tag == nullptr || a.tag[(long long)y * L.nx + x] == 0);
+  };
+  const bool interior = i >= 0 && i < L.nx && j >= 0 && j < L.ny, fluid = fluid_at(i, j);
+  if (a.has_av && i >= -1 && i <= L.nx && j >= (a.two_d ? -1 : 0) && j <= (a.two_d ? L.ny : 0)) {
+    const bool xm = fluid_at(i - 1, j), xp = fluid_at(i + 1, j), ym = a.two_d && fluid_at(i, j - 1),
+               yp = a.two_d && fluid_at(i, j + 1);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const double* lp = Unext + c * L.plane + t;
+      const double l0 = fluid ? lp[0] : 0.0;
+      double add = a.nu_x * (((xm ? lp[-1] : 0.0) - 2.0 * l0) + (xp ? lp[1] : 0.0));
+      if (a.two_d) add += a.nu_y * (((ym ? lp[-L.pitch] : 0.0) - 2.0 * l0) + (yp ? lp[L.pitch] : 0.0));
+      ub[c] = fma(bdt, add, ub[c]);
+      if (fluid && l0 != 0.0) {
+        const double* X = a.X + c * L.plane;
+        double lap = a.nu_x1 * ((X[t - 1] - 2.0 * X[t]) + X[t + 1]);
+        if (a.two_d) lap += a.nu_y1 * ((X[t - L.pitch] - 2.0 * X[t]) + X[t + L.pitch]);
+        nb += bdt * l0 * lap;
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const long long o = c * L.plane + t;
+    if (interior && !rhs_mode) {
+      const double un = Unext[o];
+      ub[c] += fluid ? rb * un : un;  // identity on fluid cells, carry on solid and ghost cells
+      if (fluid && ra != 0.0) Uacc[o] += ra * un;
+    }
+    a.Ub[o] = ub[c];
+  }
 }
 
 // =======================================================================================

@@ -32,7 +32,7 @@ namespace js {
 // the per-grid tiles; the forward launch runs 7 warps a block, the reverse launches 8, like the
 // per-grid kernels
 constexpr int BTX = TILE, BTY = TILE;
-constexpr int FNT = 224, BNT = 32 * ADJ_WARPS;
+constexpr int FNT = 224, BNT = 32 * ADJ_LINES;
 
 struct BatchArgs {
   const InstDesc* inst;
@@ -305,9 +305,9 @@ __global__ void __launch_bounds__(FNT, 2) batch_kernel(BatchArgs b) {
 //   pack U_n, lambda_{n+1}; zero Uacc
 //   forward recompute, stages 0 and 1: IB fill | halo fill | stage tiles; IB and halo fill of
 //   the stage-2 input
-//   reverse, stages 2, 1, 0: reverse tiles | transposed y halos (+ the previous stage's part of
-//   the parameter gradient is reduced before the tiles) | transposed x halos | inflow gradient +
-//   transposed IB ghosts | transposed IB sources
+//   reverse, stages 2, 1, 0: lines (the previous stage's part of the parameter gradient is reduced
+//   before them) | cells | transposed y halos | transposed x halos | inflow gradient + transposed
+//   IB ghosts | transposed IB sources
 //   unpack lambda_n (+ the last reduction)
 // The device bodies are those of the per-grid launches (js_adjoint_body.cuh, js_stage.cuh,
 // js_fill.cuh) on the same elements in the same order; the parameter gradient is reduced in a
@@ -334,7 +334,7 @@ struct BatchRevArgs {
   int count;
   const long long* pre;       // [RK_N][count + 1] prefix sums of the padded item counts
   const int* tile0;
-  const int* rtile0;          // prefix sums (count + 1) of the reverse tiles
+  const int* rblock0;         // prefix sums (count + 1) of the reverse line blocks
   RevCall call;
   unsigned* bar;
   int* err;
@@ -372,10 +372,13 @@ __device__ __forceinline__ AdjArgs rev_adj(const InstRev& r, const InstDesc& d, 
 
 // the parameter-gradient slot ranges of one reverse stage of one instance, summed into its pbar
 __device__ __forceinline__ void rev_reduce(const InstRev& r, double* pbar) {
-  const long long off[3] = {0, r.off_g, r.off_s};
-  const long long cnt[3] = {r.w_adj, r.w_g, r.w_s};
-  adj_pbar_reduce_block(r.ppart, off, cnt, 3, pbar);
+  const long long off[4] = {0, r.off_c, r.off_g, r.off_s};
+  const long long cnt[4] = {r.w_lines, r.w_c, r.w_g, r.w_s};
+  adj_pbar_reduce_block(r.ppart, off, cnt, 4, pbar);
 }
+
+// the stage constants of the SSP-RK3 step
+__device__ constexpr double REV_A[3] = {0.0, 0.75, 1.0 / 3.0}, REV_B[3] = {1.0, 0.25, 2.0 / 3.0};
 
 // The phases of one batched reverse step.  Each runs over the work items of all instances with
 // grid-stride loops, so it is correct for any grid; the persistent kernel runs them in order
@@ -386,8 +389,9 @@ enum RevPhase {
   RP_GHOST,         // IB fill of stage input s
   RP_HALO,          // halo fill of stage input s
   RP_STAGE,         // forward recompute of stage s (0, 1)
-  RP_REDUCE,        // the parameter gradient of reverse stage s+1 (before the tiles reuse its slots)
-  RP_TILES,         // reverse tiles of stage s
+  RP_REDUCE,        // the parameter gradient of reverse stage s+1 (before the lines reuse its slots)
+  RP_LINES,         // reverse of stage s: lines
+  RP_CELLS,         // cells
   RP_BCTY,          // transposed y halos
   RP_BCTX,          // transposed x halos
   RP_INFLOW_GHOST,  // inflow-state gradient + transposed IB ghosts
@@ -473,20 +477,32 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     if (s < 2 && call.pbar)
       for (int k = blockIdx.x; k < b.count; k += gridDim.x)
         if (call.pbar[k]) rev_reduce(b.rev[k], call.pbar[k]);
-  } else if constexpr (PH == RP_TILES) {
-    const double ra[3] = {0.0, 0.75, 1.0 / 3.0};
-    const double rb[3] = {1.0, 0.25, 2.0 / 3.0};
-    for (int it = blockIdx.x; it < b.rtile0[b.count]; it += gridDim.x) {
-      const int k = find_inst(b.rtile0, b.count, it);
+  } else if constexpr (PH == RP_LINES) {
+    for (int it = blockIdx.x; it < b.rblock0[b.count]; it += gridDim.x) {
+      const int k = find_inst(b.rblock0, b.count, it);
       const InstDesc& d = b.inst[k];
       const InstRev& r = b.rev[k];
       const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
       const double* src = even ? r.P0 : r.P1;
-      const int t = it - b.rtile0[k], ntx = adj_tiles_x(d.lay);
-      if (d.visc) adj_tile<true>(a, src, r.Uacc, ra[s], rb[s], call.dt[k], 0, t % ntx, t / ntx, smem, (long long)t * ADJ_WARPS);
-      else adj_tile<false>(a, src, r.Uacc, ra[s], rb[s], call.dt[k], 0, t % ntx, t / ntx, smem, (long long)t * ADJ_WARPS);
-      __syncthreads();  // the next tile reuses shared memory
+      const int t = it - b.rblock0[k], bx = adj_blocks(d.lay, 0);
+      const double bdt = REV_B[s] * call.dt[k];
+      if (d.visc) adj_lines<true>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, (long long)t * ADJ_LINES);
+      else adj_lines<false>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, (long long)t * ADJ_LINES);
+      __syncthreads();  // the next block of lines reuses shared memory
     }
+  } else if constexpr (PH == RP_CELLS) {
+    rev_items(b, RK_PLANE, [&](int k, long long t) {
+      if (k < 0) return;
+      const InstDesc& d = b.inst[k];
+      const InstRev& r = b.rev[k];
+      const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
+      const double* src = even ? r.P0 : r.P1;
+      double gb = 0.0, nb = 0.0;
+      const double bdt = REV_B[s] * call.dt[k];
+      if (d.visc) adj_cell<true>(a, src, r.Uacc, REV_A[s], REV_B[s], bdt, 0, t, gb, nb);
+      else adj_cell<false>(a, src, r.Uacc, REV_A[s], REV_B[s], bdt, 0, t, gb, nb);
+      warp_partials(a.pp, r.off_c + (t >> 5), gb, 0.0, 0.0, nb);
+    });
   } else if constexpr (PH == RP_BCTY || PH == RP_BCTX) {
     rev_items(b, PH == RP_BCTY ? RK_BCTY : RK_BCTX, [&](int k, long long t) {
       if (k < 0) return;
@@ -556,7 +572,9 @@ __global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
   for (int s = 2; s >= 0; --s) {
     rev_phase<RP_REDUCE>(b, s, smem);
     if (s < 2 && b.call.pbar && !grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_TILES>(b, s, smem);
+    rev_phase<RP_LINES>(b, s, smem);
+    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
+    rev_phase<RP_CELLS>(b, s, smem);
     if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
     rev_phase<RP_BCTY>(b, s, smem);
     if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
@@ -572,7 +590,7 @@ __global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
 
 // one phase of the reverse step as a kernel of its own (split launch)
 template <int PH>
-__global__ void __launch_bounds__(BNT, PH == RP_STAGE || PH == RP_TILES ? 2 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
+__global__ void __launch_bounds__(BNT, PH == RP_STAGE || PH == RP_LINES ? 2 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
   extern __shared__ double smem[];
   rev_phase<PH>(b, s, smem);
 }
@@ -622,7 +640,7 @@ struct js_batch {
   int rev_blocks = 0;
   int rev_split = 0;                  // 1: one launch per phase (js_batch_set_reverse_launch)
   int rev_pblocks[js::RP_N] = {};     // grid of each phase kernel of the split launch
-  int* d_rtile0 = nullptr;            // prefix sums of the reverse tiles
+  int* d_rblock0 = nullptr;            // prefix sums of the reverse line blocks
   void** d_tab = nullptr;       // call table of js_batch_step_vjp: U_n, lam_np1, lam_n, p_bar x count
   double* d_dt = nullptr;       // its step sizes
   // checkpointed rollout reverse (js_batch_rollout_vjp)
@@ -641,8 +659,9 @@ int js_internal_rev_desc(js_ctx* c, js::InstRev* d);
 
 namespace {
 size_t batch_smem() { return js::StageTile<true>::SMEM; }
-size_t rev_smem() { return std::max(batch_smem(), js::adj_smem<true>()); }
-size_t rev_phase_smem(int ph) { return ph == js::RP_STAGE ? batch_smem() : ph == js::RP_TILES ? js::adj_smem<true>() : 0; }
+constexpr size_t kLineSmem = sizeof(double) * 8 * js::AP;
+size_t rev_smem() { return std::max(batch_smem(), kLineSmem); }
+size_t rev_phase_smem(int ph) { return ph == js::RP_STAGE ? batch_smem() : ph == js::RP_LINES ? kLineSmem : 0; }
 }  // namespace
 
 namespace {
@@ -656,18 +675,19 @@ int rev_prepare(js_batch* b) {
   const int n = b->count;
   std::vector<js::InstRev> rev(n);
   std::vector<long long> pre((size_t)js::RK_N * (n + 1), 0);
-  std::vector<int> rtile0(n + 1, 0);
+  std::vector<int> rblock0(n + 1, 0);
   for (int k = 0; k < n; ++k) {
     js::InstRev& r = rev[k];
     const int rc = js_internal_rev_desc(b->ctx[k], &r);
     if (rc) return rc;
     const js::InstDesc& d = b->desc[k];
     const js::Lay& L = d.lay;
-    r.tile0 = rtile0[k];
-    const int tiles = js::adj_tiles_x(L) * js::adj_tiles_y(L);
-    rtile0[k + 1] = rtile0[k] + tiles;
-    r.w_adj = (long long)tiles * js::ADJ_WARPS;
-    r.off_g = r.w_adj;
+    const int blocks = js::adj_blocks(L, 0) + js::adj_blocks(L, 1);
+    rblock0[k + 1] = rblock0[k] + blocks;
+    r.w_lines = (long long)blocks * js::ADJ_LINES;
+    r.off_c = r.w_lines;
+    r.w_c = round32(L.plane) / 32;
+    r.off_g = r.off_c + r.w_c;
     r.w_g = round32(d.ib.n) / 32;
     r.off_s = r.off_g + r.w_g;
     r.w_s = round32(r.ibt.nsrc) / 32;
@@ -689,13 +709,14 @@ int rev_prepare(js_batch* b) {
   // the split launch: each phase kernel's own resident blocks per SM
   if (cudaFuncSetAttribute(js::batch_vjp_phase_kernel<js::RP_STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)batch_smem()) != cudaSuccess ||
-      cudaFuncSetAttribute(js::batch_vjp_phase_kernel<js::RP_TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
+      cudaFuncSetAttribute(js::batch_vjp_phase_kernel<js::RP_LINES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kLineSmem) != cudaSuccess)
     return JS_ERR_CUDA;
   const void* kern[js::RP_N] = {
       (const void*)js::batch_vjp_phase_kernel<js::RP_PACK>, (const void*)js::batch_vjp_phase_kernel<js::RP_GHOST>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_HALO>, (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE>,
-      (const void*)js::batch_vjp_phase_kernel<js::RP_REDUCE>, (const void*)js::batch_vjp_phase_kernel<js::RP_TILES>,
+      (const void*)js::batch_vjp_phase_kernel<js::RP_REDUCE>, (const void*)js::batch_vjp_phase_kernel<js::RP_LINES>,
+      (const void*)js::batch_vjp_phase_kernel<js::RP_CELLS>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_BCTY>, (const void*)js::batch_vjp_phase_kernel<js::RP_BCTX>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_INFLOW_GHOST>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_SRC>, (const void*)js::batch_vjp_phase_kernel<js::RP_UNPACK>};
@@ -709,13 +730,13 @@ int rev_prepare(js_batch* b) {
   }
   if (cudaMalloc(&b->d_rev, sizeof(js::InstRev) * n) != cudaSuccess ||
       cudaMalloc(&b->d_pre, sizeof(long long) * pre.size()) != cudaSuccess ||
-      cudaMalloc(&b->d_rtile0, sizeof(int) * (n + 1)) != cudaSuccess ||
+      cudaMalloc(&b->d_rblock0, sizeof(int) * (n + 1)) != cudaSuccess ||
       cudaMalloc(&b->d_tab, sizeof(void*) * 4 * n) != cudaSuccess ||
       cudaMalloc(&b->d_dt, sizeof(double) * n) != cudaSuccess)
     return JS_ERR_NOMEM;
   if (cudaMemcpy(b->d_rev, rev.data(), sizeof(js::InstRev) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_pre, pre.data(), sizeof(long long) * pre.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(b->d_rtile0, rtile0.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(b->d_rblock0, rblock0.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess)
     return JS_ERR_CUDA;
   b->rev_ready = true;
@@ -730,7 +751,7 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
   a.count = b->count;
   a.pre = b->d_pre;
   a.tile0 = b->d_tile0;
-  a.rtile0 = b->d_rtile0;
+  a.rblock0 = b->d_rblock0;
   a.call = call;
   a.bar = b->d_bar;
   a.err = b->d_err;
@@ -757,7 +778,8 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
     }
     for (int s = 2; s >= 0; --s) {
       if (s < 2 && call.pbar) run(js::batch_vjp_phase_kernel<js::RP_REDUCE>, js::RP_REDUCE, s);
-      run(js::batch_vjp_phase_kernel<js::RP_TILES>, js::RP_TILES, s);
+      run(js::batch_vjp_phase_kernel<js::RP_LINES>, js::RP_LINES, s);
+      run(js::batch_vjp_phase_kernel<js::RP_CELLS>, js::RP_CELLS, s);
       run(js::batch_vjp_phase_kernel<js::RP_BCTY>, js::RP_BCTY, s);
       run(js::batch_vjp_phase_kernel<js::RP_BCTX>, js::RP_BCTX, s);
       run(js::batch_vjp_phase_kernel<js::RP_INFLOW_GHOST>, js::RP_INFLOW_GHOST, s);
@@ -780,7 +802,7 @@ extern "C" {
 void js_batch_destroy(js_batch* b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream); else cudaDeviceSynchronize();
-  cudaFree(b->d_rev); cudaFree(b->d_pre); cudaFree(b->d_rtile0); cudaFree(b->d_tab); cudaFree(b->d_dt); cudaFree(b->d_order);
+  cudaFree(b->d_rev); cudaFree(b->d_pre); cudaFree(b->d_rblock0); cudaFree(b->d_tab); cudaFree(b->d_dt); cudaFree(b->d_order);
   for (double* p : b->ro_buf) cudaFree(p);
   cudaFree(b->d_ro); cudaFree(b->d_spre);
   for (js_ctx* c : b->ctx) js_destroy(c);

@@ -49,6 +49,9 @@ struct js_ctx {
   // adjoint workspace (allocated by the first vjp call)
   bool adj_ready = false;
   double* ppart = nullptr;   // block partials of the parameter gradient (js::adj_ppart_doubles)
+  double* Qb = nullptr;      // 10 planes: primitive adjoints of the x and y lines
+  double* tang = nullptr;    // 4 planes (viscous 2D grids)
+  double* strips = nullptr;  // js::adj_strip_doubles
   double* P0 = nullptr;      // 4 planes (stage adjoint ping)
   double* P1 = nullptr;      // 4 planes (pong)
   double* Uacc = nullptr;    // 4 planes
@@ -466,7 +469,7 @@ void js_destroy(js_ctx* c) {
   cudaFree(c->err); cudaFree(c->red); cudaFree(c->cfl_bmax); cudaFree(c->dtc);
   cudaFree(c->ieee.Q); cudaFree(c->ieee.F); cudaFree(c->ieee.G);
   cudaFree(c->ibt_cell); cudaFree(c->ibt_ptr); cudaFree(c->ibt_ghost); cudaFree(c->ibt_w);
-  cudaFree(c->ppart); cudaFree(c->P0); cudaFree(c->P1); cudaFree(c->Uacc);
+  cudaFree(c->ppart); cudaFree(c->Qb); cudaFree(c->tang); cudaFree(c->strips); cudaFree(c->P0); cudaFree(c->P1); cudaFree(c->Uacc);
   if (c->inflow_host) cudaFreeHost(c->inflow_host);
   cudaFree(c->nnQ); cudaFree(c->nn_partial); cudaFree(c->nn_lam); cudaFree(c->nn_fadj);
   for (void* b : c->nn_buf) cudaFree(b);
@@ -809,14 +812,16 @@ int adj_reserve(js_ctx* c) {
   if (c->adj_ready) return JS_OK;
   const size_t pl = sizeof(double) * (size_t)c->lay.plane;
   struct { double** p; size_t planes; } bufs[] = {
-      {&c->P0, 4}, {&c->P1, 4}, {&c->Uacc, 4}};
+      {&c->P0, 4}, {&c->P1, 4}, {&c->Uacc, 4}, {&c->Qb, 10}, {&c->tang, 4}};
   for (auto& b : bufs) {
     if (cudaMalloc(b.p, b.planes * pl) != cudaSuccess) return JS_ERR_NOMEM;
     JS_CUDA(cudaMemsetAsync(*b.p, 0, b.planes * pl, c->stream));  // ordered with the caller's work
   }
   const size_t tmax = (size_t)std::max(c->g.nx + 6, c->g.ny);
   const size_t npp = (size_t)js::adj_ppart_doubles(c->lay, c->n_ghost, c->n_src, js::nn_image_vjp_blocks(c->lay));
-  if (cudaMalloc(&c->ppart, sizeof(double) * npp) != cudaSuccess) return JS_ERR_NOMEM;
+  if (cudaMalloc(&c->ppart, sizeof(double) * npp) != cudaSuccess ||
+      cudaMalloc(&c->strips, sizeof(double) * (size_t)js::adj_strip_doubles(c->lay)) != cudaSuccess)
+    return JS_ERR_NOMEM;
   if (cudaMalloc(&c->inflow_part, sizeof(double) * 16 * tmax) != cudaSuccess ||
       cudaMalloc(&c->inflow_prim, 16 * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&c->qIb, sizeof(double) * 4 * (size_t)(c->n_ghost > 0 ? c->n_ghost : 1)) != cudaSuccess)
@@ -835,6 +840,9 @@ js::AdjArgs adj_args(js_ctx* c, const double* X, double* Ub, double* p_bar) {
   a.pp = c->ppart;
   a.Ub = Ub;
   a.fadj = c->nn_fadj;
+  a.Qb = c->Qb;
+  a.tang = c->tang;
+  a.strips = c->strips;
   a.splane = saved_plane(c);
   a.tpitch = transposed_pitch(c);
   a.pbar = p_bar;

@@ -61,6 +61,9 @@ struct AdjArgs {
   const double* Q;           // padded primitives (4 planes; the neural flux's reverse only)
   double* lam;               // padded lambda' (4 planes), zero outside fluid cells (likewise)
   double* Ub;                // padded conserved adjoints of X (4 planes)
+  double* Qb;                // primitive adjoints of the x and y lines (2 x 5 padded planes)
+  double* tang;              // tangential terms of the x and y lines' viscous fluxes (2 x 2 planes)
+  double* strips;            // the line warps' sums for their outer cells
   double* fadj;              // the neural flux's face-state adjoints [dir][left/right][var] planes
                              //   of splane, or nullptr without the network
   long long splane;          // plane size of fadj (>= both layouts below)
@@ -77,11 +80,10 @@ struct AdjArgs {
   double* pp;                // warp partials of pbar[0..3] of the current launch (4 per warp)
 };
 
-// the reverse tile kernel: output cells of the padded array per tile and direction, warps a block
-constexpr int ADJ_TILE = 24, ADJ_WARPS = 8;
-// tiles of a grid's padded array along x and y
-inline __host__ __device__ int adj_tiles_x(const Lay& lay) { return (lay.nx + 6 + ADJ_TILE - 1) / ADJ_TILE; }
-inline __host__ __device__ int adj_tiles_y(const Lay& lay) { return (lay.H + ADJ_TILE - 1) / ADJ_TILE; }
+// the reverse line launch: reversed cells a warp, lines (warps) a block
+constexpr int ADJ_CHUNK = 28, ADJ_LINES = 8;
+// doubles of the strips of a grid
+long long adj_strip_doubles(const Lay& lay);
 // doubles of the parameter-gradient warp partials of one reverse stage (nn_blocks = blocks of the
 // neural image reverse, 0 without it)
 long long adj_ppart_doubles(const Lay& lay, int n_ghost, int n_src, long long nn_blocks);
@@ -169,7 +171,7 @@ struct InstDesc {
 
 // reverse-pass description of one instance for the persistent batched reverse kernel
 // (js_batch.cu): the context's adjoint arguments and workspace (js_internal_rev_desc) and the
-// instance's tiles and parameter-gradient slot offsets (set by js_batch.cu)
+// instance's parameter-gradient slot offsets (set by js_batch.cu)
 struct InstRev {
   AdjArgs a;                 // X, Ub, pbar, pp are set per phase
   IbTArgs ibt;
@@ -181,9 +183,8 @@ struct InstRev {
   double* qIb;
   double* ppart;             // warp partials of the parameter gradient
   int tmax;                  // max(nx + 6, ny): inflow_part row length
-  int tile0;                 // the instance's first reverse tile
-  long long w_adj;           // warp slots of its reverse tiles
-  long long off_g, w_g, off_s, w_s;  // slots of IB ghost, IB source
+  long long w_lines;         // warp slots of its line blocks
+  long long off_c, w_c, off_g, w_g, off_s, w_s;  // slots of cells, IB ghost, IB source
 };
 
 // opaque 128-byte, 64-byte aligned tensor map (CUtensorMap) for TMA copies
