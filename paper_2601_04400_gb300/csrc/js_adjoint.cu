@@ -33,11 +33,11 @@ namespace js {
 // x line blocks, then y line blocks.  Bound by the FP64 pipe (about 200 FP64 instructions per lane
 // and direction) with the integer WENO5 forward and reverse beside it; 16 warps an SM at 128 registers.
 template <bool VISC>
-__global__ void __launch_bounds__(32 * ADJ_LINES, 2)
+__global__ void __launch_bounds__(32 * ADJ_LINES, 3)
 adj_lines_kernel(AdjArgs a, const double* __restrict__ Unext, double bdt, int bx) {
   __shared__ double smem[8 * AP];
   const int b = blockIdx.x;
-  adj_lines<VISC>(a, Unext, bdt, b < bx ? 0 : 1, b < bx ? b : b - bx, smem, (long long)b * ADJ_LINES);
+  adj_lines<VISC>(a, Unext, bdt, b < bx ? 0 : 1, b < bx ? b : b - bx, smem, b);
 }
 
 template <bool VISC>
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) adj_cells_kernel(AdjArgs a, const double*
                                                         int rhs_mode) {
   double gb = 0.0, nb = 0.0;
   adj_cell<VISC>(a, Unext, Uacc, ra, rb, bdt, rhs_mode, (long long)blockIdx.x * blockDim.x + threadIdx.x, gb, nb);
-  warp_partials(a.pp, global_warp(), gb, 0.0, 0.0, nb);
+  block_partials(a.pp, blockIdx.x, gb, 0.0, 0.0, nb);
 }
 
 // primitives of every padded cell and lambda' = bdt Unext on fluid cells (the neural flux's reverse)
@@ -113,11 +113,11 @@ unsigned ib_blocks(int n) { return n > 0 ? blocks_for(n, 128) : 0; }
 long long adj_strip_doubles(const Lay& L) { return strip_size(L, 0) + strip_size(L, 1); }
 
 long long adj_ppart_doubles(const Lay& L, int n_ghost, int n_src, long long nn_blocks) {
-  // warps: the line blocks, the neural image reverse and the cells (256 threads a block), IB (128)
-  const long long warps = (long long)ADJ_LINES * (adj_blocks(L, 0) + adj_blocks(L, 1)) + 8 * nn_blocks +
-                          8 * (long long)blocks_for(L.plane, 256) +
+  // slots: one a line block; cells one a block (per warp in the batched kernels); per warp the
+  // neural image reverse (256 threads a block) and IB (128)
+  const long long slots = adj_blocks(L, 0) + adj_blocks(L, 1) + 8 * nn_blocks + 8 * (long long)blocks_for(L.plane, 256) +
                           4 * (long long)(ib_blocks(n_ghost) + ib_blocks(n_src));
-  return 4 * warps;
+  return 4 * slots;
 }
 
 cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& ib, const IbTArgs& ibt, int wall,
@@ -128,12 +128,12 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
   const Lay& L = a.lay;
   long long n = 0;
   cudaError_t e;
-  // warp partials of pbar[0..3]: consecutive slices for the launches that produce them
+  // partials of pbar[0..3]: consecutive slices for the launches that produce them
   double* const pp0 = a0.pbar ? a0.pp : nullptr;
   long long used = 0;
-  auto slice = [&](long long warps) {
+  auto slice = [&](long long slots) {
     double* p = pp0 ? pp0 + 4 * used : nullptr;
-    used += warps;
+    used += slots;
     return p;
   };
   if (nn) {
@@ -148,12 +148,12 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
   }
   const double bdt = rhs_mode ? 1.0 : rb * dt;
   const int bx = adj_blocks(L, 0), nb = bx + adj_blocks(L, 1);
-  a.pp = slice((long long)ADJ_LINES * nb);
+  a.pp = slice(nb);
   if (a.visc) adj_lines_kernel<true><<<nb, 32 * ADJ_LINES, 0, s>>>(a, Unext, bdt, bx);
   else adj_lines_kernel<false><<<nb, 32 * ADJ_LINES, 0, s>>>(a, Unext, bdt, bx);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const unsigned gp = blocks_for(L.plane, 256);
-  a.pp = slice(8LL * gp);
+  a.pp = slice(gp);
   if (a.visc) adj_cells_kernel<true><<<gp, 256, 0, s>>>(a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
   else adj_cells_kernel<false><<<gp, 256, 0, s>>>(a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

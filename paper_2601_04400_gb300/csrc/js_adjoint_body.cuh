@@ -34,6 +34,29 @@ __device__ __forceinline__ void warp_partials(double* pp, long long w, double g,
     o[3] = n;
   }
 }
+// the same summed over the block's warps in order (at most 8 warps, all threads call it): one slot
+// per block, so that the final reduction stays short
+__device__ __forceinline__ void block_partials(double* pp, long long slot, double g, double m, double pr, double n) {
+  if (pp == nullptr) return;
+  __shared__ double part[8][4];
+  g = warp_sum(g);
+  m = warp_sum(m);
+  pr = warp_sum(pr);
+  n = warp_sum(n);
+  if ((threadIdx.x & 31) == 0) {
+    double* o = part[threadIdx.x >> 5];
+    o[0] = g;
+    o[1] = m;
+    o[2] = pr;
+    o[3] = n;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    double t = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w][threadIdx.x];
+    pp[4 * slot + threadIdx.x] = t;
+  }
+}
 __device__ __forceinline__ long long global_warp() {
   return ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
 }
@@ -84,11 +107,11 @@ __device__ __forceinline__ double* strip(const AdjArgs& a, int dir, int chunk, i
   return a.strips + (dir == 0 ? 0 : strip_size(a.lay, 0)) + ((long long)(chunk * 5 + c) * 4 + e) * nline + line;
 }
 
-// block `item` of direction dir: ADJ_LINES warps, a line each; slot0: warp slot of the block's
+// block `item` of direction dir: ADJ_LINES warps, a line each; slot: the block's slot for its
 // partials of pbar[0..3]; smem: 8 AP doubles
 template <bool VISC>
 __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __restrict__ Unext, double bdt, int dir,
-                                          int item, double* smem, long long slot0) {
+                                          int item, double* smem, long long slot) {
   const Lay& L = a.lay;
   double* sq = smem;           // rho, u, v, p
   double* sl = smem + 4 * AP;  // Unext on fluid cells
@@ -272,7 +295,7 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
     vmu *= a.inv_mu;
     vk *= a.kp;
   }
-  warp_partials(a.pp, slot0 + warp, gb, vmu, vk, 0.0);
+  block_partials(a.pp, slot, gb, vmu, vk, 0.0);
 }
 
 // the line sums of primitive c at padded cell (i, j)

@@ -4,9 +4,10 @@
 //
 // The kernel runs every phase of every step for all instances, separated by grid barriers:
 //   pack       user states -> padded buffers
-//   per step:  CFL        per-instance max wave-speed rate and min density (atomics)
-//              per stage: IB fill | halo fill | fused stage tiles (the per-grid kernel's
-//                         device function, so trajectories equal js_step's bit for bit)
+//   per step:  CFL        per-instance max wave-speed rate and min density (atomics): fast rates,
+//                         then IEEE rates near the maximum, as js_max_dt
+//              per stage: IB fill | halo fill | lines | cells (the per-grid kernels' device
+//                         functions, so trajectories equal js_step's bit for bit)
 //   unpack     padded buffers -> user states
 // Each instance's dt is computed on the device from its reduction (same arithmetic as
 // js_max_dt).  Work items (tiles, ghosts, halo cells) of all instances are distributed
@@ -29,18 +30,20 @@
 
 namespace js {
 
-// the per-grid tiles; the forward launch runs 7 warps a block, the reverse launches 8, like the
-// per-grid kernels
-constexpr int BTX = TILE, BTY = TILE;
-constexpr int FNT = 224, BNT = 32 * ADJ_LINES;
+// cell tiles of the elementwise phases; both launches run 8 warps a block, like the per-grid kernels
+constexpr int BTX = 32, BTY = 32;
+constexpr int FNT = 32 * SLINES, BNT = 32 * ADJ_LINES;
 
 struct BatchArgs {
   const InstDesc* inst;
   int count;
-  const int* tile0;           // prefix sums (count + 1) of tiles, ghosts and halo cells
+  const int* tile0;           // prefix sums (count + 1) of cell tiles, line blocks, ghosts and halo cells
+  const int* line0;
   const long long* ghost0;
   const long long* halo0;
-  unsigned long long* red;    // [2][count][2]: rate bits, rho_min bits
+  unsigned long long* red;    // [2][count][4]: bits of the IEEE rate, rho_min, the fast rate
+  double* tmax;               // largest fast rate of each tile
+  double* dtc;                // [count][DTC_N] stage constants of the current step
   unsigned* bar;              // [0] arrivals, [1] generation
   int* err;
   double* t;                  // accumulated time per instance or nullptr
@@ -54,7 +57,7 @@ struct BatchArgs {
   double* const* save;        // [n_steps][count] states after each step, or nullptr
   double* const* save1;       // [n_steps][count] stage states U1, U2 of each step (after stages
   double* const* save2;       //   1 and 2), or nullptr
-  const int* order;           // schedule: queue position -> tile number (ntiles), or nullptr
+  const int* order;           // schedule: queue position -> line block, or nullptr
 };
 
 // ---------------------------------------------------------------------------------------
@@ -124,15 +127,30 @@ __device__ __forceinline__ double inst_dt(const InstDesc& d, const unsigned long
   return dt;
 }
 
-__global__ void __launch_bounds__(FNT, 2) batch_kernel(BatchArgs b) {
+// the stage arguments that do not depend on the stage and the step size
+__device__ __forceinline__ void fill_stage_args(StageArgs& a, const InstDesc& d, const double* X, int* err) {
+  a.Uin = X;
+  a.dF = d.dF;
+  a.tag = d.tag;
+  a.dtc = nullptr;
+  a.err = err;
+  a.lay = d.lay;
+  a.gamma = d.gamma;
+  a.gm1 = d.gamma - 1.0;
+  a.g1 = 1.0 / (d.gamma - 1.0);
+  a.vx = d.vx;
+  a.vy = d.vy;
+  a.has_av = d.has_av;
+}
+
+__global__ void __launch_bounds__(FNT, 3) batch_kernel(BatchArgs b) {
   extern __shared__ double smem[];
   const int ntiles = b.tile0[b.count];
   const long long nghost = b.ghost0[b.count], nhalo = b.halo0[b.count];
   const int tid = threadIdx.x, lane = threadIdx.x & 31;
   // ---- pack user states; reset both reduction buffers
   for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-    const int q = b.order ? b.order[it] : it;
-    const int k = find_inst(b.tile0, b.count, q);
+    const int q = it, k = find_inst(b.tile0, b.count, q);
     const InstDesc& d = b.inst[k];
     const double* Uk = b.ustate ? b.ustate[k] : d.U;
     const int t = q - b.tile0[k];
@@ -148,48 +166,97 @@ __global__ void __launch_bounds__(FNT, 2) batch_kernel(BatchArgs b) {
   }
   if (blockIdx.x == 0)
     for (int k = tid; k < 2 * b.count; k += FNT) {
-      b.red[2 * k] = 0ULL;
-      b.red[2 * k + 1] = 0x7ff0000000000000ULL;
+      b.red[4 * k] = b.red[4 * k + 2] = 0ULL;
+      b.red[4 * k + 1] = 0x7ff0000000000000ULL;
     }
   if (!grid_sync(b)) return;
   for (int step = 0; step < b.n_steps; ++step) {
     const int par = step & 1;
-    unsigned long long* red = b.red + 2 * (long long)b.count * par;
+    unsigned long long* red = b.red + 4 * (long long)b.count * par;
     // ---- CFL reduction over fluid cells, per instance (skipped with given step sizes)
-    for (int it = blockIdx.x; it < (b.dt_in ? 0 : ntiles); it += gridDim.x) {
-      const int q = b.order ? b.order[it] : it;
-    const int k = find_inst(b.tile0, b.count, q);
-      const InstDesc& d = b.inst[k];
-      const int t = q - b.tile0[k];
-      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
-      double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
-      for (int e = tid; e < BTX * BTY; e += FNT) {
-        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
-        if (i >= d.lay.nx || j >= d.lay.ny) continue;
-        if (d.tag && d.tag[(long long)j * d.lay.nx + i] != 0) continue;
-        const long long p = d.lay.idx(i, j);
-        const double r = d.N[p];
-        rate = fmax(rate, cfl_rate(r, d.N[d.lay.plane + p], d.N[2 * d.lay.plane + p], d.N[3 * d.lay.plane + p],
-                                   d.gamma, d.dx, d.dy, d.lay.ny > 1));
-        rmin = fmin(rmin, r);
+    if (!b.dt_in) {
+      __shared__ double sr[FNT / 32], sm[FNT / 32];
+      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+        const int k = find_inst(b.tile0, b.count, it);
+        const InstDesc& d = b.inst[k];
+        const int t = it - b.tile0[k];
+        const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+        const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
+        double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
+        for (int e = tid; e < BTX * BTY; e += FNT) {
+          const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+          if (i >= d.lay.nx || j >= d.lay.ny) continue;
+          if (d.tag && d.tag[(long long)j * d.lay.nx + i] != 0) continue;
+          const long long p = d.lay.idx(i, j);
+          const double r = d.N[p];
+          rate = fmax(rate, cfl_rate_fast(r, d.N[d.lay.plane + p], d.N[2 * d.lay.plane + p], d.N[3 * d.lay.plane + p],
+                                          d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1));
+          rmin = fmin(rmin, r);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+          rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
+          rmin = fmin(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+        }
+        if (lane == 0) {
+          sr[tid >> 5] = rate;
+          sm[tid >> 5] = rmin;
+        }
+        __syncthreads();
+        if (tid == 0) {
+          for (int w = 1; w < FNT / 32; ++w) {
+            rate = fmax(rate, sr[w]);
+            rmin = fmin(rmin, sm[w]);
+          }
+          b.tmax[it] = rate;
+          atomicMax(red + 4 * k + 2, (unsigned long long)__double_as_longlong(rate));
+          atomicMin(red + 4 * k + 1, (unsigned long long)__double_as_longlong(rmin));
+        }
+        __syncthreads();
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
-        rmin = fmin(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+      if (!grid_sync(b)) return;
+      // the IEEE rate of the cells near the maximum, once per run of identical cells along a row
+      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+        const int k = find_inst(b.tile0, b.count, it);
+        const double thr = __longlong_as_double((long long)red[4 * k + 2]) * (1.0 - CFL_MARGIN);
+        if (!(b.tmax[it] >= thr)) continue;  // the same for the whole block
+        const InstDesc& d = b.inst[k];
+        const int t = it - b.tile0[k];
+        const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+        const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
+        double rate = 0.0;
+        for (int e = tid; e < BTX * BTY; e += FNT) {
+          const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+          if (i >= d.lay.nx || j >= d.lay.ny) continue;
+          const unsigned char* tag = d.tag ? d.tag + (long long)j * d.lay.nx + i : nullptr;
+          if (tag && tag[0] != 0) continue;
+          const double* X = d.N + d.lay.idx(i, j);
+          const long long P = d.lay.plane;
+          const double r = X[0], mx = X[P], my = X[2 * P], E = X[3 * P];
+          if (!(cfl_rate_fast(r, mx, my, E, d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1) >= thr)) continue;
+          if (i > 0 && !(tag && tag[-1] != 0) && same_bits(r, X[-1]) && same_bits(mx, X[P - 1]) &&
+              same_bits(my, X[2 * P - 1]) && same_bits(E, X[3 * P - 1]))
+            continue;
+          rate = fmax(rate, cfl_rate(r, mx, my, E, d.gamma, d.dx, d.dy, d.lay.ny > 1));
+        }
+        for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
+        if (lane == 0 && rate > 0.0) atomicMax(red + 4 * k, (unsigned long long)__double_as_longlong(rate));
       }
-      if (lane == 0) {
-        atomicMax(red + 2 * k, (unsigned long long)__double_as_longlong(rate));
-        atomicMin(red + 2 * k + 1, (unsigned long long)__double_as_longlong(rmin));
-      }
+      if (!grid_sync(b)) return;
     }
-    if (!b.dt_in && !grid_sync(b)) return;
     if (blockIdx.x == 0) {
       // the other parity was last read in the previous step: reset it for the next one
-      unsigned long long* nxt = b.red + 2 * (long long)b.count * (par ^ 1);
+      unsigned long long* nxt = b.red + 4 * (long long)b.count * (par ^ 1);
       for (int k = tid; k < b.count; k += FNT) {
-        nxt[2 * k] = 0ULL;
-        nxt[2 * k + 1] = 0x7ff0000000000000ULL;
-        const double dtk = b.dt_in ? b.dt_in[(long long)step * b.count + k] : inst_dt(b.inst[k], red + 2 * k, b.cfl);
+        nxt[4 * k] = nxt[4 * k + 2] = 0ULL;
+        nxt[4 * k + 1] = 0x7ff0000000000000ULL;
+        const InstDesc& d = b.inst[k];
+        const double dtk = b.dt_in ? b.dt_in[(long long)step * b.count + k] : inst_dt(d, red + 4 * k, b.cfl);
+        // the stage constants, read by the cell phases (grid barriers lie between)
+        double* dtc = b.dtc + (long long)DTC_N * k;
+        dtc[0] = __ddiv_rn(dtk, d.dx);
+        dtc[1] = __ddiv_rn(dtk, d.dy);
+        dtc[2] = __ddiv_rn(__dmul_rn(dtk, d.nu), __dmul_rn(d.dx, d.dx));
+        dtc[3] = __ddiv_rn(__dmul_rn(dtk, d.nu), __dmul_rn(d.dy, d.dy));
         // a non-physical fluid cell has an infinite rate (cfl_rate): dt = 0
         if (!(dtk > 0.0) || !(dtk < CUDART_INF)) atomicOr(b.err, ERR_NONPHYSICAL_BIT);
         if (b.t) b.t[k] += dtk;
@@ -213,37 +280,42 @@ __global__ void __launch_bounds__(FNT, 2) batch_kernel(BatchArgs b) {
         bc_fill_one(X, d.lay, d.bc, h - b.halo0[k]);
       }
       if (!grid_sync(b)) return;
-      // ---- stage tiles
-      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-        const int q = b.order ? b.order[it] : it;
-    const int k = find_inst(b.tile0, b.count, q);
+      // ---- lines
+      const int nlines = b.line0[b.count];
+      for (int it = blockIdx.x; it < nlines; it += gridDim.x) {
+        const int q = b.order ? b.order[it] : it, k = find_inst(b.line0, b.count, q);
         const InstDesc& d = b.inst[k];
-        const int t = q - b.tile0[k];
-        const double dt = b.dt_in ? b.dt_in[(long long)step * b.count + k] : inst_dt(d, red + 2 * k, b.cfl);
+        __shared__ StageArgs sa;  // (in registers they would cost resident warps)
+        if (tid == 0) fill_stage_args(sa, d, (s == 0) ? d.N : ((s == 1) ? d.A : d.B), b.err);
+        __syncthreads();
+        const int t = q - b.line0[k], bx = stage_blocks(d.lay, 0);
+        if (d.visc) stage_lines<true, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+        else stage_lines<false, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+        __syncthreads();  // the next block of lines reuses shared memory
+      }
+      if (!grid_sync(b)) return;
+      // ---- cells
+      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+        const int k = find_inst(b.tile0, b.count, it);
+        const InstDesc& d = b.inst[k];
+        const double* dtc = b.dtc + (long long)DTC_N * k;
         StageArgs a;
-        a.Uin = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
+        fill_stage_args(a, d, (s == 0) ? d.N : ((s == 1) ? d.A : d.B), b.err);
         a.Un = d.N;
         a.Uout = (s == 0) ? d.A : ((s == 1) ? d.B : d.N);
-        a.tag = d.tag;
-        a.dtc = nullptr;
-        a.err = b.err;
-        a.lay = d.lay;
-        a.gamma = d.gamma;
-        a.gm1 = d.gamma - 1.0;
-        a.g1 = 1.0 / (d.gamma - 1.0);
-        a.cx = dt / d.dx;
-        a.cy = dt / d.dy;
+        a.cx = dtc[0];
+        a.cy = dtc[1];
+        a.avx = dtc[2];
+        a.avy = dtc[3];
         a.rk_a = (s == 0) ? 0.0 : ((s == 1) ? 0.75 : 1.0 / 3.0);
         a.rk_b = (s == 0) ? 1.0 : ((s == 1) ? 0.25 : 2.0 / 3.0);
-        a.avx = dt * d.nu / (d.dx * d.dx);
-        a.avy = dt * d.nu / (d.dy * d.dy);
-        a.vx = d.vx;
-        a.vy = d.vy;
         a.use_un = (s > 0) ? 1 : 0;
-        a.has_av = d.has_av;
-        if (d.visc) stage_tile<true, false>(a, t % d.ntx, t / d.ntx, smem);
-        else stage_tile<false, false>(a, t % d.ntx, t / d.ntx, smem);
-        __syncthreads();  // the next tile reuses shared memory
+        const int t = it - b.tile0[k];
+        const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+        for (int e = tid; e < BTX * BTY; e += FNT) {
+          const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+          if (i < d.lay.nx && j < d.lay.ny) stage_cell<false>(a, i, j);
+        }
       }
       if (!grid_sync(b)) return;
     }
@@ -252,8 +324,7 @@ __global__ void __launch_bounds__(FNT, 2) batch_kernel(BatchArgs b) {
       // and the stage states A, B of this step (their ghost cells were refilled from fluid
       // cells, which a reverse pass that fills them again reproduces)
       for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-        const int q = b.order ? b.order[it] : it;
-        const int k = find_inst(b.tile0, b.count, q);
+        const int q = it, k = find_inst(b.tile0, b.count, q);
         const InstDesc& d = b.inst[k];
         const long long row = (long long)step * b.count + k;
         double* S = b.save ? b.save[row] : nullptr;
@@ -281,8 +352,7 @@ __global__ void __launch_bounds__(FNT, 2) batch_kernel(BatchArgs b) {
   }
   // ---- unpack
   for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-    const int q = b.order ? b.order[it] : it;
-    const int k = find_inst(b.tile0, b.count, q);
+    const int q = it, k = find_inst(b.tile0, b.count, q);
     const InstDesc& d = b.inst[k];
     double* Uk = b.ustate ? b.ustate[k] : d.U;
     const int t = q - b.tile0[k];
@@ -334,6 +404,7 @@ struct BatchRevArgs {
   int count;
   const long long* pre;       // [RK_N][count + 1] prefix sums of the padded item counts
   const int* tile0;
+  const int* line0;
   const int* rblock0;         // prefix sums (count + 1) of the reverse line blocks
   RevCall call;
   unsigned* bar;
@@ -388,7 +459,8 @@ enum RevPhase {
   RP_PACK = 0,      // pack U_n, lambda_{n+1} (and given stage states); Uacc = 0
   RP_GHOST,         // IB fill of stage input s
   RP_HALO,          // halo fill of stage input s
-  RP_STAGE,         // forward recompute of stage s (0, 1)
+  RP_STAGE,         // forward recompute of stage s (0, 1): lines
+  RP_STAGE_CELLS,   // cells
   RP_REDUCE,        // the parameter gradient of reverse stage s+1 (before the lines reuse its slots)
   RP_LINES,         // reverse of stage s: lines
   RP_CELLS,         // cells
@@ -443,35 +515,39 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       bc_fill_one(X, d.lay, d.bc, h);
     });
   } else if constexpr (PH == RP_STAGE) {
+    for (int it = blockIdx.x; it < b.line0[b.count]; it += gridDim.x) {
+      const int k = find_inst(b.line0, b.count, it);
+      const InstDesc& d = b.inst[k];
+      __shared__ StageArgs sa;
+      if (threadIdx.x == 0) fill_stage_args(sa, d, (s == 0) ? d.N : d.A, b.err);
+      __syncthreads();
+      const int t = it - b.line0[k], bx = stage_blocks(d.lay, 0);
+      if (d.visc) stage_lines<true, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+      else stage_lines<false, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+      __syncthreads();  // the next block of lines reuses shared memory
+    }
+  } else if constexpr (PH == RP_STAGE_CELLS) {
     for (int it = blockIdx.x; it < b.tile0[b.count]; it += gridDim.x) {
       const int k = find_inst(b.tile0, b.count, it);
       const InstDesc& d = b.inst[k];
-      const int t = it - b.tile0[k];
       const double dt = call.dt[k];
       StageArgs a;
-      a.Uin = (s == 0) ? d.N : d.A;
+      fill_stage_args(a, d, (s == 0) ? d.N : d.A, b.err);
       a.Un = d.N;
       a.Uout = (s == 0) ? d.A : d.B;
-      a.tag = d.tag;
-      a.err = b.err;
-      a.lay = d.lay;
-      a.gamma = d.gamma;
-      a.gm1 = d.gamma - 1.0;
-      a.g1 = 1.0 / (d.gamma - 1.0);
       a.cx = dt / d.dx;
       a.cy = dt / d.dy;
       a.rk_a = (s == 0) ? 0.0 : 0.75;
       a.rk_b = (s == 0) ? 1.0 : 0.25;
       a.avx = dt * d.nu / (d.dx * d.dx);
       a.avy = dt * d.nu / (d.dy * d.dy);
-      a.vx = d.vx;
-      a.vy = d.vy;
       a.use_un = (s > 0) ? 1 : 0;
-      a.has_av = d.has_av;
-      a.dtc = nullptr;
-      if (d.visc) stage_tile<true, false>(a, t % d.ntx, t / d.ntx, smem);
-      else stage_tile<false, false>(a, t % d.ntx, t / d.ntx, smem);
-      __syncthreads();  // the next tile reuses shared memory
+      const int t = it - b.tile0[k];
+      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+      for (int e = threadIdx.x; e < BTX * BTY; e += BNT) {
+        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+        if (i < d.lay.nx && j < d.lay.ny) stage_cell<false>(a, i, j);
+      }
     }
   } else if constexpr (PH == RP_REDUCE) {
     if (s < 2 && call.pbar)
@@ -486,8 +562,8 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       const double* src = even ? r.P0 : r.P1;
       const int t = it - b.rblock0[k], bx = adj_blocks(d.lay, 0);
       const double bdt = REV_B[s] * call.dt[k];
-      if (d.visc) adj_lines<true>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, (long long)t * ADJ_LINES);
-      else adj_lines<false>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, (long long)t * ADJ_LINES);
+      if (d.visc) adj_lines<true>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
+      else adj_lines<false>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
       __syncthreads();  // the next block of lines reuses shared memory
     }
   } else if constexpr (PH == RP_CELLS) {
@@ -567,6 +643,8 @@ __global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
     if (b.call.U1) continue;  // the stage states were given: only their ghosts and halos are filled
     rev_phase<RP_STAGE>(b, s, smem);
     if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
+    rev_phase<RP_STAGE_CELLS>(b, s, smem);
+    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
   }
   // ---- reverse through the stages 2, 1, 0: P0 -> P1 -> P0 -> P1
   for (int s = 2; s >= 0; --s) {
@@ -590,7 +668,7 @@ __global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
 
 // one phase of the reverse step as a kernel of its own (split launch)
 template <int PH>
-__global__ void __launch_bounds__(BNT, PH == RP_STAGE || PH == RP_LINES ? 2 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
+__global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
   extern __shared__ double smem[];
   rev_phase<PH>(b, s, smem);
 }
@@ -621,6 +699,10 @@ struct js_batch {
   std::vector<InstDesc> desc;    // host copy
   InstDesc* d_desc = nullptr;
   int* d_tile0 = nullptr;
+  int* d_line0 = nullptr;        // prefix sums of the stage's line blocks
+  std::vector<int> line0;
+  double* d_tmax = nullptr;      // per tile: largest fast rate
+  double* d_dtc = nullptr;       // per instance: stage constants
   long long* d_ghost0 = nullptr;
   long long* d_halo0 = nullptr;
   unsigned long long* d_red = nullptr;
@@ -658,7 +740,7 @@ void js_internal_desc(js_ctx* c, js::InstDesc* d);
 int js_internal_rev_desc(js_ctx* c, js::InstRev* d);
 
 namespace {
-size_t batch_smem() { return js::StageTile<true>::SMEM; }
+size_t batch_smem() { return js::stage_smem<true>(); }
 constexpr size_t kLineSmem = sizeof(double) * 8 * js::AP;
 size_t rev_smem() { return std::max(batch_smem(), kLineSmem); }
 size_t rev_phase_smem(int ph) { return ph == js::RP_STAGE ? batch_smem() : ph == js::RP_LINES ? kLineSmem : 0; }
@@ -684,7 +766,7 @@ int rev_prepare(js_batch* b) {
     const js::Lay& L = d.lay;
     const int blocks = js::adj_blocks(L, 0) + js::adj_blocks(L, 1);
     rblock0[k + 1] = rblock0[k] + blocks;
-    r.w_lines = (long long)blocks * js::ADJ_LINES;
+    r.w_lines = blocks;
     r.off_c = r.w_lines;
     r.w_c = round32(L.plane) / 32;
     r.off_g = r.off_c + r.w_c;
@@ -715,6 +797,7 @@ int rev_prepare(js_batch* b) {
   const void* kern[js::RP_N] = {
       (const void*)js::batch_vjp_phase_kernel<js::RP_PACK>, (const void*)js::batch_vjp_phase_kernel<js::RP_GHOST>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_HALO>, (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE>,
+      (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE_CELLS>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_REDUCE>, (const void*)js::batch_vjp_phase_kernel<js::RP_LINES>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_CELLS>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_BCTY>, (const void*)js::batch_vjp_phase_kernel<js::RP_BCTX>,
@@ -751,6 +834,7 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
   a.count = b->count;
   a.pre = b->d_pre;
   a.tile0 = b->d_tile0;
+  a.line0 = b->d_line0;
   a.rblock0 = b->d_rblock0;
   a.call = call;
   a.bar = b->d_bar;
@@ -775,6 +859,7 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
       if (s == 2) break;
       if (call.U1) continue;
       run(js::batch_vjp_phase_kernel<js::RP_STAGE>, js::RP_STAGE, s);
+      run(js::batch_vjp_phase_kernel<js::RP_STAGE_CELLS>, js::RP_STAGE_CELLS, s);
     }
     for (int s = 2; s >= 0; --s) {
       if (s < 2 && call.pbar) run(js::batch_vjp_phase_kernel<js::RP_REDUCE>, js::RP_REDUCE, s);
@@ -806,7 +891,7 @@ void js_batch_destroy(js_batch* b) {
   for (double* p : b->ro_buf) cudaFree(p);
   cudaFree(b->d_ro); cudaFree(b->d_spre);
   for (js_ctx* c : b->ctx) js_destroy(c);
-  cudaFree(b->d_desc); cudaFree(b->d_tile0); cudaFree(b->d_ghost0); cudaFree(b->d_halo0);
+  cudaFree(b->d_desc); cudaFree(b->d_tile0); cudaFree(b->d_line0); cudaFree(b->d_tmax); cudaFree(b->d_dtc); cudaFree(b->d_ghost0); cudaFree(b->d_halo0);
   cudaFree(b->d_red); cudaFree(b->d_bar); cudaFree(b->d_err);
   delete b;
 }
@@ -820,6 +905,7 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
   b->count = count;
   b->stream = (cudaStream_t)stream;
   std::vector<int> tile0(count + 1, 0);
+  b->line0.assign(1, 0);
   std::vector<long long> ghost0(count + 1, 0), halo0(count + 1, 0);
   for (int k = 0; k < count; ++k) {
     if (grids[k].ny < 2) { js_batch_destroy(b); return JS_ERR_ARG; }  // 2D instances only
@@ -833,6 +919,7 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
     d.nty = (grids[k].ny + js::BTY - 1) / js::BTY;
     b->desc.push_back(d);
     tile0[k + 1] = tile0[k] + d.ntx * d.nty;
+    b->line0.push_back(b->line0.back() + js::stage_blocks(d.lay, 0) + js::stage_blocks(d.lay, 1));
     ghost0[k + 1] = ghost0[k] + d.ib.n;
     halo0[k + 1] = halo0[k] + js::halo_count(d.lay);
     b->cells += (long long)grids[k].nx * grids[k].ny;
@@ -856,13 +943,17 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
       cudaMalloc(&b->d_tile0, sizeof(int) * (count + 1)) != cudaSuccess ||
       cudaMalloc(&b->d_ghost0, sizeof(long long) * (count + 1)) != cudaSuccess ||
       cudaMalloc(&b->d_halo0, sizeof(long long) * (count + 1)) != cudaSuccess ||
-      cudaMalloc(&b->d_red, sizeof(unsigned long long) * 4 * count) != cudaSuccess ||
+      cudaMalloc(&b->d_red, sizeof(unsigned long long) * 8 * count) != cudaSuccess ||
+      cudaMalloc(&b->d_line0, sizeof(int) * (count + 1)) != cudaSuccess ||
+      cudaMalloc(&b->d_tmax, sizeof(double) * b->ntiles) != cudaSuccess ||
+      cudaMalloc(&b->d_dtc, sizeof(double) * js::DTC_N * count) != cudaSuccess ||
       cudaMalloc(&b->d_bar, 2 * sizeof(unsigned)) != cudaSuccess ||
       cudaMalloc(&b->d_err, sizeof(int)) != cudaSuccess) {
     js_batch_destroy(b);
     return JS_ERR_NOMEM;
   }
   if (cudaMemcpy(b->d_tile0, tile0.data(), sizeof(int) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(b->d_line0, b->line0.data(), sizeof(int) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_ghost0, ghost0.data(), sizeof(long long) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_halo0, halo0.data(), sizeof(long long) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(b->d_bar, 0, 2 * sizeof(unsigned)) != cudaSuccess ||
@@ -905,9 +996,13 @@ static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, dou
   a.inst = b->d_desc;
   a.count = b->count;
   a.tile0 = b->d_tile0;
+  a.line0 = b->d_line0;
   a.ghost0 = b->d_ghost0;
   a.halo0 = b->d_halo0;
   a.red = b->d_red;
+  a.tmax = b->d_tmax;
+  a.dtc = b->d_dtc;
+  a.line0 = b->d_line0;
   a.bar = b->d_bar;
   a.err = b->d_err;
   a.t = t_dev;
@@ -1197,28 +1292,26 @@ int js_batch_sync_status(js_batch* b) {
 int js_batch_set_tuning(js_batch* b, int blocks_per_sm, int schedule) {
   if (!b || blocks_per_sm < 0 || blocks_per_sm > b->per_sm || schedule < 0 || schedule > 2) return JS_ERR_ARG;
   if (schedule != 0) {
-    // queue position -> tile number
-    std::vector<int> tile0(b->count + 1, 0);
-    for (int k = 0; k < b->count; ++k) tile0[k + 1] = tile0[k] + b->desc[k].ntx * b->desc[k].nty;
+    // queue position -> line block
+    const std::vector<int>& t0 = b->line0;
+    const int nblocks = t0[b->count];
     std::vector<int> order;
-    order.reserve(b->ntiles);
-    if (schedule == 1) {  // interleaved: tile j of every instance, then tile j + 1
+    order.reserve(nblocks);
+    if (schedule == 1) {  // interleaved: block j of every instance, then block j + 1
       int most = 0;
-      for (int k = 0; k < b->count; ++k) most = std::max(most, tile0[k + 1] - tile0[k]);
+      for (int k = 0; k < b->count; ++k) most = std::max(most, t0[k + 1] - t0[k]);
       for (int j = 0; j < most; ++j)
         for (int k = 0; k < b->count; ++k)
-          if (tile0[k] + j < tile0[k + 1]) order.push_back(tile0[k] + j);
-    } else {  // the largest instances first, each instance's tiles together
+          if (t0[k] + j < t0[k + 1]) order.push_back(t0[k] + j);
+    } else {  // the largest instances first, each instance's blocks together
       std::vector<int> inst(b->count);
       for (int k = 0; k < b->count; ++k) inst[k] = k;
-      std::stable_sort(inst.begin(), inst.end(), [&](int x, int y) {
-        return tile0[x + 1] - tile0[x] > tile0[y + 1] - tile0[y];
-      });
+      std::stable_sort(inst.begin(), inst.end(), [&](int x, int y) { return t0[x + 1] - t0[x] > t0[y + 1] - t0[y]; });
       for (int k : inst)
-        for (int t = tile0[k]; t < tile0[k + 1]; ++t) order.push_back(t);
+        for (int t = t0[k]; t < t0[k + 1]; ++t) order.push_back(t);
     }
-    if (!b->d_order && cudaMalloc(&b->d_order, sizeof(int) * b->ntiles) != cudaSuccess) return JS_ERR_NOMEM;
-    if (cudaMemcpyAsync(b->d_order, order.data(), sizeof(int) * b->ntiles, cudaMemcpyHostToDevice, b->stream) !=
+    if (!b->d_order && cudaMalloc(&b->d_order, sizeof(int) * nblocks) != cudaSuccess) return JS_ERR_NOMEM;
+    if (cudaMemcpyAsync(b->d_order, order.data(), sizeof(int) * nblocks, cudaMemcpyHostToDevice, b->stream) !=
             cudaSuccess ||
         cudaStreamSynchronize(b->stream) != cudaSuccess)
       return JS_ERR_CUDA;

@@ -5,11 +5,10 @@
 // FP64 add/mul/fma instructions:
 //   * no IEEE division or square root: reciprocals and reciprocal square roots are formed in
 //     integer arithmetic beside the FP64 pipe (js_wide.cuh), accurate to half an ulp;
-//   * WENO5 runs on the integer pipes (js_weno.cuh) but for three FP64 instructions per cell
-//     and variable; the nonlinear weights use the products of the other stencils'
+//   * WENO5 runs on the integer pipes (js_weno.cuh); the nonlinear weights use the products of the other stencils'
 //     (eps + beta)^2 instead of 1/(eps + beta)^2, so one division per face state remains;
 //   * HLLC forms the flux of the upwind side's star state (selected with integer selects),
-//     and the sound speed as gamma*p*rsqrt(gamma*p*rho).
+//     the sound speed in integer arithmetic.
 #pragma once
 #include <cstdint>
 
@@ -61,6 +60,16 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
   const s32 h = (s32)hi32(dbits(x));
   if ((u32)(h - 0x00100000) >= 0x7fe00000u) return rsqrt_plain(x);  // not positive and normal
   return rsqrt_wide(x);
+}
+
+// sound speed sqrt(gamma p / r) in integer arithmetic (it took 8 FP64 instructions)
+__device__ __forceinline__ double sound(double gamma, double p, double r) {
+  const s32 hp = (s32)hi32(dbits(p)), hr = (s32)hi32(dbits(r));
+  if ((u32)(hp - 0x00100000) >= 0x7fe00000u || (u32)(hr - 0x00100000) >= 0x7fe00000u) {
+    const double gp = gamma * p;
+    return gp * rsqrt_plain(gp * r);
+  }
+  return sound_wide(gamma, p, r);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -134,8 +143,8 @@ static __device__ __noinline__ double2 weno_plain(double qm2, double qm1, double
 }
 
 // the largest exponent of a stencil's differences up to which the integer form serves
-// (js_weno.cuh); pos: the variable is positive (density, pressure)
-__device__ __forceinline__ int weno_limit(double q0, bool pos) { return pos ? imin(expo(q0) + 3, 1500) : 1500; }
+// (js_weno.cuh); e: the cell value's exponent, pos: the variable is positive (density, pressure)
+__device__ __forceinline__ int weno_limit(int e, bool pos) { return pos ? imin(e + 3, 1500) : 1500; }
 
 __device__ __forceinline__ Sm shfl_up(const Sm& s) {
   return Sm{(u64)__shfl_up_sync(0xffffffffu, (unsigned long long)s.m, 1), __shfl_up_sync(0xffffffffu, s.x, 1)};
@@ -156,44 +165,38 @@ __device__ __forceinline__ Fx shfl_down(const Fx& d) {
 // forms the differences on both sides of its cell and the three indicators they determine, and
 // takes its s_0, s_2 and outer differences from its neighbours.
 __device__ __forceinline__ void weno_lane(const double* q, int st, bool pos, bool inner, double& Lf, double& Rf) {
-  const double q0 = q[0];
-  const Fx dm1 = fx_of(q0 - q[-st]), dp1 = fx_of(q[st] - q0);
+  const Qx x = qx_of(q[0]);
+  const Fx dm1 = fx_of(x, qx_of(q[-st])), dp1 = fx_of(qx_of(q[st]), x);
   Sm s1, s0n, s2p;
   sm_pair(dm1, dp1, s1, s0n, s2p);
   const Sm s0 = shfl_up(s0n), s2 = shfl_down(s2p);
   const Fx dm2 = shfl_up(dm1), dp2 = shfl_down(dp1);
   const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
-  if (F > weno_limit(q0, pos) && inner) {
-    const double2 r = weno_plain(q[-2 * st], q[-st], q0, q[st], q[2 * st]);
+  if (F > weno_limit(x.e, pos) && inner) {
+    const double2 r = weno_plain(q[-2 * st], q[-st], q[0], q[st], q[2 * st]);
     Lf = r.x;
     Rf = r.y;
   } else {
-    double cL, cR;
-    weno_corr(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR);
-    Lf = fma(cL, SIXTH, q0);
-    Rf = fma(cR, SIXTH, q0);
+    weno_faces(x, dm2, dm1, dp1, dp2, s0, s1, s2, F, Lf, Rf);
   }
 }
 
 // the same for a single thread (q[-2 st .. 2 st] readable): the same bits
 template <class I>
 __device__ __forceinline__ void weno_cell(const double* q, I st, bool pos, double& Lf, double& Rf) {
-  const double q0 = q[0];
-  const Fx dm2 = fx_of(q[-st] - q[-2 * st]), dm1 = fx_of(q0 - q[-st]), dp1 = fx_of(q[st] - q0), dp2 = fx_of(q[2 * st] - q[st]);
-  Sm s0, s1, s2, x, y;
-  sm_pair(dm2, dm1, x, s0, y);
-  sm_pair(dp1, dp2, x, y, s2);
-  sm_pair(dm1, dp1, s1, x, y);
+  const Qx m2 = qx_of(q[-2 * st]), m1 = qx_of(q[-st]), x = qx_of(q[0]), p1 = qx_of(q[st]), p2 = qx_of(q[2 * st]);
+  const Fx dm2 = fx_of(m1, m2), dm1 = fx_of(x, m1), dp1 = fx_of(p1, x), dp2 = fx_of(p2, p1);
+  Sm s0, s1, s2, u, v;
+  sm_pair(dm2, dm1, u, s0, v);
+  sm_pair(dp1, dp2, u, v, s2);
+  sm_pair(dm1, dp1, s1, u, v);
   const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
-  if (F > weno_limit(q0, pos)) {
-    const double2 r = weno_plain(q[-2 * st], q[-st], q0, q[st], q[2 * st]);
+  if (F > weno_limit(x.e, pos)) {
+    const double2 r = weno_plain(q[-2 * st], q[-st], q[0], q[st], q[2 * st]);
     Lf = r.x;
     Rf = r.y;
   } else {
-    double cL, cR;
-    weno_corr(dm2, dm1, dp1, dp2, s0, s1, s2, F, cL, cR);
-    Lf = fma(cL, SIXTH, q0);
-    Rf = fma(cR, SIXTH, q0);
+    weno_faces(x, dm2, dm1, dp1, dp2, s0, s1, s2, F, Lf, Rf);
   }
 }
 
@@ -208,7 +211,7 @@ __device__ __forceinline__ void weno_cell(const double* q, I st, bool pos, doubl
 //   G = m s*/(s_K - s*),  F = (G, G s* + p*, G u_t, s*/(s_K - s*) (d E - p u + p* s_K)).
 // A supersonic face (s_K on the far side of zero) has F = F_K, the same expressions with u in
 // the place of s*.  At s* = 0 both sides give (0, p*, 0, 0): the average of the branches that
-// sign(0) = 0 asks for is either of them.  35 FP64 instructions a face (19 at s* = 0, where gas
+// sign(0) = 0 asks for is either of them.  31 FP64 instructions a face (15 at s* = 0, where gas
 // at rest on both sides always lands) where building the star state and its jump took 69.
 // ---------------------------------------------------------------------------------------
 // signs and positivity from the bits: an FP64 comparison takes an FP64 issue slot
@@ -218,11 +221,9 @@ __device__ __forceinline__ bool positive(double x) { return dbits(x) - 1u < 0x7f
 
 __device__ __forceinline__ void hllc(double rL, double uL, double vL, double pL, double rR, double uR,
                                      double vR, double pR, const Gas& g, double F[4]) {
-  const double gpL = g.gamma * pL, gpR = g.gamma * pR;
-  // sound speed a = gp y
-  const double yL = rsqrt_nr(gpL * rL), yR = rsqrt_nr(gpR * rR);
-  const double sL = fmin(fma(-gpL, yL, uL), fma(-gpR, yR, uR));
-  const double sR = fmax(fma(gpL, yL, uL), fma(gpR, yR, uR));
+  const double aL = sound(g.gamma, pL, rL), aR = sound(g.gamma, pR, rR);
+  const double sL = fmin(uL - aL, uR - aR);
+  const double sR = fmax(uL + aL, uR + aR);
   // (products that a later sum or difference could be contracted with are rounded on their own:
   // every kernel that inlines this then gives the same bits)
   const double dL = sL - uL, dR = sR - uR;

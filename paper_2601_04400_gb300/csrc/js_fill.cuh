@@ -119,4 +119,29 @@ __device__ __forceinline__ double cfl_rate(double r, double mx, double my, doubl
   return s;
 }
 
+// The two-pass CFL reduction (js_forward.cu): a rate within CFL_MARGIN/2 of cfl_rate's, by the fast
+// reciprocal where the approximation's error bound holds, else cfl_rate itself
+constexpr double CFL_MARGIN = 4e-6;
+
+__device__ __forceinline__ double cfl_rate_fast(double r, double mx, double my, double E, double gamma, double dx,
+                                                double dy, double idx, double idy, bool two_d) {
+  if (!(r > 1e-290) || !(r < 1e290)) return cfl_rate(r, mx, my, E, gamma, dx, dy, two_d);
+  const double rr = recip(r);
+  const double u = mx * rr, v = my * rr;
+  const double ke = (0.5 * r) * fma(u, u, v * v);
+  const double p = (gamma - 1.0) * (E - ke);
+  // p <= 1e-8 E, p <= 0 or NaN: the approximation's error bound does not hold
+  if (!(p > 1e-8 * E) || !(E < 1e290)) return cfl_rate(r, mx, my, E, gamma, dx, dy, two_d);
+  const double c2 = (gamma * p) * rr;
+  const double a = (c2 > 1e-290) ? c2 * rsqrt_nr(c2) : sqrt(c2);
+  double s = (fabs(u) + a) * idx;
+  if (two_d) s = fma(fabs(v) + a, idy, s);
+  return s;
+}
+
+// bitwise equality of two states (identical states have identical IEEE rates)
+__device__ __forceinline__ bool same_bits(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b);
+}
+
 }  // namespace js

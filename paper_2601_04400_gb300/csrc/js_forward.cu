@@ -2,9 +2,8 @@
 //   bc_fill      domain halos (transmissive / reflective / periodic / inflow), 3 deep
 //   ib_fill      ghost-cell immersed boundary: slip-wall mirror of the bilinear image-point
 //                interpolation of fluid cells (Sec. 2, Fig. 1(c))
-//   stage2d      one fused kernel per Runge-Kutta stage: conserved tile + halo -> primitives
-//                in shared memory -> fluxes of the x lines, then of the y lines (WENO5, HLLC,
-//                viscous flux, divergence) into a shared accumulator -> RK stage combination
+//   stage        two kernels per Runge-Kutta stage: lines (primitives, WENO5, HLLC, viscous flux:
+//                flux differences of the x and y lines) and cells (divergence, RK combination)
 //   stage1d      the same along a single line (ny == 1)
 //   cfl_reduce   maximum wave speed and minimum density (bit-exact IEEE arithmetic)
 #include <cuda_runtime.h>
@@ -99,24 +98,6 @@ __global__ void prim_to_cons_kernel(const double* W, double* U, long long n, dou
 // always a pass-2 candidate, and the result is the one-pass IEEE maximum for every state.
 // A non-physical fluid cell has the rate +infinity in both passes (cfl_rate).
 // =======================================================================================
-constexpr double CFL_MARGIN = 4e-6;
-
-__device__ __forceinline__ double cfl_rate_fast(double r, double mx, double my, double E, double gamma, double dx,
-                                                double dy, double idx, double idy, bool two_d) {
-  if (!(r > 1e-290) || !(r < 1e290)) return cfl_rate(r, mx, my, E, gamma, dx, dy, two_d);
-  const double rr = recip(r);
-  const double u = mx * rr, v = my * rr;
-  const double ke = (0.5 * r) * fma(u, u, v * v);
-  const double p = (gamma - 1.0) * (E - ke);
-  // p <= 1e-8 E, p <= 0 or NaN: the approximation's error bound does not hold
-  if (!(p > 1e-8 * E) || !(E < 1e290)) return cfl_rate(r, mx, my, E, gamma, dx, dy, two_d);
-  const double c2 = (gamma * p) * rr;
-  const double a = (c2 > 1e-290) ? c2 * rsqrt_nr(c2) : sqrt(c2);
-  double s = (fabs(u) + a) * idx;
-  if (two_d) s = fma(fabs(v) + a, idy, s);
-  return s;
-}
-
 // block maximum (thread 0 holds it) and, when rmin != nullptr, block minimum
 __device__ __forceinline__ void cfl_block_reduce(double& rate, double* rmin) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -177,11 +158,6 @@ __global__ void cfl_pass1_kernel(CflSrc q, long long n, int two_d,
     atomicMax(&red[2], (unsigned long long)__double_as_longlong(rate));
     atomicMin(&red[1], (unsigned long long)__double_as_longlong(rmin));
   }
-}
-
-// bitwise equality of two states (identical states have identical IEEE rates)
-__device__ __forceinline__ bool same_bits(double a, double b) {
-  return __double_as_longlong(a) == __double_as_longlong(b);
 }
 
 // A candidate cell whose left neighbour in its row is a fluid cell with the identical state
@@ -288,27 +264,22 @@ __device__ __forceinline__ bool stage_constants(const StageArgs& a0, StageArgs& 
   return a0.dtc[4] != 0.0;
 }
 
-// persistent stage kernel of NW warps a block: blocks stride over the tiles, staged by TMA (tensor
-// map of the stage input as a grid constant) or by plain loads; with IMG the neural flux's face
-// images of the stage input go to a.img.
-// 7 warps (4 lines each in both directions), 3 blocks an SM: 21 warps at 96 registers.  14 warps
-// for grids of few tiles, where a tile's latency counts.
-template <int NW, bool VISC, bool RHS, bool TMA, bool IMG>
-__global__ void __launch_bounds__(32 * NW, NW == 7 ? 3 : 1)
-stage2d_kernel(StageArgs a0, int ntx, int ntiles, const __grid_constant__ TensorMap128 tmap) {
+// x line blocks, then y line blocks; B: resident blocks an SM the registers are allotted for
+template <bool VISC, bool IMG, int B>
+__global__ void __launch_bounds__(32 * SLINES, B) stage_lines_kernel(StageArgs a, int bx) {
+  if (a.dtc != nullptr && a.dtc[4] == 0.0) return;  // an inactive device-sized step
+  __shared__ double smem[stage_smem<VISC>() / sizeof(double)];
+  const int b = blockIdx.x;
+  stage_lines<VISC, IMG>(a, b < bx ? 0 : 1, b < bx ? b : b - bx, smem);
+}
+
+template <bool RHS>
+__global__ void __launch_bounds__(128) stage_cells_kernel(StageArgs a0) {
   StageArgs a;
   if (!stage_constants(a0, a)) return;
-  extern __shared__ __align__(128) double smem[];
-  __shared__ __align__(8) unsigned long long bar;
-  if (TMA) {
-    if (threadIdx.x == 0) mbar_init(&bar);
-    __syncthreads();
-  }
-  unsigned phase = 0;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    stage_tile<VISC, RHS, TMA, IMG>(a, t % ntx, t / ntx, smem, &tmap, &bar, &phase);
-    __syncthreads();
-  }
+  const int gi = blockIdx.x * 128 + threadIdx.x;
+  if (gi >= a.lay.nx) return;
+  for (int gj = blockIdx.y; gj < a.lay.ny; gj += gridDim.y) stage_cell<RHS>(a, gi, gj);
 }
 
 // one line (ny == 1): a warp per 28 cells
@@ -317,10 +288,10 @@ __global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
   StageArgs a;
   if (!stage_constants(a0, a)) return;
   constexpr int NPL = VISC ? 5 : 4;
-  constexpr int PS = TILE_B;
+  constexpr int PS = SB;
   __shared__ double sq[NPL * PS];
   const Gas g{a.gamma, a.gm1, a.g1};
-  const int tx0 = blockIdx.x * TILE, lane = threadIdx.x;
+  const int tx0 = blockIdx.x * SCHUNK, lane = threadIdx.x;
   const int W = a.lay.nx + 6;
   for (int col = lane; col < PS; col += 32) {
     const int gx = tx0 + col;
@@ -337,74 +308,62 @@ __global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
   }
   __syncwarp();
   const int k = lane - 2, gi = tx0 + k;
-  double dF[4], upd[4];
-  line_fluxes<VISC, false>(sq + k + 3, PS, 1, 0, 1, g, a.vx, dF);
+  double dF[4];
+  line_fluxes<VISC, false>(sq + k + 3, PS, 0, 1, g, a.vx, dF);
   if (lane < 2 || lane > 29 || gi >= a.lay.nx) return;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) upd[c] = fma(-a.cx, dF[c], RHS ? 0.0 : a.Uin[c * a.lay.plane + a.lay.idx(gi, 0)]);
-  finish_cell<RHS>(a, gi, 0, upd, sq[k + 3], sq[3 * PS + k + 3]);
+  if (!(positive(sq[k + 3]) && positive(sq[3 * PS + k + 3]))) atomicOr(a.err, ERR_NONPHYSICAL_BIT);
+  finish_cell<RHS>(a, gi, 0, dF, dF);
 }
 
 // =======================================================================================
 // launchers
 // =======================================================================================
 namespace {
-template <int NW, bool VISC, bool RHS, bool TMA, bool IMG>
-cudaError_t launch_stage2d_nw(const StageArgs& a, const TensorMap128* tmap, int ntx, int ntiles, cudaStream_t s) {
-  using S = StageTile<VISC>;
-  auto k = stage2d_kernel<NW, VISC, RHS, TMA, IMG>;
-  static int resident = 0;  // blocks resident on the whole GPU
-  if (resident == 0) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * NW, S::SMEM);
-    if (e != cudaSuccess) return e;
-    resident = sms * (per_sm > 0 ? per_sm : 1);
+// Resident blocks an SM the registers are allotted for: 4 (64 registers, 32 warps) hides the FP64
+// and integer latencies best (2048x1024 viscous step: 4 blocks 2.42 ms, 3 blocks 2.50, 2 blocks
+// 2.96).  Tuning variants 1 and 2 are 3 and 2 blocks; every variant gives the same bits.
+template <bool VISC, bool IMG>
+cudaError_t launch_lines(const StageArgs& a, int variant, cudaStream_t s) {
+  const int bx = stage_blocks(a.lay, 0), n = bx + stage_blocks(a.lay, 1);
+  if constexpr (!IMG) {
+    if (variant == 1 || variant == 2) {
+      if (variant == 1) stage_lines_kernel<VISC, IMG, 3><<<n, 32 * SLINES, 0, s>>>(a, bx);
+      else stage_lines_kernel<VISC, IMG, 2><<<n, 32 * SLINES, 0, s>>>(a, bx);
+      return cudaGetLastError();
+    }
   }
-  static const TensorMap128 none{};
-  k<<<ntiles < resident ? ntiles : resident, 32 * NW, S::SMEM, s>>>(a, ntx, ntiles, TMA ? *tmap : none);
+  stage_lines_kernel<VISC, IMG, 4><<<n, 32 * SLINES, 0, s>>>(a, bx);
   return cudaGetLastError();
 }
 
-template <bool VISC, bool RHS, bool IMG = false>
-cudaError_t launch_stage2d(const StageArgs& a, int variant, const TensorMap128* tmap, cudaStream_t s) {
-  const int ntx = (a.lay.nx + TILE - 1) / TILE, nty = (a.lay.ny + TILE - 1) / TILE, ntiles = ntx * nty;
-  if constexpr (!IMG) {
-    // blocks of 14 warps take a tile in half the time; worth it while every tile has its SM
-    const bool wide = variant == 2 || variant == 3 || (variant != 1 && variant != 4 && ntiles <= 152);
-    if (wide)
-      return tmap ? launch_stage2d_nw<14, VISC, RHS, true, IMG>(a, tmap, ntx, ntiles, s)
-                  : launch_stage2d_nw<14, VISC, RHS, false, IMG>(a, tmap, ntx, ntiles, s);
-  }
-  return tmap ? launch_stage2d_nw<7, VISC, RHS, true, IMG>(a, tmap, ntx, ntiles, s)
-              : launch_stage2d_nw<7, VISC, RHS, false, IMG>(a, tmap, ntx, ntiles, s);
+template <bool VISC, bool IMG = false>
+cudaError_t launch_stage2d(const StageArgs& a, bool rhs, int variant, cudaStream_t s) {
+  const cudaError_t e = launch_lines<VISC, IMG>(a, variant, s);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((a.lay.nx + 127) / 128, a.lay.ny < 65535 ? a.lay.ny : 65535);
+  if (rhs) stage_cells_kernel<true><<<grid, 128, 0, s>>>(a);
+  else stage_cells_kernel<false><<<grid, 128, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 template <bool VISC, bool RHS>
 cudaError_t launch_stage1d(const StageArgs& a, cudaStream_t s) {
-  stage1d_kernel<VISC, RHS><<<(a.lay.nx + TILE - 1) / TILE, 32, 0, s>>>(a);
+  stage1d_kernel<VISC, RHS><<<stage_chunks(a.lay.nx), 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 }  // namespace
 
-cudaError_t launch_stage_img(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s) {
+cudaError_t launch_stage_img(const StageArgs& a, bool visc, cudaStream_t s) {
   if (a.lay.ny == 1 || a.img == nullptr) return cudaErrorInvalidValue;
-  return visc ? launch_stage2d<true, false, true>(a, 0, tmap, s)
-              : launch_stage2d<false, false, true>(a, 0, tmap, s);
+  return visc ? launch_stage2d<true, true>(a, false, 0, s) : launch_stage2d<false, true>(a, false, 0, s);
 }
 
-cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, const TensorMap128* tmap,
-                         cudaStream_t s) {
+cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, cudaStream_t s) {
   if (a.lay.ny == 1) {
     if (visc) return rhs ? launch_stage1d<true, true>(a, s) : launch_stage1d<true, false>(a, s);
     return rhs ? launch_stage1d<false, true>(a, s) : launch_stage1d<false, false>(a, s);
   }
-  if (visc)
-    return rhs ? launch_stage2d<true, true>(a, variant, tmap, s) : launch_stage2d<true, false>(a, variant, tmap, s);
-  return rhs ? launch_stage2d<false, true>(a, variant, tmap, s) : launch_stage2d<false, false>(a, variant, tmap, s);
+  return visc ? launch_stage2d<true>(a, rhs, variant, s) : launch_stage2d<false>(a, rhs, variant, s);
 }
 
 cudaError_t launch_bc_fill(double* U, const Lay& lay, const BcArgs& bc, cudaStream_t s) {

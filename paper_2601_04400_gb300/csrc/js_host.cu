@@ -1,6 +1,5 @@
 // Host side of libjaxshock.so: solver contexts, immersed-boundary precomputation and the
 // C ABI declared in include/jaxshock.h.
-#include <cuda.h>  // tensor-map types only; the encoder is looked up at run time
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -63,6 +62,7 @@ struct js_ctx {
   // neural flux (js_set_neural)
   bool nn_on = false;
   js::NnArgs nn;
+  double* dF = nullptr;         // stage scratch: flux differences (8 padded planes; 2D)
   double* nnQ = nullptr;        // primitives of the stage input (4 planes)
   double* nn_lam = nullptr;     // reverse: lambda' of the stage (4 padded planes)
   double* nn_fadj = nullptr;    // reverse: face-state adjoints of the network (16 planes)
@@ -76,7 +76,6 @@ struct js_ctx {
   int variant = 0;  // stage-kernel tile shape (js_set_tuning)
   int arith = JS_ARITH_FAST;  // js_set_arith
   js::IeeeBufs ieee = {nullptr, nullptr, nullptr};  // workspace of JS_ARITH_IEEE
-  std::vector<std::pair<const double*, js::TensorMap128>> tmaps;  // TMA maps of stage inputs
   // tape: per slot the three filled stage states of one recorded step
   std::vector<double*> tape;
   // y slab of a decomposed grid (js_create_slab): local row k is global row
@@ -277,6 +276,7 @@ StageArgs base_args(const js_ctx* c) {
   StageArgs a;
   std::memset(&a, 0, sizeof(a));
   a.tag = c->tag;
+  a.dF = c->dF;
   a.err = c->err;
   a.lay = c->lay;
   a.gamma = c->p.gamma;
@@ -298,47 +298,6 @@ int fill_halos(js_ctx* c, double* X, bool ieee = false) {
   JS_CUDA(js::launch_bc_fill(X, c->lay, c->bc, c->stream));
   c->launches += (c->n_ghost > 0) ? 2 : 1;
   return JS_OK;
-}
-
-// cuTensorMapEncodeTiled from the driver, looked up once through the runtime
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
-  }
-  return fn;
-}
-
-// Tensor map of a padded state buffer: 3D (column, row, plane) FP64 tensor, box of the
-// 28x28 tile with its 3-cell halo and all 4 planes; reads past the array return zeros.
-const js::TensorMap128* stage_tmap(js_ctx* c, const double* buf) {
-  if (c->lay.ny == 1) return nullptr;
-  for (auto& e : c->tmaps)
-    if (e.first == buf) return &e.second;
-  EncodeTiledFn enc = encode_tiled();
-  if (!enc) return nullptr;
-  static_assert(sizeof(CUtensorMap) == sizeof(js::TensorMap128), "tensor map size");
-  js::TensorMap128 m;
-  const cuuint64_t dims[3] = {(cuuint64_t)c->lay.pitch, (cuuint64_t)c->lay.H, 4};
-  const cuuint64_t strides[2] = {(cuuint64_t)c->lay.pitch * sizeof(double), (cuuint64_t)c->lay.plane * sizeof(double)};
-  const cuuint32_t box[3] = {js::TMA_BOX, js::TMA_BOX, 4};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = enc(reinterpret_cast<CUtensorMap*>(&m), CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)buf, dims,
-                         strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return nullptr;
-  c->tmaps.push_back({buf, m});
-  return &c->tmaps.back().second;
 }
 
 // neural flux of the stage input a.Uin (before the stage kernel) and its divergence
@@ -379,13 +338,13 @@ int stage_img(js_ctx* c, StageArgs a, bool visc) {
   a.img_g1 = (float)(1.0 / (c->p.gamma - 1.0));
   const bool timed = c->profiling && c->ev_used + 2 <= (int)c->ev.size();
   if (timed) JS_CUDA(cudaEventRecord(c->ev[c->ev_used], c->stream));
-  JS_CUDA(js::launch_stage_img(a, visc, stage_tmap(c, a.Uin), c->stream));
+  JS_CUDA(js::launch_stage_img(a, visc, c->stream));
   if (timed) {
     JS_CUDA(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
     c->ev_used += 2;
   }
   JS_CUDA(js::nn_layers(c->nn, c->stream));
-  c->launches += 4;
+  c->launches += 5;
   return nn_after(c, a, false);
 }
 
@@ -396,14 +355,12 @@ int stage(js_ctx* c, const StageArgs& a, bool visc, bool rhs) {
   if (rc) return rc;
   const bool timed = c->profiling && c->ev_used + 2 <= (int)c->ev.size();
   if (timed) JS_CUDA(cudaEventRecord(c->ev[c->ev_used], c->stream));
-  // tile variants: 0 the library's choice, 1 / 3 plain loads, 2 / 4 TMA; 1, 4: 7 warps a block, 2, 3: 14
-  const js::TensorMap128* tm = (c->variant != 1 && c->variant != 3) ? stage_tmap(c, a.Uin) : nullptr;
-  JS_CUDA(js::launch_stage(a, visc, rhs, c->variant, tm, c->stream));
+  JS_CUDA(js::launch_stage(a, visc, rhs, c->variant, c->stream));
   if (timed) {
     JS_CUDA(cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
     c->ev_used += 2;
   }
-  ++c->launches;
+  c->launches += (c->g.ny > 1) ? 2 : 1;
   return nn_after(c, a, rhs);
 }
 
@@ -426,6 +383,7 @@ void js_internal_desc(js_ctx* c, js::InstDesc* d) {
   d->N = c->N;
   d->A = c->A;
   d->B = c->B;
+  d->dF = c->dF;
   d->tag = c->tag;
   d->ib = ib_args(c);
   d->bc = c->bc;
@@ -463,7 +421,7 @@ const char* js_strerror(int code) {
 void js_destroy(js_ctx* c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream); else cudaDeviceSynchronize();
-  cudaFree(c->N); cudaFree(c->A); cudaFree(c->B);
+  cudaFree(c->N); cudaFree(c->A); cudaFree(c->B); cudaFree(c->dF);
   cudaFree(c->tag);
   cudaFree(c->ib_dst); cudaFree(c->ib_src); cudaFree(c->ib_w); cudaFree(c->ib_nrm);
   cudaFree(c->err); cudaFree(c->red); cudaFree(c->cfl_bmax); cudaFree(c->dtc);
@@ -519,6 +477,7 @@ int create_ctx(const js_grid* grid, const js_params* params, const js_boundary* 
   const size_t bytes = sizeof(double) * 4 * (size_t)L.plane;
   if (cudaMalloc(&c->N, bytes) != cudaSuccess || cudaMalloc(&c->A, bytes) != cudaSuccess ||
       cudaMalloc(&c->B, bytes) != cudaSuccess || cudaMalloc(&c->err, sizeof(int)) != cudaSuccess ||
+      (grid->ny > 1 && cudaMalloc(&c->dF, 2 * bytes) != cudaSuccess) ||
       cudaMalloc(&c->red, 4 * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMalloc(&c->cfl_bmax, sizeof(double) * js::CFL_MAX_BLOCKS) != cudaSuccess ||
       cudaMalloc(&c->dtc, sizeof(double) * js::DTC_N) != cudaSuccess) {

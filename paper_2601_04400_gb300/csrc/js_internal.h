@@ -11,6 +11,7 @@ struct StageArgs {
   const double* Un;          // padded U^n (RK combination), may alias Uout
   double* Uout;              // padded stage output, or [4][ny][nx] in RHS mode
   const unsigned char* tag;  // [ny][nx] cell tags (0 fluid) or nullptr
+  double* dF;                // scratch: flux differences of the x, then of the y lines (8 padded planes)
   int* err;                  // device error flag
   Lay lay;
   double gamma, gm1, g1;
@@ -160,6 +161,7 @@ struct InstDesc {
   double* A;
   double* B;
   double* U;                 // user state [4][ny][nx]
+  double* dF;                // stage scratch (8 padded planes)
   const unsigned char* tag;
   IbArgs ib;
   BcArgs bc;
@@ -183,17 +185,9 @@ struct InstRev {
   double* qIb;
   double* ppart;             // warp partials of the parameter gradient
   int tmax;                  // max(nx + 6, ny): inflow_part row length
-  long long w_lines;         // warp slots of its line blocks
+  long long w_lines;         // slots of its line blocks
   long long off_c, w_c, off_g, w_g, off_s, w_s;  // slots of cells, IB ghost, IB source
 };
-
-// opaque 128-byte, 64-byte aligned tensor map (CUtensorMap) for TMA copies
-struct alignas(64) TensorMap128 {
-  unsigned long long opaque[16];
-};
-
-// box of the TMA-staged stage tile (28x28 cells + 3-cell halo, 4 planes)
-constexpr int TMA_BOX = 34;
 
 // IEEE-order arithmetic mode (js_ieee.cu): padded primitives Q (4 planes of lay.plane),
 // x-face fluxes F [4][ny][nx+1], y-face fluxes G [4][ny+1][nx]
@@ -209,10 +203,9 @@ cudaError_t launch_ieee_stage(const StageArgs& a, const IeeeBufs& b, double dt, 
 // (a.dtc set: dt = a.dtc[5], and the stage does nothing when a.dtc[4] == 0)
 
 constexpr int STAGE_VARIANTS = 5;
-cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, const TensorMap128* tmap,
-                         cudaStream_t s);
+cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, cudaStream_t s);
 // stage update that also writes the neural flux's face images of its input to a.img (2D)
-cudaError_t launch_stage_img(const StageArgs& a, bool visc, const TensorMap128* tmap, cudaStream_t s);
+cudaError_t launch_stage_img(const StageArgs& a, bool visc, cudaStream_t s);
 cudaError_t launch_bc_fill(double* U, const Lay& lay, const BcArgs& bc, cudaStream_t s);
 cudaError_t launch_ib_fill(double* U, const Lay& lay, const IbArgs& ib, double gamma, int wall, cudaStream_t s);
 cudaError_t launch_pack(const double* U, double* P, const Lay& lay, cudaStream_t s);

@@ -53,6 +53,29 @@ __device__ __forceinline__ const T* chan_img(const void* base, int C, int d, lon
 __device__ __forceinline__ double act_tanh(double x) { return tanh(x); }
 __device__ __forceinline__ float act_tanh(float x) { return tanhf(x); }
 
+// shared-memory addresses and mbarriers; waits are bounded (budget in SM clock cycles)
+__device__ __forceinline__ unsigned smem_u32(const void* p) {
+  return (unsigned)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+// wait for the mbarrier phase `parity` to complete, for at most `budget` SM clock cycles
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, long long budget) {
+  const long long t0 = clock64();
+  while (true) {
+    unsigned ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (clock64() - t0 > budget) return false;
+  }
+}
+
 // two floats rounded to BF16 (to nearest even) and packed, lo in the low half; eight of them as
 // one 16-byte value (built in registers, not through a local array)
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {

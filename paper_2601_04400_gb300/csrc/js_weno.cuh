@@ -2,14 +2,15 @@
 // arithmetic (js_wide.cuh says why), cell-centred: both face states of a cell share its three
 // smoothness indicators, and an indicator is formed once for the three cells it serves.
 //
-// The differences d_{j+1/2} = q_{j+1} - q_j and the two final q + c/6 stay FP64 (3 instructions a
-// cell, variable and direction, where the whole evaluation took 48); what lies between works on
-// 58- to 64-bit mantissas with explicit exponents:
-//   * the differences are brought to the largest one's exponent (of the pair for an indicator, of
-//     the stencil for the candidate corrections): absolute error 2^-59 of the largest;
+// Everything from the cell values to the face states (48 FP64 instructions a cell, variable and
+// direction) works on 58- to 64-bit mantissas with explicit exponents:
+//   * the differences d_{j+1/2} = q_{j+1} - q_j are exact, or to 2^-57 where the values' exponents
+//     differ; they are brought to the largest one's exponent (of the pair for an indicator, of the
+//     stencil for the candidate corrections): absolute error 2^-59 of the largest;
 //   * indicators, their products and squares are normalised or leave 60 bits; the weights are
 //     brought to a common scale on which their sum has 60 to 62 bits;
-//   * the quotient takes a 58-bit reciprocal and is rounded to 53 bits at the end.
+//   * the quotient takes a 58-bit reciprocal; the cell value and a sixth of the quotient are added
+//     as integers and the sum is rounded to 53 bits, the only rounding.
 // The face state's error is that of its final rounding plus about 2^-57 of the largest
 // difference: at or below the FP64 sequence's on smooth, noisy and discontinuous data alike, as
 // long as the largest difference of the stencil is below 16 |q|.  Where it is not (density or
@@ -21,17 +22,30 @@
 
 namespace js {
 
-// a first difference d as m 2^(e - 1081): |m| in [2^58, 2^59), or 0
+// a cell value as m 2^(e - 1080): |m| in [2^57, 2^58), or 0
+struct Qx {
+  s64 m;
+  s32 e;
+};
+JS_HD Qx qx_of(double q) {
+  const u64 b = dbits(q);
+  const s32 e = expo(q);
+  const u64 M = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 5;
+  const u64 s = (u64)(s64)((s32)hi32(b) >> 31);
+  return Qx{e == 0 ? 0 : (s64)((M ^ s) - s), e};
+}
+// a first difference as m 2^(e - 1081): |m| in [2^58, 2^59), or 0 with e = 0; e = 2047 where a value
+// is not finite or above 2^477
 struct Fx {
   s64 m;
   s32 e;
 };
-JS_HD Fx fx_of(double d) {
-  const u64 b = dbits(d);
-  const s32 e = expo(d);
-  const u64 M = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 6;
-  const u64 s = (u64)(s64)((s32)hi32(b) >> 31);
-  return Fx{e == 0 ? 0 : (s64)((M ^ s) - s), e};
+JS_HD Fx fx_of(const Qx& hi, const Qx& lo) {
+  const int E = imax(hi.e, lo.e);
+  const s64 d = sar(hi.m, E - hi.e) - sar(lo.m, E - lo.e);
+  const s64 sg = d >> 63;
+  const int up = clz64((u64)((d ^ sg) - sg)) - 5;
+  return Fx{(s64)((u64)d << (up & 63)), E > 1500 ? 2047 : d == 0 ? 0 : E + 1 - up};
 }
 
 // three times a smoothness indicator, 3 (4 beta_k + 4 eps) = m 2^(x - 2100), 2^63 <= m < 2^64
@@ -40,8 +54,8 @@ struct Sm {
   s32 x;
 };
 JS_HD Sm sm_norm(u64 s, int x2) {
-  const int lz = clz64(s);
-  return Sm{s << (lz & 63), x2 - lz};
+  const int lz = clz32(hi32(s));  // (never below 2^54)
+  return Sm{s << lz, x2 - lz};
 }
 
 // 3 (4 eps) 2^76, and the exponent of d at which the indicators hold it at that scale: pairs of
@@ -85,10 +99,21 @@ JS_HD Wgt weno_weights(const Sm& s0, const Sm& s1, const Sm& s2) {
   return g;
 }
 
-// c_L = 6 (q_{i+1/2}^L - q_i) and c_R = 6 (q_{i-1/2}^R - q_i) of cell i from its four differences
-// (F: the largest's exponent) and three indicators
-JS_HD void weno_corr(const Fx& dm2, const Fx& dm1, const Fx& dp1, const Fx& dp2, const Sm& s0, const Sm& s1,
-                     const Sm& s2, int F, double& cL, double& cR) {
+// q_i + num / (6 den), num on the scale 2^(F - 1081 + 62), as a double
+JS_HD double weno_face(const Qx& q0, s64 num, u64 den, int F) {
+  const u64 d3 = 3u * den;  // below 2^64
+  const int lz = clz32(hi32(d3));
+  // C 2^(x - 1080) is the correction, |C| below 2^60
+  const s64 C = mul62(limbs(num), limbs((s64)recip_top(d3 << lz)));
+  const int x = F + lz - 3;
+  const int E = imax(q0.e, x);
+  return fix_to_double(sar(q0.m, E - q0.e) + sar(C, E - x), E + 6);
+}
+
+// Face states of cell i at i+1/2 (left-biased) and i-1/2 (right-biased) from its value, its four
+// differences (F: the largest's exponent) and three indicators
+JS_HD void weno_faces(const Qx& q0, const Fx& dm2, const Fx& dm1, const Fx& dp1, const Fx& dp2, const Sm& s0,
+                      const Sm& s1, const Sm& s2, int F, double& Lf, double& Rf) {
   const Wgt g = weno_weights(s0, s1, s2);
   const s64 w6 = 6 * g.w1;
   // differences on the scale of the largest
@@ -96,19 +121,15 @@ JS_HD void weno_corr(const Fx& dm2, const Fx& dm1, const Fx& dp1, const Fx& dp2,
   const Limb l6 = limbs(w6);
   {  // linear weights 1 : 6 : 3
     const s64 w2_3 = 3 * g.w2;
-    const u64 den = (u64)(g.w0 + w6 + w2_3);
     const s64 num = mul62(limbs(g.w0), limbs(5 * b - 2 * a)) + mul62(l6, limbs(b + 2 * c)) +
                     mul62(limbs(w2_3), limbs(4 * c - d));
-    const int lz = clz32(hi32(den));
-    cL = fix_to_double(mul62(limbs(num), limbs((s64)recip_top(den << lz))), F + lz + 4);
+    Lf = weno_face(q0, num, (u64)(g.w0 + w6 + w2_3), F);
   }
   {  // 3 : 6 : 1
     const s64 w0_3 = 3 * g.w0;
-    const u64 den = (u64)(w0_3 + w6 + g.w2);
     const s64 num = mul62(limbs(w0_3), limbs(a - 4 * b)) + mul62(l6, limbs(-2 * b - c)) +
                     mul62(limbs(g.w2), limbs(2 * d - 5 * c));
-    const int lz = clz32(hi32(den));
-    cR = fix_to_double(mul62(limbs(num), limbs((s64)recip_top(den << lz))), F + lz + 4);
+    Rf = weno_face(q0, num, (u64)(w0_3 + w6 + g.w2), F);
   }
 }
 

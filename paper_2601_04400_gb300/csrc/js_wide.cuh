@@ -190,6 +190,21 @@ JS_HD double rsqrt_wide(double x) {
   return pack62(rsqrt_top(mant64(x) >> odd), 1023 - ((e + odd) >> 1));
 }
 
+// sqrt(g p / r) (rounded from about 57 bits) for positive normal g, p, r: g p and its product with
+// 1/sqrt(g p r), all in 64-bit mantissas
+JS_HD double sound_wide(double g, double p, double r) {
+  const int e = expo(g) + expo(p);
+  const u64 gp = mul_top(mant64(g), mant64(p));  // g p = gp 2^(e - 2108)
+  const u64 z = mul_top(gp, mant64(r));          // g p r = z 2^(e + e_r - 3130)
+  const int lz = clz32(hi32(z));
+  const int X = e + expo(r) - 3066 - lz, odd = X & 1;  // g p r = (n / 2^64) 2^X, X even after the shift
+  const u64 A = mul_top(gp, rsqrt_top((z << lz) >> odd) << 2);
+  const int l2 = clz32(hi32(A));
+  const u64 m = A << l2;
+  const int be = e - 1021 - l2 - ((X + odd) >> 1);
+  return bitsd(((u64)(u32)(be - 1) << 52) + (m >> 11) + ((m >> 10) & 1u));
+}
+
 // a signed fixed-point value c 2^(e - 1086) as a double (rounded at 53 bits):
 // c / 2^63 in [1/2, 1) has the biased exponent e.  Values below the normal range give 0.
 JS_HD double fix_to_double(s64 c, int e) {
