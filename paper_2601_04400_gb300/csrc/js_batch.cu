@@ -1,19 +1,18 @@
 // Batched path: many independent flow instances (uneven grids, parameters, bodies) advanced
-// together in ONE persistent cooperative kernel launch -- the GB300 counterpart of mapping the
-// solver step over a batch of problems (the paper's vmap, Sec. 1).
+// together, every launch working on all of them -- the GB300 counterpart of mapping the solver step
+// over a batch of problems (the paper's vmap, Sec. 1).
 //
-// The kernel runs every phase of every step for all instances, separated by grid barriers:
 //   pack       user states -> padded buffers
 //   per step:  CFL        per-instance max wave-speed rate and min density (atomics): fast rates,
 //                         then IEEE rates near the maximum, as js_max_dt
+//              dt         each instance's step size (js_max_dt's arithmetic) and stage constants
 //              per stage: IB fill | halo fill | lines | cells (the per-grid kernels' device
 //                         functions, so trajectories equal js_step's bit for bit)
 //   unpack     padded buffers -> user states
-// Each instance's dt is computed on the device from its reduction (same arithmetic as
-// js_max_dt).  Work items (tiles, ghosts, halo cells) of all instances are distributed
-// round-robin over the resident blocks.  Every barrier wait is bounded: a block that waits
-// longer than the budget sets JS_ERR_TIMEOUT in the error flag and returns, and the others
-// leave at their next wait.
+// The forward runs these phases as ordinary launches on the batch's stream.  The reverse step does so
+// too or runs its phases in one persistent cooperative launch separated by grid barriers; every
+// barrier wait is bounded: a block that waits longer than the budget sets JS_ERR_TIMEOUT in the error
+// flag and returns, and the others leave at their next wait.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -111,10 +110,6 @@ __device__ bool grid_sync_on(unsigned* bar, int* err, int extra_arrivals, long l
   __syncthreads();
   return s_ok != 0;
 }
-__device__ __forceinline__ bool grid_sync(const BatchArgs& b) {
-  return grid_sync_on(b.bar, b.err, b.extra_arrivals, b.budget);
-}
-
 __device__ __forceinline__ double inst_dt(const InstDesc& d, const unsigned long long* red, double cfl) {
   const double rate = __longlong_as_double((long long)red[0]);
   const double rmin = __longlong_as_double((long long)red[1]);
@@ -143,106 +138,111 @@ __device__ __forceinline__ void fill_stage_args(StageArgs& a, const InstDesc& d,
   a.has_av = d.has_av;
 }
 
-__global__ void __launch_bounds__(FNT, 3) batch_kernel(BatchArgs b) {
-  extern __shared__ double smem[];
+// The phases of one batched forward run, each a launch of its own (kernel boundaries order them): the
+// register allocation and occupancy of a phase are its own, where one persistent kernel held all of
+// them at 80 registers with spills and grid barriers between (32 instances, one step: 3.5 ms
+// persistent).  Every phase is a loop over the work items of all instances.
+enum FwdPhase { FP_PACK, FP_CFL, FP_CFL_IEEE, FP_DT, FP_GHOST, FP_HALO, FP_LINES, FP_CELLS, FP_SAVE, FP_UNPACK };
+
+// VM: the instances of the line phase (1 the viscous ones, 2 the inviscid ones: each kind's launch has
+// its own registers)
+template <int PH, int VM = 0>
+__device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, double* smem) {
   const int ntiles = b.tile0[b.count];
-  const long long nghost = b.ghost0[b.count], nhalo = b.halo0[b.count];
   const int tid = threadIdx.x, lane = threadIdx.x & 31;
-  // ---- pack user states; reset both reduction buffers
+  const int par = step & 1;
+  unsigned long long* red = b.red + 4 * (long long)b.count * par;
+  if constexpr (PH == FP_PACK) {
+    // user states; reset both reduction buffers
   for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-    const int q = it, k = find_inst(b.tile0, b.count, q);
-    const InstDesc& d = b.inst[k];
-    const double* Uk = b.ustate ? b.ustate[k] : d.U;
-    const int t = q - b.tile0[k];
-    const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
-    const long long n = (long long)d.lay.nx * d.lay.ny;
-    for (int e = tid; e < BTX * BTY; e += FNT) {
-      const int i = i0 + (e % BTX), j = j0 + (e / BTX);
-      if (i >= d.lay.nx || j >= d.lay.ny) continue;
-      const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
+      const int q = it, k = find_inst(b.tile0, b.count, q);
+      const InstDesc& d = b.inst[k];
+      const double* Uk = b.ustate ? b.ustate[k] : d.U;
+      const int t = q - b.tile0[k];
+      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+      const long long n = (long long)d.lay.nx * d.lay.ny;
+      for (int e = tid; e < BTX * BTY; e += FNT) {
+        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+        if (i >= d.lay.nx || j >= d.lay.ny) continue;
+        const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) d.N[c * d.lay.plane + p] = Uk[c * n + o];
-    }
-  }
-  if (blockIdx.x == 0)
-    for (int k = tid; k < 2 * b.count; k += FNT) {
-      b.red[4 * k] = b.red[4 * k + 2] = 0ULL;
-      b.red[4 * k + 1] = 0x7ff0000000000000ULL;
-    }
-  if (!grid_sync(b)) return;
-  for (int step = 0; step < b.n_steps; ++step) {
-    const int par = step & 1;
-    unsigned long long* red = b.red + 4 * (long long)b.count * par;
-    // ---- CFL reduction over fluid cells, per instance (skipped with given step sizes)
-    if (!b.dt_in) {
-      __shared__ double sr[FNT / 32], sm[FNT / 32];
-      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-        const int k = find_inst(b.tile0, b.count, it);
-        const InstDesc& d = b.inst[k];
-        const int t = it - b.tile0[k];
-        const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
-        const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
-        double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
-        for (int e = tid; e < BTX * BTY; e += FNT) {
-          const int i = i0 + (e % BTX), j = j0 + (e / BTX);
-          if (i >= d.lay.nx || j >= d.lay.ny) continue;
-          if (d.tag && d.tag[(long long)j * d.lay.nx + i] != 0) continue;
-          const long long p = d.lay.idx(i, j);
-          const double r = d.N[p];
-          rate = fmax(rate, cfl_rate_fast(r, d.N[d.lay.plane + p], d.N[2 * d.lay.plane + p], d.N[3 * d.lay.plane + p],
-                                          d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1));
-          rmin = fmin(rmin, r);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
-          rmin = fmin(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
-        }
-        if (lane == 0) {
-          sr[tid >> 5] = rate;
-          sm[tid >> 5] = rmin;
-        }
-        __syncthreads();
-        if (tid == 0) {
-          for (int w = 1; w < FNT / 32; ++w) {
-            rate = fmax(rate, sr[w]);
-            rmin = fmin(rmin, sm[w]);
-          }
-          b.tmax[it] = rate;
-          atomicMax(red + 4 * k + 2, (unsigned long long)__double_as_longlong(rate));
-          atomicMin(red + 4 * k + 1, (unsigned long long)__double_as_longlong(rmin));
-        }
-        __syncthreads();
+        for (int c = 0; c < 4; ++c) d.N[c * d.lay.plane + p] = Uk[c * n + o];
       }
-      if (!grid_sync(b)) return;
-      // the IEEE rate of the cells near the maximum, once per run of identical cells along a row
-      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-        const int k = find_inst(b.tile0, b.count, it);
-        const double thr = __longlong_as_double((long long)red[4 * k + 2]) * (1.0 - CFL_MARGIN);
-        if (!(b.tmax[it] >= thr)) continue;  // the same for the whole block
-        const InstDesc& d = b.inst[k];
-        const int t = it - b.tile0[k];
-        const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
-        const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
-        double rate = 0.0;
-        for (int e = tid; e < BTX * BTY; e += FNT) {
-          const int i = i0 + (e % BTX), j = j0 + (e / BTX);
-          if (i >= d.lay.nx || j >= d.lay.ny) continue;
-          const unsigned char* tag = d.tag ? d.tag + (long long)j * d.lay.nx + i : nullptr;
-          if (tag && tag[0] != 0) continue;
-          const double* X = d.N + d.lay.idx(i, j);
-          const long long P = d.lay.plane;
-          const double r = X[0], mx = X[P], my = X[2 * P], E = X[3 * P];
-          if (!(cfl_rate_fast(r, mx, my, E, d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1) >= thr)) continue;
-          if (i > 0 && !(tag && tag[-1] != 0) && same_bits(r, X[-1]) && same_bits(mx, X[P - 1]) &&
-              same_bits(my, X[2 * P - 1]) && same_bits(E, X[3 * P - 1]))
-            continue;
-          rate = fmax(rate, cfl_rate(r, mx, my, E, d.gamma, d.dx, d.dy, d.lay.ny > 1));
-        }
-        for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
-        if (lane == 0 && rate > 0.0) atomicMax(red + 4 * k, (unsigned long long)__double_as_longlong(rate));
-      }
-      if (!grid_sync(b)) return;
     }
+    if (blockIdx.x == 0)
+      for (int k = tid; k < 2 * b.count; k += FNT) {
+        b.red[4 * k] = b.red[4 * k + 2] = 0ULL;
+        b.red[4 * k + 1] = 0x7ff0000000000000ULL;
+      }
+  } else if constexpr (PH == FP_CFL) {
+    // per instance the largest fast rate and the smallest density, per tile the largest fast rate
+    __shared__ double sr[FNT / 32], sm[FNT / 32];
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+      const int k = find_inst(b.tile0, b.count, it);
+      const InstDesc& d = b.inst[k];
+      const int t = it - b.tile0[k];
+      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+      const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
+      double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
+      for (int e = tid; e < BTX * BTY; e += FNT) {
+        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+        if (i >= d.lay.nx || j >= d.lay.ny) continue;
+        if (d.tag && d.tag[(long long)j * d.lay.nx + i] != 0) continue;
+        const long long p = d.lay.idx(i, j);
+        const double r = d.N[p];
+        rate = fmax(rate, cfl_rate_fast(r, d.N[d.lay.plane + p], d.N[2 * d.lay.plane + p], d.N[3 * d.lay.plane + p],
+                                        d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1));
+        rmin = fmin(rmin, r);
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
+        rmin = fmin(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+      }
+      if (lane == 0) {
+        sr[tid >> 5] = rate;
+        sm[tid >> 5] = rmin;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        for (int w = 1; w < FNT / 32; ++w) {
+          rate = fmax(rate, sr[w]);
+          rmin = fmin(rmin, sm[w]);
+        }
+        b.tmax[it] = rate;
+        atomicMax(red + 4 * k + 2, (unsigned long long)__double_as_longlong(rate));
+        atomicMin(red + 4 * k + 1, (unsigned long long)__double_as_longlong(rmin));
+      }
+      __syncthreads();
+    }
+  } else if constexpr (PH == FP_CFL_IEEE) {
+    // the IEEE rate of the cells near the maximum, once per run of identical cells along a row
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+      const int k = find_inst(b.tile0, b.count, it);
+      const double thr = __longlong_as_double((long long)red[4 * k + 2]) * (1.0 - CFL_MARGIN);
+      if (!(b.tmax[it] >= thr)) continue;  // the same for the whole block
+      const InstDesc& d = b.inst[k];
+      const int t = it - b.tile0[k];
+      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+      const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
+      double rate = 0.0;
+      for (int e = tid; e < BTX * BTY; e += FNT) {
+        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+        if (i >= d.lay.nx || j >= d.lay.ny) continue;
+        const unsigned char* tag = d.tag ? d.tag + (long long)j * d.lay.nx + i : nullptr;
+        if (tag && tag[0] != 0) continue;
+        const double* X = d.N + d.lay.idx(i, j);
+        const long long P = d.lay.plane;
+        const double r = X[0], mx = X[P], my = X[2 * P], E = X[3 * P];
+        if (!(cfl_rate_fast(r, mx, my, E, d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1) >= thr)) continue;
+        if (i > 0 && !(tag && tag[-1] != 0) && same_bits(r, X[-1]) && same_bits(mx, X[P - 1]) &&
+            same_bits(my, X[2 * P - 1]) && same_bits(E, X[3 * P - 1]))
+          continue;
+        rate = fmax(rate, cfl_rate(r, mx, my, E, d.gamma, d.dx, d.dy, d.lay.ny > 1));
+      }
+      for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
+      if (lane == 0 && rate > 0.0) atomicMax(red + 4 * k, (unsigned long long)__double_as_longlong(rate));
+    }
+  } else if constexpr (PH == FP_DT) {
     if (blockIdx.x == 0) {
       // the other parity was last read in the previous step: reset it for the next one
       unsigned long long* nxt = b.red + 4 * (long long)b.count * (par ^ 1);
@@ -263,109 +263,114 @@ __global__ void __launch_bounds__(FNT, 3) batch_kernel(BatchArgs b) {
         if (b.dt_log) b.dt_log[(long long)step * b.count + k] = dtk;
       }
     }
-    for (int s = 0; s < 3; ++s) {
-      // ---- immersed-boundary ghosts of the stage input
-      for (long long g = (long long)blockIdx.x * FNT + tid; g < nghost; g += (long long)gridDim.x * FNT) {
-        const int k = find_inst64(b.ghost0, b.count, g);
-        const InstDesc& d = b.inst[k];
-        double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
-        ib_fill_one(X, d.lay, d.ib, d.gamma, d.wall, (int)(g - b.ghost0[k]));
-      }
-      if (!grid_sync(b)) return;
-      // ---- domain halos
-      for (long long h = (long long)blockIdx.x * FNT + tid; h < nhalo; h += (long long)gridDim.x * FNT) {
-        const int k = find_inst64(b.halo0, b.count, h);
-        const InstDesc& d = b.inst[k];
-        double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
-        bc_fill_one(X, d.lay, d.bc, h - b.halo0[k]);
-      }
-      if (!grid_sync(b)) return;
-      // ---- lines
-      const int nlines = b.line0[b.count];
-      for (int it = blockIdx.x; it < nlines; it += gridDim.x) {
-        const int q = b.order ? b.order[it] : it, k = find_inst(b.line0, b.count, q);
-        const InstDesc& d = b.inst[k];
-        __shared__ StageArgs sa;  // (in registers they would cost resident warps)
-        if (tid == 0) fill_stage_args(sa, d, (s == 0) ? d.N : ((s == 1) ? d.A : d.B), b.err);
-        __syncthreads();
-        const int t = q - b.line0[k], bx = stage_blocks(d.lay, 0);
-        if (d.visc) stage_lines<true, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
-        else stage_lines<false, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
-        __syncthreads();  // the next block of lines reuses shared memory
-      }
-      if (!grid_sync(b)) return;
-      // ---- cells
-      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-        const int k = find_inst(b.tile0, b.count, it);
-        const InstDesc& d = b.inst[k];
-        const double* dtc = b.dtc + (long long)DTC_N * k;
-        StageArgs a;
-        fill_stage_args(a, d, (s == 0) ? d.N : ((s == 1) ? d.A : d.B), b.err);
-        a.Un = d.N;
-        a.Uout = (s == 0) ? d.A : ((s == 1) ? d.B : d.N);
-        a.cx = dtc[0];
-        a.cy = dtc[1];
-        a.avx = dtc[2];
-        a.avy = dtc[3];
-        a.rk_a = (s == 0) ? 0.0 : ((s == 1) ? 0.75 : 1.0 / 3.0);
-        a.rk_b = (s == 0) ? 1.0 : ((s == 1) ? 0.25 : 2.0 / 3.0);
-        a.use_un = (s > 0) ? 1 : 0;
-        const int t = it - b.tile0[k];
-        const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
-        for (int e = tid; e < BTX * BTY; e += FNT) {
-          const int i = i0 + (e % BTX), j = j0 + (e / BTX);
-          if (i < d.lay.nx && j < d.lay.ny) stage_cell<false>(a, i, j);
-        }
-      }
-      if (!grid_sync(b)) return;
+  } else if constexpr (PH == FP_GHOST) {
+    const long long nghost = b.ghost0[b.count];
+    for (long long g = (long long)blockIdx.x * FNT + tid; g < nghost; g += (long long)gridDim.x * FNT) {
+      const int k = find_inst64(b.ghost0, b.count, g);
+      const InstDesc& d = b.inst[k];
+      double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
+      ib_fill_one(X, d.lay, d.ib, d.gamma, d.wall, (int)(g - b.ghost0[k]));
     }
-    if (b.save || b.save1) {
-      // the state after this step (ghost cells included), before the next step refills them,
-      // and the stage states A, B of this step (their ghost cells were refilled from fluid
-      // cells, which a reverse pass that fills them again reproduces)
-      for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-        const int q = it, k = find_inst(b.tile0, b.count, q);
-        const InstDesc& d = b.inst[k];
-        const long long row = (long long)step * b.count + k;
-        double* S = b.save ? b.save[row] : nullptr;
-        double* S1 = b.save1 ? b.save1[row] : nullptr;
-        double* S2 = b.save1 ? b.save2[row] : nullptr;
-        const int t = q - b.tile0[k];
-        const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
-        const long long n = (long long)d.lay.nx * d.lay.ny;
-        for (int e = tid; e < BTX * BTY; e += FNT) {
-          const int i = i0 + (e % BTX), j = j0 + (e / BTX);
-          if (i >= d.lay.nx || j >= d.lay.ny) continue;
-          const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
+  } else if constexpr (PH == FP_HALO) {
+    const long long nhalo = b.halo0[b.count];
+    for (long long h = (long long)blockIdx.x * FNT + tid; h < nhalo; h += (long long)gridDim.x * FNT) {
+      const int k = find_inst64(b.halo0, b.count, h);
+      const InstDesc& d = b.inst[k];
+      double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
+      bc_fill_one(X, d.lay, d.bc, h - b.halo0[k]);
+    }
+  } else if constexpr (PH == FP_LINES) {
+    const int nlines = b.line0[b.count];
+    for (int it = blockIdx.x; it < nlines; it += gridDim.x) {
+      const int q = b.order ? b.order[it] : it, k = find_inst(b.line0, b.count, q);
+      const InstDesc& d = b.inst[k];
+      if ((VM == 1) != (d.visc != 0)) continue;  // the other launch's instance
+      __shared__ StageArgs sa;  // (in registers they would cost resident warps)
+      if (tid == 0) fill_stage_args(sa, d, (s == 0) ? d.N : ((s == 1) ? d.A : d.B), b.err);
+      __syncthreads();
+      const int t = q - b.line0[k], bx = stage_blocks(d.lay, 0);
+      stage_lines<VM == 1, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+      __syncthreads();  // the next block of lines reuses shared memory
+    }
+  } else if constexpr (PH == FP_CELLS) {
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+      const int k = find_inst(b.tile0, b.count, it);
+      const InstDesc& d = b.inst[k];
+      const double* dtc = b.dtc + (long long)DTC_N * k;
+      StageArgs a;
+      fill_stage_args(a, d, (s == 0) ? d.N : ((s == 1) ? d.A : d.B), b.err);
+      a.Un = d.N;
+      a.Uout = (s == 0) ? d.A : ((s == 1) ? d.B : d.N);
+      a.cx = dtc[0];
+      a.cy = dtc[1];
+      a.avx = dtc[2];
+      a.avy = dtc[3];
+      a.rk_a = (s == 0) ? 0.0 : ((s == 1) ? 0.75 : 1.0 / 3.0);
+      a.rk_b = (s == 0) ? 1.0 : ((s == 1) ? 0.25 : 2.0 / 3.0);
+      a.use_un = (s > 0) ? 1 : 0;
+      const int t = it - b.tile0[k];
+      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+      for (int e = tid; e < BTX * BTY; e += FNT) {
+        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+        if (i < d.lay.nx && j < d.lay.ny) stage_cell<false>(a, i, j);
+      }
+    }
+  } else if constexpr (PH == FP_SAVE) {
+    // the state after this step (ghost cells included), before the next step refills them,
+    // and the stage states A, B of this step (their ghost cells were refilled from fluid
+    // cells, which a reverse pass that fills them again reproduces)
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+      const int q = it, k = find_inst(b.tile0, b.count, q);
+      const InstDesc& d = b.inst[k];
+      const long long row = (long long)step * b.count + k;
+      double* S = b.save ? b.save[row] : nullptr;
+      double* S1 = b.save1 ? b.save1[row] : nullptr;
+      double* S2 = b.save1 ? b.save2[row] : nullptr;
+      const int t = q - b.tile0[k];
+      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+      const long long n = (long long)d.lay.nx * d.lay.ny;
+      for (int e = tid; e < BTX * BTY; e += FNT) {
+        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+        if (i >= d.lay.nx || j >= d.lay.ny) continue;
+        const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            if (S) S[c * n + o] = d.N[c * d.lay.plane + p];
-            if (S1) {
-              S1[c * n + o] = d.A[c * d.lay.plane + p];
-              S2[c * n + o] = d.B[c * d.lay.plane + p];
-            }
+        for (int c = 0; c < 4; ++c) {
+          if (S) S[c * n + o] = d.N[c * d.lay.plane + p];
+          if (S1) {
+            S1[c * n + o] = d.A[c * d.lay.plane + p];
+            S2[c * n + o] = d.B[c * d.lay.plane + p];
           }
         }
       }
-      if (!grid_sync(b)) return;
     }
-  }
-  // ---- unpack
+  } else {
   for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
-    const int q = it, k = find_inst(b.tile0, b.count, q);
-    const InstDesc& d = b.inst[k];
-    double* Uk = b.ustate ? b.ustate[k] : d.U;
-    const int t = q - b.tile0[k];
-    const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
-    const long long n = (long long)d.lay.nx * d.lay.ny;
-    for (int e = tid; e < BTX * BTY; e += FNT) {
-      const int i = i0 + (e % BTX), j = j0 + (e / BTX);
-      if (i >= d.lay.nx || j >= d.lay.ny) continue;
-      const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
+      const int q = it, k = find_inst(b.tile0, b.count, q);
+      const InstDesc& d = b.inst[k];
+      double* Uk = b.ustate ? b.ustate[k] : d.U;
+      const int t = q - b.tile0[k];
+      const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
+      const long long n = (long long)d.lay.nx * d.lay.ny;
+      for (int e = tid; e < BTX * BTY; e += FNT) {
+        const int i = i0 + (e % BTX), j = j0 + (e / BTX);
+        if (i >= d.lay.nx || j >= d.lay.ny) continue;
+        const long long o = (long long)j * d.lay.nx + i, p = d.lay.idx(i, j);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) Uk[c * n + o] = d.N[c * d.lay.plane + p];
+        for (int c = 0; c < 4; ++c) Uk[c * n + o] = d.N[c * d.lay.plane + p];
+      }
     }
   }
+}
+
+template <int PH, int VM = 0>
+__global__ void __launch_bounds__(FNT, PH == FP_LINES ? 4 : 1) batch_phase_kernel(BatchArgs b, int step, int s) {
+  extern __shared__ double smem[];
+  fwd_phase<PH, VM>(b, step, s, smem);
+}
+
+// one grid barrier of the persistent reverse launch (js_batch_test_timeout)
+__global__ void __launch_bounds__(FNT) batch_barrier_kernel(BatchArgs b) {
+  grid_sync_on(b.bar, b.err, b.extra_arrivals, b.budget);
 }
 
 // =======================================================================================
@@ -472,7 +477,8 @@ enum RevPhase {
   RP_N
 };
 
-template <int PH>
+// VM: the instances of the line phases (0 all, 1 the viscous ones, 2 the inviscid ones)
+template <int PH, int VM = 0>
 __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* smem) {
   const RevCall& call = b.call;
   const bool even = (s == 2) || (s == 0);  // reverse stages 2 and 0 read P0, write P1
@@ -518,12 +524,13 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     for (int it = blockIdx.x; it < b.line0[b.count]; it += gridDim.x) {
       const int k = find_inst(b.line0, b.count, it);
       const InstDesc& d = b.inst[k];
+      if ((VM == 1 && !d.visc) || (VM == 2 && d.visc)) continue;  // the other launch's instance
       __shared__ StageArgs sa;
       if (threadIdx.x == 0) fill_stage_args(sa, d, (s == 0) ? d.N : d.A, b.err);
       __syncthreads();
       const int t = it - b.line0[k], bx = stage_blocks(d.lay, 0);
-      if (d.visc) stage_lines<true, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
-      else stage_lines<false, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+      if (VM == 1 || (VM == 0 && d.visc)) stage_lines<true, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+      if (VM == 2 || (VM == 0 && !d.visc)) stage_lines<false, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
       __syncthreads();  // the next block of lines reuses shared memory
     }
   } else if constexpr (PH == RP_STAGE_CELLS) {
@@ -557,13 +564,16 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     for (int it = blockIdx.x; it < b.rblock0[b.count]; it += gridDim.x) {
       const int k = find_inst(b.rblock0, b.count, it);
       const InstDesc& d = b.inst[k];
+      if ((VM == 1 && !d.visc) || (VM == 2 && d.visc)) continue;  // the other launch's instance
       const InstRev& r = b.rev[k];
-      const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
+      __shared__ AdjArgs a;  // (in registers it would cost resident warps)
+      if (threadIdx.x == 0) a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
+      __syncthreads();
       const double* src = even ? r.P0 : r.P1;
       const int t = it - b.rblock0[k], bx = adj_blocks(d.lay, 0);
       const double bdt = REV_B[s] * call.dt[k];
-      if (d.visc) adj_lines<true>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
-      else adj_lines<false>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
+      if (VM == 1 || (VM == 0 && d.visc)) adj_lines<true>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
+      if (VM == 2 || (VM == 0 && !d.visc)) adj_lines<false>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
       __syncthreads();  // the next block of lines reuses shared memory
     }
   } else if constexpr (PH == RP_CELLS) {
@@ -667,10 +677,10 @@ __global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
 }
 
 // one phase of the reverse step as a kernel of its own (split launch)
-template <int PH>
+template <int PH, int VM = 0>
 __global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
   extern __shared__ double smem[];
-  rev_phase<PH>(b, s, smem);
+  rev_phase<PH, VM>(b, s, smem);
 }
 
 // one launch copying every instance's state: dst[k][i] = src[k][i], i < pre[k+1] - pre[k]
@@ -708,7 +718,9 @@ struct js_batch {
   unsigned long long* d_red = nullptr;
   unsigned* d_bar = nullptr;
   int* d_err = nullptr;
-  int blocks = 0;          // persistent blocks of the forward launch (tuning: blocks per SM x SMs)
+  int blocks = 0;          // blocks of the forward's line launch (tuning: blocks per SM x SMs)
+  bool blocks_set = false;  // tuned: that many blocks stride over the lines
+  long long nghost = 0, nhalo = 0;
   int sms = 0, per_sm = 0;  // SMs and the forward kernel's resident blocks per SM
   int schedule = 0;        // tile order of the forward launch (js_batch_set_tuning)
   int* d_order = nullptr;  // its queue -> tile table (schedules 1 and 2)
@@ -723,6 +735,8 @@ struct js_batch {
   int rev_split = 0;                  // 1: one launch per phase (js_batch_set_reverse_launch)
   int rev_pblocks[js::RP_N] = {};     // grid of each phase kernel of the split launch
   int* d_rblock0 = nullptr;            // prefix sums of the reverse line blocks
+  std::vector<int> rblock0;
+  bool has_visc = false, has_inv = false;  // the batch holds viscous / inviscid instances
   void** d_tab = nullptr;       // call table of js_batch_step_vjp: U_n, lam_np1, lam_n, p_bar x count
   double* d_dt = nullptr;       // its step sizes
   // checkpointed rollout reverse (js_batch_rollout_vjp)
@@ -743,7 +757,6 @@ namespace {
 size_t batch_smem() { return js::stage_smem<true>(); }
 constexpr size_t kLineSmem = sizeof(double) * 8 * js::AP;
 size_t rev_smem() { return std::max(batch_smem(), kLineSmem); }
-size_t rev_phase_smem(int ph) { return ph == js::RP_STAGE ? batch_smem() : ph == js::RP_LINES ? kLineSmem : 0; }
 }  // namespace
 
 namespace {
@@ -757,7 +770,8 @@ int rev_prepare(js_batch* b) {
   const int n = b->count;
   std::vector<js::InstRev> rev(n);
   std::vector<long long> pre((size_t)js::RK_N * (n + 1), 0);
-  std::vector<int> rblock0(n + 1, 0);
+  std::vector<int>& rblock0 = b->rblock0;
+  rblock0.assign(n + 1, 0);
   for (int k = 0; k < n; ++k) {
     js::InstRev& r = rev[k];
     const int rc = js_internal_rev_desc(b->ctx[k], &r);
@@ -789,23 +803,18 @@ int rev_prepare(js_batch* b) {
   if (per_sm < 1) return JS_ERR_CUDA;
   b->rev_blocks = sms * per_sm;
   // the split launch: each phase kernel's own resident blocks per SM
-  if (cudaFuncSetAttribute(js::batch_vjp_phase_kernel<js::RP_STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)batch_smem()) != cudaSuccess ||
-      cudaFuncSetAttribute(js::batch_vjp_phase_kernel<js::RP_LINES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kLineSmem) != cudaSuccess)
-    return JS_ERR_CUDA;
   const void* kern[js::RP_N] = {
       (const void*)js::batch_vjp_phase_kernel<js::RP_PACK>, (const void*)js::batch_vjp_phase_kernel<js::RP_GHOST>,
-      (const void*)js::batch_vjp_phase_kernel<js::RP_HALO>, (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE>,
+      (const void*)js::batch_vjp_phase_kernel<js::RP_HALO>, (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE, 1>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE_CELLS>,
-      (const void*)js::batch_vjp_phase_kernel<js::RP_REDUCE>, (const void*)js::batch_vjp_phase_kernel<js::RP_LINES>,
+      (const void*)js::batch_vjp_phase_kernel<js::RP_REDUCE>, (const void*)js::batch_vjp_phase_kernel<js::RP_LINES, 1>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_CELLS>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_BCTY>, (const void*)js::batch_vjp_phase_kernel<js::RP_BCTX>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_INFLOW_GHOST>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_SRC>, (const void*)js::batch_vjp_phase_kernel<js::RP_UNPACK>};
   for (int ph = 0; ph < js::RP_N; ++ph) {
     int ps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern[ph], js::BNT, rev_phase_smem(ph)) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern[ph], js::BNT, 0) !=
             cudaSuccess ||
         ps < 1)
       return JS_ERR_CUDA;
@@ -847,9 +856,16 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
     // one launch per phase, in the persistent kernel's order; kernel boundaries take the place
     // of its grid barriers
     bool ok = true;
+    // the line phases: a block an item, viscous and inviscid instances apart
+    auto run_lines = [&](auto visc, auto inv, int blocks, size_t smem, int s) {
+      if (!ok) return;
+      if (b->has_visc) visc<<<blocks, js::BNT, smem, b->stream>>>(a, s);
+      if (b->has_inv) inv<<<blocks, js::BNT, smem, b->stream>>>(a, s);
+      ok = cudaGetLastError() == cudaSuccess;
+    };
     auto run = [&](auto kernel, int ph, int s) {
       if (!ok) return;
-      kernel<<<b->rev_pblocks[ph], js::BNT, rev_phase_smem(ph), b->stream>>>(a, s);
+      kernel<<<b->rev_pblocks[ph], js::BNT, 0, b->stream>>>(a, s);
       ok = cudaGetLastError() == cudaSuccess;
     };
     run(js::batch_vjp_phase_kernel<js::RP_PACK>, js::RP_PACK, 0);
@@ -858,12 +874,14 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
       run(js::batch_vjp_phase_kernel<js::RP_HALO>, js::RP_HALO, s);
       if (s == 2) break;
       if (call.U1) continue;
-      run(js::batch_vjp_phase_kernel<js::RP_STAGE>, js::RP_STAGE, s);
+      run_lines(js::batch_vjp_phase_kernel<js::RP_STAGE, 1>, js::batch_vjp_phase_kernel<js::RP_STAGE, 2>, b->line0.back(),
+                batch_smem(), s);
       run(js::batch_vjp_phase_kernel<js::RP_STAGE_CELLS>, js::RP_STAGE_CELLS, s);
     }
     for (int s = 2; s >= 0; --s) {
       if (s < 2 && call.pbar) run(js::batch_vjp_phase_kernel<js::RP_REDUCE>, js::RP_REDUCE, s);
-      run(js::batch_vjp_phase_kernel<js::RP_LINES>, js::RP_LINES, s);
+      run_lines(js::batch_vjp_phase_kernel<js::RP_LINES, 1>, js::batch_vjp_phase_kernel<js::RP_LINES, 2>,
+                b->rblock0.back(), kLineSmem, s);
       run(js::batch_vjp_phase_kernel<js::RP_CELLS>, js::RP_CELLS, s);
       run(js::batch_vjp_phase_kernel<js::RP_BCTY>, js::RP_BCTY, s);
       run(js::batch_vjp_phase_kernel<js::RP_BCTX>, js::RP_BCTX, s);
@@ -918,6 +936,7 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
     d.ntx = (grids[k].nx + js::BTX - 1) / js::BTX;
     d.nty = (grids[k].ny + js::BTY - 1) / js::BTY;
     b->desc.push_back(d);
+    (d.visc ? b->has_visc : b->has_inv) = true;
     tile0[k + 1] = tile0[k] + d.ntx * d.nty;
     b->line0.push_back(b->line0.back() + js::stage_blocks(d.lay, 0) + js::stage_blocks(d.lay, 1));
     ghost0[k + 1] = ghost0[k] + d.ib.n;
@@ -925,8 +944,10 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
     b->cells += (long long)grids[k].nx * grids[k].ny;
   }
   b->ntiles = tile0[count];
+  b->nghost = ghost0[count];
+  b->nhalo = halo0[count];
   const size_t smem = batch_smem();
-  if (cudaFuncSetAttribute(js::batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (cudaFuncSetAttribute(js::batch_phase_kernel<js::FP_LINES, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     js_batch_destroy(b);
     return JS_ERR_CUDA;
   }
@@ -934,7 +955,7 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, js::batch_kernel, js::FNT, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, js::batch_phase_kernel<js::FP_LINES, 1>, js::FNT, smem);
   if (!coop || per_sm < 1) { js_batch_destroy(b); return JS_ERR_CUDA; }
   b->sms = sms;
   b->per_sm = per_sm;
@@ -1010,14 +1031,43 @@ static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, dou
   a.cfl = cfl;
   a.n_steps = n_steps;
   a.extra_arrivals = extra;
-  int dev = 0, khz = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
-  a.budget = (long long)(budget_s * 1e3 * (khz > 0 ? khz : 2000000));
-  void* args[] = {&a};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)js::batch_kernel, dim3(b->blocks), dim3(js::FNT), args,
-                                                    batch_smem(), b->stream);
-  return e == cudaSuccess ? JS_OK : JS_ERR_CUDA;
+  if (extra > 0) {
+    int dev = 0, khz = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
+    a.budget = (long long)(budget_s * 1e3 * (khz > 0 ? khz : 2000000));
+    void* args[] = {&a};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)js::batch_barrier_kernel, dim3(b->sms), dim3(js::FNT),
+                                                      args, 0, b->stream);
+    return e == cudaSuccess ? JS_OK : JS_ERR_CUDA;
+  }
+  using namespace js;
+  const long long nghost = b->nghost, nhalo = b->nhalo;
+  // grids: the elementwise phases a few resident blocks an SM, striding over their items; the lines one
+  // block an item (the hardware's queue balances them), or the tuned blocks per SM striding over them
+  const unsigned wide = (unsigned)(8 * b->sms);
+  const unsigned tiles = (unsigned)std::min<long long>(b->ntiles, 4LL * wide);
+  const unsigned lines = b->blocks_set ? (unsigned)std::min(b->blocks, b->line0.back()) : (unsigned)b->line0.back();
+  auto grid = [&](long long items) { return (unsigned)std::max(1LL, std::min((long long)wide, (items + FNT - 1) / FNT)); };
+  cudaStream_t st = b->stream;
+  if (n_steps > 0) batch_phase_kernel<FP_PACK><<<tiles, FNT, 0, st>>>(a, 0, 0);
+  for (int k = 0; k < n_steps; ++k) {
+    if (!a.dt_in) {
+      batch_phase_kernel<FP_CFL><<<tiles, FNT, 0, st>>>(a, k, 0);
+      batch_phase_kernel<FP_CFL_IEEE><<<tiles, FNT, 0, st>>>(a, k, 0);
+    }
+    batch_phase_kernel<FP_DT><<<1, FNT, 0, st>>>(a, k, 0);
+    for (int s = 0; s < 3; ++s) {
+      if (nghost > 0) batch_phase_kernel<FP_GHOST><<<grid(nghost), FNT, 0, st>>>(a, k, s);
+      batch_phase_kernel<FP_HALO><<<grid(nhalo), FNT, 0, st>>>(a, k, s);
+      if (b->has_visc) batch_phase_kernel<FP_LINES, 1><<<lines, FNT, stage_smem<true>(), st>>>(a, k, s);
+      if (b->has_inv) batch_phase_kernel<FP_LINES, 2><<<lines, FNT, stage_smem<false>(), st>>>(a, k, s);
+      batch_phase_kernel<FP_CELLS><<<tiles, FNT, 0, st>>>(a, k, s);
+    }
+    if (a.save || a.save1) batch_phase_kernel<FP_SAVE><<<tiles, FNT, 0, st>>>(a, k, 0);
+  }
+  if (n_steps > 0) batch_phase_kernel<FP_UNPACK><<<tiles, FNT, 0, st>>>(a, 0, 0);
+  return cudaGetLastError() == cudaSuccess ? JS_OK : JS_ERR_CUDA;
 }
 
 int js_batch_step(js_batch* b, double cfl, int n_steps, double* t_dev, double* dt_log) {
@@ -1318,6 +1368,7 @@ int js_batch_set_tuning(js_batch* b, int blocks_per_sm, int schedule) {
   }
   b->schedule = schedule;
   b->blocks = b->sms * (blocks_per_sm == 0 ? b->per_sm : blocks_per_sm);
+  b->blocks_set = blocks_per_sm != 0;
   return JS_OK;
 }
 
