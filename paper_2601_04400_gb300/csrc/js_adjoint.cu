@@ -73,15 +73,15 @@ __global__ void adj_bcT_kernel(AdjArgs a, BcArgs bc, int phase_y, double* inflow
   adj_bcT_one(a, bc, phase_y, inflow_part, tmax, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-__global__ void __launch_bounds__(128) adj_inflow_kernel(AdjArgs a, BcArgs bc, const double* inflow_part, int tmax,
-                                                         const double* inflow_prim) {
-  adj_inflow_block(a, bc, inflow_part, tmax, inflow_prim);
-}
-
-__global__ void __launch_bounds__(256) adj_pbar_reduce_kernel(const double* __restrict__ pp, long long nslot,
-                                                              double* pbar) {
+// the parameter gradient of one stage: the inflow states, then the partials' sums
+constexpr int kSumThreads = 512;
+__global__ void __launch_bounds__(kSumThreads) adj_sums_kernel(AdjArgs a, BcArgs bc, const double* inflow_part,
+                                                               int tmax, const double* inflow_prim,
+                                                               const double* __restrict__ pp, long long nslot,
+                                                               int inflow) {
+  if (inflow) adj_inflow_block(a, bc, inflow_part, tmax, inflow_prim);
   const long long off = 0;
-  adj_pbar_reduce_block(pp, &off, &nslot, 1, pbar);
+  adj_pbar_reduce_block<kSumThreads>(pp, &off, &nslot, 1, a.pbar);
 }
 
 __global__ void adj_ib_ghost_kernel(AdjArgs a, IbArgs ib, int wall, double* qIb) {
@@ -107,7 +107,7 @@ __global__ void adj_unpack_add_kernel(const double* __restrict__ P, const double
 // =======================================================================================
 namespace {
 unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
-unsigned ib_blocks(int n) { return n > 0 ? blocks_for(n, 128) : 0; }
+unsigned ib_blocks(int n) { return n > 0 ? blocks_for(4LL * n, 128) : 0; }  // a quad of lanes an item
 }  // namespace
 
 long long adj_strip_doubles(const Lay& L) { return strip_size(L, 0) + strip_size(L, 1); }
@@ -162,12 +162,11 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
   a.pp = nullptr;
   const int tmax = std::max(L.nx + 6, L.ny);
   if (two_d) {
-    adj_bcT_kernel<<<blocks_for(6LL * (L.nx + 6), 128), 128, 0, s>>>(a, bc, 1, inflow_part, tmax);
+    adj_bcT_kernel<<<blocks_for(8LL * (L.nx + 6), 128), 128, 0, s>>>(a, bc, 1, inflow_part, tmax);
     ++n;
   }
-  adj_bcT_kernel<<<blocks_for(6LL * L.ny, 128), 128, 0, s>>>(a, bc, 0, inflow_part, tmax);
-  adj_inflow_kernel<<<1, 128, 0, s>>>(a, bc, inflow_part, tmax, inflow_prim);
-  n += 2;
+  adj_bcT_kernel<<<blocks_for(8LL * L.ny, 128), 128, 0, s>>>(a, bc, 0, inflow_part, tmax);
+  ++n;
   if (ib.n > 0) {
     a.pp = slice(4LL * ib_blocks(ib.n));
     adj_ib_ghost_kernel<<<ib_blocks(ib.n), 128, 0, s>>>(a, ib, wall, qIb);
@@ -178,7 +177,8 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
     n += 2;
   }
   if (pp0) {
-    adj_pbar_reduce_kernel<<<1, 256, 0, s>>>(pp0, used, a0.pbar);
+    const int inflow = bc.kind[0] == 3 || bc.kind[1] == 3 || bc.kind[2] == 3 || bc.kind[3] == 3;
+    adj_sums_kernel<<<1, kSumThreads, 0, s>>>(a, bc, inflow_part, tmax, inflow_prim, pp0, used, inflow);
     ++n;
   }
   if (launches) *launches += n;

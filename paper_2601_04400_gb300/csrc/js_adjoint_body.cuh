@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "js_adjoint_device.cuh"
+#include "js_fill.cuh"
 #include "js_internal.h"
 
 namespace js {
@@ -384,66 +385,67 @@ __device__ __forceinline__ void adj_cell(const AdjArgs& a, const double* __restr
 // transposed halo fill (gathers).  y sides first: targets are cells of interior rows (all
 // padded columns); then x sides: targets are interior cells.
 // =======================================================================================
-__device__ __forceinline__ bool halo_source(int kind, int k, int n, bool low, int& src, bool& flip) {
-  flip = false;
-  switch (kind) {
-    case 0: src = low ? 0 : n - 1; return true;
-    case 1: src = low ? k - 1 : n - k; flip = true; return true;
-    case 2: src = low ? n - k : k - 1; return true;
-    default: return false;  // inflow
-  }
-}
-
 __device__ __forceinline__ void adj_bcT_one(const AdjArgs& a, const BcArgs& bc, int phase_y, double* inflow_part,
                                             int tmax, long long t) {
   const Lay& L = a.lay;
-  // targets: 6 source rows/columns next to each boundary
+  // targets: 6 source rows/columns next to each boundary, a run of ntan threads each (a warp takes
+  // one branch; along a row its loads are consecutive)
   const int ntan = phase_y ? L.nx + 6 : L.ny;
-  if (t < 6LL * ntan) {
-    const int r = (int)(t % 6);
-    const int tan = (int)(t / 6) - (phase_y ? 3 : 0);
-    const int n = phase_y ? L.ny : L.nx;
+  const int r = (int)(t / ntan);
+  const int tpos = (int)(t - (long long)r * ntan), tan = tpos - (phase_y ? 3 : 0);
+  const int n = phase_y ? L.ny : L.nx;
+  if (r < 6) {
     const int tgt = (r < 3) ? r : n - 6 + r;  // 0,1,2, n-3,n-2,n-1
     const int comp = phase_y ? 2 : 1;          // momentum component normal to the side
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int s = 0; s < 2; ++s) {
-      const int side = (phase_y ? 2 : 0) + s;
-      for (int k = 1; k <= 3; ++k) {
-        int src;
-        bool flip;
-        if (!halo_source(bc.kind[side], k, n, s == 0, src, flip) || src != tgt) continue;
-        const int h = (s == 0) ? -k : n - 1 + k;
-        const long long hid = phase_y ? L.idx(tan, h) : L.idx(h, tan);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const double v = a.Ub[c * L.plane + hid];
-          acc[c] += (flip && c == comp) ? -v : v;
-        }
-      }
-    }
     const long long tid = phase_y ? L.idx(tan, tgt) : L.idx(tgt, tan);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, own[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) a.Ub[c * L.plane + tid] += acc[c];
-  }
-  // inflow sides: the halo adjoints of each (side, tangential position), its three layers in
-  // order, into inflow_part[side][position] (summed over positions by adj_inflow_kernel)
-  if (t < 2LL * ntan) {
-    const int s = (int)(t % 2);
-    const int tpos = (int)(t / 2);  // 0 .. ntan - 1
-    const int tan = tpos - (phase_y ? 3 : 0);
-    const int side = (phase_y ? 2 : 0) + s;
-    if (bc.kind[side] == 3) {
-      const int n = phase_y ? L.ny : L.nx;
-      double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int k = 1; k <= 3; ++k) {
-        const int h = (s == 0) ? -k : n - 1 + k;
-        const long long hid = phase_y ? L.idx(tan, h) : L.idx(h, tan);
+    for (int c = 0; c < 4; ++c) own[c] = a.Ub[c * L.plane + tid];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[c] += a.Ub[c * L.plane + hid];
+    for (int s = 0; s < 2; ++s) {
+      const int kind = bc.kind[(phase_y ? 2 : 0) + s];
+      // the halo layers k = ka .. kb of this side that copy the target row
+      int ka, kb;
+      if (kind == 0) {
+        ka = 1;
+        kb = (tgt == (s == 0 ? 0 : n - 1)) ? 3 : 0;
+      } else {
+        const bool near_low = (kind == 1) == (s == 0);  // layer k holds row k - 1, else n - k
+        ka = kb = near_low ? tgt + 1 : n - tgt;
+      }
+      if (kind == 3 || ka > 3 || kb < ka) continue;
+      double h[3][4];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int l = min(ka + k, kb), hl = (s == 0) ? -l : n - 1 + l;
+        const long long hid = phase_y ? L.idx(tan, hl) : L.idx(hl, tan);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) h[k][c] = a.Ub[c * L.plane + hid];
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) inflow_part[((long long)side * tmax + tpos) * 4 + c] = acc[c];
+      for (int k = 0; k < 3; ++k)
+        if (ka + k <= kb)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[c] += (kind == 1 && c == comp) ? -h[k][c] : h[k][c];
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) a.Ub[c * L.plane + tid] = own[c] + acc[c];
+  } else if (r < 8) {
+    // inflow sides: the halo adjoints of each (side, tangential position), its three layers in
+    // order, into inflow_part[side][position] (summed over positions by adj_inflow_block)
+    const int s = r - 6, side = (phase_y ? 2 : 0) + s;
+    if (bc.kind[side] != 3) return;
+    double h[3][4];
+#pragma unroll
+    for (int k = 1; k <= 3; ++k) {
+      const int hl = (s == 0) ? -k : n - 1 + k;
+      const long long hid = phase_y ? L.idx(tan, hl) : L.idx(hl, tan);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) h[k - 1][c] = a.Ub[c * L.plane + hid];
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      inflow_part[((long long)side * tmax + tpos) * 4 + c] = ((0.0 + h[0][c]) + h[1][c]) + h[2][c];
   }
 }
 
@@ -457,6 +459,7 @@ __device__ __forceinline__ void adj_inflow_block(const AdjArgs& a, const BcArgs&
   if (side < 4 && bc.kind[side] == 3 && a.pbar != nullptr) {
     const int ntan = (side < 2) ? L.ny : L.nx + 6;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
     for (int k = lane; k < ntan; k += 32)
 #pragma unroll
       for (int c = 0; c < 4; ++c) v[c] += inflow_part[((long long)side * tmax + k) * 4 + c];
@@ -467,30 +470,35 @@ __device__ __forceinline__ void adj_inflow_block(const AdjArgs& a, const BcArgs&
       for (int c = 0; c < 4; ++c) S[side][c] = v[c];
   }
   __syncthreads();
-  if (threadIdx.x != 0 || a.pbar == nullptr) return;
-  for (int sd = 0; sd < 4; ++sd) {
-    if (bc.kind[sd] != 3) continue;
+  if (a.pbar == nullptr) return;
+  // U = (r, r u, r v, p/(gamma-1) + r (u^2 + v^2)/2): a thread per side and parameter
+  if (threadIdx.x < 16 && bc.kind[threadIdx.x >> 2] == 3) {
+    const int sd = threadIdx.x >> 2, m = threadIdx.x & 3;
     const double* s = S[sd];
-    const double r = inflow_prim[4 * sd], u = inflow_prim[4 * sd + 1], v = inflow_prim[4 * sd + 2],
-                 p = inflow_prim[4 * sd + 3];
-    // U = (r, r u, r v, p/(gamma-1) + r (u^2 + v^2)/2)
-    a.pbar[4 + 4 * sd + 0] += s[0] + s[1] * u + s[2] * v + s[3] * 0.5 * (u * u + v * v);
-    a.pbar[4 + 4 * sd + 1] += s[1] * r + s[3] * r * u;
-    a.pbar[4 + 4 * sd + 2] += s[2] * r + s[3] * r * v;
-    a.pbar[4 + 4 * sd + 3] += s[3] * a.gas.g1;
-    a.pbar[0] += -s[3] * p * a.gas.g1 * a.gas.g1;
+    const double r = inflow_prim[4 * sd], u = inflow_prim[4 * sd + 1], v = inflow_prim[4 * sd + 2];
+    const double e = pick4(m, s[0] + s[1] * u + s[2] * v + s[3] * 0.5 * (u * u + v * v), s[1] * r + s[3] * r * u,
+                           s[2] * r + s[3] * r * v, s[3] * a.gas.g1);
+    a.pbar[4 + 4 * sd + m] += e;
+  }
+  if (threadIdx.x == 32) {
+    double g = a.pbar[0];
+    for (int sd = 0; sd < 4; ++sd)
+      if (bc.kind[sd] == 3) g += -S[sd][3] * inflow_prim[4 * sd + 3] * a.gas.g1 * a.gas.g1;
+    a.pbar[0] = g;
   }
 }
 
 // pbar[0..3] += the warp partials pp[4 * b + k] of the slot ranges [off[r], off[r] + cnt[r]),
 // r < nr: each thread over a fixed set of slots, then a fixed reduction tree over the block
 // (blockDim.x a power of two, at most 256)
+template <int NT = 256>
 __device__ __forceinline__ void adj_pbar_reduce_block(const double* __restrict__ pp, const long long* off,
                                                       const long long* cnt, int nr, double* pbar) {
-  __shared__ double red[4][256];
+  __shared__ double red[4][NT];
   const int nt = blockDim.x;
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   for (int r = 0; r < nr; ++r)
+#pragma unroll 4
     for (long long b = threadIdx.x; b < cnt[r]; b += nt)
 #pragma unroll
       for (int k = 0; k < 4; ++k) v[k] += pp[4 * (off[r] + b) + k];
@@ -510,47 +518,26 @@ __device__ __forceinline__ void adj_pbar_reduce_block(const double* __restrict__
 // =======================================================================================
 // transposed immersed-boundary fill
 // =======================================================================================
-__device__ __forceinline__ void adj_ib_ghost_one(const AdjArgs& a, const IbArgs& ib, int wall, double* qIb, int k,
+// item t = 4 k + m: ghost k, lane m of a quad
+__device__ __forceinline__ void adj_ib_ghost_one(const AdjArgs& a, const IbArgs& ib, int wall, double* qIb, int t,
                                                  double& gb) {
-  if (k < ib.n) {
+  if (t < 4 * ib.n) {
+    const int k = t >> 2, m = t & 3;
     const Lay& L = a.lay;
-    const double gamma = a.gas.gamma;
-    double q[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const double w = ib.w[4 * k + m];
-      if (w == 0.0) continue;
-      const long long s = ib.src[4 * k + m];
-      const double r = a.X[s], u = a.X[L.plane + s] / r, v = a.X[2 * L.plane + s] / r;
-      const double p = (gamma - 1.0) * (a.X[3 * L.plane + s] - 0.5 * r * (u * u + v * v));
-      q[0] += w * r;
-      q[1] += w * u;
-      q[2] += w * v;
-      q[3] += w * p;
-    }
-    const double nx = ib.nrm[2 * k], ny = ib.nrm[2 * k + 1];
-    double ug, vg;
-    if (wall == 0) {
-      const double vn = q[1] * nx + q[2] * ny;
-      ug = q[1] - 2.0 * vn * nx;
-      vg = q[2] - 2.0 * vn * ny;
-    } else {
-      ug = -q[1];
-      vg = -q[2];
-    }
-    const long long d = ib.dst[k];
+    const long long d = m * L.plane + ib.dst[k];
+    const double own = a.Ub[d];
+    a.Ub[d] = 0.0;  // the ghost's own input value is overwritten by the fill
+    double q[4], nx, ny, ug, vg;
+    ib_image(a.X, L, ib, a.gas.gm1, wall, k, m, q, nx, ny, ug, vg);
     double G[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      G[c] = a.Ub[c * L.plane + d];
-      a.Ub[c * L.plane + d] = 0.0;  // the ghost's own input value is overwritten by the fill
-    }
+    for (int c = 0; c < 4; ++c) G[c] = __shfl_sync(0xfu << (threadIdx.x & 28), own, c, 4);
     // G = (r, r ug, r vg, p/(gamma-1) + r (ug^2 + vg^2)/2)
     const double br = G[0] + G[1] * ug + G[2] * vg + G[3] * 0.5 * (ug * ug + vg * vg);
     const double bug = G[1] * q[0] + G[3] * q[0] * ug;
     const double bvg = G[2] * q[0] + G[3] * q[0] * vg;
     const double g1 = a.gas.g1;
-    gb -= G[3] * q[3] * g1 * g1;
+    if (m == 0) gb -= G[3] * q[3] * g1 * g1;
     double bu, bv;
     if (wall == 0) {  // (ug, vg) = (I - 2 n n^T)(u, v): symmetric
       const double bn = bug * nx + bvg * ny;
@@ -560,33 +547,31 @@ __device__ __forceinline__ void adj_ib_ghost_one(const AdjArgs& a, const IbArgs&
       bu = -bug;
       bv = -bvg;
     }
-    qIb[4 * k] = br;
-    qIb[4 * k + 1] = bu;
-    qIb[4 * k + 2] = bv;
-    qIb[4 * k + 3] = G[3] * g1;
+    qIb[t] = pick4(m, br, bu, bv, G[3] * g1);
   }
 }
 
-__device__ __forceinline__ void adj_ib_src_one(const AdjArgs& a, const IbTArgs& tb, const double* qIb, int s,
+// item t = 4 s + m: source cell s, lane m of a quad sums and writes component m
+__device__ __forceinline__ void adj_ib_src_one(const AdjArgs& a, const IbTArgs& tb, const double* qIb, int t,
                                                double& gb) {
-  if (s < tb.nsrc) {
-    double S[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int e = tb.ptr[s]; e < tb.ptr[s + 1]; ++e) {
-      const int k = tb.ghost[e];
-      const double w = tb.w[e];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) S[c] += w * qIb[4 * k + c];
-    }
+  if (t < 4 * tb.nsrc) {
+    const int s = t >> 2, m = t & 3;
     const Lay& L = a.lay;
     const long long id = tb.cell[s];
-    // the fill used IEEE-rounded primitives; their derivative is the same map
-    double ub[4];
-    double u, v, p, T;
-    const double r = a.X[id];
-    cons_to_prim(r, a.X[L.plane + id], a.X[2 * L.plane + id], a.X[3 * L.plane + id], a.gas, u, v, p, T);
-    prim_vjp(r, u, v, p, a.gas, S, ub, gb);
+    const int e0 = tb.ptr[s], e1 = tb.ptr[s + 1];
+    const double r = a.X[id], mx = a.X[L.plane + id], my = a.X[2 * L.plane + id], E = a.X[3 * L.plane + id];
+    const double own = a.Ub[m * L.plane + id];
+    double sm = 0.0;
+#pragma unroll 4
+    for (int e = e0; e < e1; ++e) sm += tb.w[e] * qIb[4 * tb.ghost[e] + m];
+    double S[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int c = 0; c < 4; ++c) a.Ub[c * L.plane + id] += ub[c];
+    for (int c = 0; c < 4; ++c) S[c] = __shfl_sync(0xfu << (threadIdx.x & 28), sm, c, 4);
+    double ub[4], u, v, p, T, g = 0.0;
+    cons_to_prim(r, mx, my, E, a.gas, u, v, p, T);
+    prim_vjp(r, u, v, p, a.gas, S, ub, g);
+    if (m == 0) gb += g;
+    a.Ub[m * L.plane + id] = own + pick4(m, ub[0], ub[1], ub[2], ub[3]);
   }
 }
 

@@ -264,12 +264,12 @@ __device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, d
       }
     }
   } else if constexpr (PH == FP_GHOST) {
-    const long long nghost = b.ghost0[b.count];
+    const long long nghost = 4 * b.ghost0[b.count];  // (a quad of lanes a ghost)
     for (long long g = (long long)blockIdx.x * FNT + tid; g < nghost; g += (long long)gridDim.x * FNT) {
-      const int k = find_inst64(b.ghost0, b.count, g);
+      const int k = find_inst64(b.ghost0, b.count, g >> 2);
       const InstDesc& d = b.inst[k];
       double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
-      ib_fill_one(X, d.lay, d.ib, d.gamma, d.wall, (int)(g - b.ghost0[k]));
+      ib_fill_one(X, d.lay, d.ib, d.gamma, d.wall, (int)(g - 4 * b.ghost0[k]));
     }
   } else if constexpr (PH == FP_HALO) {
     const long long nhalo = b.halo0[b.count];
@@ -508,7 +508,7 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     rev_items(b, RK_GHOST, [&](int k, long long g) {
       if (k < 0) return;
       const InstDesc& d = b.inst[k];
-      if (g >= d.ib.n) return;
+      if (g >= 4LL * d.ib.n) return;
       double* X = (s == 0) ? d.N : ((s == 1) ? d.A : d.B);
       ib_fill_one(X, d.lay, d.ib, d.gamma, d.wall, (int)g);
     });
@@ -784,12 +784,12 @@ int rev_prepare(js_batch* b) {
     r.off_c = r.w_lines;
     r.w_c = round32(L.plane) / 32;
     r.off_g = r.off_c + r.w_c;
-    r.w_g = round32(d.ib.n) / 32;
+    r.w_g = round32(4LL * d.ib.n) / 32;  // (a quad of lanes a ghost and a source)
     r.off_s = r.off_g + r.w_g;
-    r.w_s = round32(r.ibt.nsrc) / 32;
+    r.w_s = round32(4LL * r.ibt.nsrc) / 32;
     const long long cnt[js::RK_N] = {
-        round32(L.plane), round32(4LL * L.nx * L.ny), round32(d.ib.n), round32(js::halo_count(L)),
-        round32(6LL * (L.nx + 6)), round32(6LL * L.ny), round32(r.ibt.nsrc)};
+        round32(L.plane), round32(4LL * L.nx * L.ny), round32(4LL * d.ib.n), round32(js::halo_count(L)),
+        round32(8LL * (L.nx + 6)), round32(8LL * L.ny), round32(4LL * r.ibt.nsrc)};
     for (int q = 0; q < js::RK_N; ++q) pre[(size_t)q * (n + 1) + k + 1] = pre[(size_t)q * (n + 1) + k] + cnt[q];
   }
   const size_t smem = rev_smem();
@@ -1058,7 +1058,7 @@ static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, dou
     }
     batch_phase_kernel<FP_DT><<<1, FNT, 0, st>>>(a, k, 0);
     for (int s = 0; s < 3; ++s) {
-      if (nghost > 0) batch_phase_kernel<FP_GHOST><<<grid(nghost), FNT, 0, st>>>(a, k, s);
+      if (nghost > 0) batch_phase_kernel<FP_GHOST><<<grid(4 * nghost), FNT, 0, st>>>(a, k, s);
       batch_phase_kernel<FP_HALO><<<grid(nhalo), FNT, 0, st>>>(a, k, s);
       if (b->has_visc) batch_phase_kernel<FP_LINES, 1><<<lines, FNT, stage_smem<true>(), st>>>(a, k, s);
       if (b->has_inv) batch_phase_kernel<FP_LINES, 2><<<lines, FNT, stage_smem<false>(), st>>>(a, k, s);

@@ -69,38 +69,58 @@ __device__ __forceinline__ void bc_fill_one(double* __restrict__ U, const Lay& l
   for (int c = 0; c < 4; ++c) U[c * lay.plane + d] = v[c];
 }
 
-// Ghost cell k: slip-wall (or no-slip) mirror of the bilinear interpolation of fluid cells
-// at its image point.
-__device__ __forceinline__ void ib_fill_one(double* __restrict__ U, const Lay& lay, const IbArgs& ib, double gamma,
-                                            int wall, int k) {
-  double q[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const double w = ib.w[4 * k + m];
-    if (w == 0.0) continue;
-    const long long s = ib.src[4 * k + m];
-    const double r = U[s], u = U[lay.plane + s] / r, v = U[2 * lay.plane + s] / r;
-    const double p = (gamma - 1.0) * (U[3 * lay.plane + s] - 0.5 * r * (u * u + v * v));
-    q[0] += w * r;
-    q[1] += w * u;
-    q[2] += w * v;
-    q[3] += w * p;
+// sum over the four lanes of a quad (the same value on each: (0 + 1) + (2 + 3))
+__device__ __forceinline__ double quad_sum(double x) {
+  const unsigned m = 0xfu << (threadIdx.x & 28);
+  x += __shfl_xor_sync(m, x, 1);
+  return x + __shfl_xor_sync(m, x, 2);
+}
+__device__ __forceinline__ double pick4(int c, double a, double b, double d, double e) {
+  return c < 2 ? (c == 0 ? a : b) : (c == 2 ? d : e);
+}
+
+// The image point of ghost cell k: primitives q = (rho, u, v, p) interpolated from its four source
+// cells, lane m of the quad taking source m, and the velocity (ug, vg) mirrored at the wall.  A cell
+// of weight 0 is not read.  Bound by latency: one load of weights and cells, one of states, one
+// reciprocal, then sums over the quad.
+__device__ __forceinline__ void ib_image(const double* __restrict__ U, const Lay& lay, const IbArgs& ib, double gm1,
+                                         int wall, int k, int m, double q[4], double& nx, double& ny, double& ug,
+                                         double& vg) {
+  const double w = ib.w[4 * k + m];
+  const long long s = ib.src[4 * k + m];
+  nx = ib.nrm[2 * k];
+  ny = ib.nrm[2 * k + 1];
+  q[0] = q[1] = q[2] = q[3] = 0.0;
+  if (w != 0.0) {
+    const double r = U[s], mx = U[lay.plane + s], my = U[2 * lay.plane + s], E = U[3 * lay.plane + s];
+    const double ir = recip(r), u = mx * ir, v = my * ir;
+    q[0] = w * r;
+    q[1] = w * u;
+    q[2] = w * v;
+    q[3] = w * (gm1 * (E - 0.5 * r * fma(u, u, v * v)));
   }
-  const double nx = ib.nrm[2 * k], ny = ib.nrm[2 * k + 1];
-  double ug, vg;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) q[c] = quad_sum(q[c]);
   if (wall == 0) {
-    const double vn = q[1] * nx + q[2] * ny;
-    ug = q[1] - 2.0 * vn * nx;
-    vg = q[2] - 2.0 * vn * ny;
+    const double vn = fma(q[1], nx, q[2] * ny);
+    ug = fma(-2.0 * vn, nx, q[1]);
+    vg = fma(-2.0 * vn, ny, q[2]);
   } else {
     ug = -q[1];
     vg = -q[2];
   }
-  const long long d = ib.dst[k];
-  U[d] = q[0];
-  U[lay.plane + d] = q[0] * ug;
-  U[2 * lay.plane + d] = q[0] * vg;
-  U[3 * lay.plane + d] = q[3] / (gamma - 1.0) + 0.5 * q[0] * (ug * ug + vg * vg);
+}
+
+// Ghost cell t / 4, by lane t % 4 of a quad (t a multiple of 4 on the quad's first lane): slip-wall
+// (or no-slip) mirror of the bilinear interpolation of fluid cells at its image point.
+__device__ __forceinline__ void ib_fill_one(double* __restrict__ U, const Lay& lay, const IbArgs& ib, double gamma,
+                                            int wall, int t) {
+  const int k = t >> 2, m = t & 3;
+  const double gm1 = gamma - 1.0;
+  double q[4], nx, ny, ug, vg;
+  ib_image(U, lay, ib, gm1, wall, k, m, q, nx, ny, ug, vg);
+  const double e = fma(q[3], recip(gm1), 0.5 * q[0] * fma(ug, ug, vg * vg));
+  U[m * lay.plane + ib.dst[k]] = pick4(m, q[0], q[0] * ug, q[0] * vg, e);
 }
 
 // CFL rate (|u| + a)/dx [+ (|v| + a)/dy] of one cell with conserved values (r, mx, my, E),

@@ -28,8 +28,8 @@ __global__ void bc_fill_kernel(double* __restrict__ U, Lay lay, BcArgs bc) {
 // immersed-boundary ghost states
 // =======================================================================================
 __global__ void ib_fill_kernel(double* __restrict__ U, Lay lay, IbArgs ib, double gamma, int wall) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < ib.n) ib_fill_one(U, lay, ib, gamma, wall, k);
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < 4 * ib.n) ib_fill_one(U, lay, ib, gamma, wall, t);
 }
 
 // =======================================================================================
@@ -376,7 +376,7 @@ cudaError_t launch_bc_fill(double* U, const Lay& lay, const BcArgs& bc, cudaStre
 cudaError_t launch_ib_fill(double* U, const Lay& lay, const IbArgs& ib, double gamma, int wall, cudaStream_t s) {
   if (ib.n == 0) return cudaSuccess;
   const int bs = 128;
-  ib_fill_kernel<<<(ib.n + bs - 1) / bs, bs, 0, s>>>(U, lay, ib, gamma, wall);
+  ib_fill_kernel<<<(4 * ib.n + bs - 1) / bs, bs, 0, s>>>(U, lay, ib, gamma, wall);
   return cudaGetLastError();
 }
 
