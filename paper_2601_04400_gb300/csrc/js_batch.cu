@@ -183,6 +183,8 @@ __device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, d
       const int t = it - b.tile0[k];
       const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
       const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
+      const CflF cf = cfl_f32(d.gamma, idx, idy, d.lay.ny > 1);
+      float rf = 0.0f;
       double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
       for (int e = tid; e < BTX * BTY; e += FNT) {
         const int i = i0 + (e % BTX), j = j0 + (e / BTX);
@@ -190,10 +192,11 @@ __device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, d
         if (d.tag && d.tag[(long long)j * d.lay.nx + i] != 0) continue;
         const long long p = d.lay.idx(i, j);
         const double r = d.N[p];
-        rate = fmax(rate, cfl_rate_fast(r, d.N[d.lay.plane + p], d.N[2 * d.lay.plane + p], d.N[3 * d.lay.plane + p],
-                                        d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1));
+        cfl_rate_max(r, d.N[d.lay.plane + p], d.N[2 * d.lay.plane + p], d.N[3 * d.lay.plane + p], d.gamma, d.dx, d.dy,
+                     idx, idy, cf, d.lay.ny > 1, rf, rate);
         rmin = fmin(rmin, r);
       }
+      rate = fmax(rate, (double)rf);
       for (int o = 16; o > 0; o >>= 1) {
         rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
         rmin = fmin(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
@@ -224,6 +227,7 @@ __device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, d
       const int t = it - b.tile0[k];
       const int i0 = (t % d.ntx) * BTX, j0 = (t / d.ntx) * BTY;
       const double idx = 1.0 / d.dx, idy = 1.0 / d.dy;
+      const CflF cf = cfl_f32(d.gamma, idx, idy, d.lay.ny > 1);
       double rate = 0.0;
       for (int e = tid; e < BTX * BTY; e += FNT) {
         const int i = i0 + (e % BTX), j = j0 + (e / BTX);
@@ -233,7 +237,7 @@ __device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, d
         const double* X = d.N + d.lay.idx(i, j);
         const long long P = d.lay.plane;
         const double r = X[0], mx = X[P], my = X[2 * P], E = X[3 * P];
-        if (!(cfl_rate_fast(r, mx, my, E, d.gamma, d.dx, d.dy, idx, idy, d.lay.ny > 1) >= thr)) continue;
+        if (!cfl_reaches(r, mx, my, E, d.gamma, d.dx, d.dy, idx, idy, cf, d.lay.ny > 1, thr)) continue;
         if (i > 0 && !(tag && tag[-1] != 0) && same_bits(r, X[-1]) && same_bits(mx, X[P - 1]) &&
             same_bits(my, X[2 * P - 1]) && same_bits(E, X[3 * P - 1]))
           continue;

@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "js_device.cuh"
 #include "js_internal.h"
 #include "js_fill.cuh"
@@ -86,16 +88,17 @@ __global__ void prim_to_cons_kernel(const double* W, double* U, long long n, dou
 // =======================================================================================
 // CFL reduction: rate = (|u| + a)/dx [+ (|v| + a)/dy] and rho over fluid cells, the rate in
 // IEEE-rounded intrinsics in the oracle's operation order, so equal states give equal dt.
-// Two passes keep that result while taking the IEEE rate of few cells: pass 1 takes every
-// fluid cell's rate with the fast reciprocal and reciprocal square root, the exact minimum
-// density, the maximum of these approximate rates and each block's maximum; pass 2 takes the
+// Small grids take every cell's IEEE rate in one launch.  On larger ones two passes keep that result
+// while taking the IEEE rate of few cells: pass 1 takes every fluid cell's rate in FP32, the exact
+// minimum density, the maximum of these approximate rates and each block's maximum; pass 2 takes the
 // IEEE rate only in blocks, and of cells, whose approximate rate reaches (1 - CFL_MARGIN) of
 // that maximum (once per run of cells with identical states along a row).
-// The approximation's relative error is a few ulp plus the pressure's cancellation error,
-// about (E/p) ulp.  Pass 1 therefore uses it only where p > 1e-8 E (error below 1e-7) and takes
-// the IEEE rate itself elsewhere (near-vacuum or hypersonic cells, non-physical ones), so every
+// The approximation's relative error is that of FP32 times the pressure's cancellation E/p.  Pass 1
+// takes FP32 only where the internal energy is above E/16, FP64 with the fast reciprocal only where
+// p > 1e-8 E, and the IEEE rate itself elsewhere (near-vacuum cells, non-physical ones), so every
 // pass-1 rate is within CFL_MARGIN/2 of the IEEE rate, the cell of the largest IEEE rate is
 // always a pass-2 candidate, and the result is the one-pass IEEE maximum for every state.
+// The last block of the last launch turns the maximum into the step size (cfl_finish).
 // A non-physical fluid cell has the rate +infinity in both passes (cfl_rate).
 // =======================================================================================
 // block maximum (thread 0 holds it) and, when rmin != nullptr, block minimum
@@ -134,6 +137,86 @@ __device__ __forceinline__ long long cfl_at(const CflSrc& q, long long t) {
   return PADDED ? q.off + (t / q.nx) * q.pitch + t % q.nx : t;
 }
 
+// Device step size from the CFL reduction in red, with js_max_dt's arithmetic (the same IEEE
+// operations in the same order): dt = cfl / rate, capped by the viscous limit
+// cfl hmin^2 rho_min / (2 mu lim); clipped to t_end - t when t + dt > t_end (t: running time,
+// or nullptr), the step inactive once t reaches t_end or when dt is not a positive number
+// (a non-physical state: the error flag is set).  Writes the stage constants dtc and dt_log[k].
+// Run by the block whose ticket is the last; it leaves red ready for the next step.
+__device__ __forceinline__ void cfl_reset(unsigned long long* red) {
+  red[0] = 0ULL;                    // IEEE rate maximum
+  red[1] = 0x7ff0000000000000ULL;   // density minimum
+  red[2] = 0ULL;                    // approximate rate maximum
+  red[3] = 0ULL;                    // tickets
+}
+__device__ __forceinline__ void cfl_finish(unsigned long long* red, const CflStep& q) {
+  if (q.dtc == nullptr) return;
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(&red[3], 1ULL) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
+  const int lane = threadIdx.x;
+  const double rate = __longlong_as_double((long long)__ldcg(&red[0]));
+  const double rmin = __longlong_as_double((long long)__ldcg(&red[1]));
+  double dt = __ddiv_rn(q.cfl, rate);
+  if (q.visc) {
+    const double dtv = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(q.cfl, q.hmin), q.hmin), rmin),
+                                 __dmul_rn(__dmul_rn(2.0, q.mu), q.lim));
+    dt = (dtv < dt) ? dtv : dt;
+  }
+  bool active = dt > 0.0 && dt < CUDART_INF;
+  if (!active && lane == 0) atomicOr(q.err, ERR_NONPHYSICAL_BIT);
+  double tc = 0.0;
+  if (q.t != nullptr) {
+    tc = *q.t;
+    if (active && q.t_end > 0.0) {
+      if (!(tc < q.t_end)) active = false;
+      else if (__dadd_rn(tc, dt) > q.t_end) dt = __dsub_rn(q.t_end, tc);
+    }
+  }
+  if (!active) dt = 0.0;
+  __syncwarp();
+  if (lane < 4) {  // dt/dx, dt/dy, dt nu/dx^2, dt nu/dy^2
+    const double h = (lane & 1) ? q.dy : q.dx;
+    q.dtc[lane] = __ddiv_rn(lane < 2 ? dt : __dmul_rn(dt, q.nu), lane < 2 ? h : __dmul_rn(h, h));
+  }
+  if (lane == 4) {
+    if (active && q.t != nullptr) *q.t = __dadd_rn(tc, dt);
+    q.dtc[4] = active ? 1.0 : 0.0;
+    q.dtc[5] = dt;
+    if (q.dt_log) q.dt_log[q.k] = dt;
+    cfl_reset(red);
+  }
+}
+
+__global__ void cfl_init_kernel(unsigned long long* red) { cfl_reset(red); }
+
+// Every cell's IEEE rate, a cell a thread (small grids).
+template <bool PADDED>
+__global__ void __launch_bounds__(128) cfl_one_kernel(CflSrc q, long long n, int two_d,
+                                                      const unsigned char* __restrict__ tag, double gamma, double dx,
+                                                      double dy, unsigned long long* __restrict__ red, CflStep st) {
+  double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < n && !(tag && tag[t] != 0)) {
+    const long long e = cfl_at<PADDED>(q, t);
+    rmin = q.U[e];
+    rate = cfl_rate(rmin, q.U[q.plane + e], q.U[2 * q.plane + e], q.U[3 * q.plane + e], gamma, dx, dy, two_d != 0);
+  }
+  rmin = fmin(rmin, __longlong_as_double(0x7ff0000000000000LL));
+  cfl_block_reduce(rate, &rmin);
+  if (threadIdx.x == 0) {
+    atomicMax(&red[0], (unsigned long long)__double_as_longlong(rate));
+    atomicMin(&red[1], (unsigned long long)__double_as_longlong(rmin));
+  }
+  cfl_finish(red, st);
+}
+
+// (1024x1024 cells: 14 us; with every rate in FP64 56 us, bound by the FP64 pipe)
 template <bool PADDED>
 __global__ void cfl_pass1_kernel(CflSrc q, long long n, int two_d,
                                  const unsigned char* __restrict__ tag, double gamma, double dx, double dy,
@@ -142,14 +225,17 @@ __global__ void cfl_pass1_kernel(CflSrc q, long long n, int two_d,
   double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
   const double* __restrict__ U = q.U;
   const long long P = q.plane;
+  const CflF cf = cfl_f32(gamma, idx, idy, two_d != 0);
+  float rf = 0.0f;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
     if (tag && tag[t] != 0) continue;
     const long long e = cfl_at<PADDED>(q, t);
     const double r = U[e];
-    rate = fmax(rate, cfl_rate_fast(r, U[P + e], U[2 * P + e], U[3 * P + e], gamma, dx, dy, idx, idy, two_d != 0));
+    cfl_rate_max(r, U[P + e], U[2 * P + e], U[3 * P + e], gamma, dx, dy, idx, idy, cf, two_d != 0, rf, rate);
     rmin = fmin(rmin, r);
   }
+  rate = fmax(rate, (double)rf);
   cfl_block_reduce(rate, &rmin);
   if (threadIdx.x == 0) {
     // non-negative doubles order like their bit patterns (a negative density is a non-physical
@@ -168,9 +254,13 @@ template <bool PADDED>
 __global__ void cfl_pass2_kernel(CflSrc q, long long n, int nx, int two_d,
                                  const unsigned char* __restrict__ tag, double gamma, double dx, double dy,
                                  double idx, double idy, unsigned long long* __restrict__ red,
-                                 const double* __restrict__ bmax) {
+                                 const double* __restrict__ bmax, CflStep st) {
   const double thr = __longlong_as_double((long long)red[2]) * (1.0 - CFL_MARGIN);
-  if (!(bmax[blockIdx.x] >= thr)) return;  // the same for the whole block
+  if (!(bmax[blockIdx.x] >= thr)) {  // the same for the whole block
+    cfl_finish(red, st);
+    return;
+  }
+  const CflF cf = cfl_f32(gamma, idx, idy, two_d != 0);
   const int lane = threadIdx.x & 31;
   const double* __restrict__ U = q.U;
   const long long P = q.plane;
@@ -200,7 +290,7 @@ __global__ void cfl_pass2_kernel(CflSrc q, long long n, int nx, int two_d,
       myl = U[2 * P + e];
       El = U[3 * P + e];
     }
-    if (in && fl && cfl_rate_fast(r, mx, my, E, gamma, dx, dy, idx, idy, two_d != 0) >= thr) {
+    if (in && fl && cfl_reaches(r, mx, my, E, gamma, dx, dy, idx, idy, cf, two_d != 0, thr)) {
       const bool same = (t % nx != 0) && fll && same_bits(r, rl) && same_bits(mx, mxl) && same_bits(my, myl) &&
                         same_bits(E, El);
       if (!same) rate = fmax(rate, cfl_rate(r, mx, my, E, gamma, dx, dy, two_d != 0));
@@ -208,49 +298,7 @@ __global__ void cfl_pass2_kernel(CflSrc q, long long n, int nx, int two_d,
   }
   cfl_block_reduce(rate, nullptr);
   if (threadIdx.x == 0) atomicMax(&red[0], (unsigned long long)__double_as_longlong(rate));
-}
-
-// Device step size from the CFL reduction in red, with js_max_dt's arithmetic (the same IEEE
-// operations in the same order): dt = cfl / rate, capped by the viscous limit
-// cfl hmin^2 rho_min / (2 mu lim); clipped to t_end - t when t + dt > t_end (t: running time,
-// or nullptr), the step inactive once t reaches t_end or when dt is not a positive number
-// (a non-physical state: the error flag is set).  Writes the stage constants dtc and dt_log[k].
-__global__ void cfl_dt_kernel(const unsigned long long* __restrict__ red, double cfl, double dx, double dy,
-                              double nu, int visc, double mu, double lim, double hmin, double* t, double t_end,
-                              double* __restrict__ dtc, double* __restrict__ dt_log, int k, int* err) {
-  const double rate = __longlong_as_double((long long)red[0]);
-  const double rmin = __longlong_as_double((long long)red[1]);
-  double dt = __ddiv_rn(cfl, rate);
-  if (visc) {
-    const double dtv = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(cfl, hmin), hmin), rmin),
-                                 __dmul_rn(__dmul_rn(2.0, mu), lim));
-    dt = (dtv < dt) ? dtv : dt;
-  }
-  bool active = true;
-  if (!(dt > 0.0) || !(dt < CUDART_INF)) {
-    atomicOr(err, ERR_NONPHYSICAL_BIT);
-    active = false;
-  }
-  if (active && t != nullptr && t_end > 0.0) {
-    const double tc = *t;
-    if (!(tc < t_end)) active = false;
-    else if (__dadd_rn(tc, dt) > t_end) dt = __dsub_rn(t_end, tc);
-  }
-  if (!active) dt = 0.0;
-  if (active && t != nullptr) *t = __dadd_rn(*t, dt);
-  dtc[0] = __ddiv_rn(dt, dx);
-  dtc[1] = __ddiv_rn(dt, dy);
-  dtc[2] = __ddiv_rn(__dmul_rn(dt, nu), __dmul_rn(dx, dx));
-  dtc[3] = __ddiv_rn(__dmul_rn(dt, nu), __dmul_rn(dy, dy));
-  dtc[4] = active ? 1.0 : 0.0;
-  dtc[5] = dt;
-  if (dt_log) dt_log[k] = dt;
-}
-
-__global__ void cfl_init_kernel(unsigned long long* red) {
-  red[0] = 0ULL;                    // IEEE rate maximum
-  red[1] = 0x7ff0000000000000ULL;   // density minimum
-  red[2] = 0ULL;                    // approximate rate maximum
+  cfl_finish(red, st);
 }
 
 // the stage constants of a launch: the arguments, or those of the device step size
@@ -417,35 +465,42 @@ cudaError_t launch_prim_to_cons(const double* W, double* U, long long n, double 
   return cudaGetLastError();
 }
 
-cudaError_t launch_cfl_dt(const unsigned long long* red, double cfl, double dx, double dy, double nu, double mu,
-                          double lim, double hmin, double* t, double t_end, double* dtc, double* dt_log, int k,
-                          int* err, cudaStream_t s) {
-  cfl_dt_kernel<<<1, 1, 0, s>>>(red, cfl, dx, dy, nu, mu > 0.0 ? 1 : 0, mu, lim, hmin, t, t_end, dtc, dt_log, k,
-                                err);
+cudaError_t launch_cfl_init(unsigned long long* red, cudaStream_t s) {
+  cfl_init_kernel<<<1, 1, 0, s>>>(red);
   return cudaGetLastError();
 }
 
-cudaError_t launch_cfl(const double* U, const Lay& lay, const unsigned char* tag, double gamma, double dx,
-                       double dy, unsigned long long* red, double* bmax, cudaStream_t s, bool padded) {
-  cfl_init_kernel<<<1, 1, 0, s>>>(red);
-  const long long n = (long long)lay.nx * lay.ny;
-  const int bs = 256;
-  long long blocks = (n + bs - 1) / bs;
-  if (blocks > CFL_MAX_BLOCKS) blocks = CFL_MAX_BLOCKS;
+// Cells up to which every rate is taken in IEEE arithmetic at once: one launch in place of two, each of
+// which is latency on such grids.  A step of 128x64 cells takes 89 us with one launch and 95 with two,
+// of 256x128 116 and 120; from there the FP64 pipe decides: 256x256 155 and 153, 400x320 222 and 216.
+constexpr long long CFL_ONE_CELLS = 32768;
+
+namespace {
+template <bool PADDED>
+void cfl_launches(const CflSrc& q, long long n, const Lay& lay, const unsigned char* tag, double gamma, double dx,
+                  double dy, unsigned long long* red, double* bmax, const CflStep& st, cudaStream_t s) {
   const int two_d = lay.ny > 1 ? 1 : 0;
-  const CflSrc q{U, padded ? lay.plane : n, padded ? lay.idx(0, 0) : 0, lay.nx, padded ? lay.pitch : lay.nx};
-  // both passes on the same grid: a block of pass 2 visits the cells its pass-1 maximum covers
-  if (padded) {
-    cfl_pass1_kernel<true><<<(unsigned)blocks, bs, 0, s>>>(q, n, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red,
-                                                            bmax);
-    cfl_pass2_kernel<true><<<(unsigned)blocks, bs, 0, s>>>(q, n, lay.nx, two_d, tag, gamma, dx, dy, 1.0 / dx,
-                                                            1.0 / dy, red, bmax);
-  } else {
-    cfl_pass1_kernel<false><<<(unsigned)blocks, bs, 0, s>>>(q, n, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red,
-                                                             bmax);
-    cfl_pass2_kernel<false><<<(unsigned)blocks, bs, 0, s>>>(q, n, lay.nx, two_d, tag, gamma, dx, dy, 1.0 / dx,
-                                                             1.0 / dy, red, bmax);
+  if (n <= CFL_ONE_CELLS) {
+    cfl_one_kernel<PADDED><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(q, n, two_d, tag, gamma, dx, dy, red, st);
+    return;
   }
+  const int bs = 256;
+  const unsigned blocks = (unsigned)std::min<long long>((n + bs - 1) / bs, CFL_MAX_BLOCKS);
+  // both passes on the same grid: a block of pass 2 visits the cells its pass-1 maximum covers
+  cfl_pass1_kernel<PADDED><<<blocks, bs, 0, s>>>(q, n, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red, bmax);
+  cfl_pass2_kernel<PADDED><<<blocks, bs, 0, s>>>(q, n, lay.nx, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red,
+                                                 bmax, st);
+}
+}  // namespace
+
+int cfl_launch_count(const Lay& lay) { return (long long)lay.nx * lay.ny <= CFL_ONE_CELLS ? 1 : 2; }
+
+cudaError_t launch_cfl(const double* U, const Lay& lay, const unsigned char* tag, double gamma, double dx, double dy,
+                       unsigned long long* red, double* bmax, const CflStep& st, cudaStream_t s, bool padded) {
+  const long long n = (long long)lay.nx * lay.ny;
+  const CflSrc q{U, padded ? lay.plane : n, padded ? lay.idx(0, 0) : 0, lay.nx, padded ? lay.pitch : lay.nx};
+  if (padded) cfl_launches<true>(q, n, lay, tag, gamma, dx, dy, red, bmax, st, s);
+  else cfl_launches<false>(q, n, lay, tag, gamma, dx, dy, red, bmax, st, s);
   return cudaGetLastError();
 }
 

@@ -626,8 +626,10 @@ int js_rhs(js_ctx* c, const double* U, double* dUdt) {
 
 int js_max_dt(js_ctx* c, const double* U, double cfl, double* dt_out) {
   if (!c || !U || !dt_out || !(cfl > 0.0)) return JS_ERR_ARG;
-  JS_CUDA(js::launch_cfl(U, c->lay, c->tag, c->p.gamma, c->g.dx, c->g.dy, c->red, c->cfl_bmax, c->stream));
-  c->launches += 3;
+  JS_CUDA(js::launch_cfl_init(c->red, c->stream));
+  JS_CUDA(js::launch_cfl(U, c->lay, c->tag, c->p.gamma, c->g.dx, c->g.dy, c->red, c->cfl_bmax, js::CflStep{}, c->stream,
+                         false));
+  c->launches += 1 + js::cfl_launch_count(c->lay);
   unsigned long long h[2];
   JS_CUDA(cudaMemcpyAsync(h, c->red, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
   JS_CUDA(cudaStreamSynchronize(c->stream));
@@ -694,13 +696,14 @@ int js_step_cfl(js_ctx* c, double* U, double cfl, int n_steps, double* t_dev, do
   if (n_steps == 0) return JS_OK;
   // the state stays in the padded buffer N from the first step to the last
   JS_CUDA(js::launch_pack(U, c->N, c->lay, c->stream));
-  ++c->launches;
+  JS_CUDA(js::launch_cfl_init(c->red, c->stream));
+  c->launches += 2;
+  js::CflStep st{cfl, c->g.dx, c->g.dy, c->p.nu, c->p.mu, lim, hmin, t_end, t_dev, c->dtc, dt_log, c->err, 0, visc ? 1 : 0};
   for (int k = 0; k < n_steps; ++k) {
-    JS_CUDA(js::launch_cfl(c->N, c->lay, c->tag, c->p.gamma, c->g.dx, c->g.dy, c->red, c->cfl_bmax, c->stream,
+    st.k = k;
+    JS_CUDA(js::launch_cfl(c->N, c->lay, c->tag, c->p.gamma, c->g.dx, c->g.dy, c->red, c->cfl_bmax, st, c->stream,
                            true));
-    JS_CUDA(js::launch_cfl_dt(c->red, cfl, c->g.dx, c->g.dy, c->p.nu, c->p.mu, lim, hmin, t_dev, t_end, c->dtc,
-                              dt_log, k, c->err, c->stream));
-    c->launches += 4;
+    c->launches += js::cfl_launch_count(c->lay);
     for (int s = 0; s < 3; ++s) {
       int rc = fill_halos(c, in[s], ieee);
       if (rc) return rc;

@@ -216,17 +216,23 @@ cudaError_t launch_prim_to_cons(const double* W, double* U, long long n, double 
 cudaError_t launch_rows_pack(double* U, int nx, int ny, int row0, int nrows, double* buf, int zero, cudaStream_t s);
 cudaError_t launch_rows_unpack(double* U, int nx, int ny, int row0, int nrows, const double* buf, int add,
                                cudaStream_t s);
-// CFL reduction of U (user layout): red[0] = bits of the largest rate, red[1] = bits of the
-// smallest density over fluid cells (red: 3 words; bmax: CFL_MAX_BLOCKS doubles of scratch)
+// The step that follows a CFL reduction (dtc null: none): its size on the device with js_max_dt's
+// arithmetic (viscous cap when visc with lim = max(4/3, gamma/Pr), hmin = min(dx, dy) in 2D), clipped
+// to t_end with the running time t (or t == nullptr), into the stage constants dtc[DTC_N] and dt_log[k]
+struct CflStep {
+  double cfl, dx, dy, nu, mu, lim, hmin, t_end;
+  double *t, *dtc, *dt_log;
+  int* err;
+  int k, visc;
+};
+// CFL reduction of U: red[0] = bits of the largest rate, red[1] = bits of the smallest density over
+// fluid cells (red: 4 words, reset by launch_cfl_init before the first reduction and after one
+// without a step; bmax: CFL_MAX_BLOCKS doubles of scratch).
+// padded: U is a context's padded buffer, e.g. the state N between the steps of js_step_cfl.
 constexpr int CFL_MAX_BLOCKS = 152 * 8;
-// the step size of the reduction in red on the device (js_max_dt's arithmetic; viscous cap when
-// mu > 0 with lim = max(4/3, gamma/Pr), hmin = min(dx, dy) in 2D), clipped to t_end with the
-// running time t (or t == nullptr), into the stage constants dtc[DTC_N] and dt_log[k]
-cudaError_t launch_cfl_dt(const unsigned long long* red, double cfl, double dx, double dy, double nu, double mu,
-                          double lim, double hmin, double* t, double t_end, double* dtc, double* dt_log, int k,
-                          int* err, cudaStream_t s);
-// (padded: U is a context's padded buffer, e.g. the state N between the steps of js_step_cfl)
-cudaError_t launch_cfl(const double* U, const Lay& lay, const unsigned char* tag, double gamma, double dx,
-                       double dy, unsigned long long* red, double* bmax, cudaStream_t s, bool padded = false);
+cudaError_t launch_cfl_init(unsigned long long* red, cudaStream_t s);
+cudaError_t launch_cfl(const double* U, const Lay& lay, const unsigned char* tag, double gamma, double dx, double dy,
+                       unsigned long long* red, double* bmax, const CflStep& st, cudaStream_t s, bool padded);
+int cfl_launch_count(const Lay& lay);
 
 }  // namespace js
