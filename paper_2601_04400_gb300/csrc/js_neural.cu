@@ -124,18 +124,19 @@ __global__ void nn_prims_kernel(const double* __restrict__ U, double* __restrict
   Q[3 * L.plane + t] = p;
 }
 
-// The image kernels work on 32 x 32 tiles of (line h, face f) pixels: the FP64 face-state
+// The image kernels work on tiles of 32 lines h x 8 faces f, a pixel a thread: the face-state
 // arithmetic runs with consecutive threads on consecutive lines, the direction along which the
-// stage's stored WENO5 internals and the face adjoints are contiguous in both directions, and the
-// image values (contiguous along f) pass through a shared-memory tile.
-constexpr int IT = 32;
+// face adjoints are contiguous in both directions, and the image values (contiguous along f) pass
+// through a shared-memory tile.  A pixel is a chain of eight reconstructions, so a small grid is
+// latency: tiles of 32 faces, four pixels a thread, took 50 us (reverse: 65) at 128x96.
+constexpr int IT = 32, IF = 8;
 
 template <class T>
 __global__ void __launch_bounds__(256) nn_image_kernel(NnArgs n, const double* __restrict__ Q, long long qplane) {
-  __shared__ T sx[4][IT][IT + 1];
+  __shared__ T sx[4][IT][IF + 1];
   const int d = blockIdx.z;
   const int H = n.H[d], Wd = n.W[d];
-  const int f0 = blockIdx.x * IT, h0 = blockIdx.y * IT;
+  const int f0 = blockIdx.x * IF, h0 = blockIdx.y * IT;
   if (f0 >= Wd || h0 >= H) return;  // uniform per block
   const long long pix = (long long)H * Wd;
   const int hl = threadIdx.x % IT;
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(256) nn_image_kernel(NnArgs n, const double* _
     mean[k] = (T)n.mean[k];
     isd[k] = (T)n.inv_sd[k];
   }
-  for (int fl = threadIdx.x / IT; fl < IT; fl += 256 / IT) {
+  for (int fl = threadIdx.x / IT; fl < IF; fl += 256 / IT) {
     const int h = h0 + hl, f = f0 + fl;
     if (h >= H || f >= Wd) continue;
     double wl[4], wr[4];
@@ -158,9 +159,9 @@ __global__ void __launch_bounds__(256) nn_image_kernel(NnArgs n, const double* _
   }
   __syncthreads();
   T* X = chan_img<T>(n.X, 4, d, n.pix0);
-  for (int e = threadIdx.x; e < 4 * IT * IT; e += 256) {
-    const int k = e / (IT * IT), r = e % (IT * IT), h = h0 + r / IT, f = f0 + r % IT;
-    if (h < H && f < Wd) X[k * pix + (long long)h * Wd + f] = sx[k][r / IT][r % IT];
+  for (int e = threadIdx.x; e < 4 * IT * IF; e += 256) {
+    const int k = e / (IT * IF), r = e % (IT * IF), h = h0 + r / IF, f = f0 + r % IF;
+    if (h < H && f < Wd) X[k * pix + (long long)h * Wd + f] = sx[k][r / IF][r % IF];
   }
 }
 
@@ -206,173 +207,29 @@ __global__ void __launch_bounds__(NTHR) nn_conv_kernel(NnArgs n, const void* in,
   }
 }
 
-// FP32 layer with register blocking: 128 threads per 16x16 tile, each computing 2 adjacent
-// pixels for all output channels; weights tap-major with the output channels contiguous, so
-// one 16-byte shared load feeds 8 fused multiply-adds
-constexpr int PB = 2;                 // pixels per thread (along the tile row)
-constexpr int NTHR_F = NTHR / PB;     // 128
-
-template <int CIN, int COUT, int ACT>
-__global__ void __launch_bounds__(NTHR_F) nn_conv_f32_kernel(NnArgs n, const void* in, void* out, int woff,
-                                                             void* outh) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  static_assert(COUT % 4 == 0, "output channels in groups of 4");
-  float* sw = reinterpret_cast<float*>(smem_raw);  // [CIN*9][COUT]
-  float* sb = sw + CIN * 9 * COUT;                  // [COUT]
-  float* sx = sb + COUT;                            // [CIN][18][18]
-  const int d = blockIdx.z;
-  const int H = n.H[d], Wd = n.W[d];
-  const int x0 = blockIdx.x * TILE, y0 = blockIdx.y * TILE;
-  if (x0 >= Wd || y0 >= H) return;
-  const long long pix = (long long)H * Wd;
-  const float* X = chan_img<float>(in, CIN, d, n.pix0);
-  float* Y = out ? chan_img<float>(out, COUT, d, n.pix0) : nullptr;  // FP32 output (optional)
-  for (int k = threadIdx.x; k < COUT * CIN * 9; k += NTHR_F) {
-    const int co = k / (CIN * 9), r = k % (CIN * 9);
-    sw[r * COUT + co] = (float)n.w[woff + k];
-  }
-  for (int k = threadIdx.x; k < COUT; k += NTHR_F) sb[k] = (float)n.w[woff + COUT * CIN * 9 + k];
-  for (int k = threadIdx.x; k < CIN * TH * TH; k += NTHR_F) {
-    const int ci = k / (TH * TH), r = k % (TH * TH);
-    const int gy = y0 + r / TH - 1, gx = x0 + r % TH - 1;
-    sx[k] = (gy >= 0 && gy < H && gx >= 0 && gx < Wd) ? X[ci * pix + (long long)gy * Wd + gx] : 0.0f;
-  }
-  __syncthreads();
-  const int ty = threadIdx.x / (TILE / PB), tx0 = (threadIdx.x % (TILE / PB)) * PB;
-  float acc[PB][COUT];
-#pragma unroll
-  for (int q = 0; q < PB; ++q)
-#pragma unroll
-    for (int co = 0; co < COUT; ++co) acc[q][co] = sb[co];
-  for (int ci = 0; ci < CIN; ++ci)
-#pragma unroll
-    for (int ky = 0; ky < 3; ++ky) {
-      const float* row = sx + ci * TH * TH + (ty + ky) * TH + tx0;
-      float x[PB + 2];
-#pragma unroll
-      for (int j = 0; j < PB + 2; ++j) x[j] = row[j];
-#pragma unroll
-      for (int kx = 0; kx < 3; ++kx) {
-        const float4* w4 = reinterpret_cast<const float4*>(sw + ((ci * 3 + ky) * 3 + kx) * COUT);
-#pragma unroll
-        for (int c4 = 0; c4 < COUT / 4; ++c4) {
-          const float4 wv = w4[c4];
-#pragma unroll
-          for (int q = 0; q < PB; ++q) {
-            const float v = x[q + kx];
-            acc[q][4 * c4 + 0] = fmaf(wv.x, v, acc[q][4 * c4 + 0]);
-            acc[q][4 * c4 + 1] = fmaf(wv.y, v, acc[q][4 * c4 + 1]);
-            acc[q][4 * c4 + 2] = fmaf(wv.z, v, acc[q][4 * c4 + 2]);
-            acc[q][4 * c4 + 3] = fmaf(wv.w, v, acc[q][4 * c4 + 3]);
-          }
-        }
-      }
-    }
-  const int gy = y0 + ty;
-#pragma unroll
-  for (int q = 0; q < PB; ++q) {
-    const int gx = x0 + tx0 + q;
-    if (gx < Wd && gy < H) {
-      const long long o = (long long)gy * Wd + gx;
-#pragma unroll
-      for (int co = 0; co < COUT; ++co) {
-        const float v = acc[q][co];
-        acc[q][co] = (ACT == 0) ? (v > 0.0f ? v : 0.0f) : tanhf(v);
-        if (Y) Y[co * pix + o] = acc[q][co];
-      }
-      if (outh) {
-        // BF16 pixel-major copy (the tensor-core layer's input), 8 channels per 16-byte store
-        __nv_bfloat16* Yh = static_cast<__nv_bfloat16*>(outh) + (d == 0 ? 0LL : (long long)COUT * n.pix0);
-#pragma unroll
-        for (int c8 = 0; c8 < COUT / 8; ++c8) {
-          *reinterpret_cast<uint4*>(Yh + o * COUT + 8 * c8) = pack_bf16x8(&acc[q][8 * c8]);
-        }
-      }
-    }
-  }
+// FP32 layer, forward or data gradient, with register blocking: 256 threads per 16x16 tile, each
+// computing PX pixels of a tile column for CG output channels from shared memory: weights
+// [input channel][tap][output channel], so that a 16-byte load feeds CG/4 * PX fused multiply-adds,
+// and the tile with its halo, of a pitch that spreads a warp's two row groups over the banks.
+//   forward:  out[co] = act(b[co] + sum_ci,ky,kx w[co][ci][ky][kx] in[ci][h+ky-1][x+kx-1])
+//   gradient: out[ci] = sum_co,ky,kx w[co][ci][ky][kx] in[co][h-ky+1][x-kx+1], times the ReLU mask of
+//             the layer below (MODE 2)
+// MODE 0: ReLU, 1: tanh, 2: gradient with mask, 3: gradient.  Sums run in the order written.
+// A tile is one block, and a small grid holds fewer tiles than the chip SMs: what counts is the
+// latency of a block.  At 128x96 the 16 -> 32 layer takes 15 us and its gradient 24; with two pixels
+// and all channels a thread (four warps a block) they took 24 and 41.  1024x1024, three stages: 3.9 ms
+// against 4.5.
+constexpr int LTHR = 256;
+template <int KO>
+struct LayerTile {
+  static constexpr int PX = KO >= 32 ? 4 : 2, CG = KO >= 8 ? 8 : 2, G = KO / CG;
+  static constexpr int PITCH = PX == 4 ? 20 : 24, WP = KO >= 8 ? KO + 4 : KO;
+  static_assert(TILE * (TILE / PX) * G == LTHR, "256 threads a tile");
+};
+template <int KI, int KO>
+constexpr size_t layer_smem() {
+  return sizeof(float) * (KI * 9 * LayerTile<KO>::WP + KO + KI * TH * LayerTile<KO>::PITCH);
 }
-
-// FP32 data gradient with the same blocking: weights [co][ky][kx][ci], input channels
-// contiguous; the ReLU mask of the layer below is applied when MASK
-template <int CIN, int COUT, bool MASK>
-__global__ void __launch_bounds__(NTHR_F) nn_dgrad_f32_kernel(NnArgs n, const void* gout, const void* aprev, void* gin,
-                                                              int woff) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  static_assert(CIN % 4 == 0, "input channels in groups of 4");
-  float* sw = reinterpret_cast<float*>(smem_raw);  // [COUT*9][CIN]
-  float* sg = sw + COUT * 9 * CIN;                  // [COUT][18][18]
-  const int d = blockIdx.z;
-  const int H = n.H[d], Wd = n.W[d];
-  const int x0 = blockIdx.x * TILE, y0 = blockIdx.y * TILE;
-  if (x0 >= Wd || y0 >= H) return;
-  const long long pix = (long long)H * Wd;
-  const float* G = chan_img<float>(gout, COUT, d, n.pix0);
-  float* D = chan_img<float>(gin, CIN, d, n.pix0);
-  for (int k = threadIdx.x; k < COUT * CIN * 9; k += NTHR_F) {
-    const int co = k / (CIN * 9), r = k % (CIN * 9), ci = r / 9, t = r % 9;
-    sw[(co * 9 + t) * CIN + ci] = (float)n.w[woff + k];
-  }
-  for (int k = threadIdx.x; k < COUT * TH * TH; k += NTHR_F) {
-    const int co = k / (TH * TH), r = k % (TH * TH);
-    const int gy = y0 + r / TH - 1, gx = x0 + r % TH - 1;
-    sg[k] = (gy >= 0 && gy < H && gx >= 0 && gx < Wd) ? G[co * pix + (long long)gy * Wd + gx] : 0.0f;
-  }
-  __syncthreads();
-  const int ty = threadIdx.x / (TILE / PB), tx0 = (threadIdx.x % (TILE / PB)) * PB;
-  float acc[PB][CIN];
-#pragma unroll
-  for (int q = 0; q < PB; ++q)
-#pragma unroll
-    for (int ci = 0; ci < CIN; ++ci) acc[q][ci] = 0.0f;
-  for (int co = 0; co < COUT; ++co)
-#pragma unroll
-    for (int ky = 0; ky < 3; ++ky) {
-      // gout at (ty - ky + 1, tx - kx + 1): tile row ty - ky + 2, columns tx0 .. tx0 + 5
-      const float* row = sg + co * TH * TH + (ty - ky + 2) * TH + tx0;
-      float x[PB + 2];
-#pragma unroll
-      for (int j = 0; j < PB + 2; ++j) x[j] = row[j];
-#pragma unroll
-      for (int kx = 0; kx < 3; ++kx) {
-        const float4* w4 = reinterpret_cast<const float4*>(sw + ((co * 3 + ky) * 3 + kx) * CIN);
-#pragma unroll
-        for (int c4 = 0; c4 < CIN / 4; ++c4) {
-          const float4 wv = w4[c4];
-#pragma unroll
-          for (int q = 0; q < PB; ++q) {
-            const float v = x[q + 2 - kx];
-            acc[q][4 * c4 + 0] = fmaf(wv.x, v, acc[q][4 * c4 + 0]);
-            acc[q][4 * c4 + 1] = fmaf(wv.y, v, acc[q][4 * c4 + 1]);
-            acc[q][4 * c4 + 2] = fmaf(wv.z, v, acc[q][4 * c4 + 2]);
-            acc[q][4 * c4 + 3] = fmaf(wv.w, v, acc[q][4 * c4 + 3]);
-          }
-        }
-      }
-    }
-  const int gy = y0 + ty;
-  const float* A = MASK ? chan_img<float>(aprev, CIN, d, n.pix0) : nullptr;
-#pragma unroll
-  for (int q = 0; q < PB; ++q) {
-    const int gx = x0 + tx0 + q;
-    if (gx < Wd && gy < H) {
-      const long long o = (long long)gy * Wd + gx;
-#pragma unroll
-      for (int ci = 0; ci < CIN; ++ci) {
-        float v = acc[q][ci];
-        if (MASK && !(A[ci * pix + o] > 0.0f)) v = 0.0f;
-        D[ci * pix + o] = v;
-      }
-    }
-  }
-}
-
-// FP32 weight gradient: a work item is (group of 4 output channels, input channel, kernel
-// row) with 4 x 3 sums (the three kernel columns); per pixel one 16-byte load of the output
-// gradient and one input value slid along the row.  The tile's 16 rows are split into R
-// parts so that every thread carries exactly 3 (item, part) units (NI * R = 768 for the three
-// layers); the parts, and the bias sums (every thread sums a strided subset of the tile's
-// pixels for one channel), are added in shared memory in a fixed order at the end.
-constexpr int WG_UNITS = 3 * NTHR;
 
 // 4-byte asynchronous global -> shared copy (zero-filled, nothing read, when !valid; src must
 // still be a valid address), and its group commit / wait
@@ -385,6 +242,117 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+
+template <int KI, int KO, int MODE>
+__global__ void __launch_bounds__(LTHR) nn_layer_f32_kernel(NnArgs n, const void* in, const void* aprev, void* out,
+                                                            int woff, void* outh) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  using P = LayerTile<KO>;
+  constexpr bool GRAD = MODE >= 2;
+  constexpr int PX = P::PX, CG = P::CG, NW = KI * KO * 9;
+  float* sw = reinterpret_cast<float*>(smem_raw);  // [KI*9][WP]
+  float* sb = sw + KI * 9 * P::WP;                 // [KO]
+  float* sx = sb + KO;                             // [KI][18][PITCH]
+  const int d = blockIdx.z;
+  const int H = n.H[d], Wd = n.W[d];
+  const int x0 = blockIdx.x * TILE, y0 = blockIdx.y * TILE;
+  if (x0 >= Wd || y0 >= H) return;  // the grid covers the larger image
+  const long long pix = (long long)H * Wd;
+  const float* X = chan_img<float>(in, KI, d, n.pix0);
+  float* Y = out ? chan_img<float>(out, KO, d, n.pix0) : nullptr;  // (optional in the forward)
+  for (int k = threadIdx.x; k < KI * TH * TH; k += LTHR) {
+    const int ci = k / (TH * TH), r = k % (TH * TH), ry = r / TH, rx = r % TH;
+    const int gy = y0 + ry - 1, gx = x0 + rx - 1;
+    const bool ok = gy >= 0 && gy < H && gx >= 0 && gx < Wd;
+    cp_async4(sx + (ci * TH + ry) * P::PITCH + rx, X + ci * pix + (ok ? (long long)gy * Wd + gx : 0), ok);
+  }
+  cp_async_commit();
+  const int tx = threadIdx.x % TILE, ty = (threadIdx.x / TILE) % (TILE / PX) * PX;
+  const int c0 = threadIdx.x / (TILE * TILE / PX) * CG;
+  const int gx = x0 + tx;
+  unsigned mask = 0;  // the ReLU mask's bits, read before the sums (the stores could alias it)
+  if constexpr (MODE == 2) {
+    const float* A = chan_img<float>(aprev, KO, d, n.pix0);
+#pragma unroll
+    for (int q = 0; q < PX; ++q)
+#pragma unroll
+      for (int c = 0; c < CG; ++c) {
+        const int gy = y0 + ty + q;
+        if (gx < Wd && gy < H && A[(c0 + c) * pix + (long long)gy * Wd + gx] > 0.0f) mask |= 1u << (q * CG + c);
+      }
+  }
+#pragma unroll 6
+  for (int k = threadIdx.x; k < NW; k += LTHR) {
+    const float w = (float)n.w[woff + k];
+    const int row = GRAD ? (k / (9 * KO)) * 9 + k % 9 : k % (KI * 9), ch = GRAD ? (k / 9) % KO : k / (KI * 9);
+    sw[row * P::WP + ch] = w;
+  }
+  if (!GRAD)
+    for (int k = threadIdx.x; k < KO; k += LTHR) sb[k] = (float)n.w[woff + NW + k];
+  cp_async_wait<0>();
+  __syncthreads();
+  float acc[PX][CG];
+#pragma unroll
+  for (int q = 0; q < PX; ++q)
+#pragma unroll
+    for (int c = 0; c < CG; ++c) acc[q][c] = GRAD ? 0.0f : sb[c0 + c];
+#pragma unroll 1
+  for (int ci = 0; ci < KI; ++ci) {
+    float x[PX + 2][3];
+#pragma unroll
+    for (int r = 0; r < PX + 2; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) x[r][k] = sx[(ci * TH + ty + r) * P::PITCH + tx + k];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      const int ky = t / 3, kx = t % 3;
+      const float* wr = sw + (ci * 9 + t) * P::WP + c0;
+      float w[CG];
+      if constexpr (CG == 8) {
+        const float4 a = *reinterpret_cast<const float4*>(wr), b = *reinterpret_cast<const float4*>(wr + 4);
+        w[0] = a.x, w[1] = a.y, w[2] = a.z, w[3] = a.w, w[4] = b.x, w[5] = b.y, w[6] = b.z, w[7] = b.w;
+      } else {
+        const float2 a = *reinterpret_cast<const float2*>(wr);
+        w[0] = a.x, w[1] = a.y;
+      }
+#pragma unroll
+      for (int q = 0; q < PX; ++q) {
+        const float v = GRAD ? x[q + 2 - ky][2 - kx] : x[q + ky][kx];
+#pragma unroll
+        for (int c = 0; c < CG; ++c) acc[q][c] = fmaf(w[c], v, acc[q][c]);
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < PX; ++q) {
+    const int gy = y0 + ty + q;
+    if (gx >= Wd || gy >= H) continue;
+    const long long o = (long long)gy * Wd + gx;
+#pragma unroll
+    for (int c = 0; c < CG; ++c) {
+      float v = acc[q][c];
+      if (MODE == 0) v = v > 0.0f ? v : 0.0f;
+      if (MODE == 1) v = tanhf(v);
+      if (MODE == 2 && !(mask >> (q * CG + c) & 1)) v = 0.0f;
+      acc[q][c] = v;
+      if (Y) Y[(c0 + c) * pix + o] = v;
+    }
+    if constexpr (CG == 8) {
+      // BF16 pixel-major copy (the tensor-core layer's input), 8 channels per 16-byte store
+      if (outh)
+        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(outh) + (d == 0 ? 0LL : (long long)KO * n.pix0) +
+                                  o * KO + c0) = pack_bf16x8(acc[q]);
+    }
+  }
+}
+
+// FP32 weight gradient: a work item is (group of 4 output channels, input channel, kernel
+// row) with 4 x 3 sums (the three kernel columns); per pixel one 16-byte load of the output
+// gradient and one input value slid along the row.  The tile's 16 rows are split into R
+// parts so that every thread carries exactly 3 (item, part) units (NI * R = 768 for the three
+// layers); the parts, and the bias sums (every thread sums a strided subset of the tile's
+// pixels for one channel), are added in shared memory in a fixed order at the end.
+constexpr int WG_UNITS = 3 * NTHR;
 
 template <int CIN, int COUT>
 __host__ __device__ constexpr int wgrad_tile_floats() {
@@ -1334,18 +1302,19 @@ __global__ void nn_unload_kernel(const T* __restrict__ G, double* __restrict__ G
 // stage output (or RHS) minus the neural flux divergence on fluid cells
 template <class T>
 __global__ void __launch_bounds__(256) nn_apply_kernel(NnArgs n, StageArgs a, int rhs) {
-  // 32 x 32 cells per block: the tile's y-face fluxes (image 1: line = column i, face = row j)
-  // pass through shared memory, so both images are read along their contiguous axis
-  __shared__ T sy[4][IT][IT + 2];
+  // 32 x 8 cells per block, a cell a thread: the tile's y-face fluxes (image 1: line = column i,
+  // face = row j) pass through shared memory, so both images are read along their contiguous axis
+  __shared__ T sy[4][IT][IF + 2];
   const Lay& L = a.lay;
-  const int i0 = blockIdx.x * IT, j0 = blockIdx.y * IT;
+  const int nbx = (L.nx + IT - 1) / IT;
+  const int i0 = (int)(blockIdx.x % nbx) * IT, j0 = (int)(blockIdx.x / nbx) * IF;
   const long long ncell = (long long)L.nx * L.ny;
   const bool two = n.nimg > 1;
   if (two) {
     const T* Fy = chan_img<T>(n.T3, 4, 1, n.pix0);
     const long long py = (long long)n.H[1] * n.W[1];
-    for (int e = threadIdx.x; e < 4 * IT * (IT + 1); e += 256) {
-      const int k = e / (IT * (IT + 1)), r = e % (IT * (IT + 1)), il = r / (IT + 1), jl = r % (IT + 1);
+    for (int e = threadIdx.x; e < 4 * IT * (IF + 1); e += 256) {
+      const int k = e / (IT * (IF + 1)), r = e % (IT * (IF + 1)), il = r / (IF + 1), jl = r % (IF + 1);
       const int i = i0 + il, j = j0 + jl;
       sy[k][il][jl] = (i < L.nx && j <= L.ny) ? Fy[k * py + (long long)i * n.W[1] + j] : (T)0;
     }
@@ -1358,7 +1327,7 @@ __global__ void __launch_bounds__(256) nn_apply_kernel(NnArgs n, StageArgs a, in
   const float cxf = (float)a.cx, cyf = (float)a.cy;
   const float scf[4] = {(float)n.scale[0], (float)n.scale[1], (float)n.scale[2], (float)n.scale[3]};
   const int il = threadIdx.x % IT;
-  for (int jl = threadIdx.x / IT; jl < IT; jl += 256 / IT) {
+  for (int jl = threadIdx.x / IT; jl < IF; jl += 256 / IT) {
     const int i = i0 + il, j = j0 + jl;
     if (i >= L.nx || j >= L.ny) continue;
     const long long o = (long long)j * L.nx + i;
@@ -1539,11 +1508,18 @@ __global__ void __launch_bounds__(NTHR) nn_wgrad_kernel(NnArgs n, const void* go
   }
 }
 
-__global__ void nn_wreduce_kernel(NnArgs n) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= NN_NPARAM) return;
+// the partial weight gradients summed: 32 parameters a block, eight threads each
+__global__ void __launch_bounds__(256) nn_wreduce_kernel(NnArgs n) {
+  __shared__ double part[8][32];
+  const int kl = threadIdx.x % 32, p = threadIdx.x / 32, k = blockIdx.x * 32 + kl;
   double s = 0.0;
-  for (int b = 0; b < n.nwblk; ++b) s += n.partial[(long long)b * NN_NPARAM + k];
+  if (k < NN_NPARAM)
+#pragma unroll 4
+    for (int b = p; b < n.nwblk; b += 8) s += n.partial[(long long)b * NN_NPARAM + k];
+  part[p][kl] = s;
+  __syncthreads();
+  if (p != 0 || k >= NN_NPARAM) return;
+  for (int q = 1; q < 8; ++q) s += part[q][kl];
   n.w_bar[k] += s;
 }
 
@@ -1556,10 +1532,10 @@ __device__ __forceinline__ double nn_warp_sum(double v) {
 // d/dgamma of the face energies (added to pbar[0]); 32 x 32 pixel tiles as nn_image_kernel
 template <class T>
 __global__ void __launch_bounds__(256) nn_image_vjp_kernel(NnArgs n, AdjArgs a) {
-  __shared__ T sx[4][IT][IT + 1];
+  __shared__ T sx[4][IT][IF + 1];
   const int d = blockIdx.z;
   const int H = n.H[d], Wd = n.W[d];
-  const int f0 = blockIdx.x * IT, h0 = blockIdx.y * IT;
+  const int f0 = blockIdx.x * IF, h0 = blockIdx.y * IT;
   // per-warp partials of pbar[0] (gamma; the other three entries 0), summed with the other
   // partials of the stage in a fixed order: warp w of block b writes pp[4 (8 b + w) + k]
   const long long blk = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
@@ -1570,16 +1546,16 @@ __global__ void __launch_bounds__(256) nn_image_vjp_kernel(NnArgs n, AdjArgs a) 
   }
   const long long pix = (long long)H * Wd;
   const T* dX = chan_img<T>(n.G4, 4, d, n.pix0);
-  for (int e = threadIdx.x; e < 4 * IT * IT; e += 256) {
-    const int k = e / (IT * IT), r = e % (IT * IT), h = h0 + r / IT, f = f0 + r % IT;
-    sx[k][r / IT][r % IT] = (h < H && f < Wd) ? dX[k * pix + (long long)h * Wd + f] : (T)0;
+  for (int e = threadIdx.x; e < 4 * IT * IF; e += 256) {
+    const int k = e / (IT * IF), r = e % (IT * IF), h = h0 + r / IF, f = f0 + r % IF;
+    sx[k][r / IF][r % IF] = (h < H && f < Wd) ? dX[k * pix + (long long)h * Wd + f] : (T)0;
   }
   __syncthreads();
   double gbar = 0.0;
   const int hl = threadIdx.x % IT;
   const int un = (d == 0) ? 1 : 2, ut = (d == 0) ? 2 : 1;
   const int fdir = d * 8;
-  for (int fl = threadIdx.x / IT; fl < IT; fl += 256 / IT) {
+  for (int fl = threadIdx.x / IT; fl < IF; fl += 256 / IT) {
     const int h = h0 + hl, f = f0 + fl;
     if (h >= H || f >= Wd) continue;
     double wl[4], wr[4];
@@ -1623,7 +1599,7 @@ dim3 image_grid(const NnArgs& n) {
     W = W > n.W[1] ? W : n.W[1];
     H = H > n.H[1] ? H : n.H[1];
   }
-  return dim3(cdiv(W, IT), cdiv(H, IT), n.nimg);
+  return dim3(cdiv(W, IF), cdiv(H, IT), n.nimg);
 }
 
 dim3 tile_grid(const NnArgs& n) {
@@ -1638,11 +1614,11 @@ dim3 tile_grid(const NnArgs& n) {
 template <class T, int CIN, int COUT, int ACT>
 cudaError_t conv(const NnArgs& n, const void* in, void* out, int woff, cudaStream_t s, void* outh = nullptr) {
   if (std::is_same<T, float>::value) {
-    const size_t sm = sizeof(float) * (CIN * 9 * COUT + COUT + CIN * TH * TH);
-    auto k = nn_conv_f32_kernel<CIN, COUT, ACT>;
+    const size_t sm = layer_smem<CIN, COUT>();
+    auto k = nn_layer_f32_kernel<CIN, COUT, ACT>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k<<<tile_grid(n), NTHR_F, sm, s>>>(n, in, out, woff, outh);
+    k<<<tile_grid(n), LTHR, sm, s>>>(n, in, nullptr, out, woff, outh);
     return cudaGetLastError();
   }
   constexpr int NW = COUT * CIN * 9 + COUT;
@@ -1657,11 +1633,11 @@ cudaError_t conv(const NnArgs& n, const void* in, void* out, int woff, cudaStrea
 template <class T, int CIN, int COUT, bool MASK>
 cudaError_t dgrad(const NnArgs& n, const void* gout, const void* aprev, void* gin, int woff, cudaStream_t s) {
   if (std::is_same<T, float>::value) {
-    const size_t sm = sizeof(float) * (COUT * 9 * CIN + COUT * TH * TH);
-    auto k = nn_dgrad_f32_kernel<CIN, COUT, MASK>;
+    const size_t sm = layer_smem<COUT, CIN>();
+    auto k = nn_layer_f32_kernel<COUT, CIN, MASK ? 2 : 3>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k<<<tile_grid(n), NTHR_F, sm, s>>>(n, gout, aprev, gin, woff);
+    k<<<tile_grid(n), LTHR, sm, s>>>(n, gout, aprev, gin, woff, nullptr);
     return cudaGetLastError();
   }
   constexpr int NWW = COUT * CIN * 9;
@@ -1823,7 +1799,7 @@ cudaError_t layers_vjp_t(const NnArgs& n, cudaStream_t s) {
   if ((e = dgrad<T, 4, 16, false>(n, n.G16, nullptr, n.G4, NN_OFF1, s)) != cudaSuccess) return e;  // G4 = dX
   if (n.w_bar) {
     if ((e = wgrad<T, 4, 16>(n, n.G16, n.X, NN_OFF1, s)) != cudaSuccess) return e;
-    nn_wreduce_kernel<<<cdiv(NN_NPARAM, 256), 256, 0, s>>>(n);
+    nn_wreduce_kernel<<<cdiv(NN_NPARAM, 32), 256, 0, s>>>(n);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1892,7 +1868,7 @@ cudaError_t nn_eval_vjp(const NnArgs& n, const double* X, int H, int W, const do
 }
 
 cudaError_t nn_apply(const NnArgs& n, const StageArgs& a, bool rhs, cudaStream_t s) {
-  const dim3 grid(cdiv(a.lay.nx, IT), cdiv(a.lay.ny, IT));
+  const unsigned grid = cdiv(a.lay.nx, IT) * cdiv(a.lay.ny, IF);
   if (n.fp32) nn_apply_kernel<float><<<grid, 256, 0, s>>>(n, a, rhs ? 1 : 0);
   else nn_apply_kernel<double><<<grid, 256, 0, s>>>(n, a, rhs ? 1 : 0);
   return cudaGetLastError();
