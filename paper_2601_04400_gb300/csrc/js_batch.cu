@@ -581,18 +581,24 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       __syncthreads();  // the next block of lines reuses shared memory
     }
   } else if constexpr (PH == RP_CELLS) {
-    rev_items(b, RK_PLANE, [&](int k, long long t) {
-      if (k < 0) return;
+    // (the planes' items are padded to whole blocks: one instance a block)
+    const long long* pre = b.pre + (long long)RK_PLANE * (b.count + 1);
+    __shared__ AdjArgs a;  // (in registers it would cost resident warps)
+    for (long long base = (long long)blockIdx.x * BNT; base < pre[b.count]; base += (long long)gridDim.x * BNT) {
+      const int k = find_inst64(pre, b.count, base);
       const InstDesc& d = b.inst[k];
       const InstRev& r = b.rev[k];
-      const AdjArgs a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
+      const long long t = base + threadIdx.x - pre[k];
+      __syncthreads();  // the previous block's readers of a
+      if (threadIdx.x == 0) a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
+      __syncthreads();
       const double* src = even ? r.P0 : r.P1;
       double gb = 0.0, nb = 0.0;
       const double bdt = REV_B[s] * call.dt[k];
       if (d.visc) adj_cell<true>(a, src, r.Uacc, REV_A[s], REV_B[s], bdt, 0, t, gb, nb);
       else adj_cell<false>(a, src, r.Uacc, REV_A[s], REV_B[s], bdt, 0, t, gb, nb);
       warp_partials(a.pp, r.off_c + (t >> 5), gb, 0.0, 0.0, nb);
-    });
+    }
   } else if constexpr (PH == RP_BCTY || PH == RP_BCTX) {
     rev_items(b, PH == RP_BCTY ? RK_BCTY : RK_BCTX, [&](int k, long long t) {
       if (k < 0) return;
@@ -682,7 +688,7 @@ __global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
 
 // one phase of the reverse step as a kernel of its own (split launch)
 template <int PH, int VM = 0>
-__global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
+__global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 : PH == RP_CELLS ? 4 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
   extern __shared__ double smem[];
   rev_phase<PH, VM>(b, s, smem);
 }
@@ -786,13 +792,14 @@ int rev_prepare(js_batch* b) {
     rblock0[k + 1] = rblock0[k] + blocks;
     r.w_lines = blocks;
     r.off_c = r.w_lines;
-    r.w_c = round32(L.plane) / 32;
+    const long long plane = (L.plane + js::BNT - 1) / js::BNT * js::BNT;  // (whole blocks)
+    r.w_c = plane / 32;
     r.off_g = r.off_c + r.w_c;
     r.w_g = round32(4LL * d.ib.n) / 32;  // (a quad of lanes a ghost and a source)
     r.off_s = r.off_g + r.w_g;
     r.w_s = round32(4LL * r.ibt.nsrc) / 32;
     const long long cnt[js::RK_N] = {
-        round32(L.plane), round32(4LL * L.nx * L.ny), round32(4LL * d.ib.n), round32(js::halo_count(L)),
+        plane, round32(4LL * L.nx * L.ny), round32(4LL * d.ib.n), round32(js::halo_count(L)),
         round32(8LL * (L.nx + 6)), round32(8LL * L.ny), round32(4LL * r.ibt.nsrc)};
     for (int q = 0; q < js::RK_N; ++q) pre[(size_t)q * (n + 1) + k + 1] = pre[(size_t)q * (n + 1) + k] + cnt[q];
   }
