@@ -9,10 +9,7 @@
 //              per stage: IB fill | halo fill | lines | cells (the per-grid kernels' device
 //                         functions, so trajectories equal js_step's bit for bit)
 //   unpack     padded buffers -> user states
-// The forward runs these phases as ordinary launches on the batch's stream.  The reverse step does so
-// too or runs its phases in one persistent cooperative launch separated by grid barriers; every
-// barrier wait is bounded: a block that waits longer than the budget sets JS_ERR_TIMEOUT in the error
-// flag and returns, and the others leave at their next wait.
+// Forward and reverse run their phases as ordinary launches on the batch's stream.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -372,15 +369,14 @@ __global__ void __launch_bounds__(FNT, PH == FP_LINES ? 4 : 1) batch_phase_kerne
   fwd_phase<PH, VM>(b, step, s, smem);
 }
 
-// one grid barrier of the persistent reverse launch (js_batch_test_timeout)
+// one bounded grid barrier (js_batch_test_timeout)
 __global__ void __launch_bounds__(FNT) batch_barrier_kernel(BatchArgs b) {
   grid_sync_on(b.bar, b.err, b.extra_arrivals, b.budget);
 }
 
 // =======================================================================================
-// persistent batched reverse: one launch reverses one SSP-RK3 step of every instance (the
-// gradient chain rule of Sec. 2 per instance) -- the per-grid js_step_vjp's phases, each run
-// over the work items of all instances, separated by grid barriers:
+// batched reverse of one SSP-RK3 step of every instance (the gradient chain rule of Sec. 2 per
+// instance) -- the per-grid js_step_vjp's phases, each run over the work items of all instances:
 //   pack U_n, lambda_{n+1}; zero Uacc
 //   forward recompute, stages 0 and 1: IB fill | halo fill | stage tiles; IB and halo fill of
 //   the stage-2 input
@@ -390,8 +386,8 @@ __global__ void __launch_bounds__(FNT) batch_barrier_kernel(BatchArgs b) {
 //   unpack lambda_n (+ the last reduction)
 // The device bodies are those of the per-grid launches (js_adjoint_body.cuh, js_stage.cuh,
 // js_fill.cuh) on the same elements in the same order; the parameter gradient is reduced in a
-// fixed order too.  Work items of every instance are padded to whole warps, so a warp never spans
-// two instances.
+// fixed order too.  Work items of every instance are padded to whole warps (planes: to whole blocks),
+// so a warp never spans two instances.
 // =======================================================================================
 enum RevKind { RK_PLANE = 0, RK_USER4, RK_GHOST, RK_HALO, RK_BCTY, RK_BCTX, RK_SRC, RK_N };
 
@@ -416,9 +412,7 @@ struct BatchRevArgs {
   const int* line0;
   const int* rblock0;         // prefix sums (count + 1) of the reverse line blocks
   RevCall call;
-  unsigned* bar;
   int* err;
-  long long budget;
 };
 
 // every item g of kind K over all instances: f(k, local) with k = -1 past the end (whole
@@ -460,10 +454,11 @@ __device__ __forceinline__ void rev_reduce(const InstRev& r, double* pbar) {
 // the stage constants of the SSP-RK3 step
 __device__ constexpr double REV_A[3] = {0.0, 0.75, 1.0 / 3.0}, REV_B[3] = {1.0, 0.25, 2.0 / 3.0};
 
-// The phases of one batched reverse step.  Each runs over the work items of all instances with
-// grid-stride loops, so it is correct for any grid; the persistent kernel runs them in order
-// with grid barriers between them, the split launch as one kernel per phase (each with its own
-// register allocation and occupancy).
+// The phases of one batched reverse step, a kernel each with its own registers and occupancy; they run
+// over the work items of all instances with grid-stride loops, so any grid is correct.  One persistent
+// cooperative kernel with grid barriers between them, at the registers of the heaviest, took 9.3 ms for
+// 16 instances of 128x128 to 512x256 where the launches take 7.6, and no less for one 32x24 instance
+// (0.95 and 0.92 ms).
 enum RevPhase {
   RP_PACK = 0,      // pack U_n, lambda_{n+1} (and given stage states); Uacc = 0
   RP_GHOST,         // IB fill of stage input s
@@ -481,7 +476,7 @@ enum RevPhase {
   RP_N
 };
 
-// VM: the instances of the line phases (0 all, 1 the viscous ones, 2 the inviscid ones)
+// VM: the instances of the line phases (1 the viscous ones, 2 the inviscid ones)
 template <int PH, int VM = 0>
 __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* smem) {
   const RevCall& call = b.call;
@@ -528,13 +523,12 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     for (int it = blockIdx.x; it < b.line0[b.count]; it += gridDim.x) {
       const int k = find_inst(b.line0, b.count, it);
       const InstDesc& d = b.inst[k];
-      if ((VM == 1 && !d.visc) || (VM == 2 && d.visc)) continue;  // the other launch's instance
+      if ((VM == 1) != (d.visc != 0)) continue;  // the other launch's instance
       __shared__ StageArgs sa;
       if (threadIdx.x == 0) fill_stage_args(sa, d, (s == 0) ? d.N : d.A, b.err);
       __syncthreads();
       const int t = it - b.line0[k], bx = stage_blocks(d.lay, 0);
-      if (VM == 1 || (VM == 0 && d.visc)) stage_lines<true, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
-      if (VM == 2 || (VM == 0 && !d.visc)) stage_lines<false, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
+      stage_lines<VM == 1, false>(sa, t < bx ? 0 : 1, t < bx ? t : t - bx, smem);
       __syncthreads();  // the next block of lines reuses shared memory
     }
   } else if constexpr (PH == RP_STAGE_CELLS) {
@@ -568,7 +562,7 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     for (int it = blockIdx.x; it < b.rblock0[b.count]; it += gridDim.x) {
       const int k = find_inst(b.rblock0, b.count, it);
       const InstDesc& d = b.inst[k];
-      if ((VM == 1 && !d.visc) || (VM == 2 && d.visc)) continue;  // the other launch's instance
+      if ((VM == 1) != (d.visc != 0)) continue;  // the other launch's instance
       const InstRev& r = b.rev[k];
       __shared__ AdjArgs a;  // (in registers it would cost resident warps)
       if (threadIdx.x == 0) a = rev_adj(r, d, s, call, k, even ? r.P1 : r.P0, true);
@@ -576,8 +570,7 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
       const double* src = even ? r.P0 : r.P1;
       const int t = it - b.rblock0[k], bx = adj_blocks(d.lay, 0);
       const double bdt = REV_B[s] * call.dt[k];
-      if (VM == 1 || (VM == 0 && d.visc)) adj_lines<true>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
-      if (VM == 2 || (VM == 0 && !d.visc)) adj_lines<false>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
+      adj_lines<VM == 1>(a, src, bdt, t < bx ? 0 : 1, t < bx ? t : t - bx, smem, t);
       __syncthreads();  // the next block of lines reuses shared memory
     }
   } else if constexpr (PH == RP_CELLS) {
@@ -649,44 +642,7 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
   }
 }
 
-__global__ void __launch_bounds__(BNT, 2) batch_vjp_kernel(BatchRevArgs b) {
-  extern __shared__ double smem[];
-  rev_phase<RP_PACK>(b, 0, smem);
-  if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-  // ---- forward recompute of the stage inputs X0 = N, X1 = A, X2 = B
-  for (int s = 0; s < 3; ++s) {
-    rev_phase<RP_GHOST>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_HALO>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    if (s == 2) break;
-    if (b.call.U1) continue;  // the stage states were given: only their ghosts and halos are filled
-    rev_phase<RP_STAGE>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_STAGE_CELLS>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-  }
-  // ---- reverse through the stages 2, 1, 0: P0 -> P1 -> P0 -> P1
-  for (int s = 2; s >= 0; --s) {
-    rev_phase<RP_REDUCE>(b, s, smem);
-    if (s < 2 && b.call.pbar && !grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_LINES>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_CELLS>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_BCTY>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_BCTX>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_INFLOW_GHOST>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-    rev_phase<RP_SRC>(b, s, smem);
-    if (!grid_sync_on(b.bar, b.err, 0, b.budget)) return;
-  }
-  rev_phase<RP_UNPACK>(b, 0, smem);
-}
-
-// one phase of the reverse step as a kernel of its own (split launch)
+// one phase of the reverse step
 template <int PH, int VM = 0>
 __global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 : PH == RP_CELLS ? 4 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
   extern __shared__ double smem[];
@@ -737,13 +693,12 @@ struct js_batch {
   int ntiles = 0;
   long long cells = 0;
   bool states_set = false;
-  // persistent reverse (prepared by the first reverse call)
+  // reverse (prepared by the first reverse call)
   bool rev_ready = false;
   js::InstRev* d_rev = nullptr;
   long long* d_pre = nullptr;   // [RK_N][count + 1]
-  int rev_blocks = 0;
-  int rev_split = 0;                  // 1: one launch per phase (js_batch_set_reverse_launch)
-  int rev_pblocks[js::RP_N] = {};     // grid of each phase kernel of the split launch
+  int rev_split = 0;                  // js_batch_set_reverse_launch (both forms run the same launches)
+  int rev_pblocks[js::RP_N] = {};     // grid of each phase kernel
   int* d_rblock0 = nullptr;            // prefix sums of the reverse line blocks
   std::vector<int> rblock0;
   bool has_visc = false, has_inv = false;  // the batch holds viscous / inviscid instances
@@ -766,7 +721,6 @@ int js_internal_rev_desc(js_ctx* c, js::InstRev* d);
 namespace {
 size_t batch_smem() { return js::stage_smem<true>(); }
 constexpr size_t kLineSmem = sizeof(double) * 8 * js::AP;
-size_t rev_smem() { return std::max(batch_smem(), kLineSmem); }
 }  // namespace
 
 namespace {
@@ -803,17 +757,10 @@ int rev_prepare(js_batch* b) {
         round32(8LL * (L.nx + 6)), round32(8LL * L.ny), round32(4LL * r.ibt.nsrc)};
     for (int q = 0; q < js::RK_N; ++q) pre[(size_t)q * (n + 1) + k + 1] = pre[(size_t)q * (n + 1) + k] + cnt[q];
   }
-  const size_t smem = rev_smem();
-  if (cudaFuncSetAttribute(js::batch_vjp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return JS_ERR_CUDA;
-  int dev = 0, sms = 0, per_sm = 0;
+  int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, js::batch_vjp_kernel, js::BNT, smem);
-  if (per_sm < 1) return JS_ERR_CUDA;
-  b->rev_blocks = sms * per_sm;
-  // the split launch: each phase kernel's own resident blocks per SM
+  // each phase kernel's own resident blocks
   const void* kern[js::RP_N] = {
       (const void*)js::batch_vjp_phase_kernel<js::RP_PACK>, (const void*)js::batch_vjp_phase_kernel<js::RP_GHOST>,
       (const void*)js::batch_vjp_phase_kernel<js::RP_HALO>, (const void*)js::batch_vjp_phase_kernel<js::RP_STAGE, 1>,
@@ -846,7 +793,7 @@ int rev_prepare(js_batch* b) {
   return JS_OK;
 }
 
-// one persistent cooperative launch reversing one step of every instance
+// the launches reversing one step of every instance; kernel boundaries order the phases
 int rev_launch(js_batch* b, const js::RevCall& call) {
   js::BatchRevArgs a;
   a.inst = b->d_desc;
@@ -857,56 +804,42 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
   a.line0 = b->d_line0;
   a.rblock0 = b->d_rblock0;
   a.call = call;
-  a.bar = b->d_bar;
   a.err = b->d_err;
-  int dev = 0, khz = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
-  a.budget = (long long)(2.0 * (khz > 0 ? khz : 2000000) * 1e3);  // 2 s of SM clock cycles
-  if (b->rev_split) {
-    // one launch per phase, in the persistent kernel's order; kernel boundaries take the place
-    // of its grid barriers
-    bool ok = true;
-    // the line phases: a block an item, viscous and inviscid instances apart
-    auto run_lines = [&](auto visc, auto inv, int blocks, size_t smem, int s) {
-      if (!ok) return;
-      if (b->has_visc) visc<<<blocks, js::BNT, smem, b->stream>>>(a, s);
-      if (b->has_inv) inv<<<blocks, js::BNT, smem, b->stream>>>(a, s);
-      ok = cudaGetLastError() == cudaSuccess;
-    };
-    auto run = [&](auto kernel, int ph, int s) {
-      if (!ok) return;
-      kernel<<<b->rev_pblocks[ph], js::BNT, 0, b->stream>>>(a, s);
-      ok = cudaGetLastError() == cudaSuccess;
-    };
-    run(js::batch_vjp_phase_kernel<js::RP_PACK>, js::RP_PACK, 0);
-    for (int s = 0; s < 3; ++s) {
-      run(js::batch_vjp_phase_kernel<js::RP_GHOST>, js::RP_GHOST, s);
-      run(js::batch_vjp_phase_kernel<js::RP_HALO>, js::RP_HALO, s);
-      if (s == 2) break;
-      if (call.U1) continue;
-      run_lines(js::batch_vjp_phase_kernel<js::RP_STAGE, 1>, js::batch_vjp_phase_kernel<js::RP_STAGE, 2>, b->line0.back(),
-                batch_smem(), s);
-      run(js::batch_vjp_phase_kernel<js::RP_STAGE_CELLS>, js::RP_STAGE_CELLS, s);
-    }
-    for (int s = 2; s >= 0; --s) {
-      if (s < 2 && call.pbar) run(js::batch_vjp_phase_kernel<js::RP_REDUCE>, js::RP_REDUCE, s);
-      run_lines(js::batch_vjp_phase_kernel<js::RP_LINES, 1>, js::batch_vjp_phase_kernel<js::RP_LINES, 2>,
-                b->rblock0.back(), kLineSmem, s);
-      run(js::batch_vjp_phase_kernel<js::RP_CELLS>, js::RP_CELLS, s);
-      run(js::batch_vjp_phase_kernel<js::RP_BCTY>, js::RP_BCTY, s);
-      run(js::batch_vjp_phase_kernel<js::RP_BCTX>, js::RP_BCTX, s);
-      run(js::batch_vjp_phase_kernel<js::RP_INFLOW_GHOST>, js::RP_INFLOW_GHOST, s);
-      run(js::batch_vjp_phase_kernel<js::RP_SRC>, js::RP_SRC, s);
-    }
-    run(js::batch_vjp_phase_kernel<js::RP_UNPACK>, js::RP_UNPACK, 0);
-    return ok ? JS_OK : JS_ERR_CUDA;
+  bool ok = true;
+  // the line phases: a block an item, viscous and inviscid instances apart
+  auto run_lines = [&](auto visc, auto inv, int blocks, size_t smem, int s) {
+    if (!ok) return;
+    if (b->has_visc) visc<<<blocks, js::BNT, smem, b->stream>>>(a, s);
+    if (b->has_inv) inv<<<blocks, js::BNT, smem, b->stream>>>(a, s);
+    ok = cudaGetLastError() == cudaSuccess;
+  };
+  auto run = [&](auto kernel, int ph, int s) {
+    if (!ok) return;
+    kernel<<<b->rev_pblocks[ph], js::BNT, 0, b->stream>>>(a, s);
+    ok = cudaGetLastError() == cudaSuccess;
+  };
+  run(js::batch_vjp_phase_kernel<js::RP_PACK>, js::RP_PACK, 0);
+  for (int s = 0; s < 3; ++s) {
+    run(js::batch_vjp_phase_kernel<js::RP_GHOST>, js::RP_GHOST, s);
+    run(js::batch_vjp_phase_kernel<js::RP_HALO>, js::RP_HALO, s);
+    if (s == 2) break;
+    if (call.U1) continue;
+    run_lines(js::batch_vjp_phase_kernel<js::RP_STAGE, 1>, js::batch_vjp_phase_kernel<js::RP_STAGE, 2>, b->line0.back(),
+              batch_smem(), s);
+    run(js::batch_vjp_phase_kernel<js::RP_STAGE_CELLS>, js::RP_STAGE_CELLS, s);
   }
-  void* args[] = {&a};
-  if (cudaLaunchCooperativeKernel((void*)js::batch_vjp_kernel, dim3(b->rev_blocks), dim3(js::BNT), args,
-                                  rev_smem(), b->stream) != cudaSuccess)
-    return JS_ERR_CUDA;
-  return JS_OK;
+  for (int s = 2; s >= 0; --s) {
+    if (s < 2 && call.pbar) run(js::batch_vjp_phase_kernel<js::RP_REDUCE>, js::RP_REDUCE, s);
+    run_lines(js::batch_vjp_phase_kernel<js::RP_LINES, 1>, js::batch_vjp_phase_kernel<js::RP_LINES, 2>,
+              b->rblock0.back(), kLineSmem, s);
+    run(js::batch_vjp_phase_kernel<js::RP_CELLS>, js::RP_CELLS, s);
+    run(js::batch_vjp_phase_kernel<js::RP_BCTY>, js::RP_BCTY, s);
+    run(js::batch_vjp_phase_kernel<js::RP_BCTX>, js::RP_BCTX, s);
+    run(js::batch_vjp_phase_kernel<js::RP_INFLOW_GHOST>, js::RP_INFLOW_GHOST, s);
+    run(js::batch_vjp_phase_kernel<js::RP_SRC>, js::RP_SRC, s);
+  }
+  run(js::batch_vjp_phase_kernel<js::RP_UNPACK>, js::RP_UNPACK, 0);
+  return ok ? JS_OK : JS_ERR_CUDA;
 }
 
 }  // namespace
