@@ -40,17 +40,21 @@ __device__ __forceinline__ void warp_partials(double* pp, long long w, double g,
 }
 // the same summed over the block's warps in order (at most 8 warps, all threads call it): one slot
 // per block, so that the final reduction stays short
-__device__ __forceinline__ void block_partials(double* pp, long long slot, double g, double m, double pr, double n) {
-  if (pp == nullptr) return;
+// the block's sums of the four values, value k on thread k < 4 (the other threads return nothing)
+__device__ __forceinline__ double block_sum4(double a, double b, double c, double d) {
   __shared__ double part[8][4];
-  const double v = warp_sum4(g, m, pr, n);
+  const double v = warp_sum4(a, b, c, d);
   if ((threadIdx.x & 7) == 0) part[threadIdx.x >> 5][(threadIdx.x & 31) >> 3] = v;
   __syncthreads();
-  if (threadIdx.x < 4) {
-    double t = 0.0;
+  double t = 0.0;
+  if (threadIdx.x < 4)
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w][threadIdx.x];
-    pp[4 * slot + threadIdx.x] = t;
-  }
+  return t;
+}
+__device__ __forceinline__ void block_partials(double* pp, long long slot, double g, double m, double pr, double n) {
+  if (pp == nullptr) return;
+  const double t = block_sum4(g, m, pr, n);
+  if (threadIdx.x < 4) pp[4 * slot + threadIdx.x] = t;
 }
 __device__ __forceinline__ long long global_warp() {
   return ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -155,7 +159,7 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
     const bool own = lane >= 2;  // (with face) the warp's faces: lanes 2..29
     const bool rev = lane >= 2 && lane < 30;
     double bL[4], bR[4], dl[VISC ? 5 : 4], dr[VISC ? 5 : 4];
-    bool straight;
+    bool fell;  // a face of the warp fell back to first order
     {
       double Lq[4], Rq[4];
 #pragma unroll 1
@@ -194,7 +198,7 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
         bL[m] = fallback || !face ? 0.0 : bL[m];
         bR[m] = fallback || !face ? 0.0 : bR[m];
       }
-      straight = VISC || __any_sync(0xffffffffu, fallback && face);
+      fell = __any_sync(0xffffffffu, fallback && face);
       if (VISC) {
         // F[n] -= tnn; F[t] -= tnt; F[3] -= 0.5 (sbn tnn + sbt tnt) + ck dT
         const double Tc = q[3 * AP] * recip(q[0]);
@@ -203,23 +207,23 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
         const double dun = ub - ua, dut = tb - ta;
         double tnn, tnt;
         if (a.two_d) {
-          const double sun = (un[AB] - un[-AB]) + (un[AB + 1] - un[1 - AB]);
-          const double sut = (ut[AB] - ut[-AB]) + (ut[AB + 1] - ut[1 - AB]);
+          const double cun = un[AB] - un[-AB], cut = ut[AB] - ut[-AB];
+          const double sun = cun + __shfl_down_sync(0xffffffffu, cun, 1), sut = cut + __shfl_down_sync(0xffffffffu, cut, 1);
           tnn = fma(vc.c43n, dun, -vc.c23t * sut);
           tnt = fma(vc.cn, dut, vc.ct * sun);
         } else {
           tnn = vc.c43n * dun;
           tnt = vc.cn * dut;
         }
-        const double h3 = 0.5 * Fb[3];
+        const double h3 = half_of(Fb[3]);
         const double btnn = fma(-h3, ua + ub, -Fb[1]), btnt = fma(-h3, ta + tb, -Fb[2]);
         const double bT = Fb[3] * vc.ck, ckk = -bT * dT;
         const double bdun = vc.c43n * btnn, bdut = vc.cn * btnt;
         if (own && face) {
-          dl[1] += fma(-h3, tnn, -bdun);
-          dr[1] += fma(-h3, tnn, bdun);
-          dl[2] += fma(-h3, tnt, -bdut);
-          dr[2] += fma(-h3, tnt, bdut);
+          const double l1 = fma(-h3, tnn, -bdun), r1 = fma(-h3, tnn, bdun), l2 = fma(-h3, tnt, -bdut),
+                       r2 = fma(-h3, tnt, bdut);
+          if (fell) dl[1] += l1, dr[1] += r1, dl[2] += l2, dr[2] += r2;
+          else dl[1] = l1, dr[1] = r1, dl[2] = l2, dr[2] = r2;
           vmu = fma(btnn, tnn, fma(btnt, tnt, ckk));
           vk = ckk;
         }
@@ -254,9 +258,10 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
       bL[m] = rev ? bL[m] : 0.0;
       bR[m] = rev ? up : 0.0;
     }
-    if (straight) {
+    if (VISC || fell) {
 #pragma unroll
       for (int m = 0; m < (VISC ? 5 : 4); ++m) {
+        if ((m == 0 || m == 3) && !fell) continue;  // no such term
         const double up = __shfl_up_sync(0xffffffffu, dr[m], 1);
         dl[m] += lane > 0 ? up : 0.0;
       }
@@ -279,18 +284,20 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
                        (__shfl_down_sync(0xffffffffu, w[1], 1) + __shfl_down_sync(0xffffffffu, w[0], 2));
       const double tm = __shfl_up_sync(0xffffffffu, t, 1);
       double v = fma(SIXTH, (lane > 0 ? tm : 0.0) - t, Lb + Rb);
-      if (straight) v += (k == 0) ? dl[0] : (k == 1) ? dl[1] : (k == 2) ? dl[2] : dl[3];
+      if (fell || (VISC && (k == 1 || k == 2))) v += (k == 0) ? dl[0] : (k == 1) ? dl[1] : (k == 2) ? dl[2] : dl[3];
       if (in) qo[c * qs] = v;
     }
     if (VISC && in) qo[4 * qs] = dl[VISC ? 4 : 0];
   }
-  double gb = gs2 / g.gamma - gs1 * g.g1 * g.g1;
-  if (VISC) {
-    gb += a.kg * vk;
-    vmu *= a.inv_mu;
-    vk *= a.kp;
+  if (a.pp == nullptr) return;
+  // gamma, mu and Pr from the block's sums
+  const double t = block_sum4(gs1, gs2, vmu, vk);
+  if (threadIdx.x < 4) {
+    const double s1 = __shfl_sync(0xfu, t, 0), s2 = __shfl_sync(0xfu, t, 1), sm = __shfl_sync(0xfu, t, 2), sk = __shfl_sync(0xfu, t, 3);
+    const double gb = s2 / g.gamma - s1 * g.g1 * g.g1;
+    a.pp[4 * slot + threadIdx.x] =
+        threadIdx.x == 0 ? (VISC ? fma(a.kg, sk, gb) : gb) : !VISC || threadIdx.x == 3 ? 0.0 : threadIdx.x == 1 ? sm * a.inv_mu : sk * a.kp;
   }
-  block_partials(a.pp, slot, gb, vmu, vk, 0.0);
 }
 
 // the line sums of primitive c at padded cell (i, j)
