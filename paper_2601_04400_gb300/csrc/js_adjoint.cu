@@ -35,6 +35,7 @@ namespace js {
 template <bool VISC>
 __global__ void __launch_bounds__(32 * ADJ_LINES, 3)
 adj_lines_kernel(AdjArgs a, const double* __restrict__ Unext, double bdt, int bx) {
+  pdl_enter();
   __shared__ double smem[8 * AP];
   const int b = blockIdx.x;
   adj_lines<VISC>(a, Unext, bdt, b < bx ? 0 : 1, b < bx ? b : b - bx, smem, b);
@@ -45,6 +46,7 @@ template <bool VISC>
 __global__ void __launch_bounds__(kCellThreads) adj_cells_kernel(AdjArgs a, const double* __restrict__ Unext,
                                                         double* __restrict__ Uacc, double ra, double rb, double bdt,
                                                         int rhs_mode) {
+  pdl_enter();
   double gb = 0.0, nb = 0.0;
   adj_cell<VISC>(a, Unext, Uacc, ra, rb, bdt, rhs_mode, (long long)blockIdx.x * blockDim.x + threadIdx.x, gb, nb);
   block_partials(a.pp, blockIdx.x, gb, 0.0, 0.0, nb);
@@ -52,6 +54,7 @@ __global__ void __launch_bounds__(kCellThreads) adj_cells_kernel(AdjArgs a, cons
 
 // primitives of every padded cell and lambda' = bdt Unext on fluid cells (the neural flux's reverse)
 __global__ void adj_nn_seed_kernel(AdjArgs a, double* __restrict__ Q, const double* __restrict__ Unext, double bdt) {
+  pdl_enter();
   const Lay& L = a.lay;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= L.plane) return;
@@ -71,6 +74,7 @@ __global__ void adj_nn_seed_kernel(AdjArgs a, double* __restrict__ Q, const doub
 }
 
 __global__ void adj_bcT_kernel(AdjArgs a, BcArgs bc, int phase_y, double* inflow_part, int tmax) {
+  pdl_enter();
   adj_bcT_one(a, bc, phase_y, inflow_part, tmax, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -80,18 +84,21 @@ __global__ void __launch_bounds__(kSumThreads) adj_sums_kernel(AdjArgs a, BcArgs
                                                                int tmax, const double* inflow_prim,
                                                                const double* __restrict__ pp, long long nslot,
                                                                int inflow) {
+  pdl_enter();
   if (inflow) adj_inflow_block(a, bc, inflow_part, tmax, inflow_prim);
   const long long off = 0;
   adj_pbar_reduce_block<kSumThreads>(pp, &off, &nslot, 1, a.pbar);
 }
 
 __global__ void adj_ib_ghost_kernel(AdjArgs a, IbArgs ib, int wall, double* qIb) {
+  pdl_enter();
   double gb = 0.0;
   adj_ib_ghost_one(a, ib, wall, qIb, blockIdx.x * blockDim.x + threadIdx.x, gb);
   warp_partials(a.pp, global_warp(), gb, 0.0, 0.0, 0.0);
 }
 
 __global__ void adj_ib_src_kernel(AdjArgs a, IbTArgs tb, const double* qIb) {
+  pdl_enter();
   double gb = 0.0;
   adj_ib_src_one(a, tb, qIb, blockIdx.x * blockDim.x + threadIdx.x, gb);
   warp_partials(a.pp, global_warp(), gb, 0.0, 0.0, 0.0);
@@ -99,6 +106,7 @@ __global__ void adj_ib_src_kernel(AdjArgs a, IbTArgs tb, const double* qIb) {
 
 __global__ void adj_unpack_add_kernel(const double* __restrict__ P, const double* __restrict__ P2,
                                       double* __restrict__ U, Lay lay) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < 4LL * lay.nx * lay.ny) adj_unpack_add_one(P, P2, U, lay, t);
 }
@@ -139,7 +147,7 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
   };
   if (nn) {
     // the neural flux: its face-state adjoints join the HLLC ones before the WENO5 reverse
-    adj_nn_seed_kernel<<<blocks_for(L.plane, 256), 256, 0, s>>>(a, const_cast<double*>(a.Q), Unext,
+    launch(adj_nn_seed_kernel, blocks_for(L.plane, 256), 256, 0, s, a, const_cast<double*>(a.Q), Unext,
                                                                  rhs_mode ? 1.0 : rb * dt);
     a.pp = slice(8 * nn_image_vjp_blocks(L));
     if ((e = nn_reverse(*nn, a, s)) != cudaSuccess) return e;
@@ -150,36 +158,36 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
   const double bdt = rhs_mode ? 1.0 : rb * dt;
   const int bx = adj_blocks(L, 0), nb = bx + adj_blocks(L, 1);
   a.pp = slice(nb);
-  if (a.visc) adj_lines_kernel<true><<<nb, 32 * ADJ_LINES, 0, s>>>(a, Unext, bdt, bx);
-  else adj_lines_kernel<false><<<nb, 32 * ADJ_LINES, 0, s>>>(a, Unext, bdt, bx);
+  if (a.visc) launch(adj_lines_kernel<true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+  else launch(adj_lines_kernel<false>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const unsigned gp = blocks_for(L.plane, kCellThreads);
   a.pp = slice(gp);
-  if (a.visc) adj_cells_kernel<true><<<gp, kCellThreads, 0, s>>>(a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
-  else adj_cells_kernel<false><<<gp, kCellThreads, 0, s>>>(a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
+  if (a.visc) launch(adj_cells_kernel<true>, gp, kCellThreads, 0, s, a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
+  else launch(adj_cells_kernel<false>, gp, kCellThreads, 0, s, a, Unext, Uacc, ra, rb, bdt, rhs_mode ? 1 : 0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   n += 2;
   const bool two_d = L.ny > 1;
   a.pp = nullptr;
   const int tmax = std::max(L.nx + 6, L.ny);
   if (two_d) {
-    adj_bcT_kernel<<<blocks_for(8LL * (L.nx + 6), 128), 128, 0, s>>>(a, bc, 1, inflow_part, tmax);
+    launch(adj_bcT_kernel, blocks_for(8LL * (L.nx + 6), 128), 128, 0, s, a, bc, 1, inflow_part, tmax);
     ++n;
   }
-  adj_bcT_kernel<<<blocks_for(8LL * L.ny, 128), 128, 0, s>>>(a, bc, 0, inflow_part, tmax);
+  launch(adj_bcT_kernel, blocks_for(8LL * L.ny, 128), 128, 0, s, a, bc, 0, inflow_part, tmax);
   ++n;
   if (ib.n > 0) {
     a.pp = slice(4LL * ib_blocks(ib.n));
-    adj_ib_ghost_kernel<<<ib_blocks(ib.n), 128, 0, s>>>(a, ib, wall, qIb);
+    launch(adj_ib_ghost_kernel, ib_blocks(ib.n), 128, 0, s, a, ib, wall, qIb);
     if (ibt.nsrc > 0) {
       a.pp = slice(4LL * ib_blocks(ibt.nsrc));
-      adj_ib_src_kernel<<<ib_blocks(ibt.nsrc), 128, 0, s>>>(a, ibt, qIb);
+      launch(adj_ib_src_kernel, ib_blocks(ibt.nsrc), 128, 0, s, a, ibt, qIb);
     }
     n += 2;
   }
   if (pp0) {
     const int inflow = bc.kind[0] == 3 || bc.kind[1] == 3 || bc.kind[2] == 3 || bc.kind[3] == 3;
-    adj_sums_kernel<<<1, kSumThreads, 0, s>>>(a, bc, inflow_part, tmax, inflow_prim, pp0, used, inflow);
+    launch(adj_sums_kernel, 1, kSumThreads, 0, s, a, bc, inflow_part, tmax, inflow_prim, pp0, used, inflow);
     ++n;
   }
   if (launches) *launches += n;
@@ -187,7 +195,7 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
 }
 
 cudaError_t launch_adj_unpack(const double* P, const double* P2, double* U, const Lay& lay, cudaStream_t s) {
-  adj_unpack_add_kernel<<<blocks_for(4LL * lay.nx * lay.ny, 256), 256, 0, s>>>(P, P2, U, lay);
+  launch(adj_unpack_add_kernel, blocks_for(4LL * lay.nx * lay.ny, 256), 256, 0, s, P, P2, U, lay);
   return cudaGetLastError();
 }
 

@@ -365,6 +365,7 @@ __device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, d
 
 template <int PH, int VM = 0>
 __global__ void __launch_bounds__(FNT, PH == FP_LINES ? 4 : 1) batch_phase_kernel(BatchArgs b, int step, int s) {
+  pdl_enter();
   extern __shared__ double smem[];
   fwd_phase<PH, VM>(b, step, s, smem);
 }
@@ -645,6 +646,7 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
 // one phase of the reverse step
 template <int PH, int VM = 0>
 __global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 : PH == RP_CELLS ? 4 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
+  pdl_enter();
   extern __shared__ double smem[];
   rev_phase<PH, VM>(b, s, smem);
 }
@@ -652,6 +654,7 @@ __global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 :
 // one launch copying every instance's state: dst[k][i] = src[k][i], i < pre[k+1] - pre[k]
 __global__ void batch_copy_kernel(const double* const* src, double* const* dst, const long long* __restrict__ pre,
                                   int count) {
+  pdl_enter();
   const long long total = pre[count];
   for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < total;
        g += (long long)gridDim.x * blockDim.x) {
@@ -809,13 +812,13 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
   // the line phases: a block an item, viscous and inviscid instances apart
   auto run_lines = [&](auto visc, auto inv, int blocks, size_t smem, int s) {
     if (!ok) return;
-    if (b->has_visc) visc<<<blocks, js::BNT, smem, b->stream>>>(a, s);
-    if (b->has_inv) inv<<<blocks, js::BNT, smem, b->stream>>>(a, s);
+    if (b->has_visc) js::launch(visc, blocks, js::BNT, smem, b->stream, a, s);
+    if (b->has_inv) js::launch(inv, blocks, js::BNT, smem, b->stream, a, s);
     ok = cudaGetLastError() == cudaSuccess;
   };
   auto run = [&](auto kernel, int ph, int s) {
     if (!ok) return;
-    kernel<<<b->rev_pblocks[ph], js::BNT, 0, b->stream>>>(a, s);
+    js::launch(kernel, b->rev_pblocks[ph], js::BNT, 0, b->stream, a, s);
     ok = cudaGetLastError() == cudaSuccess;
   };
   run(js::batch_vjp_phase_kernel<js::RP_PACK>, js::RP_PACK, 0);
@@ -994,23 +997,23 @@ static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, dou
   const unsigned lines = b->blocks_set ? (unsigned)std::min(b->blocks, b->line0.back()) : (unsigned)b->line0.back();
   auto grid = [&](long long items) { return (unsigned)std::max(1LL, std::min((long long)wide, (items + FNT - 1) / FNT)); };
   cudaStream_t st = b->stream;
-  if (n_steps > 0) batch_phase_kernel<FP_PACK><<<tiles, FNT, 0, st>>>(a, 0, 0);
+  if (n_steps > 0) launch(batch_phase_kernel<FP_PACK>, tiles, FNT, 0, st, a, 0, 0);
   for (int k = 0; k < n_steps; ++k) {
     if (!a.dt_in) {
-      batch_phase_kernel<FP_CFL><<<tiles, FNT, 0, st>>>(a, k, 0);
-      batch_phase_kernel<FP_CFL_IEEE><<<tiles, FNT, 0, st>>>(a, k, 0);
+      launch(batch_phase_kernel<FP_CFL>, tiles, FNT, 0, st, a, k, 0);
+      launch(batch_phase_kernel<FP_CFL_IEEE>, tiles, FNT, 0, st, a, k, 0);
     }
-    batch_phase_kernel<FP_DT><<<1, FNT, 0, st>>>(a, k, 0);
+    launch(batch_phase_kernel<FP_DT>, 1, FNT, 0, st, a, k, 0);
     for (int s = 0; s < 3; ++s) {
-      if (nghost > 0) batch_phase_kernel<FP_GHOST><<<grid(4 * nghost), FNT, 0, st>>>(a, k, s);
-      batch_phase_kernel<FP_HALO><<<grid(nhalo), FNT, 0, st>>>(a, k, s);
-      if (b->has_visc) batch_phase_kernel<FP_LINES, 1><<<lines, FNT, stage_smem<true>(), st>>>(a, k, s);
-      if (b->has_inv) batch_phase_kernel<FP_LINES, 2><<<lines, FNT, stage_smem<false>(), st>>>(a, k, s);
-      batch_phase_kernel<FP_CELLS><<<tiles, FNT, 0, st>>>(a, k, s);
+      if (nghost > 0) launch(batch_phase_kernel<FP_GHOST>, grid(4 * nghost), FNT, 0, st, a, k, s);
+      launch(batch_phase_kernel<FP_HALO>, grid(nhalo), FNT, 0, st, a, k, s);
+      if (b->has_visc) launch(batch_phase_kernel<FP_LINES, 1>, lines, FNT, stage_smem<true>(), st, a, k, s);
+      if (b->has_inv) launch(batch_phase_kernel<FP_LINES, 2>, lines, FNT, stage_smem<false>(), st, a, k, s);
+      launch(batch_phase_kernel<FP_CELLS>, tiles, FNT, 0, st, a, k, s);
     }
-    if (a.save || a.save1) batch_phase_kernel<FP_SAVE><<<tiles, FNT, 0, st>>>(a, k, 0);
+    if (a.save || a.save1) launch(batch_phase_kernel<FP_SAVE>, tiles, FNT, 0, st, a, k, 0);
   }
-  if (n_steps > 0) batch_phase_kernel<FP_UNPACK><<<tiles, FNT, 0, st>>>(a, 0, 0);
+  if (n_steps > 0) launch(batch_phase_kernel<FP_UNPACK>, tiles, FNT, 0, st, a, 0, 0);
   return cudaGetLastError() == cudaSuccess ? JS_OK : JS_ERR_CUDA;
 }
 
@@ -1058,7 +1061,7 @@ namespace {
 // one launch copying the states of table src into those of table dst (device tables of count
 // pointers)
 int batch_copy(js_batch* b, void* const* src, void* const* dst) {
-  js::batch_copy_kernel<<<4 * 152, 256, 0, b->stream>>>(reinterpret_cast<const double* const*>(src),
+  js::launch(js::batch_copy_kernel, 4 * 152, 256, 0, b->stream, reinterpret_cast<const double* const*>(src),
                                                         reinterpret_cast<double* const*>(dst), b->d_spre, b->count);
   return cudaGetLastError() == cudaSuccess ? JS_OK : JS_ERR_CUDA;
 }

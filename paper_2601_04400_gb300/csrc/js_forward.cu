@@ -22,6 +22,7 @@ namespace js {
 // domain halo
 // =======================================================================================
 __global__ void bc_fill_kernel(double* __restrict__ U, Lay lay, BcArgs bc) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < halo_count(lay)) bc_fill_one(U, lay, bc, t);
 }
@@ -30,6 +31,7 @@ __global__ void bc_fill_kernel(double* __restrict__ U, Lay lay, BcArgs bc) {
 // immersed-boundary ghost states
 // =======================================================================================
 __global__ void ib_fill_kernel(double* __restrict__ U, Lay lay, IbArgs ib, double gamma, int wall) {
+  pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < 4 * ib.n) ib_fill_one(U, lay, ib, gamma, wall, t);
 }
@@ -38,6 +40,7 @@ __global__ void ib_fill_kernel(double* __restrict__ U, Lay lay, IbArgs ib, doubl
 // layout conversion
 // =======================================================================================
 __global__ void pack_kernel(const double* __restrict__ U, double* __restrict__ P, Lay lay) {
+  pdl_enter();
   const long long n = (long long)lay.nx * lay.ny;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * n) return;
@@ -48,6 +51,7 @@ __global__ void pack_kernel(const double* __restrict__ U, double* __restrict__ P
 }
 
 __global__ void unpack_kernel(const double* __restrict__ P, double* __restrict__ U, Lay lay) {
+  pdl_enter();
   const long long n = (long long)lay.nx * lay.ny;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * n) return;
@@ -60,6 +64,7 @@ __global__ void unpack_kernel(const double* __restrict__ P, double* __restrict__
 // row blocks of a [4][ny][nx] state for the halo exchange of a y-decomposed grid
 __global__ void rows_pack_kernel(double* __restrict__ U, long long plane, long long off, long long m,
                                  double* __restrict__ buf, int zero) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * m) return;
   const long long k = (t / m) * plane + off + t % m;
@@ -69,6 +74,7 @@ __global__ void rows_pack_kernel(double* __restrict__ U, long long plane, long l
 
 __global__ void rows_unpack_kernel(double* __restrict__ U, long long plane, long long off, long long m,
                                    const double* __restrict__ buf, int add) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * m) return;
   const long long k = (t / m) * plane + off + t % m;
@@ -76,6 +82,7 @@ __global__ void rows_unpack_kernel(double* __restrict__ U, long long plane, long
 }
 
 __global__ void prim_to_cons_kernel(const double* W, double* U, long long n, double g1) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const double r = W[t], u = W[n + t], v = W[2 * n + t], p = W[3 * n + t];
@@ -193,13 +200,17 @@ __device__ __forceinline__ void cfl_finish(unsigned long long* red, const CflSte
   }
 }
 
-__global__ void cfl_init_kernel(unsigned long long* red) { cfl_reset(red); }
+__global__ void cfl_init_kernel(unsigned long long* red) {
+  pdl_enter();
+  cfl_reset(red);
+}
 
 // Every cell's IEEE rate, a cell a thread (small grids).
 template <bool PADDED>
 __global__ void __launch_bounds__(128) cfl_one_kernel(CflSrc q, long long n, int two_d,
                                                       const unsigned char* __restrict__ tag, double gamma, double dx,
                                                       double dy, unsigned long long* __restrict__ red, CflStep st) {
+  pdl_enter();
   double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n && !(tag && tag[t] != 0)) {
@@ -222,6 +233,7 @@ __global__ void cfl_pass1_kernel(CflSrc q, long long n, int two_d,
                                  const unsigned char* __restrict__ tag, double gamma, double dx, double dy,
                                  double idx, double idy, unsigned long long* __restrict__ red,
                                  double* __restrict__ bmax) {
+  pdl_enter();
   double rate = 0.0, rmin = __longlong_as_double(0x7ff0000000000000LL);
   const double* __restrict__ U = q.U;
   const long long P = q.plane;
@@ -255,6 +267,7 @@ __global__ void cfl_pass2_kernel(CflSrc q, long long n, int nx, int two_d,
                                  const unsigned char* __restrict__ tag, double gamma, double dx, double dy,
                                  double idx, double idy, unsigned long long* __restrict__ red,
                                  const double* __restrict__ bmax, CflStep st) {
+  pdl_enter();
   const double thr = __longlong_as_double((long long)red[2]) * (1.0 - CFL_MARGIN);
   if (!(bmax[blockIdx.x] >= thr)) {  // the same for the whole block
     cfl_finish(red, st);
@@ -315,6 +328,7 @@ __device__ __forceinline__ bool stage_constants(const StageArgs& a0, StageArgs& 
 // x line blocks, then y line blocks; B: resident blocks an SM the registers are allotted for
 template <bool VISC, bool IMG, int B>
 __global__ void __launch_bounds__(32 * SLINES, B) stage_lines_kernel(StageArgs a, int bx) {
+  pdl_enter();
   if (a.dtc != nullptr && a.dtc[4] == 0.0) return;  // an inactive device-sized step
   __shared__ double smem[stage_smem<VISC>() / sizeof(double)];
   const int b = blockIdx.x;
@@ -323,6 +337,7 @@ __global__ void __launch_bounds__(32 * SLINES, B) stage_lines_kernel(StageArgs a
 
 template <bool RHS>
 __global__ void __launch_bounds__(128) stage_cells_kernel(StageArgs a0) {
+  pdl_enter();
   StageArgs a;
   if (!stage_constants(a0, a)) return;
   const int gi = blockIdx.x * 128 + threadIdx.x;
@@ -333,6 +348,7 @@ __global__ void __launch_bounds__(128) stage_cells_kernel(StageArgs a0) {
 // one line (ny == 1): a warp per 28 cells
 template <bool VISC, bool RHS>
 __global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
+  pdl_enter();
   StageArgs a;
   if (!stage_constants(a0, a)) return;
   constexpr int NPL = VISC ? 5 : 4;
@@ -375,12 +391,12 @@ cudaError_t launch_lines(const StageArgs& a, int variant, cudaStream_t s) {
   const int bx = stage_blocks(a.lay, 0), n = bx + stage_blocks(a.lay, 1);
   if constexpr (!IMG) {
     if (variant == 1 || variant == 2) {
-      if (variant == 1) stage_lines_kernel<VISC, IMG, 3><<<n, 32 * SLINES, 0, s>>>(a, bx);
-      else stage_lines_kernel<VISC, IMG, 2><<<n, 32 * SLINES, 0, s>>>(a, bx);
+      if (variant == 1) launch(stage_lines_kernel<VISC, IMG, 3>, n, 32 * SLINES, 0, s, a, bx);
+      else launch(stage_lines_kernel<VISC, IMG, 2>, n, 32 * SLINES, 0, s, a, bx);
       return cudaGetLastError();
     }
   }
-  stage_lines_kernel<VISC, IMG, 4><<<n, 32 * SLINES, 0, s>>>(a, bx);
+  launch(stage_lines_kernel<VISC, IMG, 4>, n, 32 * SLINES, 0, s, a, bx);
   return cudaGetLastError();
 }
 
@@ -389,14 +405,14 @@ cudaError_t launch_stage2d(const StageArgs& a, bool rhs, int variant, cudaStream
   const cudaError_t e = launch_lines<VISC, IMG>(a, variant, s);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.lay.nx + 127) / 128, a.lay.ny < 65535 ? a.lay.ny : 65535);
-  if (rhs) stage_cells_kernel<true><<<grid, 128, 0, s>>>(a);
-  else stage_cells_kernel<false><<<grid, 128, 0, s>>>(a);
+  if (rhs) launch(stage_cells_kernel<true>, grid, 128, 0, s, a);
+  else launch(stage_cells_kernel<false>, grid, 128, 0, s, a);
   return cudaGetLastError();
 }
 
 template <bool VISC, bool RHS>
 cudaError_t launch_stage1d(const StageArgs& a, cudaStream_t s) {
-  stage1d_kernel<VISC, RHS><<<stage_chunks(a.lay.nx), 32, 0, s>>>(a);
+  launch(stage1d_kernel<VISC, RHS>, stage_chunks(a.lay.nx), 32, 0, s, a);
   return cudaGetLastError();
 }
 }  // namespace
@@ -417,35 +433,35 @@ cudaError_t launch_stage(const StageArgs& a, bool visc, bool rhs, int variant, c
 cudaError_t launch_bc_fill(double* U, const Lay& lay, const BcArgs& bc, cudaStream_t s) {
   const long long n = halo_count(lay);
   const int bs = 256;
-  bc_fill_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(U, lay, bc);
+  launch(bc_fill_kernel, (unsigned)((n + bs - 1) / bs), bs, 0, s, U, lay, bc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ib_fill(double* U, const Lay& lay, const IbArgs& ib, double gamma, int wall, cudaStream_t s) {
   if (ib.n == 0) return cudaSuccess;
   const int bs = 128;
-  ib_fill_kernel<<<(4 * ib.n + bs - 1) / bs, bs, 0, s>>>(U, lay, ib, gamma, wall);
+  launch(ib_fill_kernel, (4 * ib.n + bs - 1) / bs, bs, 0, s, U, lay, ib, gamma, wall);
   return cudaGetLastError();
 }
 
 cudaError_t launch_pack(const double* U, double* P, const Lay& lay, cudaStream_t s) {
   const long long n = 4LL * lay.nx * lay.ny;
   const int bs = 256;
-  pack_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(U, P, lay);
+  launch(pack_kernel, (unsigned)((n + bs - 1) / bs), bs, 0, s, U, P, lay);
   return cudaGetLastError();
 }
 
 cudaError_t launch_unpack(const double* P, double* U, const Lay& lay, cudaStream_t s) {
   const long long n = 4LL * lay.nx * lay.ny;
   const int bs = 256;
-  unpack_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(P, U, lay);
+  launch(unpack_kernel, (unsigned)((n + bs - 1) / bs), bs, 0, s, P, U, lay);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rows_pack(double* U, int nx, int ny, int row0, int nrows, double* buf, int zero, cudaStream_t s) {
   const long long m = (long long)nrows * nx;
   if (m == 0) return cudaSuccess;
-  rows_pack_kernel<<<(unsigned)((4 * m + 255) / 256), 256, 0, s>>>(U, (long long)nx * ny, (long long)row0 * nx, m,
+  launch(rows_pack_kernel, (unsigned)((4 * m + 255) / 256), 256, 0, s, U, (long long)nx * ny, (long long)row0 * nx, m,
                                                                    buf, zero);
   return cudaGetLastError();
 }
@@ -454,19 +470,19 @@ cudaError_t launch_rows_unpack(double* U, int nx, int ny, int row0, int nrows, c
                                cudaStream_t s) {
   const long long m = (long long)nrows * nx;
   if (m == 0) return cudaSuccess;
-  rows_unpack_kernel<<<(unsigned)((4 * m + 255) / 256), 256, 0, s>>>(U, (long long)nx * ny, (long long)row0 * nx,
+  launch(rows_unpack_kernel, (unsigned)((4 * m + 255) / 256), 256, 0, s, U, (long long)nx * ny, (long long)row0 * nx,
                                                                      m, buf, add);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prim_to_cons(const double* W, double* U, long long n, double gamma, cudaStream_t s) {
   const int bs = 256;
-  prim_to_cons_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(W, U, n, 1.0 / (gamma - 1.0));
+  launch(prim_to_cons_kernel, (unsigned)((n + bs - 1) / bs), bs, 0, s, W, U, n, 1.0 / (gamma - 1.0));
   return cudaGetLastError();
 }
 
 cudaError_t launch_cfl_init(unsigned long long* red, cudaStream_t s) {
-  cfl_init_kernel<<<1, 1, 0, s>>>(red);
+  launch(cfl_init_kernel, 1, 1, 0, s, red);
   return cudaGetLastError();
 }
 
@@ -481,14 +497,14 @@ void cfl_launches(const CflSrc& q, long long n, const Lay& lay, const unsigned c
                   double dy, unsigned long long* red, double* bmax, const CflStep& st, cudaStream_t s) {
   const int two_d = lay.ny > 1 ? 1 : 0;
   if (n <= CFL_ONE_CELLS) {
-    cfl_one_kernel<PADDED><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(q, n, two_d, tag, gamma, dx, dy, red, st);
+    launch(cfl_one_kernel<PADDED>, (unsigned)((n + 127) / 128), 128, 0, s, q, n, two_d, tag, gamma, dx, dy, red, st);
     return;
   }
   const int bs = 256;
   const unsigned blocks = (unsigned)std::min<long long>((n + bs - 1) / bs, CFL_MAX_BLOCKS);
   // both passes on the same grid: a block of pass 2 visits the cells its pass-1 maximum covers
-  cfl_pass1_kernel<PADDED><<<blocks, bs, 0, s>>>(q, n, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red, bmax);
-  cfl_pass2_kernel<PADDED><<<blocks, bs, 0, s>>>(q, n, lay.nx, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red,
+  launch(cfl_pass1_kernel<PADDED>, blocks, bs, 0, s, q, n, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red, bmax);
+  launch(cfl_pass2_kernel<PADDED>, blocks, bs, 0, s, q, n, lay.nx, two_d, tag, gamma, dx, dy, 1.0 / dx, 1.0 / dy, red,
                                                  bmax, st);
 }
 }  // namespace

@@ -6,6 +6,29 @@
 
 namespace js {
 
+// A launch whose setup overlaps the end of the kernel before it on the stream, for the chains of short
+// kernels that small grids are: its blocks start as the predecessor's last ones leave and wait in
+// pdl_enter, the first statement of every kernel launched this way, until the predecessor has
+// completed and its writes are visible.  128x64 cylinder, 13 launches a step: 101 us a step with plain
+// launches, 73 so.  The predecessor does not release its successor early: waiting blocks would crowd
+// on the SMs that are free while it still runs (128x96 training step: 4.2 ms, 6.8 released early, 5.2
+// with plain launches).
+__device__ __forceinline__ void pdl_enter() { cudaGridDependencySynchronize(); }
+template <class... P, class... A>
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 struct StageArgs {
   const double* Uin;         // padded stage input (halo and IB ghosts filled)
   const double* Un;          // padded U^n (RK combination), may alias Uout

@@ -111,6 +111,7 @@ __device__ __forceinline__ void face_states(const Lay& L, const double* Q, long 
 // forward
 // ---------------------------------------------------------------------------------------
 __global__ void nn_prims_kernel(const double* __restrict__ U, double* __restrict__ Q, Lay L, Gas g) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= L.plane) return;
   const int col = (int)(t % L.pitch), row = (int)(t / L.pitch);
@@ -133,6 +134,7 @@ constexpr int IT = 32, IF = 8;
 
 template <class T>
 __global__ void __launch_bounds__(256) nn_image_kernel(NnArgs n, const double* __restrict__ Q, long long qplane) {
+  pdl_enter();
   __shared__ T sx[4][IT][IF + 1];
   const int d = blockIdx.z;
   const int H = n.H[d], Wd = n.W[d];
@@ -168,6 +170,7 @@ __global__ void __launch_bounds__(256) nn_image_kernel(NnArgs n, const double* _
 // one 3x3 layer on a 16x16 pixel tile per block; ACT 0: ReLU, 1: tanh
 template <class T, int CIN, int COUT, int ACT>
 __global__ void __launch_bounds__(NTHR) nn_conv_kernel(NnArgs n, const void* in, void* out, int woff) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NW = COUT * CIN * 9 + COUT;
   T* sw = reinterpret_cast<T*>(smem_raw);
@@ -246,6 +249,7 @@ __device__ __forceinline__ void cp_async_wait() {
 template <int KI, int KO, int MODE>
 __global__ void __launch_bounds__(LTHR) nn_layer_f32_kernel(NnArgs n, const void* in, const void* aprev, void* out,
                                                             int woff, void* outh) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using P = LayerTile<KO>;
   constexpr bool GRAD = MODE >= 2;
@@ -361,6 +365,7 @@ __host__ __device__ constexpr int wgrad_tile_floats() {
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(NTHR) nn_wgrad_f32_kernel(NnArgs n, const void* gout, const void* ain, int woff) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NI = (COUT / 4) * CIN * 3;          // work items
   constexpr int R = WG_UNITS / NI;                  // row parts per item
@@ -557,6 +562,7 @@ constexpr int TC_ROWS = 16;
 template <int CIN, int COUT, int ACT, int MODE = 0, int CINR = CIN>
 __global__ void __launch_bounds__(128) nn_conv_tc_kernel(NnArgs n, const void* inh, void* out, int woff,
                                                          void* outh, const void* aprev) {
+  pdl_enter();
   static_assert(CIN % 16 == 0, "input channels in groups of 16 (K of one MMA)");
   static_assert(CINR <= CIN, "present channels within the padded ones");
   constexpr int N = (COUT + 15) / 16 * 16;   // MMA N (multiple of 16 for M = 128)
@@ -763,6 +769,7 @@ constexpr int NF_SMEM = NF_OFF_BIAS + (16 + 32 + 4) * 4;
 __host__ __device__ constexpr int nf_slot3(int r) { return (r + 15) % 3; }   // rows >= -15
 
 __global__ void __launch_bounds__(128) nn_net_tc_kernel(NnArgs n, int band) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* sA1 = smem_raw;
   unsigned char* sA2 = smem_raw + NF_OFF_A2;
@@ -1053,6 +1060,7 @@ __device__ __forceinline__ uint4 bf16x8(const float v[8]) { return pack_bf16x8(v
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(WNT) nn_wgrad_tc_kernel(NnArgs n, const float* __restrict__ gout,
                                                           const float* __restrict__ ain, int woff) {
+  pdl_enter();
   using P = WgTc<CIN, COUT>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar[2];
@@ -1248,6 +1256,7 @@ __global__ void __launch_bounds__(WNT) nn_wgrad_tc_kernel(NnArgs n, const float*
 // the FP32 network input X (planar, 4 channels) as the first tensor-core layer's input: BF16
 // pixel-major, 16 channels per pixel (4 and 12 zeros)
 __global__ void nn_x16_kernel(NnArgs n, __nv_bfloat16* __restrict__ Xh) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long pix = n.pix0 + (n.nimg > 1 ? (long long)n.H[1] * n.W[1] : 0LL);
   if (t >= pix) return;
@@ -1262,11 +1271,13 @@ __global__ void nn_x16_kernel(NnArgs n, __nv_bfloat16* __restrict__ Xh) {
 // network input from an FP64 image / scaled FP64 output (js_nn_eval)
 template <class T>
 __global__ void nn_load_kernel(const double* __restrict__ Xd, T* __restrict__ X, long long n4) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n4) X[t] = (T)Xd[t];
 }
 template <class T>
 __global__ void nn_store_kernel(const T* __restrict__ T3, double* __restrict__ Y, long long pix, NnArgs n) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < 4 * pix) Y[t] = n.scale[t / pix] * (double)T3[t];
 }
@@ -1275,6 +1286,7 @@ __global__ void nn_store_kernel(const T* __restrict__ T3, double* __restrict__ Y
 // optional BF16 pixel-major copy padded to 16 channels, and the input gradient back to FP64
 template <class T>
 __global__ void nn_seed_eval_kernel(NnArgs n, const double* __restrict__ GY, long long pix, __nv_bfloat16* gh) {
+  pdl_enter();
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= pix) return;
   const T* t3 = static_cast<const T*>(n.T3);
@@ -1295,6 +1307,7 @@ __global__ void nn_seed_eval_kernel(NnArgs n, const double* __restrict__ GY, lon
 }
 template <class T>
 __global__ void nn_unload_kernel(const T* __restrict__ G, double* __restrict__ GX, long long n4) {
+  pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n4) GX[t] = (double)G[t];
 }
@@ -1302,6 +1315,7 @@ __global__ void nn_unload_kernel(const T* __restrict__ G, double* __restrict__ G
 // stage output (or RHS) minus the neural flux divergence on fluid cells
 template <class T>
 __global__ void __launch_bounds__(256) nn_apply_kernel(NnArgs n, StageArgs a, int rhs) {
+  pdl_enter();
   // 32 x 8 cells per block, a cell a thread: the tile's y-face fluxes (image 1: line = column i,
   // face = row j) pass through shared memory, so both images are read along their contiguous axis
   __shared__ T sy[4][IT][IF + 2];
@@ -1365,6 +1379,7 @@ __global__ void __launch_bounds__(256) nn_apply_kernel(NnArgs n, StageArgs a, in
 // tensor-core data gradient of the last layer)
 template <class T>
 __global__ void nn_seed_kernel(NnArgs n, AdjArgs a, __nv_bfloat16* gh) {
+  pdl_enter();
   const int d = blockIdx.y;
   const int Wd = n.W[d];
   const long long pix = (long long)n.H[d] * Wd;
@@ -1399,6 +1414,7 @@ __global__ void nn_seed_kernel(NnArgs n, AdjArgs a, __nv_bfloat16* gh) {
 template <class T, int CIN, int COUT, bool MASK>
 __global__ void __launch_bounds__(NTHR) nn_dgrad_kernel(NnArgs n, const void* gout, const void* aprev, void* gin,
                                                         int woff) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NWW = COUT * CIN * 9;
   T* sw = reinterpret_cast<T*>(smem_raw);
@@ -1447,6 +1463,7 @@ __global__ void __launch_bounds__(NTHR) nn_dgrad_kernel(NnArgs n, const void* go
 // per-thread sums of the weights they own; each block writes its sums to partial[block]
 template <class T, int CIN, int COUT>
 __global__ void __launch_bounds__(NTHR) nn_wgrad_kernel(NnArgs n, const void* gout, const void* ain, int woff) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NW = COUT * CIN * 9 + COUT;
   constexpr int PER = (NW + NTHR - 1) / NTHR;
@@ -1510,6 +1527,7 @@ __global__ void __launch_bounds__(NTHR) nn_wgrad_kernel(NnArgs n, const void* go
 
 // the partial weight gradients summed: 32 parameters a block, eight threads each
 __global__ void __launch_bounds__(256) nn_wreduce_kernel(NnArgs n) {
+  pdl_enter();
   __shared__ double part[8][32];
   const int kl = threadIdx.x % 32, p = threadIdx.x / 32, k = blockIdx.x * 32 + kl;
   double s = 0.0;
@@ -1532,6 +1550,7 @@ __device__ __forceinline__ double nn_warp_sum(double v) {
 // d/dgamma of the face energies (added to pbar[0]); 32 x 32 pixel tiles as nn_image_kernel
 template <class T>
 __global__ void __launch_bounds__(256) nn_image_vjp_kernel(NnArgs n, AdjArgs a) {
+  pdl_enter();
   __shared__ T sx[4][IT][IF + 1];
   const int d = blockIdx.z;
   const int H = n.H[d], Wd = n.W[d];
@@ -1618,7 +1637,7 @@ cudaError_t conv(const NnArgs& n, const void* in, void* out, int woff, cudaStrea
     auto k = nn_layer_f32_kernel<CIN, COUT, ACT>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k<<<tile_grid(n), LTHR, sm, s>>>(n, in, nullptr, out, woff, outh);
+    launch(k, tile_grid(n), LTHR, sm, s, n, in, nullptr, out, woff, outh);
     return cudaGetLastError();
   }
   constexpr int NW = COUT * CIN * 9 + COUT;
@@ -1626,7 +1645,7 @@ cudaError_t conv(const NnArgs& n, const void* in, void* out, int woff, cudaStrea
   auto k = nn_conv_kernel<T, CIN, COUT, ACT>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k<<<tile_grid(n), NTHR, sm, s>>>(n, in, out, woff);
+  launch(k, tile_grid(n), NTHR, sm, s, n, in, out, woff);
   return cudaGetLastError();
 }
 
@@ -1637,7 +1656,7 @@ cudaError_t dgrad(const NnArgs& n, const void* gout, const void* aprev, void* gi
     auto k = nn_layer_f32_kernel<COUT, CIN, MASK ? 2 : 3>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k<<<tile_grid(n), LTHR, sm, s>>>(n, gout, aprev, gin, woff, nullptr);
+    launch(k, tile_grid(n), LTHR, sm, s, n, gout, aprev, gin, woff, nullptr);
     return cudaGetLastError();
   }
   constexpr int NWW = COUT * CIN * 9;
@@ -1645,7 +1664,7 @@ cudaError_t dgrad(const NnArgs& n, const void* gout, const void* aprev, void* gi
   auto k = nn_dgrad_kernel<T, CIN, COUT, MASK>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k<<<tile_grid(n), NTHR, sm, s>>>(n, gout, aprev, gin, woff);
+  launch(k, tile_grid(n), NTHR, sm, s, n, gout, aprev, gin, woff);
   return cudaGetLastError();
 }
 
@@ -1656,7 +1675,7 @@ cudaError_t wgrad_tc(const NnArgs& n, const void* gout, const void* ain, int wof
   auto k = nn_wgrad_tc_kernel<CIN, COUT>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, P::SMEM);
   if (e != cudaSuccess) return e;
-  k<<<n.nwblk, WNT, P::SMEM, s>>>(n, static_cast<const float*>(gout), static_cast<const float*>(ain), woff);
+  launch(k, n.nwblk, WNT, P::SMEM, s, n, static_cast<const float*>(gout), static_cast<const float*>(ain), woff);
   return cudaGetLastError();
 }
 
@@ -1671,14 +1690,14 @@ cudaError_t wgrad(const NnArgs& n, const void* gout, const void* ain, int woff, 
     auto k = nn_wgrad_f32_kernel<CIN, COUT>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k<<<n.nwblk, NTHR, sm, s>>>(n, gout, ain, woff);
+    launch(k, n.nwblk, NTHR, sm, s, n, gout, ain, woff);
     return cudaGetLastError();
   }
   const size_t sm = sizeof(T) * (COUT * NTHR + CIN * TH * TH);
   auto k = nn_wgrad_kernel<T, CIN, COUT>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k<<<n.nwblk, NTHR, sm, s>>>(n, gout, ain, woff);
+  launch(k, n.nwblk, NTHR, sm, s, n, gout, ain, woff);
   return cudaGetLastError();
 }
 
@@ -1695,7 +1714,7 @@ cudaError_t conv_tc(const NnArgs& n, const void* inh, void* out, int woff, cudaS
   // co-schedules; each block allocates its 32 tensor-memory columns once and frees them
   long long items = 0;
   for (int d = 0; d < n.nimg; ++d) items += (long long)cdiv(n.W[d], TC_M) * cdiv(n.H[d], TC_ROWS);
-  k<<<(unsigned)items, 128, sm, s>>>(n, inh, out, woff, outh, aprev);
+  launch(k, (unsigned)items, 128, sm, s, n, inh, out, woff, outh, aprev);
   return cudaGetLastError();
 }
 
@@ -1718,7 +1737,7 @@ cudaError_t net_tc(const NnArgs& n, cudaStream_t s) {
   band = band < 16 ? 16 : (band > hmax ? hmax : band);
   long long items = 0;
   for (int d = 0; d < n.nimg; ++d) items += (long long)cdiv(n.W[d], NF_OUT) * ((n.H[d] + band - 1) / band);
-  k<<<(unsigned)items, 128, NF_SMEM, s>>>(n, (int)band);
+  launch(k, (unsigned)items, 128, NF_SMEM, s, n, (int)band);
   return cudaGetLastError();
 }
 
@@ -1735,7 +1754,7 @@ cudaError_t layers_t(const NnArgs& n, cudaStream_t s) {
     void* a2 = n.keep ? n.A2 : nullptr;
     const long long pix = n.pix0 + (n.nimg > 1 ? (long long)n.H[1] * n.W[1] : 0LL);
     __nv_bfloat16* xh = static_cast<__nv_bfloat16*>(n.G16);
-    nn_x16_kernel<<<(unsigned)((pix + 255) / 256), 256, 0, s>>>(n, xh);
+    launch(nn_x16_kernel, (unsigned)((pix + 255) / 256), 256, 0, s, n, xh);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = conv_tc<16, 16, 0, 0, 4>(n, xh, a1, NN_OFF1, s, n.A1h)) != cudaSuccess) return e;
     if ((e = conv_tc<16, 32, 0>(n, n.A1h, a2, NN_OFF2, s, n.A2h)) != cudaSuccess) return e;
@@ -1748,7 +1767,7 @@ cudaError_t layers_t(const NnArgs& n, cudaStream_t s) {
 
 template <class T>
 cudaError_t forward_t(const NnArgs& n, const double* Q, long long qplane, cudaStream_t s) {
-  nn_image_kernel<T><<<image_grid(n), 256, 0, s>>>(n, Q, qplane);
+  launch(nn_image_kernel<T>, image_grid(n), 256, 0, s, n, Q, qplane);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return layers_t<T>(n, s);
@@ -1762,11 +1781,11 @@ cudaError_t eval_t(const NnArgs& n0, const double* X, int H, int W, double* Y, c
   n.W[0] = W;
   n.pix0 = (long long)H * W;
   const long long pix = n.pix0;
-  nn_load_kernel<T><<<cdiv(4 * pix, 256), 256, 0, s>>>(X, static_cast<T*>(n.X), 4 * pix);
+  launch(nn_load_kernel<T>, cdiv(4 * pix, 256), 256, 0, s, X, static_cast<T*>(n.X), 4 * pix);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if ((e = layers_t<T>(n, s)) != cudaSuccess) return e;
-  nn_store_kernel<T><<<cdiv(4 * pix, 256), 256, 0, s>>>(static_cast<const T*>(n.T3), Y, pix, n);
+  launch(nn_store_kernel<T>, cdiv(4 * pix, 256), 256, 0, s, static_cast<const T*>(n.T3), Y, pix, n);
   return cudaGetLastError();
 }
 
@@ -1799,7 +1818,7 @@ cudaError_t layers_vjp_t(const NnArgs& n, cudaStream_t s) {
   if ((e = dgrad<T, 4, 16, false>(n, n.G16, nullptr, n.G4, NN_OFF1, s)) != cudaSuccess) return e;  // G4 = dX
   if (n.w_bar) {
     if ((e = wgrad<T, 4, 16>(n, n.G16, n.X, NN_OFF1, s)) != cudaSuccess) return e;
-    nn_wreduce_kernel<<<cdiv(NN_NPARAM, 32), 256, 0, s>>>(n);
+    launch(nn_wreduce_kernel, cdiv(NN_NPARAM, 32), 256, 0, s, n);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1813,10 +1832,10 @@ cudaError_t reverse_t(const NnArgs& n0, const AdjArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const dim3 pg(cdiv(max_pix(n), 256), n.nimg);
   const bool tc = std::is_same<T, float>::value && n.bf16;
-  nn_seed_kernel<T><<<pg, 256, 0, s>>>(n, a, tc ? static_cast<__nv_bfloat16*>(n.A1h) : nullptr);  // G4 = dZ3
+  launch(nn_seed_kernel<T>, pg, 256, 0, s, n, a, tc ? static_cast<__nv_bfloat16*>(n.A1h) : nullptr);  // G4 = dZ3
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = layers_vjp_t<T>(n, s)) != cudaSuccess) return e;
-  nn_image_vjp_kernel<T><<<image_grid(n), 256, 0, s>>>(n, a);
+  launch(nn_image_vjp_kernel<T>, image_grid(n), 256, 0, s, n, a);
   return cudaGetLastError();
 }
 
@@ -1831,22 +1850,22 @@ cudaError_t eval_vjp_t(const NnArgs& n0, const double* X, int H, int W, const do
   n = capped_wblocks(n);
   n.keep = 1;
   const long long pix = n.pix0;
-  nn_load_kernel<T><<<cdiv(4 * pix, 256), 256, 0, s>>>(X, static_cast<T*>(n.X), 4 * pix);
+  launch(nn_load_kernel<T>, cdiv(4 * pix, 256), 256, 0, s, X, static_cast<T*>(n.X), 4 * pix);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if ((e = layers_t<T>(n, s)) != cudaSuccess) return e;
   const bool tc = std::is_same<T, float>::value && n.bf16;
-  nn_seed_eval_kernel<T><<<cdiv(pix, 256), 256, 0, s>>>(n, GY, pix, tc ? static_cast<__nv_bfloat16*>(n.A1h) : nullptr);
+  launch(nn_seed_eval_kernel<T>, cdiv(pix, 256), 256, 0, s, n, GY, pix, tc ? static_cast<__nv_bfloat16*>(n.A1h) : nullptr);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = layers_vjp_t<T>(n, s)) != cudaSuccess) return e;
-  nn_unload_kernel<T><<<cdiv(4 * pix, 256), 256, 0, s>>>(static_cast<const T*>(n.G4), GX, 4 * pix);
+  launch(nn_unload_kernel<T>, cdiv(4 * pix, 256), 256, 0, s, static_cast<const T*>(n.G4), GX, 4 * pix);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t nn_prims(const double* U, double* Q, const Lay& lay, double gamma, cudaStream_t s) {
-  nn_prims_kernel<<<cdiv(lay.plane, 256), 256, 0, s>>>(U, Q, lay, Gas{gamma, gamma - 1.0, 1.0 / (gamma - 1.0)});
+  launch(nn_prims_kernel, cdiv(lay.plane, 256), 256, 0, s, U, Q, lay, Gas{gamma, gamma - 1.0, 1.0 / (gamma - 1.0)});
   return cudaGetLastError();
 }
 
@@ -1869,8 +1888,8 @@ cudaError_t nn_eval_vjp(const NnArgs& n, const double* X, int H, int W, const do
 
 cudaError_t nn_apply(const NnArgs& n, const StageArgs& a, bool rhs, cudaStream_t s) {
   const unsigned grid = cdiv(a.lay.nx, IT) * cdiv(a.lay.ny, IF);
-  if (n.fp32) nn_apply_kernel<float><<<grid, 256, 0, s>>>(n, a, rhs ? 1 : 0);
-  else nn_apply_kernel<double><<<grid, 256, 0, s>>>(n, a, rhs ? 1 : 0);
+  if (n.fp32) launch(nn_apply_kernel<float>, grid, 256, 0, s, n, a, rhs ? 1 : 0);
+  else launch(nn_apply_kernel<double>, grid, 256, 0, s, n, a, rhs ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -1896,6 +1915,7 @@ cudaError_t nn_reverse(const NnArgs& n, const AdjArgs& a, cudaStream_t s) {
 namespace {
 __global__ void block_average_kernel(const double* __restrict__ U, int nx, int ny, int fx, int fy,
                                      double* __restrict__ out) {
+  pdl_enter();
   const int cx = nx / fx, cy = ny / fy;
   const long long n = (long long)cx * cy;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1913,7 +1933,7 @@ __global__ void block_average_kernel(const double* __restrict__ U, int nx, int n
 
 cudaError_t launch_block_average(const double* U, int nx, int ny, int fx, int fy, double* out, cudaStream_t s) {
   const long long n = 4LL * (nx / fx) * (ny / fy);
-  block_average_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(U, nx, ny, fx, fy, out);
+  launch(block_average_kernel, (unsigned)((n + 255) / 256), 256, 0, s, U, nx, ny, fx, fy, out);
   return cudaGetLastError();
 }
 
