@@ -326,13 +326,13 @@ __device__ __forceinline__ bool stage_constants(const StageArgs& a0, StageArgs& 
 }
 
 // x line blocks, then y line blocks; B: resident blocks an SM the registers are allotted for
-template <bool VISC, bool IMG, int B>
+template <bool VISC, bool IMG, int B, bool SPLIT = false>
 __global__ void __launch_bounds__(32 * SLINES, B) stage_lines_kernel(StageArgs a, int bx) {
   pdl_enter();
   if (a.dtc != nullptr && a.dtc[4] == 0.0) return;  // an inactive device-sized step
-  __shared__ double smem[stage_smem<VISC>() / sizeof(double)];
+  __shared__ double smem[stage_smem<VISC, SPLIT>() / sizeof(double)];
   const int b = blockIdx.x;
-  stage_lines<VISC, IMG>(a, b < bx ? 0 : 1, b < bx ? b : b - bx, smem);
+  stage_lines<VISC, IMG, SPLIT>(a, b < bx ? 0 : 1, b < bx ? b : b - bx, smem);
 }
 
 template <bool RHS>
@@ -345,19 +345,20 @@ __global__ void __launch_bounds__(128) stage_cells_kernel(StageArgs a0) {
   for (int gj = blockIdx.y; gj < a.lay.ny; gj += gridDim.y) stage_cell<RHS>(a, gi, gj);
 }
 
-// one line (ny == 1): a warp per 28 cells
+// one line (ny == 1): four warps per 28 cells, a variable's reconstruction each.  Latency up to some
+// 30000 cells (one warp per 28 cells: 200 cells 38 us a step, four 30), equal at 70000 and above.
 template <bool VISC, bool RHS>
-__global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
+__global__ void __launch_bounds__(128) stage1d_kernel(StageArgs a0) {
   pdl_enter();
   StageArgs a;
   if (!stage_constants(a0, a)) return;
   constexpr int NPL = VISC ? 5 : 4;
   constexpr int PS = SB;
-  __shared__ double sq[NPL * PS];
+  __shared__ double sq[NPL * PS + 256];
   const Gas g{a.gamma, a.gm1, a.g1};
-  const int tx0 = blockIdx.x * SCHUNK, lane = threadIdx.x;
+  const int tx0 = blockIdx.x * SCHUNK, lane = threadIdx.x & 31;
   const int W = a.lay.nx + 6;
-  for (int col = lane; col < PS; col += 32) {
+  for (int col = threadIdx.x; col < PS; col += 128) {
     const int gx = tx0 + col;
     const int gc = (gx < W) ? gx : W - 1;
     const double r = a.Uin[gc], mx = a.Uin[a.lay.plane + gc], my = a.Uin[2 * a.lay.plane + gc],
@@ -370,10 +371,10 @@ __global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
     sq[3 * PS + col] = p;
     if (NPL == 5) sq[4 * PS + col] = T;
   }
-  __syncwarp();
+  __syncthreads();
   const int k = lane - 2, gi = tx0 + k;
   double dF[4];
-  line_fluxes<VISC, false>(sq + k + 3, PS, 0, 1, g, a.vx, dF);
+  if (!line_fluxes<VISC, false>(sq + k + 3, PS, 0, 1, g, a.vx, dF, sq + NPL * PS)) return;
   if (lane < 2 || lane > 29 || gi >= a.lay.nx) return;
   if (!(positive(sq[k + 3]) && positive(sq[3 * PS + k + 3]))) atomicOr(a.err, ERR_NONPHYSICAL_BIT);
   finish_cell<RHS>(a, gi, 0, dF, dF);
@@ -383,12 +384,21 @@ __global__ void __launch_bounds__(32) stage1d_kernel(StageArgs a0) {
 // launchers
 // =======================================================================================
 namespace {
+// Blocks of eight lines up to which four warps share a line: about one block an SM, where a warp's
+// chain of four reconstructions is the time.  Per step, shared and not: 96x64 47 and 61 us, 128x128 66
+// and 73; then the chip fills: 200x128 (253 blocks) 85 and 80, 250x190 115 and 100.
+constexpr int SPLIT_BLOCKS = 160;
 // Resident blocks an SM the registers are allotted for: 4 (64 registers, 32 warps) hides the FP64
 // and integer latencies best (2048x1024 viscous step: 4 blocks 2.42 ms, 3 blocks 2.50, 2 blocks
 // 2.96).  Tuning variants 1 and 2 are 3 and 2 blocks; every variant gives the same bits.
 template <bool VISC, bool IMG>
 cudaError_t launch_lines(const StageArgs& a, int variant, cudaStream_t s) {
   const int bx = stage_blocks(a.lay, 0), n = bx + stage_blocks(a.lay, 1);
+  if (n <= SPLIT_BLOCKS && variant != 1 && variant != 2) {
+    const int sx = stage_blocks(a.lay, 0, SPLIT_LINES);
+    return launch(stage_lines_kernel<VISC, IMG, 2, true>, sx + stage_blocks(a.lay, 1, SPLIT_LINES), 32 * SLINES, 0, s, a,
+                  sx);
+  }
   if constexpr (!IMG) {
     if (variant == 1 || variant == 2) {
       if (variant == 1) launch(stage_lines_kernel<VISC, IMG, 3>, n, 32 * SLINES, 0, s, a, bx);
@@ -412,8 +422,7 @@ cudaError_t launch_stage2d(const StageArgs& a, bool rhs, int variant, cudaStream
 
 template <bool VISC, bool RHS>
 cudaError_t launch_stage1d(const StageArgs& a, cudaStream_t s) {
-  launch(stage1d_kernel<VISC, RHS>, stage_chunks(a.lay.nx), 32, 0, s, a);
-  return cudaGetLastError();
+  return launch(stage1d_kernel<VISC, RHS>, stage_chunks(a.lay.nx), 128, 0, s, a);
 }
 }  // namespace
 

@@ -40,9 +40,12 @@ struct NoFace {
 // warp calls it, consecutive lanes on consecutive cells; q[-1 .. 1] is readable for each.
 // face(ql, qr), when given, receives the two WENO5 states of face i+1/2 before any positivity
 // fallback (lanes 1..29).
+// fb null: the warp takes the line alone.  Else four warps share it, warp k (of the block's, mod 4)
+// reconstructing variable k into fb ([8][32], one per line) and warp 0 going on after a barrier of the
+// block: the same values with a quarter of the reconstructions' latency.  False for the other warps.
 template <bool VISC, bool HAS_T, class Face = NoFace>
-__device__ __forceinline__ void line_fluxes(const double* q, int ps, int ts, int pn, const Gas& g,
-                                            const ViscC& vc, double dF[4], Face face = Face{}) {
+__device__ __forceinline__ bool line_fluxes(const double* q, int ps, int ts, int pn, const Gas& g, const ViscC& vc,
+                                            double dF[4], double* fb, Face face = Face{}) {
   constexpr bool FI = !std::is_same<Face, NoFace>::value;
   constexpr int st = 1;
   const int lane = threadIdx.x & 31;
@@ -50,20 +53,35 @@ __device__ __forceinline__ void line_fluxes(const double* q, int ps, int ts, int
   const int pt = 3 - pn;
   // face states of the cell in the line's frame: rho, normal, tangential velocity, p
   double L[4], R[4];
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    const int c = (k == 1) ? pn : (k == 2) ? pt : k;
+  if (fb != nullptr) {
+    const int k = (threadIdx.x >> 5) & 3;
     double Lf, Rf;
-    weno_lane(q + c * ps, st, k == 0 || k == 3, inner, Lf, Rf);
+    weno_lane(q + ((k == 1) ? pn : (k == 2) ? pt : k) * ps, st, k == 0 || k == 3, inner, Lf, Rf);
+    fb[32 * k + lane] = Lf;
+    fb[32 * (4 + k) + lane] = Rf;
+    __syncthreads();
+    if (k != 0) return false;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      L[m] = (k == m) ? Lf : L[m];
-      R[m] = (k == m) ? Rf : R[m];
+      L[m] = fb[32 * m + lane];
+      R[m] = fb[32 * (4 + m) + min(lane + 1, 31)];
     }
-  }
-  // face i+1/2: the cell's left-biased state, its neighbour's right-biased one
+  } else {
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+      const int c = (k == 1) ? pn : (k == 2) ? pt : k;
+      double Lf, Rf;
+      weno_lane(q + c * ps, st, k == 0 || k == 3, inner, Lf, Rf);
 #pragma unroll
-  for (int m = 0; m < 4; ++m) R[m] = shfl_down(R[m]);
+      for (int m = 0; m < 4; ++m) {
+        L[m] = (k == m) ? Lf : L[m];
+        R[m] = (k == m) ? Rf : R[m];
+      }
+    }
+    // face i+1/2: the cell's left-biased state, its neighbour's right-biased one
+#pragma unroll
+    for (int m = 0; m < 4; ++m) R[m] = shfl_down(R[m]);
+  }
   const double* un = q + pn * ps;
   const double* ut = q + pt * ps;
   if (FI) {
@@ -105,6 +123,7 @@ __device__ __forceinline__ void line_fluxes(const double* q, int ps, int ts, int
   dF[1] = pn == 1 ? D[1] : D[2];
   dF[2] = pn == 1 ? D[2] : D[1];
   dF[3] = D[3];
+  return true;
 }
 
 // =======================================================================================
@@ -112,16 +131,17 @@ __device__ __forceinline__ void line_fluxes(const double* q, int ps, int ts, int
 // =======================================================================================
 constexpr int SCHUNK = 28, SLINES = 8;  // cells a warp, lines (warps) a block
 constexpr int SB = SCHUNK + 6;          // positions of a line's box: lane l at l + 1
-constexpr int SL = SLINES + 2;          // lines of a block's box: its own and one on either side
-constexpr int SP = SB * SL;             // plane of the box, [line][position] in both directions
+constexpr int SPLIT_LINES = SLINES / 4;  // lines a block where four warps share one
+// plane of a block's box, [line][position] in both directions: nl lines and one on either side
+__host__ __device__ constexpr int stage_plane(int nl) { return SB * (nl + 2); }
 
 __host__ __device__ inline int stage_chunks(int n) { return (n + SCHUNK - 1) / SCHUNK; }
-__host__ __device__ inline int stage_blocks(const Lay& L, int dir) {
-  return dir == 0 ? (L.ny + SLINES - 1) / SLINES * stage_chunks(L.nx) : (L.nx + SLINES - 1) / SLINES * stage_chunks(L.ny);
+__host__ __device__ inline int stage_blocks(const Lay& L, int dir, int nl = SLINES) {
+  return dir == 0 ? (L.ny + nl - 1) / nl * stage_chunks(L.nx) : (L.nx + nl - 1) / nl * stage_chunks(L.ny);
 }
-template <bool VISC>
+template <bool VISC, bool SPLIT = false>
 __host__ __device__ constexpr size_t stage_smem() {
-  return sizeof(double) * (size_t)((VISC ? 5 : 4) * SP);
+  return sizeof(double) * (size_t)((VISC ? 5 : 4) * stage_plane(SPLIT ? SPLIT_LINES : SLINES) + (SPLIT ? SPLIT_LINES * 256 : 0));
 }
 
 // face image of the neural flux (IMG: a.img, FP32 [4][ny][nx+1] for x faces then [4][nx][ny+1]
@@ -140,15 +160,16 @@ __device__ __forceinline__ void put_image(const StageArgs& a, int dir, int line,
   for (int k = 0; k < 4; ++k) X[k * pix] = m[k];
 }
 
-// block `item` of direction dir (0: x lines): SLINES warps, a line each; writes the flux differences
-// to a.dF (4 padded planes for x, 4 for y)
-template <bool VISC, bool IMG>
+// block `item` of direction dir (0: x lines): SLINES warps, a line each (SPLIT: four warps a line);
+// writes the flux differences to a.dF (4 padded planes for x, 4 for y)
+template <bool VISC, bool IMG, bool SPLIT = false>
 __device__ __forceinline__ void stage_lines(const StageArgs& a, int dir, int item, double* sq) {
+  constexpr int NL = SPLIT ? SPLIT_LINES : SLINES, SL = NL + 2, SP = stage_plane(NL);
   const Lay& L = a.lay;
   const Gas g{a.gamma, a.gm1, a.g1};
   const int nline = dir == 0 ? L.ny : L.nx, ncell = dir == 0 ? L.nx : L.ny;
   const int nch = stage_chunks(ncell);
-  const int i0 = SCHUNK * (item % nch), line0 = item / nch * SLINES;
+  const int i0 = SCHUNK * (item % nch), line0 = item / nch * NL;
   const int gyl = dir == 0 ? L.gy : 3, gyc = dir == 0 ? 3 : L.gy;  // ghost layers across / along the line
   for (int e = threadIdx.x; e < SP; e += 32 * SLINES) {
     // consecutive threads along x in both directions
@@ -171,22 +192,24 @@ __device__ __forceinline__ void stage_lines(const StageArgs& a, int dir, int ite
     if (VISC) sq[4 * SP + o] = T;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int line = line0 + warp, cell = i0 - 2 + lane;
-  if (line >= nline) return;
-  const double* q = sq + (warp + 1) * SB + lane + 1;
+  const int lane = threadIdx.x & 31, ln = (threadIdx.x >> 5) / (SPLIT ? 4 : 1);
+  const int line = line0 + ln, cell = i0 - 2 + lane;
+  if (!SPLIT && line >= nline) return;  // (the shared lines' warps meet at a barrier)
+  const double* q = sq + (ln + 1) * SB + lane + 1;
+  double* const fb = SPLIT ? sq + (VISC ? 5 : 4) * SP + 256 * ln : nullptr;
   double dF[4];
   const ViscC& vc = dir == 0 ? a.vx : a.vy;
   if constexpr (IMG) {
-    line_fluxes<VISC, true>(q, SP, SB, dir + 1, g, vc, dF, [&](const double* ql, const double* qr) {
+    const bool mine = line_fluxes<VISC, true>(q, SP, SB, dir + 1, g, vc, dF, fb, [&](const double* ql, const double* qr) {
       // face cell + 1; the chunk's outer face belongs to the next chunk unless it is the line's last
       const int f = cell + 1;
-      if (lane >= 1 && f <= ncell && (lane <= 28 || (lane == 29 && f == ncell))) put_image(a, dir, line, f, ql, qr);
+      if (line < nline && lane >= 1 && f <= ncell && (lane <= 28 || (lane == 29 && f == ncell))) put_image(a, dir, line, f, ql, qr);
     });
+    if (!mine) return;
   } else {
-    line_fluxes<VISC, true>(q, SP, SB, dir + 1, g, vc, dF);
+    if (!line_fluxes<VISC, true>(q, SP, SB, dir + 1, g, vc, dF, fb)) return;
   }
-  if (lane >= 2 && lane < 30 && cell < ncell) {
+  if (line < nline && lane >= 2 && lane < 30 && cell < ncell) {
     const int i = dir == 0 ? cell : line, j = dir == 0 ? line : cell;
     const long long t = L.idx(i, j);
     if (dir == 0 && !(positive(q[0]) && positive(q[3 * SP])) &&
