@@ -107,8 +107,7 @@ __global__ void adj_ib_src_kernel(AdjArgs a, IbTArgs tb, const double* qIb) {
 __global__ void adj_unpack_add_kernel(const double* __restrict__ P, const double* __restrict__ P2,
                                       double* __restrict__ U, Lay lay) {
   pdl_enter();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < 4LL * lay.nx * lay.ny) adj_unpack_add_one(P, P2, U, lay, t);
+  adj_unpack_add_one(P, P2, U, lay, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // =======================================================================================
@@ -195,7 +194,7 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
 }
 
 cudaError_t launch_adj_unpack(const double* P, const double* P2, double* U, const Lay& lay, cudaStream_t s) {
-  launch(adj_unpack_add_kernel, blocks_for(4LL * lay.nx * lay.ny, 256), 256, 0, s, P, P2, U, lay);
+  launch(adj_unpack_add_kernel, blocks_for((long long)lay.nx * lay.ny, 256), 256, 0, s, P, P2, U, lay);
   return cudaGetLastError();
 }
 

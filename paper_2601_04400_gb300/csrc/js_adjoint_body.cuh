@@ -579,15 +579,18 @@ __device__ __forceinline__ void adj_ib_src_one(const AdjArgs& a, const IbTArgs& 
 // =======================================================================================
 // small elementwise helpers
 // =======================================================================================
+// cell t (fewer than 2^31), its four planes
 __device__ __forceinline__ void adj_unpack_add_one(const double* __restrict__ P, const double* __restrict__ P2,
-                                                   double* __restrict__ U, const Lay& lay, long long t) {
-  const long long n = (long long)lay.nx * lay.ny;
-  if (t >= 4 * n) return;
-  const int c = (int)(t / n);
-  const long long o = t % n;
-  const int i = (int)(o % lay.nx), j = (int)(o / lay.nx);
-  const long long id = c * lay.plane + lay.idx(i, j);
-  U[t] = P2 ? P[id] + P2[id] : P[id];
+                                                   double* __restrict__ U, const Lay& lay, unsigned t) {
+  const unsigned n = (unsigned)lay.nx * (unsigned)lay.ny;
+  if (t >= n) return;
+  const int i = (int)(t % (unsigned)lay.nx), j = (int)(t / (unsigned)lay.nx);
+  const long long id = lay.idx(i, j);
+  double v[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) v[c] = P2 ? P[c * lay.plane + id] + P2[c * lay.plane + id] : P[c * lay.plane + id];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) U[(long long)c * n + t] = v[c];
 }
 
 }  // namespace js

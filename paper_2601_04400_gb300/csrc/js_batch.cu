@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(FNT) batch_barrier_kernel(BatchArgs b) {
 // fixed order too.  Work items of every instance are padded to whole warps (planes: to whole blocks),
 // so a warp never spans two instances.
 // =======================================================================================
-enum RevKind { RK_PLANE = 0, RK_USER4, RK_GHOST, RK_HALO, RK_BCTY, RK_BCTX, RK_SRC, RK_N };
+enum RevKind { RK_PLANE = 0, RK_USER, RK_GHOST, RK_HALO, RK_BCTY, RK_BCTX, RK_SRC, RK_N };
 
 struct RevCall {
   const double* const* Un;    // [count] user states U_n
@@ -483,19 +483,25 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
   const RevCall& call = b.call;
   const bool even = (s == 2) || (s == 0);  // reverse stages 2 and 0 read P0, write P1
   if constexpr (PH == RP_PACK) {
-    rev_items(b, RK_USER4, [&](int k, long long t) {
+    rev_items(b, RK_USER, [&](int k, long long t) {
       if (k < 0) return;
       const InstDesc& d = b.inst[k];
-      const long long n = (long long)d.lay.nx * d.lay.ny;
-      if (t >= 4 * n) return;
-      const int c = (int)(t / n);
-      const long long o = t % n;
-      const long long p = c * d.lay.plane + d.lay.idx((int)(o % d.lay.nx), (int)(o / d.lay.nx));
-      d.N[p] = call.Un[k][t];
-      b.rev[k].P0[p] = call.lam1[k][t];
-      if (call.U1) {
-        d.A[p] = call.U1[k][t];
-        d.B[p] = call.U2[k][t];
+      const unsigned n = (unsigned)d.lay.nx * (unsigned)d.lay.ny, q = (unsigned)t;
+      if (q >= n) return;
+      const long long p0 = d.lay.idx((int)(q % (unsigned)d.lay.nx), (int)(q / (unsigned)d.lay.nx));
+      const double *Un = call.Un[k] + q, *lam = call.lam1[k] + q, *U1 = nullptr, *U2 = nullptr;
+      if (call.U1) U1 = call.U1[k] + q, U2 = call.U2[k] + q;
+      double* P0 = b.rev[k].P0;
+      double v[4], l[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = Un[(long long)c * n], l[c] = lam[(long long)c * n];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) d.N[c * d.lay.plane + p0] = v[c], P0[c * d.lay.plane + p0] = l[c];
+      if (U1) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = U1[(long long)c * n], l[c] = U2[(long long)c * n];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) d.A[c * d.lay.plane + p0] = v[c], d.B[c * d.lay.plane + p0] = l[c];
       }
     });
     rev_items(b, RK_PLANE, [&](int k, long long t) {
@@ -631,11 +637,10 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
     });
   } else if constexpr (PH == RP_UNPACK) {
     // lambda_n = P1 + Uacc (stage 0 wrote P1); the last stage's parameter gradient
-    rev_items(b, RK_USER4, [&](int k, long long t) {
+    rev_items(b, RK_USER, [&](int k, long long t) {
       if (k < 0) return;
       const InstDesc& d = b.inst[k];
-      if (t >= 4LL * d.lay.nx * d.lay.ny) return;
-      adj_unpack_add_one(b.rev[k].P1, b.rev[k].Uacc, call.lam0[k], d.lay, t);
+      adj_unpack_add_one(b.rev[k].P1, b.rev[k].Uacc, call.lam0[k], d.lay, (unsigned)t);
     });
     if (call.pbar)
       for (int k = blockIdx.x; k < b.count; k += gridDim.x)
@@ -756,7 +761,7 @@ int rev_prepare(js_batch* b) {
     r.off_s = r.off_g + r.w_g;
     r.w_s = round32(4LL * r.ibt.nsrc) / 32;
     const long long cnt[js::RK_N] = {
-        plane, round32(4LL * L.nx * L.ny), round32(4LL * d.ib.n), round32(js::halo_count(L)),
+        plane, round32((long long)L.nx * L.ny), round32(4LL * d.ib.n), round32(js::halo_count(L)),
         round32(8LL * (L.nx + 6)), round32(8LL * L.ny), round32(4LL * r.ibt.nsrc)};
     for (int q = 0; q < js::RK_N; ++q) pre[(size_t)q * (n + 1) + k + 1] = pre[(size_t)q * (n + 1) + k] + cnt[q];
   }
