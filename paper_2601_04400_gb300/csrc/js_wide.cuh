@@ -207,9 +207,11 @@ JS_HD double sound_wide(double g, double p, double r) {
 
 // a signed fixed-point value c 2^(e - 1086) as a double (rounded at 53 bits):
 // c / 2^63 in [1/2, 1) has the biased exponent e.  Values below the normal range give 0.
+// c is the floor of the value meant (right shifts brought it there), so a negative one's magnitude is
+// -c - 1 and a fraction: the complement rounds it as a positive value's floor does.
 JS_HD double fix_to_double(s64 c, int e) {
   const s64 sg = c >> 63;
-  u64 m = (u64)((c ^ sg) - sg);
+  u64 m = (u64)(c ^ sg);
   const int lz = clz64(m);
   m <<= (lz & 63);
   const int be = e - lz;  // biased exponent of the leading bit
