@@ -925,7 +925,9 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
     js_batch_destroy(b);
     return JS_ERR_NOMEM;
   }
-  if (cudaMemcpy(b->d_tile0, tile0.data(), sizeof(int) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+  // (the reverse takes its states per call: the instances must be on the device before js_batch_set_states)
+  if (cudaMemcpy(b->d_desc, b->desc.data(), sizeof(InstDesc) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(b->d_tile0, tile0.data(), sizeof(int) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_line0, b->line0.data(), sizeof(int) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_ghost0, ghost0.data(), sizeof(long long) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_halo0, halo0.data(), sizeof(long long) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
