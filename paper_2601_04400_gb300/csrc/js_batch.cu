@@ -1322,7 +1322,9 @@ int js_batch_set_tuning(js_batch* b, int blocks_per_sm, int schedule) {
   }
   b->schedule = schedule;
   b->blocks = b->sms * (blocks_per_sm == 0 ? b->per_sm : blocks_per_sm);
-  b->blocks_set = blocks_per_sm != 0;
+  // the most that fit: a launched block an item, which the hardware balances better than resident blocks
+  // striding over them (256 instances, one step: 18.5 ms against 23.4)
+  b->blocks_set = blocks_per_sm != 0 && blocks_per_sm < b->per_sm;
   return JS_OK;
 }
 
