@@ -102,8 +102,8 @@ __device__ __forceinline__ bool line_fluxes(const double* q, int ps, int ts, int
     const double dun = ub - ua, dut = tb - ta, dT = Tq[st] - Tq[0];
     double tnn, tnt;
     if (HAS_T) {
-      const double sun = (un[ts] - un[-ts]) + (un[st + ts] - un[st - ts]);
-      const double sut = (ut[ts] - ut[-ts]) + (ut[st + ts] - ut[st - ts]);
+      const double cun = un[ts] - un[-ts], cut = ut[ts] - ut[-ts];
+      const double sun = cun + shfl_down(cun), sut = cut + shfl_down(cut);
       tnn = fma(vc.c43n, dun, -vc.c23t * sut);
       tnt = fma(vc.cn, dut, vc.ct * sun);
     } else {
@@ -111,10 +111,9 @@ __device__ __forceinline__ bool line_fluxes(const double* q, int ps, int ts, int
       tnt = vc.cn * dut;
     }
     const double sbn = ua + ub, sbt = ta + tb;
-    const double e = fma(0.5, fma(sbn, tnn, sbt * tnt), vc.ck * dT);
     F[1] -= tnn;
     F[2] -= tnt;
-    F[3] -= e;
+    F[3] = fma(-0.5, fma(sbn, tnn, sbt * tnt), fma(-vc.ck, dT, F[3]));
   }
   double D[4];
 #pragma unroll
