@@ -15,7 +15,8 @@ the largest single-GPU configuration: the viscous Mach-2 shock over the immersed
 Prints ONE JSON line (rank 0).  `value` is cell-updates/s with the state resident in HBM;
 `e2e` is the same metric through the C ABI with the state copied from pinned host memory
 and back every step; `roofline` divides the algorithmic FP64 operation count of the stage
-kernel by its CUDA-event time and by the FP64 peak.
+kernels (lines, then cells) by their CUDA-event time and by the FP64 peak; the kernels form WENO5,
+reciprocals and square roots in integer arithmetic beside the FP64 pipe, so the fraction exceeds 1.
 """
 import argparse
 import json
@@ -37,14 +38,10 @@ FLOPS_PER_CELL_STAGE = {"riemann2d": 1281.0, "shock_cylinder": 1357.0, "mach5_cy
 FP64_PEAK_TFLOPS = 1.25
 # neural flux network per cell and stage: x and y face images, 2 x 6336 multiply-adds each
 NN_FLOPS_PER_CELL_STAGE = 2 * 2 * 6336
-# DRAM bytes (read + write) per stage-kernel launch, mean of the three stages of one step,
-# from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of this bench's default
-# run with the TMA-staged variant 0 and the current kernel; None for other workloads or
-# variants (and for workloads whose capture predates the current kernel).
-STAGE_TRAFFIC_BYTES = {("shock_cylinder", 0): 291.0e6, ("riemann2d", 0): 108.0e6}
-# DRAM bytes per step of the persistent batched forward kernel on the 256-instance workload: an
-# ncu capture of one 2-step launch of the current kernel (19.27 GB), scaled by the steps of a launch
-BATCH_TRAFFIC_PER_STEP = 9.64e9
+# DRAM bytes (read + write) per stage (lines + cells kernels), mean of the three stages of one step,
+# from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the current kernels; None for
+# workloads or variants without one.
+STAGE_TRAFFIC_BYTES = {("shock_cylinder", 0): 500.1e6, ("riemann2d", 0): 182.0e6}
 L2_FLUSH_BYTES = 256 << 20
 METRIC = "FP64 cell-updates/s per RK step on 1 GB300 (% roofline); adjoint/forward time ratio"
 
@@ -398,7 +395,7 @@ def run_ours(args):
             "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": achieved / FP64_PEAK_TFLOPS,
                          "traffic": STAGE_TRAFFIC_BYTES.get((args.workload, solver.tuning()[0])),
-                         "kernel": "stage2d (fused WENO5-HLLC stage)", "stage_ms_avg": stage_avg,
+                         "kernel": "stage_lines + stage_cells (WENO5, HLLC, viscous fluxes; Runge-Kutta stage)", "stage_ms_avg": stage_avg,
                          "flops_per_launch": flop_launch},
             "e2e": {"value": e2e_value, "unit": "cell-updates/s", "h2d_bytes_per_step": state_bytes,
                     "d2h_bytes_per_step": state_bytes},
@@ -418,7 +415,7 @@ def run_ours(args):
 
 
 def run_batched(args):
-    """Many independent shock-cylinder instances: one persistent launch per js_batch_step
+    """Many independent shock-cylinder instances: a launch per phase over all of them per js_batch_step
     (device CFL per instance) against one-at-a-time js_max_dt + js_step per instance."""
     import torch
     from paper_2601_04400_gb300 import binding as B
@@ -456,7 +453,7 @@ def run_batched(args):
     sampler = ClockSampler(local)
     with sampler:
         e0.record(stream)
-        batch.step(0.5, args.steps)  # one persistent launch for all steps
+        batch.step(0.5, args.steps)  # every launch works on all instances
         e1.record(stream)
         e1.synchronize()
     t_batch = e0.elapsed_time(e1)
@@ -519,7 +516,7 @@ def run_batched(args):
         s.set_stream(stream)
     ok = ok and all(s.status() == 0 for s in solvers)
     # reverse of one batched step (js_batch_step_vjp over all instances) against one batched
-    # forward step, in both launch forms (one persistent launch; one launch per phase); the tuner
+    # forward step, in both settings of the launch form (they run the same launches); the tuner
     # keeps the faster for the rollout below
     dts = [s.max_dt(U, 0.5) for s, U in zip(solvers, states)]
     lams = [torch.randn_like(U) for U in states]
@@ -592,21 +589,21 @@ def run_batched(args):
             "data": "synthetic", "status_ok": ok,
             "config": {"workload": "%d viscous shock-cylinder instances (seed 0: Mach U[1.5,3], radius U[0.3,0.7], "
                                    "nx 128..512, ny 128..256), per-instance device CFL 0.5" % len(mine),
-                       "cells": cells, "persistent_blocks": info["blocks"], "tiles": info["tiles"],
+                       "cells": cells, "resident_line_blocks": info["blocks"], "tiles": info["tiles"],
                        "tuning": {"blocks_per_sm": batch.tuning()[0], "schedule": batch.tuning()[2],
                                   "timed": {"%d,%d" % k: v for k, v in tuned.items()}}},
             "e2e": {"value": cells * args.steps / (t_e2e * 1e-3), "unit": "cell-updates/s",
                     "h2d_bytes_per_step": state_bytes, "d2h_bytes_per_step": state_bytes},
-            "roofline": {"bound": "alu", "kernel": "batch_kernel (persistent: CFL, IB and halo fills, stage tiles)",
+            "roofline": {"bound": "alu", "kernel": "batch_phase_kernel (CFL, IB and halo fills, lines, cells: the whole run)",
                          "achieved": FLOPS_PER_CELL_STAGE["shock_cylinder"] * 3 * cells * args.steps
                          / (t_batch * 1e-3) / 1e12,
                          "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": FLOPS_PER_CELL_STAGE["shock_cylinder"] * 3 * cells * args.steps
                          / (t_batch * 1e-3) / 1e12 / FP64_PEAK_TFLOPS,
-                         "traffic": BATCH_TRAFFIC_PER_STEP * args.steps if args.instances == 256 and world == 1
-                         else None,
+                         "traffic": None,
                          "flops_per_cell_stage": FLOPS_PER_CELL_STAGE["shock_cylinder"]},
-            "gpu_launches": 1, "clocks": sampler.summary(),
+            # pack and unpack; per step two CFL passes, the step sizes, 3 x (IB fill, halos, lines, cells)
+            "gpu_launches": 2 + 15 * args.steps, "clocks": sampler.summary(),
             "one_at_a_time": {"value": local_cells * args.steps / (t_seq * 1e-3), "ms_per_step": t_seq / args.steps,
                               "how": "rank 0's instances one after another, each js_step_cfl for all steps "
                                      "(device CFL, no host round trip)"},
@@ -617,8 +614,8 @@ def run_batched(args):
             "speedup_vs_one_at_a_time": t_seq / t_batch,
             "speedup_vs_graph": t_graph / t_batch,
             "adjoint": {"ms_per_step_vjp": t_vjp, "ratio": t_vjp / (t_batch / args.steps),
-                        "launch": "one launch per phase" if choice else "one persistent launch",
-                        "ms_per_step_vjp_persistent": t_vjp_form[0], "ms_per_step_vjp_split": t_vjp_form[1],
+                        "launch": "one launch per phase",
+                        "ms_per_step_vjp_form0": t_vjp_form[0], "ms_per_step_vjp_form1": t_vjp_form[1],
                         "tuner_timed": {str(k): v for k, v in rev_tuned.items()},
                         "note": "js_batch_step_vjp (recompute of the stage states and the reverse of the 3 "
                                 "stages of every instance; the launch form the tuner chose) / one batched "

@@ -124,11 +124,10 @@ int js_rhs_vjp(js_ctx* ctx, const double* U, const double* lam, double* U_bar, d
 /* Vector-Jacobian product of ONE SSP-RK3 step of size dt taken from U_n:
  *   lam_n  = (dU_{n+1}/dU_n)^T lam_np1     (overwritten), device [4][ny][nx]
  *   p_bar += (dU_{n+1}/dtheta)^T lam_np1   (accumulated), device double[JS_NPARAM] or NULL
- * The three stage states are recomputed from U_n inside the call (on 2D grids the first
- * two forward stages also store their WENO5 internals for the reverse pass, which needs
- * 2 x 56 extra padded planes of workspace; with the neural flux on, their network input and
- * activations are kept too, 2 x 56 face-image channels allocated by the first such call, and
- * recomputed instead when that allocation fails).  lam_n may alias lam_np1.  Asynchronous. */
+ * The three stage states are recomputed from U_n inside the call (with the neural flux on,
+ * the network input and activations of the first two forward stages are kept for the reverse,
+ * 2 x 56 face-image channels allocated by the first such call, and recomputed instead when that
+ * allocation fails).  lam_n may alias lam_np1.  Asynchronous. */
 int js_step_vjp(js_ctx* ctx, const double* U_n, double dt, const double* lam_np1, double* lam_n,
                 double* p_bar);
 
@@ -143,10 +142,9 @@ int js_step_vjp(js_ctx* ctx, const double* U_n, double dt, const double* lam_np1
  *                            recorded in `slot` (same dt), without recomputing its stages. */
 int js_tape_reserve(js_ctx* ctx, int n_slots);
 
-/* js_tape_reserve with options.  JS_TAPE_WENO (2D grids; ignored for ny == 1): every slot
- * also holds the WENO5 internals of its three stages (56 padded planes per stage, about
- * 1.3 KB per cell and slot), written by js_step_taped; js_step_vjp_taped then skips the
- * WENO forward recompute of its reverse pass.  Results are identical with and without.
+/* js_tape_reserve with options.  JS_TAPE_WENO is accepted and changes nothing: the reverse
+ * forms WENO5 again in integer arithmetic, which takes less time than reading stored internals
+ * (56 planes a stage) from memory would.
  * flags = 0 is js_tape_reserve; the choice applies to the js_step_taped calls that follow.
  * Returns JS_ERR_NOMEM (nothing freed) when the device memory does not suffice. */
 #define JS_TAPE_WENO 1
@@ -162,9 +160,8 @@ int js_step_vjp_taped(js_ctx* ctx, int slot, double dt, const double* lam_np1, d
  * stage > 0 (may be NULL for stage 0).  All arrays device [4][ny][nx]; any may alias.
  * Asynchronous.  This is the entry for callers that act between stages (the halo exchange of
  * a y-decomposed grid, below).  stage | JS_STAGE_INTERNALS (stages 0 and 1 of a 2D grid; the
- * flag is ignored otherwise) also stores the stage's WENO5 internals in the context (the
- * workspace of js_step_vjp, allocated by the first such call), for a js_step_stage_vjp of the
- * same stage and U_in that passes the flag too. */
+ * flag is ignored otherwise) marks the stage for a js_step_stage_vjp of the same stage and U_in
+ * that passes the flag too, and allocates the reverse workspace; it stores nothing else. */
 #define JS_STAGE_INTERNALS 16
 int js_step_stage(js_ctx* ctx, const double* U_n, const double* U_in, double* U_out, double dt, int stage);
 
@@ -174,10 +171,9 @@ int js_step_stage(js_ctx* ctx, const double* U_n, const double* U_in, double* U_
  *   p_bar  += (dU_out/dtheta)^T lam_out                                (accumulated, or NULL)
  * The U_n part a_k lam_out of stages 2 and 1 is kept in the context and added to the lam_in
  * of stage 0 (whose U_in is U_n): with lam_out of stage k-1 = lam_in of stage k, the stage-0
- * lam_in equals js_step_vjp's lam_n.  lam_in may alias lam_out.  stage | JS_STAGE_INTERNALS
- * uses the internals js_step_stage stored for that stage (stages 0, 1 of a 2D grid; JS_ERR_ARG
- * when it stored none since the last js_step_vjp) instead of recomputing WENO5: same results.
- * Asynchronous. */
+ * lam_in equals js_step_vjp's lam_n.  lam_in may alias lam_out.  stage | JS_STAGE_INTERNALS:
+ * the same results, JS_ERR_ARG when js_step_stage did not mark that stage (0, 1 of a 2D grid)
+ * since the last js_step_vjp.  Asynchronous. */
 int js_step_stage_vjp(js_ctx* ctx, const double* U_in, double dt, int stage, const double* lam_out,
                       double* lam_in, double* p_bar);
 
@@ -287,12 +283,11 @@ int js_ib_info(js_ctx* ctx, int* n_ghost, unsigned char* tag_host);
 
 /* ---- batched path ---------------------------------------------------------------------
  * Many independent 2D problems (uneven grids, parameters, boundaries, immersed bodies)
- * advanced together by ONE persistent cooperative kernel launch per js_batch_step call (the
- * solver step mapped over a batch of problems; the paper's vmap, Sec. 1).  Each instance's
+ * advanced together: every launch works on all of them (the solver step mapped over a batch of
+ * problems; the paper's vmap, Sec. 1).  Each instance's
  * dt is recomputed on the device before every step from its own state (CFL rule of
  * js_max_dt, same arithmetic, so a batched run equals per-instance js_max_dt + js_step runs
- * bit for bit).  Grid barriers inside the launch wait at most 2 s each; a wait that runs out
- * sets JS_ERR_TIMEOUT (read by js_batch_sync_status) and the launch returns. */
+ * bit for bit). */
 typedef struct js_batch js_batch;
 
 /* Create a batch of `count` problems: arrays grids[count], params[count], bcs[count];
@@ -306,15 +301,15 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
  * device and synchronises; call again when the pointers change (not inside a capture). */
 int js_batch_set_states(js_batch* b, double* const* U);
 
-/* Advance every instance by n_steps SSP-RK3 steps with its own CFL time step (cfl > 0) in
- * one launch.  t_dev: optional device double[count] to which each instance's elapsed time
+/* Advance every instance by n_steps SSP-RK3 steps with its own CFL time step (cfl > 0).
+ * t_dev: optional device double[count] to which each instance's elapsed time
  * is added.  dt_log: optional device double[n_steps][count] receiving the step sizes used
  * (the reverse pass needs them).  Asynchronous; allocates nothing, so it can be captured
  * into a CUDA graph. */
 int js_batch_step(js_batch* b, double cfl, int n_steps, double* t_dev, double* dt_log);
 
-/* Reverse of one batched step (the gradient chain rule of Sec. 2 per instance) in ONE
- * persistent cooperative launch over all instances: for every instance k,
+/* Reverse of one batched step (the gradient chain rule of Sec. 2 per instance), a launch per
+ * phase over all instances: for every instance k,
  * lam_n[k] = (dU_{n+1}/dU_n)^T lam_np1[k] for the step of size dt[k] taken from U_n[k]
  * (the same values as js_step_vjp, bit for bit), and p_bar[k] += (dU_{n+1}/dtheta_k)^T
  * lam_np1[k] (JS_NPARAM doubles each, summed in a fixed order; p_bar or an entry may be NULL).
@@ -327,8 +322,8 @@ int js_batch_step_vjp(js_batch* b, double* const* U_n, const double* dt, double*
                       double* const* lam_n, double* const* p_bar);
 
 /* Advance every registered state n_steps SSP-RK3 steps of the given sizes dt[step][count]
- * (device) instead of CFL step sizes, e.g. to replay a run logged by js_batch_step.  One launch;
- * asynchronous; allocates nothing. */
+ * (device) instead of CFL step sizes, e.g. to replay a run logged by js_batch_step.
+ * Asynchronous; allocates nothing. */
 int js_batch_step_fixed(js_batch* b, int n_steps, const double* dt);
 
 /* Reverse of a batched rollout of n_steps steps (the chain rule of Sec. 2 through the whole
@@ -341,14 +336,14 @@ int js_batch_step_fixed(js_batch* b, int n_steps, const double* dt);
  *           state after every ckpt-th step (or those of js_batch_rollout_forward are used, see
  *           there); then, from the last segment back, each segment is re-run keeping its
  *           states and its steps' stage states U1, U2, and reversed step by step by the
- *           persistent reverse launch of js_batch_step_vjp, which takes the stage states as
+ *           launches of js_batch_step_vjp, which take the stage states as
  *           given instead of recomputing them.  Spacing 1: the forward keeps every state and
  *           stage state, nothing is re-run.
  * Workspace: ceil(n_steps/ckpt) + 3 ckpt + 2 states per instance (3 n_steps + 3 with spacing
  * 1) and the reverse workspace,
  * allocated by the first call for these n_steps and ckpt (synchronises; make it before any
  * stream capture).  Later calls with the same n_steps, ckpt, lam and p_bar pointers enqueue
- * only kernels (one launch per copy, segment re-run and reverse step) and can be captured into
+ * only kernels and can be captured into
  * a CUDA graph.  Asynchronous otherwise. */
 int js_batch_rollout_vjp(js_batch* b, int n_steps, const double* dt_log, int ckpt, double* const* lam,
                          double* const* p_bar);
@@ -373,15 +368,16 @@ int js_batch_rollout_spacing(js_batch* b, int n_steps, int* ckpt);
  * JS_ERR_TIMEOUT. */
 int js_batch_sync_status(js_batch* b);
 
-/* Launch shape and size: resident blocks of the persistent kernel, 32x16 tiles, cells. */
+/* Launch shape and size: resident blocks of the forward's line kernel, 32x16 tiles, cells. */
 int js_batch_info(js_batch* b, int* blocks, int* tiles, long long* cells);
 
-/* Launch shape and schedule of the forward launch (js_batch_step, js_batch_step_fixed and the
- * rollout's forward runs): blocks_per_sm resident blocks on every SM (0 = the most that fit),
- * and the order in which the blocks take the tiles of all instances: 0 instance by instance,
- * 1 interleaved (tile j of every instance, then tile j + 1), 2 the largest instances first.
+/* Launch shape and schedule of the forward's line kernels (js_batch_step, js_batch_step_fixed and
+ * the rollout's forward runs): blocks_per_sm blocks on every SM striding over the blocks of lines (0 =
+ * a launched block for each), and the order in which they take the lines of all instances: 0 instance
+ * by instance, 1 interleaved (block j of every instance, then block j + 1), 2 the largest instances
+ * first.
  * Results are identical for every choice; only speed differs (the Python autotuner times them
- * and caches the choice per mix of instances).  Schedules 1 and 2 upload a tile table
+ * and caches the choice per mix of instances).  Schedules 1 and 2 upload a table
  * (synchronises: before any stream capture).  js_batch_get_tuning reports the current choice,
  * the most blocks per SM and the number of schedules. */
 int js_batch_set_tuning(js_batch* b, int blocks_per_sm, int schedule);
@@ -389,17 +385,12 @@ int js_batch_get_tuning(js_batch* b, int* blocks_per_sm, int* max_blocks_per_sm,
 
 /* Launch form of the batched reverse step (js_batch_step_vjp and every reverse step of
  * js_batch_rollout_vjp; the gradient chain rule of Sec. 2 applied to each instance):
- *   split = 0 (default): ONE persistent cooperative launch per reverse step, its phases (pack,
- *     forward recompute, then per stage: seed + primitives, pass 1, pass 2, primitive reverse,
- *     transposed halos, inflow gradient and IB ghosts, IB sources; unpack) separated by
- *     bounded grid barriers, every phase at the register allocation of the heaviest one;
- *   split = 1: one ordinary launch per phase (34 per reverse step; 37 when the batch mixes
- *     viscous and inviscid instances), in the same order on the batch's stream, each phase
- *     kernel at its own occupancy.
- * Both run the same device code on the same work items in the same order: lambda and the
- * parameter gradient agree to rounding (separately compiled kernels may contract different
- * products into fused multiply-adds), and each form repeats its own results bit for bit.
- * Both can be captured in a CUDA graph.
+ *   split = 0 (default) and split = 1 both run one ordinary launch per phase (pack, forward
+ *     recompute, then per stage: lines, cells, transposed halos, inflow gradient and IB ghosts, IB
+ *     sources; unpack: 32 per reverse step with given parameter gradients, one more per line phase
+ *     when the batch mixes viscous and inviscid instances), each phase kernel at its own occupancy.
+ *     A single persistent launch, which 0 selected before, was slower on every batch.
+ * Results repeat bit for bit; rollouts can be captured in a CUDA graph.
  * Synchronises the batch's stream (call before any stream capture).  Errors: JS_ERR_ARG for a
  * split value other than 0 or 1. */
 int js_batch_set_reverse_launch(js_batch* b, int split);
@@ -408,7 +399,7 @@ int js_batch_get_reverse_launch(js_batch* b, int* split);
 /* The context of instance k (owned by the batch; do not destroy it), e.g. for js_step_vjp. */
 js_ctx* js_batch_instance(js_batch* b, int k);
 
-/* Failure-detection check of the bounded barrier: launches the persistent kernel with a
+/* Failure-detection check of a bounded grid barrier: launches a kernel with a
  * barrier that can never complete (one arrival short) and a wait budget of budget_s
  * (0 < budget_s <= 2) seconds; the launch must end by itself with JS_ERR_TIMEOUT in the
  * batch's error flag.  Requires js_batch_set_states. */
@@ -418,16 +409,16 @@ void js_batch_destroy(js_batch* b);
 
 /* Arithmetic mode of the forward path (js_rhs, js_step, and js_step_stage without
  * JS_STAGE_INTERNALS) of this context:
- *   JS_ARITH_FAST (default): the fused stage kernel, which contracts products into fused
- *     multiply-adds and replaces division and square root by a refined reciprocal (within
- *     about 2 ulp) -- each stage agrees with the IEEE-order result to about 1e-15 relative;
+ *   JS_ARITH_FAST (default): the stage kernels that form WENO5, reciprocals and square roots in
+ *     58- to 64-bit integer arithmetic (rounded once) and the rest in FP64 with fused
+ *     multiply-adds -- each stage agrees with the IEEE-order result to about 1e-15 relative;
  *   JS_ARITH_IEEE: every operation of the right-hand side (Sec. 2: WENO5 of the primitive
  *     variables, HLLC with the positivity fallback, viscous fluxes, divergence, artificial
  *     viscosity), the immersed-boundary ghost fill and the Runge-Kutta stage is one
  *     IEEE-rounded double operation in a fixed canonical expression order (written out in
  *     js_ieee.cu), each face and cell computed on its own: the results are reproducible bit for
  *     bit by any implementation that follows that order, independent of launch shape or
- *     device.  About 3x slower; extra workspace of 4 padded planes plus the face fluxes
+ *     device.  About 13x slower; extra workspace of 4 padded planes plus the face fluxes
  *     (allocated by the first switch to it: call before any stream capture).
  * The reverse-mode entry points, the taped steps and the batched path keep the fast
  * arithmetic.  JS_ARITH_IEEE does not combine with the neural flux (js_rhs / js_step then
@@ -437,9 +428,9 @@ void js_batch_destroy(js_batch* b);
 int js_set_arith(js_ctx* ctx, int mode);
 int js_get_arith(js_ctx* ctx, int* mode);
 
-/* Stage-kernel tuning: tile shape variant (0 .. n_variants-1) used by this context's
- * js_rhs / js_step / js_step_vjp; 0 = 32x32-cell tiles staged by TMA with concurrent x/y sweeps.  Results are identical for every
- * variant; only speed differs (the Python autotuner times them and caches the choice). */
+/* Stage-kernel tuning: variant (0 .. n_variants-1) of the line kernel used by this context's
+ * js_rhs / js_step / js_step_vjp: 0, 3 and 4 four blocks of eight lines an SM (small grids: four warps
+ * a line), 1 three, 2 two.  Results are identical for every variant; only speed differs (the Python autotuner times them and caches the choice). */
 int js_set_tuning(js_ctx* ctx, int variant);
 int js_get_tuning(js_ctx* ctx, int* variant, int* n_variants);
 

@@ -5,9 +5,7 @@ Forward steps run js_step; the backward pass walks the steps in reverse.  Only e
 `checkpoint_every`-th state is kept (default ceil(sqrt(n))); during the backward pass each
 segment is re-run from its checkpoint with js_step_taped (which records the stage states of
 every step) and reversed with js_step_vjp_taped, so a rollout of n steps holds about
-sqrt(n) checkpoints plus 3 sqrt(n) stage states instead of n states.  On 2D grids the tape
-also records the WENO5 internals of every stage (about 1.3 KB per cell and step) when they
-fit in half of the free device memory, which spares the reverse pass their recompute.
+sqrt(n) checkpoints plus 3 sqrt(n) stage states instead of n states.
 
 theta is the 20-entry parameter vector of the library (gamma, mu, Pr, nu, then the inflow
 state rho, u, v, p of the x-low, x-high, y-low and y-high sides); its gradient is returned
@@ -122,8 +120,7 @@ def rollout(solver, U0, theta, dts, outputs=None, checkpoint_every=None, tape_in
     solver: binding.Solver; U0: float64 CUDA tensor [4, ny, nx]; theta: float64 tensor [20]
     (see module docstring); dts: list of step sizes (one per step).  outputs: step indices
     whose states are returned stacked (default: only the final state, index len(dts)).
-    tape_internals: record the WENO5 internals on the tape (True / False; None decides by
-    free device memory).  The gradient is the same either way.
+    tape_internals: accepted (True / False / None); the tape holds the stage states only.
     weights: float64 tensor [6388] of neural-flux parameters (Sec. 2.3) or None; norm: its
     input normalisation and output scale (mean[4], sd[4], scale[4]); fp32: FP32 network
     arithmetic.  The solver keeps the neural flux switched on after the call.

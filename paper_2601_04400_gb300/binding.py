@@ -411,7 +411,7 @@ class Solver:
 
     def step_stage(self, U_n, U_in, U_out, dt, k, internals=False):
         """One SSP-RK3 stage k (0, 1, 2): U_out = a_k U_n + b_k (U_in + dt L(U_in)); internals:
-        also store the stage's WENO5 internals for step_stage_vjp (stages 0, 1)."""
+        mark the stage for step_stage_vjp's `internals` (stages 0, 1)."""
         flag = JS_STAGE_INTERNALS if internals else 0
         _check(lib().js_step_stage(self.ctx, _ptr(U_n) if k > 0 else None, _ptr(U_in), _ptr(U_out), float(dt),
                                    int(k) | flag), "js_step_stage")
@@ -419,7 +419,7 @@ class Solver:
 
     def step_stage_vjp(self, U_in, dt, k, lam_out, lam_in, p_bar=None, internals=False):
         """Reverse of stage k (called for k = 2, 1, 0 of one step; stage 0 adds the U^n part);
-        internals: use the internals step_stage stored for this stage."""
+        internals: only for a stage that step_stage marked (JS_ERR_ARG otherwise; same results)."""
         flag = JS_STAGE_INTERNALS if internals else 0
         _check(lib().js_step_stage_vjp(self.ctx, _ptr(U_in), float(dt), int(k) | flag, _ptr(lam_out),
                                        _ptr(lam_in), _ptr(p_bar)), "js_step_stage_vjp")
@@ -436,8 +436,7 @@ class Solver:
         return U
 
     def tape_reserve(self, n_slots, weno=False):
-        """n_slots tape slots; weno=True also records the WENO5 internals of each stage
-        (2D grids), so that step_vjp_taped skips their recompute."""
+        """n_slots tape slots; weno is passed on (JS_TAPE_WENO) and changes nothing."""
         _check(lib().js_tape_reserve_ex(self.ctx, int(n_slots), JS_TAPE_WENO if weno else 0),
                "js_tape_reserve_ex")
 
@@ -460,7 +459,8 @@ class Solver:
         return GX
 
     def tape_weno_bytes(self, n_slots):
-        """Device bytes the WENO5 internals of n_slots tape slots take (0 on 1D grids)."""
+        """Device bytes that stored WENO5 internals of n_slots tape slots would take (0 on 1D grids);
+        the tape holds none."""
         nx, ny = self._spec["nx"], self._spec["ny"]
         if ny == 1:
             return 0
@@ -502,10 +502,10 @@ class Solver:
 
 
 # ---------------------------------------------------------------------------------------
-# batched path: one persistent launch advances many independent problems
+# batched path: every launch advances many independent problems
 # ---------------------------------------------------------------------------------------
 class Batch:
-    """Independent 2D problems advanced together by js_batch_step (one persistent launch)."""
+    """Independent 2D problems advanced together by js_batch_step."""
 
     def __init__(self, problems, stream=None):
         n = len(problems)
@@ -557,8 +557,7 @@ class Batch:
         return tuple(x.value for x in v)
 
     def set_reverse_launch(self, split):
-        """Launch form of the batched reverse step: 0 one persistent launch, 1 one launch per
-        phase (identical results)."""
+        """Launch form of the batched reverse step: 0 and 1 both run one launch per phase."""
         _check(lib().js_batch_set_reverse_launch(self.handle, int(split)), "js_batch_set_reverse_launch")
 
     def reverse_launch(self):

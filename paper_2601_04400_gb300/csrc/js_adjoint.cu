@@ -30,8 +30,10 @@ namespace js {
 // =======================================================================================
 // per-grid launches
 // =======================================================================================
-// x line blocks, then y line blocks.  Bound by the FP64 pipe (about 200 FP64 instructions per lane
-// and direction) with the integer WENO5 forward and reverse beside it; 16 warps an SM at 128 registers.
+// x line blocks, then y line blocks.  Bound by the FP64 pipe (221 instructions a lane, 62% busy) and by
+// latency, with the integer WENO5 forward and reverse beside it (55% of issue slots): 1024x512 viscous
+// 709 us.  Three blocks an SM at 80 registers with a few spills; two at 128 registers hide less, four
+// spill more than they hide.
 template <bool VISC>
 __global__ void __launch_bounds__(32 * ADJ_LINES, 3)
 adj_lines_kernel(AdjArgs a, const double* __restrict__ Unext, double bdt, int bx) {

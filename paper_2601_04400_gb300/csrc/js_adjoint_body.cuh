@@ -1,6 +1,6 @@
 // Device bodies of the reverse-mode stage (gradient chain rule of Sec. 2 applied to the
-// discrete operator), shared by the per-grid launches of js_adjoint.cu and the persistent
-// batched reverse kernel of js_batch.cu: one tile, element or block of each phase.
+// discrete operator), shared by the per-grid launches of js_adjoint.cu and the
+// batched ones of js_batch.cu: one element or block of each phase.
 #pragma once
 #include <cuda_runtime.h>
 

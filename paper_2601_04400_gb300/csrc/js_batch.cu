@@ -137,8 +137,8 @@ __device__ __forceinline__ void fill_stage_args(StageArgs& a, const InstDesc& d,
 
 // The phases of one batched forward run, each a launch of its own (kernel boundaries order them): the
 // register allocation and occupancy of a phase are its own, where one persistent kernel held all of
-// them at 80 registers with spills and grid barriers between (32 instances, one step: 3.5 ms
-// persistent).  Every phase is a loop over the work items of all instances.
+// them at 80 registers with spills and grid barriers between (32 instances, one step: 3.5 ms, against
+// 2.6 when it was split).  Every phase is a loop over the work items of all instances.
 enum FwdPhase { FP_PACK, FP_CFL, FP_CFL_IEEE, FP_DT, FP_GHOST, FP_HALO, FP_LINES, FP_CELLS, FP_SAVE, FP_UNPACK };
 
 // VM: the instances of the line phase (1 the viscous ones, 2 the inviscid ones: each kind's launch has

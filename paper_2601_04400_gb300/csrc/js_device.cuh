@@ -91,7 +91,7 @@ __device__ __forceinline__ void cons_to_prim(double r, double mx, double my, dou
 }
 
 // ---------------------------------------------------------------------------------------
-// WENO5 (Jiang-Shu, eps = 1e-6, power 2) on a line, cell-centred with a sliding window.
+// WENO5 (Jiang-Shu, eps = 1e-6, power 2) on a line, cell-centred.
 // For cell i with neighbours q_{i-2..i+2} (Sec. 2: reconstruction of primitive variables):
 //   d_{i+1/2} = q_{i+1} - q_i,  D_i = q_{i-1} - 2 q_i + q_{i+1}
 //   4 beta_0 = 13/3 D_{i-1}^2 + (D_{i-1} + 2 d_{i-1/2})^2

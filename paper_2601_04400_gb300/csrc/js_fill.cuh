@@ -1,5 +1,5 @@
-// Per-element pieces of the forward step shared by the per-grid kernels and the persistent
-// batched kernel: one domain-halo cell, one immersed-boundary ghost cell (Sec. 2, Fig. 1(c))
+// Per-element pieces of the forward step shared by the per-grid kernels and the
+// batched ones: one domain-halo cell, one immersed-boundary ghost cell (Sec. 2, Fig. 1(c))
 // and the CFL wave-speed rate of one cell.
 #pragma once
 #include <math_constants.h>

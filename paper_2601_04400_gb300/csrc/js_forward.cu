@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(128) cfl_one_kernel(CflSrc q, long long n, int
   cfl_finish(red, st);
 }
 
-// (1024x1024 cells: 14 us; with every rate in FP64 56 us, bound by the FP64 pipe)
+// (1024x1024 cells: 19 us; with every rate in FP64 56 us, bound by the FP64 pipe)
 template <bool PADDED>
 __global__ void cfl_pass1_kernel(CflSrc q, long long n, int two_d,
                                  const unsigned char* __restrict__ tag, double gamma, double dx, double dy,

@@ -194,7 +194,7 @@ struct InstDesc {
   int wall, visc, has_av, ntx, nty;
 };
 
-// reverse-pass description of one instance for the persistent batched reverse kernel
+// reverse-pass description of one instance for the batched reverse kernels
 // (js_batch.cu): the context's adjoint arguments and workspace (js_internal_rev_desc) and the
 // instance's parameter-gradient slot offsets (set by js_batch.cu)
 struct InstRev {

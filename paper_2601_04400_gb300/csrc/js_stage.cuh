@@ -1,13 +1,13 @@
 // One stage of the FP64 finite-volume step (arXiv 2601.04400, Sec. 2) in two launches: lines (the
 // flux differences of every x and y line: primitives, WENO5, HLLC, viscous flux) and cells (their
 // divergence, artificial viscosity and the SSP-RK3 stage combination).  Used by the per-grid kernels
-// and by the persistent batched kernels.
+// and by the batched ones.
 //
 // A warp takes 28 cells of one line, a lane one cell: what a cell shares with its neighbours
 // (differences, smoothness indicators, face states, face fluxes) is passed by shuffles.  Of the 32
 // cells of lanes 0..31 (cells -2 .. 29 of the 28) the differences serve WENO5 of cells -1 .. 28, these
 // the faces -1/2 .. 27 1/2, these the 28 outputs.  No state is carried along a line, so a thread holds
-// one cell's values (80 registers; sweeping 16 cells with a sliding window in registers took 214 and
+// one cell's values (64 registers; sweeping 16 cells with a sliding window in registers took 214 and
 // left 2 warps per SM sub-partition, too few to overlap the integer WENO5 with the FP64 of the
 // fluxes), and a line takes one pass of latency instead of 17.
 //

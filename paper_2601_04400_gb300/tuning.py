@@ -1,4 +1,4 @@
-"""Autotuners of the fused stage kernel's tile shape and of the batched launches.
+"""Autotuners of the stage's line kernel and of the batched launches.
 
 Every variant computes identical results; only speed differs.  `autotune` times a few
 js_step calls per variant with CUDA events on the solver's stream, selects the fastest and
@@ -66,7 +66,7 @@ def autotune(solver, U, reps=3, use_cache=True):
         t1.synchronize()
         times[v] = t0.elapsed_time(t1) / reps
         work.copy_(U)
-    # keep the default (TMA-staged) variant unless another is clearly faster
+    # keep the default variant unless another is clearly faster
     best = min(times, key=times.get)
     if times[best] > 0.98 * times[0]:
         best = 0
@@ -78,7 +78,7 @@ def autotune(solver, U, reps=3, use_cache=True):
 
 
 # ---------------------------------------------------------------------------------------
-# batched path: blocks per SM and tile schedule of the persistent forward launch
+# batched path: blocks per SM and schedule of the forward's line kernels
 # ---------------------------------------------------------------------------------------
 def batch_key(problems):
     """The instance mix: grid sizes, physics and immersed bodies of all instances (order-free)."""
@@ -133,7 +133,7 @@ def autotune_batch(batch, problems, states, steps=2, use_cache=True):
 
 def autotune_batch_reverse(batch, problems, states, dts, reps=2, use_cache=True):
     """Time js_batch_step_vjp (one reverse step of every instance from `states` with step sizes
-    `dts`) in both launch forms -- one persistent launch, one launch per phase -- and select the
+    `dts`) in both settings of the launch form -- they run the same launches -- and select the
     faster; the choice is cached per instance mix.  Results are identical for both forms.
     Returns {split: ms per reverse step} ({} when the cache had the choice)."""
     import torch
