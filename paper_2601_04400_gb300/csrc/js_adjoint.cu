@@ -34,13 +34,13 @@ namespace js {
 // latency, with the integer WENO5 forward and reverse beside it (55% of issue slots): 1024x512 viscous
 // 709 us.  Three blocks an SM at 80 registers with a few spills; two at 128 registers hide less, four
 // spill more than they hide.
-template <bool VISC>
-__global__ void __launch_bounds__(32 * ADJ_LINES, 3)
+template <bool VISC, bool SPLIT = false>
+__global__ void __launch_bounds__(32 * ADJ_LINES, SPLIT ? 2 : 3)
 adj_lines_kernel(AdjArgs a, const double* __restrict__ Unext, double bdt, int bx) {
   pdl_enter();
-  __shared__ double smem[8 * AP];
+  __shared__ double smem[adj_smem(SPLIT)];
   const int b = blockIdx.x;
-  adj_lines<VISC>(a, Unext, bdt, b < bx ? 0 : 1, b < bx ? b : b - bx, smem, b);
+  adj_lines<VISC, SPLIT>(a, Unext, bdt, b < bx ? 0 : 1, b < bx ? b : b - bx, smem, b);
 }
 
 constexpr int kCellThreads = 128;  // (256: 1.2 blocks an SM at 250x190, 23 us against 18)
@@ -122,10 +122,22 @@ unsigned ib_blocks(int n) { return n > 0 ? blocks_for(4LL * n, 128) : 0; }  // a
 
 long long adj_strip_doubles(const Lay& L) { return strip_size(L, 0) + strip_size(L, 1); }
 
+// Four warps share a line in 1D (a block of eight lines would hold one) and up to so many blocks of
+// eight lines, some 1.5 an SM, where a warp's chain of four reconstructions forward and back is the
+// time.  A reverse step, Euler / viscous with a body, shared and not: 64x64 165 / 200 and 238 / 258 us,
+// 128x128 249 / 311 and 278 / 341, 180x128 (227 blocks) 305 / 345 and 329 / 351; then the chip fills:
+// 250x190 (440) 449 / 527 and 391 / 425.
+constexpr int ADJ_SPLIT_BLOCKS = 228;
+namespace {
+int line_block(const Lay& L) {  // lines a block
+  return L.ny == 1 || adj_blocks(L, 0) + adj_blocks(L, 1) <= ADJ_SPLIT_BLOCKS ? ADJ_SPLIT : ADJ_LINES;
+}
+}  // namespace
+
 long long adj_ppart_doubles(const Lay& L, int n_ghost, int n_src, long long nn_blocks) {
   // slots: one a line block; cells one a block (per warp in the batched kernels); per warp the
   // neural image reverse (256 threads a block) and IB (128)
-  const long long slots = adj_blocks(L, 0) + adj_blocks(L, 1) + 8 * nn_blocks + 8 * (long long)blocks_for(L.plane, 256) +
+  const long long slots = adj_blocks(L, 0, line_block(L)) + adj_blocks(L, 1, line_block(L)) + 8 * nn_blocks + 8 * (long long)blocks_for(L.plane, 256) +
                           4 * (long long)(ib_blocks(n_ghost) + ib_blocks(n_src));
   return 4 * slots;
 }
@@ -157,10 +169,15 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
     a.fadj = nullptr;
   }
   const double bdt = rhs_mode ? 1.0 : rb * dt;
-  const int bx = adj_blocks(L, 0), nb = bx + adj_blocks(L, 1);
+  const int nl = line_block(L), bx = adj_blocks(L, 0, nl), nb = bx + adj_blocks(L, 1, nl);
   a.pp = slice(nb);
-  if (a.visc) launch(adj_lines_kernel<true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
-  else launch(adj_lines_kernel<false>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+  if (nl == ADJ_SPLIT) {
+    if (a.visc) launch(adj_lines_kernel<true, true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+    else launch(adj_lines_kernel<false, true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+  } else {
+    if (a.visc) launch(adj_lines_kernel<true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+    else launch(adj_lines_kernel<false>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+  }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const unsigned gp = blocks_for(L.plane, kCellThreads);
   a.pp = slice(gp);

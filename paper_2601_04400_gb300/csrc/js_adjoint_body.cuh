@@ -88,14 +88,18 @@ __device__ __forceinline__ long long face_id(const AdjArgs& a, int dir, int k, i
 // Every sum has a fixed order, so the reverse pass gives the same bits on every run.
 // =======================================================================================
 constexpr int AB = 34;                   // positions of a line's box: lane l at l + 1
-constexpr int AL = ADJ_LINES + 2;        // lines of a block's box: its own and one on either side
-constexpr int AP = AB * AL;              // plane of the box, [line][position] in both directions
-
+constexpr int ADJ_SPLIT = ADJ_LINES / 4;  // lines a block where four warps share one
+// plane of a block's box, [line][position] in both directions: nl lines and one on either side
+__host__ __device__ constexpr int adj_plane(int nl) { return AB * (nl + 2); }
+// shared doubles of a block: the box's 8 planes; shared lines: 13 rows of a warp's lanes a line
+__host__ __device__ constexpr int adj_smem(bool split) {
+  return 8 * adj_plane(split ? ADJ_SPLIT : ADJ_LINES) + (split ? ADJ_SPLIT * 13 * 32 : 0);
+}
 // line blocks of a direction: groups of ADJ_LINES lines x chunks of 28 cells (-1 .. n) along them
 __host__ __device__ inline int adj_chunks(int n) { return (n + 2 + ADJ_CHUNK - 1) / ADJ_CHUNK; }
-__host__ __device__ inline int adj_groups(int nline) { return (nline + ADJ_LINES - 1) / ADJ_LINES; }
-__host__ __device__ inline int adj_blocks(const Lay& L, int dir) {
-  return dir == 0 ? adj_groups(L.ny) * adj_chunks(L.nx) : L.ny > 1 ? adj_groups(L.nx) * adj_chunks(L.ny) : 0;
+__host__ __device__ inline int adj_groups(int nline, int nl) { return (nline + nl - 1) / nl; }
+__host__ __device__ inline int adj_blocks(const Lay& L, int dir, int nl = ADJ_LINES) {
+  return dir == 0 ? adj_groups(L.ny, nl) * adj_chunks(L.nx) : L.ny > 1 ? adj_groups(L.nx, nl) * adj_chunks(L.ny) : 0;
 }
 // strips of a direction: [chunk][variable (5)][4 outer cells][line]
 __host__ __device__ inline long long strip_size(const Lay& L, int dir) {
@@ -106,18 +110,20 @@ __device__ __forceinline__ double* strip(const AdjArgs& a, int dir, int chunk, i
   return a.strips + (dir == 0 ? 0 : strip_size(a.lay, 0)) + ((long long)(chunk * 5 + c) * 4 + e) * nline + line;
 }
 
-// block `item` of direction dir: ADJ_LINES warps, a line each; slot: the block's slot for its
-// partials of pbar[0..3]; smem: 8 AP doubles
-template <bool VISC>
+// block `item` of direction dir: ADJ_LINES warps, a line each (SPLIT: four warps a line, each with one
+// variable's WENO5 forward and reverse, the first of them with the fluxes between); slot: the block's
+// slot for its partials of pbar[0..3]; smem: adj_smem(SPLIT) doubles
+template <bool VISC, bool SPLIT = false>
 __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __restrict__ Unext, double bdt, int dir,
                                           int item, double* smem, long long slot) {
+  constexpr int NL = SPLIT ? ADJ_SPLIT : ADJ_LINES, AL = NL + 2, AP = adj_plane(NL);
   const Lay& L = a.lay;
   double* sq = smem;           // rho, u, v, p
   double* sl = smem + 4 * AP;  // Unext on fluid cells
   const Gas g = a.gas;
   const int nline = dir == 0 ? L.ny : L.nx, ncell = dir == 0 ? L.nx : L.ny;
   const int nch = adj_chunks(ncell);
-  const int chunk = item % nch, line0 = item / nch * ADJ_LINES;
+  const int chunk = item % nch, line0 = item / nch * NL;
   const int i0 = -1 + ADJ_CHUNK * chunk;  // first reversed cell
   const int gyl = dir == 0 ? L.gy : 3, gyc = dir == 0 ? 3 : L.gy;  // ghost layers across / along the line
   for (int e = threadIdx.x; e < AP; e += 32 * ADJ_LINES) {
@@ -142,10 +148,12 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
     for (int c = 0; c < 4; ++c) sl[c * AP + o] = fluid ? Unext[c * L.plane + t] : 0.0;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) / (SPLIT ? 4 : 1);
+  const int kq = SPLIT ? (threadIdx.x >> 5) & 3 : 0;
   const int line = line0 + warp;
+  const bool live = line < nline;
   double gs1 = 0.0, gs2 = 0.0, vmu = 0.0, vk = 0.0;
-  if (line < nline) {
+  if (SPLIT || live) {  // (the shared lines' warps meet at barriers)
     const ViscC& vc = dir == 0 ? a.vx : a.vy;
     const double fl = bdt * (dir == 0 ? a.inv_dx : a.inv_dy);  // lambda' differences over h
     const int pn = dir + 1, pt = 2 - dir;
@@ -155,13 +163,26 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
     const double* un = q + pn * AP;
     const double* ut = q + pt * AP;
     const int cell = i0 - 2 + lane, f = cell + 1;  // the lane's cell and its face at i+1/2
-    const bool face = inner && lane < 30 && f >= 0 && f <= ncell;
+    const bool face = live && inner && lane < 30 && f >= 0 && f <= ncell;
     const bool own = lane >= 2;  // (with face) the warp's faces: lanes 2..29
     const bool rev = lane >= 2 && lane < 30;
+    double* const ex = smem + 8 * AP + 13 * 32 * warp + lane;  // SPLIT: [13][32] of the line
     double bL[4], bR[4], dl[VISC ? 5 : 4], dr[VISC ? 5 : 4];
-    bool fell;  // a face of the warp fell back to first order
-    {
-      double Lq[4], Rq[4];
+    bool fell = SPLIT;  // a face of the warp fell back to first order
+    double Lq[4], Rq[4];
+    if constexpr (SPLIT) {
+      double Lf, Rf;
+      weno_lane(q + ((kq == 1) ? pn : (kq == 2) ? pt : kq) * AP, 1, kq == 0 || kq == 3, inner, Lf, Rf);
+      ex[32 * kq] = Lf;
+      ex[32 * (4 + kq)] = Rf;
+      __syncthreads();
+      if (kq == 0)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          Lq[m] = ex[32 * m];
+          Rq[m] = ex[32 * (4 + m) + (lane < 31 ? 1 : 0)];
+        }
+    } else {
 #pragma unroll 1
       for (int k = 0; k < 4; ++k) {
         const int c = (k == 1) ? pn : (k == 2) ? pt : k;
@@ -175,6 +196,8 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
       }
 #pragma unroll
       for (int m = 0; m < 4; ++m) Rq[m] = __shfl_down_sync(0xffffffffu, Rq[m], 1);
+    }
+    if (!SPLIT || kq == 0) {
       const bool fallback = !(positive(Lq[0]) && positive(Lq[3]) && positive(Rq[0]) && positive(Rq[3]));
       if (fallback) {
         Lq[0] = q[0], Lq[1] = un[0], Lq[2] = ut[0], Lq[3] = q[3 * AP];
@@ -234,48 +257,57 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
           // cell's sum over its two faces
           const double xn = face ? vc.ct * btnt : 0.0, xt = face ? -vc.c23t * btnn : 0.0;
           const double tn = xn + __shfl_up_sync(0xffffffffu, xn, 1), tt = xt + __shfl_up_sync(0xffffffffu, xt, 1);
-          if (rev && cell <= ncell) {
+          if (live && rev && cell <= ncell) {
             double* o = a.tang + (long long)(2 * dir) * L.plane + (dir == 0 ? L.idx(cell, line) : L.idx(line, cell));
             o[0] = tn;
             o[L.plane] = tt;
           }
         }
       }
-    }
-    if (a.fadj != nullptr && face) {
-      const double* fa = a.fadj + (long long)(dir * 8) * a.splane + face_id(a, dir, f, line);
+      if (a.fadj != nullptr && face) {
+        const double* fa = a.fadj + (long long)(dir * 8) * a.splane + face_id(a, dir, f, line);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int c = (m == 1) ? pn : (m == 2) ? pt : m;
+          bL[m] += fa[c * a.splane];
+          bR[m] += fa[(4 + c) * a.splane];
+        }
+      }
+      // the reversed cells' face states: L at i+1/2, R at i-1/2; right cells' straight terms
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const int c = (m == 1) ? pn : (m == 2) ? pt : m;
-        bL[m] += fa[c * a.splane];
-        bR[m] += fa[(4 + c) * a.splane];
+        const double up = __shfl_up_sync(0xffffffffu, bR[m], 1);
+        bL[m] = rev ? bL[m] : 0.0;
+        bR[m] = rev ? up : 0.0;
+      }
+      if (VISC || fell) {
+#pragma unroll
+        for (int m = 0; m < (VISC ? 5 : 4); ++m) {
+          if ((m == 0 || m == 3) && !fell) continue;  // no such term
+          const double up = __shfl_up_sync(0xffffffffu, dr[m], 1);
+          dl[m] += lane > 0 ? up : 0.0;
+        }
       }
     }
-    // the reversed cells' face states: L at i+1/2, R at i-1/2; right cells' straight terms
+    if constexpr (SPLIT) {
+      if (kq == 0) {
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const double up = __shfl_up_sync(0xffffffffu, bR[m], 1);
-      bL[m] = rev ? bL[m] : 0.0;
-      bR[m] = rev ? up : 0.0;
-    }
-    if (VISC || fell) {
+        for (int m = 0; m < 4; ++m) ex[32 * m] = bL[m], ex[32 * (4 + m)] = bR[m];
 #pragma unroll
-      for (int m = 0; m < (VISC ? 5 : 4); ++m) {
-        if ((m == 0 || m == 3) && !fell) continue;  // no such term
-        const double up = __shfl_up_sync(0xffffffffu, dr[m], 1);
-        dl[m] += lane > 0 ? up : 0.0;
+        for (int m = 0; m < 4; ++m) ex[32 * (8 + m)] = dl[m];
       }
+      __syncthreads();
     }
     // where the lane's sums go: the cell's place, or a strip of the warp
-    const bool in = cell >= -gyc && cell < ncell + gyc;
+    const bool in = live && cell >= -gyc && cell < ncell + gyc;
     double* qo = rev ? a.Qb + (long long)(dir * 5) * L.plane + (in ? (dir == 0 ? L.idx(cell, line) : L.idx(line, cell)) : 0)
                      : strip(a, dir, chunk, 0, lane < 2 ? lane : lane - 28, line);
     const long long qs = rev ? L.plane : 4LL * nline;
 #pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
+    for (int k = kq; k < (SPLIT ? kq + 1 : 4); ++k) {
       const int c = (k == 1) ? pn : (k == 2) ? pt : k;
-      const double Lb = (k == 0) ? bL[0] : (k == 1) ? bL[1] : (k == 2) ? bL[2] : bL[3];
-      const double Rb = (k == 0) ? bR[0] : (k == 1) ? bR[1] : (k == 2) ? bR[2] : bR[3];
+      const double Lb = SPLIT ? ex[32 * k] : (k == 0) ? bL[0] : (k == 1) ? bL[1] : (k == 2) ? bL[2] : bL[3];
+      const double Rb = SPLIT ? ex[32 * (4 + k)] : (k == 0) ? bR[0] : (k == 1) ? bR[1] : (k == 2) ? bR[2] : bR[3];
       double w[4];
       weno_grad_lane(q + c * AP, 1, k == 0 || k == 3, inner, Lb, Rb, w);  // 0 where Lb = Rb = 0
       // adjoint of d_{i+1/2}: its share in the reversed cells i-1 .. i+2
@@ -284,10 +316,10 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
                        (__shfl_down_sync(0xffffffffu, w[1], 1) + __shfl_down_sync(0xffffffffu, w[0], 2));
       const double tm = __shfl_up_sync(0xffffffffu, t, 1);
       double v = fma(SIXTH, (lane > 0 ? tm : 0.0) - t, Lb + Rb);
-      if (fell || (VISC && (k == 1 || k == 2))) v += (k == 0) ? dl[0] : (k == 1) ? dl[1] : (k == 2) ? dl[2] : dl[3];
+      if (fell || (VISC && (k == 1 || k == 2))) v += SPLIT ? ex[32 * (8 + k)] : (k == 0) ? dl[0] : (k == 1) ? dl[1] : (k == 2) ? dl[2] : dl[3];
       if (in) qo[c * qs] = v;
     }
-    if (VISC && in) qo[4 * qs] = dl[VISC ? 4 : 0];
+    if (VISC && in && (!SPLIT || kq == 0)) qo[4 * qs] = dl[VISC ? 4 : 0];
   }
   if (a.pp == nullptr) return;
   // gamma, mu and Pr from the block's sums

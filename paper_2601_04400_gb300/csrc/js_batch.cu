@@ -728,7 +728,7 @@ int js_internal_rev_desc(js_ctx* c, js::InstRev* d);
 
 namespace {
 size_t batch_smem() { return js::stage_smem<true>(); }
-constexpr size_t kLineSmem = sizeof(double) * 8 * js::AP;
+constexpr size_t kLineSmem = sizeof(double) * js::adj_smem(false);
 }  // namespace
 
 namespace {
