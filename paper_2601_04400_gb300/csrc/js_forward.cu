@@ -500,8 +500,9 @@ cudaError_t launch_cfl_init(unsigned long long* red, cudaStream_t s) {
 }
 
 // Cells up to which every rate is taken in IEEE arithmetic at once: one launch in place of two, each of
-// which is latency on such grids.  A step of 128x64 cells takes 89 us with one launch and 95 with two,
-// of 256x128 116 and 120; from there the FP64 pipe decides: 256x256 155 and 153, 400x320 222 and 216.
+// which is latency on such grids.  A step of 128x64 cells took 89 us with one launch and 95 with two,
+// of 256x128 116 and 120; from there the FP64 pipe decides: 256x256 155 and 153, 400x320 222 and 216
+// (before the launches overlapped).
 constexpr long long CFL_ONE_CELLS = 32768;
 
 namespace {

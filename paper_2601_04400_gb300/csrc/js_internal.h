@@ -10,7 +10,7 @@ namespace js {
 // kernels that small grids are: its blocks start as the predecessor's last ones leave and wait in
 // pdl_enter, the first statement of every kernel launched this way, until the predecessor has
 // completed and its writes are visible.  128x64 cylinder, 13 launches a step: 101 us a step with plain
-// launches, 73 so.  The predecessor does not release its successor early: waiting blocks would crowd
+// launches and 73 so when it was introduced (61 since).  The predecessor does not release its successor early: waiting blocks would crowd
 // on the SMs that are free while it still runs (128x96 training step: 4.2 ms, 6.8 released early, 5.2
 // with plain launches).
 __device__ __forceinline__ void pdl_enter() { cudaGridDependencySynchronize(); }
