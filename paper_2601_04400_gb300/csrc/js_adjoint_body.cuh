@@ -484,50 +484,57 @@ __device__ __forceinline__ void adj_bcT_one(const AdjArgs& a, const BcArgs& bc, 
 
 // inflow halo adjoints (conserved) -> gradient of the inflow primitive state and gamma; one
 // warp per side sums its partials in a fixed order, then one thread adds to pbar side by side
-__device__ __forceinline__ void adj_inflow_block(const AdjArgs& a, const BcArgs& bc, const double* inflow_part,
-                                                 int tmax, const double* inflow_prim) {
-  __shared__ double S[4][4];
-  const int side = threadIdx.x >> 5, lane = threadIdx.x & 31;  // (at least four warps)
+// S[side] = the sums of a side's inflow halo adjoints (warp `side` of the first four)
+__device__ __forceinline__ void adj_inflow_sums(const AdjArgs& a, const BcArgs& bc, const double* inflow_part, int tmax,
+                                                double S[4][4]) {
+  const int side = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Lay& L = a.lay;
-  if (side < 4 && bc.kind[side] == 3 && a.pbar != nullptr) {
+  if (side < 4 && bc.kind[side] == 3) {
     const int ntan = (side < 2) ? L.ny : L.nx + 6;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 4
     for (int k = lane; k < ntan; k += 32)
 #pragma unroll
       for (int c = 0; c < 4; ++c) v[c] += inflow_part[((long long)side * tmax + k) * 4 + c];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = warp_sum(v[c]);
-    if (lane == 0)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) S[side][c] = v[c];
+    const double t = warp_sum4(v[0], v[1], v[2], v[3]);
+    if ((lane & 7) == 0) S[side][lane >> 3] = t;
   }
+}
+// the inflow states' gradient, a thread (of the first 16) per side and parameter, from
+// U = (r, r u, r v, p/(gamma-1) + r (u^2 + v^2)/2)
+__device__ __forceinline__ void adj_inflow_states(const AdjArgs& a, const BcArgs& bc, const double* inflow_prim,
+                                                  const double S[4][4]) {
+  if (threadIdx.x >= 16 || bc.kind[threadIdx.x >> 2] != 3) return;
+  const int sd = threadIdx.x >> 2, m = threadIdx.x & 3;
+  const double* s = S[sd];
+  const double r = inflow_prim[4 * sd], u = inflow_prim[4 * sd + 1], v = inflow_prim[4 * sd + 2];
+  a.pbar[4 + 4 * sd + m] += pick4(m, s[0] + s[1] * u + s[2] * v + s[3] * 0.5 * (u * u + v * v), s[1] * r + s[3] * r * u,
+                                  s[2] * r + s[3] * r * v, s[3] * a.gas.g1);
+}
+// and their part of gamma's
+__device__ __forceinline__ double adj_inflow_gamma(const AdjArgs& a, const BcArgs& bc, const double* inflow_prim,
+                                                   const double S[4][4]) {
+  double g = 0.0;
+  for (int sd = 0; sd < 4; ++sd)
+    if (bc.kind[sd] == 3) g += -S[sd][3] * inflow_prim[4 * sd + 3] * a.gas.g1 * a.gas.g1;
+  return g;
+}
+__device__ __forceinline__ void adj_inflow_block(const AdjArgs& a, const BcArgs& bc, const double* inflow_part,
+                                                 int tmax, const double* inflow_prim) {
+  __shared__ double S[4][4];
+  if (a.pbar != nullptr) adj_inflow_sums(a, bc, inflow_part, tmax, S);
   __syncthreads();
   if (a.pbar == nullptr) return;
-  // U = (r, r u, r v, p/(gamma-1) + r (u^2 + v^2)/2): a thread per side and parameter
-  if (threadIdx.x < 16 && bc.kind[threadIdx.x >> 2] == 3) {
-    const int sd = threadIdx.x >> 2, m = threadIdx.x & 3;
-    const double* s = S[sd];
-    const double r = inflow_prim[4 * sd], u = inflow_prim[4 * sd + 1], v = inflow_prim[4 * sd + 2];
-    const double e = pick4(m, s[0] + s[1] * u + s[2] * v + s[3] * 0.5 * (u * u + v * v), s[1] * r + s[3] * r * u,
-                           s[2] * r + s[3] * r * v, s[3] * a.gas.g1);
-    a.pbar[4 + 4 * sd + m] += e;
-  }
-  if (threadIdx.x == 32) {
-    double g = a.pbar[0];
-    for (int sd = 0; sd < 4; ++sd)
-      if (bc.kind[sd] == 3) g += -S[sd][3] * inflow_prim[4 * sd + 3] * a.gas.g1 * a.gas.g1;
-    a.pbar[0] = g;
-  }
+  adj_inflow_states(a, bc, inflow_prim, S);
+  if (threadIdx.x == 32) a.pbar[0] += adj_inflow_gamma(a, bc, inflow_prim, S);
 }
 
 // pbar[0..3] += the warp partials pp[4 * b + k] of the slot ranges [off[r], off[r] + cnt[r]),
 // r < nr: each thread over a fixed set of slots, then a fixed reduction tree over the block
 // (blockDim.x a power of two, at most 256)
-template <int NT = 256>
 __device__ __forceinline__ void adj_pbar_reduce_block(const double* __restrict__ pp, const long long* off,
                                                       const long long* cnt, int nr, double* pbar) {
-  __shared__ double red[4][NT];
+  __shared__ double red[4][256];
   const int nt = blockDim.x;
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   for (int r = 0; r < nr; ++r)
