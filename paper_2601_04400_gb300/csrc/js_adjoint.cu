@@ -32,10 +32,9 @@ namespace js {
 // =======================================================================================
 // x line blocks, then y line blocks.  Bound by the FP64 pipe (221 instructions a lane, 62% busy) and by
 // latency, with the integer WENO5 forward and reverse beside it (55% of issue slots): 1024x512 viscous
-// 709 us.  Three blocks an SM at 80 registers with a few spills; two at 128 registers hide less, four
-// spill more than they hide.
-template <bool VISC, bool SPLIT = false>
-__global__ void __launch_bounds__(32 * ADJ_LINES, SPLIT ? 2 : 3)
+// 709 us at B = 3 blocks an SM.  B: the resident blocks the registers are allotted for (ADJ_THREE_BLOCKS).
+template <bool VISC, bool SPLIT, int B>
+__global__ void __launch_bounds__(32 * ADJ_LINES, B)
 adj_lines_kernel(AdjArgs a, const double* __restrict__ Unext, double bdt, int bx) {
   pdl_enter();
   __shared__ double smem[adj_smem(SPLIT)];
@@ -190,11 +189,14 @@ cudaError_t launch_adj_stage(const AdjArgs& a0, const BcArgs& bc, const IbArgs& 
   const int nl = line_block(L), bx = adj_blocks(L, 0, nl), nb = bx + adj_blocks(L, 1, nl);
   a.pp = slice(nb);
   if (nl == ADJ_SPLIT) {
-    if (a.visc) launch(adj_lines_kernel<true, true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
-    else launch(adj_lines_kernel<false, true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+    if (a.visc) launch(adj_lines_kernel<true, true, 2>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+    else launch(adj_lines_kernel<false, true, 2>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+  } else if (nb <= ADJ_THREE_BLOCKS) {
+    if (a.visc) launch(adj_lines_kernel<true, false, 3>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+    else launch(adj_lines_kernel<false, false, 3>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
   } else {
-    if (a.visc) launch(adj_lines_kernel<true>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
-    else launch(adj_lines_kernel<false>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+    if (a.visc) launch(adj_lines_kernel<true, false, 4>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
+    else launch(adj_lines_kernel<false, false, 4>, nb, 32 * ADJ_LINES, 0, s, a, Unext, bdt, bx);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const unsigned gp = blocks_for(L.plane, kCellThreads);

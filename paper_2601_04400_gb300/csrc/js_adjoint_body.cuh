@@ -101,6 +101,12 @@ __host__ __device__ inline int adj_groups(int nline, int nl) { return (nline + n
 __host__ __device__ inline int adj_blocks(const Lay& L, int dir, int nl = ADJ_LINES) {
   return dir == 0 ? adj_groups(L.ny, nl) * adj_chunks(L.nx) : L.ny > 1 ? adj_groups(L.nx, nl) * adj_chunks(L.ny) : 0;
 }
+// Blocks of eight lines that three an SM hold at once.  Up to here the line kernels take 80 registers
+// (three blocks an SM), above 64 with more spills (four).  A reverse step with four and with three, Euler /
+// viscous with a body: 256x200 (450 blocks) 462 / 490 and 424 / 499 us, 300x200 (579) 475 / 499 and 483 /
+// 511, 512x512 1358 / 1545 and 1367 / 1572, 900x600 2576 / 2944 and 2589 / 3008; 16 instances 5.30 and
+// 5.42 ms.  Two blocks (128 registers, no spills): 512x512 viscous 1681.
+constexpr int ADJ_THREE_BLOCKS = 456;
 // strips of a direction: [chunk][variable (5)][4 outer cells][line]
 __host__ __device__ inline long long strip_size(const Lay& L, int dir) {
   return dir == 0 ? 20LL * adj_chunks(L.nx) * L.ny : L.ny > 1 ? 20LL * adj_chunks(L.ny) * L.nx : 0;

@@ -649,8 +649,8 @@ __device__ __forceinline__ void rev_phase(const BatchRevArgs& b, int s, double* 
 }
 
 // one phase of the reverse step
-template <int PH, int VM = 0>
-__global__ void __launch_bounds__(BNT, PH == RP_STAGE ? 4 : PH == RP_LINES ? 3 : PH == RP_CELLS ? 4 : 1) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
+template <int PH, int VM = 0, int B = PH == RP_STAGE || PH == RP_CELLS ? 4 : PH == RP_LINES ? 3 : 1>
+__global__ void __launch_bounds__(BNT, B) batch_vjp_phase_kernel(BatchRevArgs b, int s) {
   pdl_enter();
   extern __shared__ double smem[];
   rev_phase<PH, VM>(b, s, smem);
@@ -838,8 +838,12 @@ int rev_launch(js_batch* b, const js::RevCall& call) {
   }
   for (int s = 2; s >= 0; --s) {
     if (s < 2 && call.pbar) run(js::batch_vjp_phase_kernel<js::RP_REDUCE>, js::RP_REDUCE, s);
-    run_lines(js::batch_vjp_phase_kernel<js::RP_LINES, 1>, js::batch_vjp_phase_kernel<js::RP_LINES, 2>,
-              b->rblock0.back(), kLineSmem, s);
+    if (b->rblock0.back() <= js::ADJ_THREE_BLOCKS)
+      run_lines(js::batch_vjp_phase_kernel<js::RP_LINES, 1>, js::batch_vjp_phase_kernel<js::RP_LINES, 2>,
+                b->rblock0.back(), kLineSmem, s);
+    else
+      run_lines(js::batch_vjp_phase_kernel<js::RP_LINES, 1, 4>, js::batch_vjp_phase_kernel<js::RP_LINES, 2, 4>,
+                b->rblock0.back(), kLineSmem, s);
     run(js::batch_vjp_phase_kernel<js::RP_CELLS>, js::RP_CELLS, s);
     run(js::batch_vjp_phase_kernel<js::RP_BCTY>, js::RP_BCTY, s);
     run(js::batch_vjp_phase_kernel<js::RP_BCTX>, js::RP_BCTX, s);
