@@ -135,8 +135,9 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
   for (int e = threadIdx.x; e < AP; e += 32 * ADJ_LINES) {
     // consecutive threads along x in both directions
     const int ln = dir == 0 ? e / AB : e % AL, pos = dir == 0 ? e % AB : e / AL;
-    const int line = line0 - 1 + ln, cell = i0 - 3 + pos;
-    const bool in = line >= -gyl && line < nline + gyl && cell >= -gyc && cell < ncell + gyc;
+    // past the array a line goes on with its outer cell's state (as in the stage kernel)
+    const int line = line0 - 1 + ln, cell = imax(imin(i0 - 3 + pos, ncell + gyc - 1), -gyc);
+    const bool in = line >= -gyl && line < nline + gyl;
     const int i = dir == 0 ? cell : line, j = dir == 0 ? line : cell;
     const long long t = in ? L.idx(i, j) : 0;
     double r = 1.0, u = 0.0, v = 0.0, p = 1.0, T;
@@ -178,7 +179,7 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
     double Lq[4], Rq[4];
     if constexpr (SPLIT) {
       double Lf, Rf;
-      weno_lane(q + ((kq == 1) ? pn : (kq == 2) ? pt : kq) * AP, 1, kq == 0 || kq == 3, inner, Lf, Rf);
+      weno_lane(q + ((kq == 1) ? pn : (kq == 2) ? pt : kq) * AP, 1, inner, Lf, Rf);
       ex[32 * kq] = Lf;
       ex[32 * (4 + kq)] = Rf;
       __syncthreads();
@@ -193,7 +194,7 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
       for (int k = 0; k < 4; ++k) {
         const int c = (k == 1) ? pn : (k == 2) ? pt : k;
         double Lf, Rf;
-        weno_lane(q + c * AP, 1, k == 0 || k == 3, inner, Lf, Rf);
+        weno_lane(q + c * AP, 1, inner, Lf, Rf);
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
           Lq[m] = (k == m) ? Lf : Lq[m];
@@ -315,7 +316,7 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
       const double Lb = SPLIT ? ex[32 * k] : (k == 0) ? bL[0] : (k == 1) ? bL[1] : (k == 2) ? bL[2] : bL[3];
       const double Rb = SPLIT ? ex[32 * (4 + k)] : (k == 0) ? bR[0] : (k == 1) ? bR[1] : (k == 2) ? bR[2] : bR[3];
       double w[4];
-      weno_grad_lane(q + c * AP, 1, k == 0 || k == 3, inner, Lb, Rb, w);  // 0 where Lb = Rb = 0
+      weno_grad_lane(q + c * AP, 1, inner, Lb, Rb, w);  // 0 where Lb = Rb = 0
       // adjoint of d_{i+1/2}: its share in the reversed cells i-1 .. i+2
       const double u3 = __shfl_up_sync(0xffffffffu, w[3], 1);
       const double t = (w[2] + (lane > 0 ? u3 : 0.0)) +

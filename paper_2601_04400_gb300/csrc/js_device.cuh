@@ -142,10 +142,6 @@ static __device__ __noinline__ double2 weno_plain(double qm2, double qm1, double
   return make_double2(fma(quot(nL, w0 + w6 + w2_3), SIXTH, q0), fma(quot(nR, w0_3 + w6 + w2), SIXTH, q0));
 }
 
-// the largest exponent of a stencil's differences up to which the integer form serves
-// (js_weno.cuh); e: the cell value's exponent, pos: the variable is positive (density, pressure)
-__device__ __forceinline__ int weno_limit(int e, bool pos) { return pos ? imin(e + 3, 1500) : 1500; }
-
 __device__ __forceinline__ Sm shfl_up(const Sm& s) {
   return Sm{(u64)__shfl_up_sync(0xffffffffu, (unsigned long long)s.m, 1), __shfl_up_sync(0xffffffffu, s.x, 1)};
 }
@@ -164,39 +160,39 @@ __device__ __forceinline__ Fx shfl_down(const Fx& d) {
 // readable; q[-2 st], q[2 st] too in the inner lanes 1..30, where the result is valid).  A lane
 // forms the differences on both sides of its cell and the three indicators they determine, and
 // takes its s_0, s_2 and outer differences from its neighbours.
-__device__ __forceinline__ void weno_lane(const double* q, int st, bool pos, bool inner, double& Lf, double& Rf) {
+__device__ __forceinline__ void weno_lane(const double* q, int st, bool inner, double& Lf, double& Rf) {
   const Qx x = qx_of(q[0]);
   const Fx dm1 = fx_of(x, qx_of(q[-st])), dp1 = fx_of(qx_of(q[st]), x);
   Sm s1, s0n, s2p;
   sm_pair(dm1, dp1, s1, s0n, s2p);
   const Sm s0 = shfl_up(s0n), s2 = shfl_down(s2p);
   const Fx dm2 = shfl_up(dm1), dp2 = shfl_down(dp1);
-  const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
-  if (F > weno_limit(x.e, pos) && inner) {
+  const int EL = imax(dm2.e, dm1.e), EM = imax(dm1.e, dp1.e), ER = imax(dp1.e, dp2.e), F = imax(EL, ER);
+  if (F > 1500 && inner) {
     const double2 r = weno_plain(q[-2 * st], q[-st], q[0], q[st], q[2 * st]);
     Lf = r.x;
     Rf = r.y;
   } else {
-    weno_faces(x, dm2, dm1, dp1, dp2, s0, s1, s2, F, Lf, Rf);
+    weno_faces(x, dm2, dm1, dp1, dp2, s0, s1, s2, F, Lf, Rf, weno_fits(x, EL, EM, ER, F));
   }
 }
 
 // the same for a single thread (q[-2 st .. 2 st] readable): the same bits
 template <class I>
-__device__ __forceinline__ void weno_cell(const double* q, I st, bool pos, double& Lf, double& Rf) {
+__device__ __forceinline__ void weno_cell(const double* q, I st, double& Lf, double& Rf) {
   const Qx m2 = qx_of(q[-2 * st]), m1 = qx_of(q[-st]), x = qx_of(q[0]), p1 = qx_of(q[st]), p2 = qx_of(q[2 * st]);
   const Fx dm2 = fx_of(m1, m2), dm1 = fx_of(x, m1), dp1 = fx_of(p1, x), dp2 = fx_of(p2, p1);
   Sm s0, s1, s2, u, v;
   sm_pair(dm2, dm1, u, s0, v);
   sm_pair(dp1, dp2, u, v, s2);
   sm_pair(dm1, dp1, s1, u, v);
-  const int F = imax(imax(dm2.e, dm1.e), imax(dp1.e, dp2.e));
-  if (F > weno_limit(x.e, pos)) {
+  const int EL = imax(dm2.e, dm1.e), EM = imax(dm1.e, dp1.e), ER = imax(dp1.e, dp2.e), F = imax(EL, ER);
+  if (F > 1500) {
     const double2 r = weno_plain(q[-2 * st], q[-st], q[0], q[st], q[2 * st]);
     Lf = r.x;
     Rf = r.y;
   } else {
-    weno_faces(x, dm2, dm1, dp1, dp2, s0, s1, s2, F, Lf, Rf);
+    weno_faces(x, dm2, dm1, dp1, dp2, s0, s1, s2, F, Lf, Rf, weno_fits(x, EL, EM, ER, F));
   }
 }
 

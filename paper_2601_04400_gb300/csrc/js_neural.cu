@@ -97,8 +97,8 @@ __device__ __forceinline__ void face_states(const Lay& L, const double* Q, long 
 #pragma unroll 1
   for (int c = 0; c < 4; ++c) {
     double l, r, unused;
-    weno_cell(q + c * qplane - st, st, c == 0 || c == 3, l, unused);
-    weno_cell(q + c * qplane, st, c == 0 || c == 3, unused, r);
+    weno_cell(q + c * qplane - st, st, l, unused);
+    weno_cell(q + c * qplane, st, unused, r);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       wl[m] = (c == m) ? l : wl[m];

@@ -56,7 +56,7 @@ __device__ __forceinline__ bool line_fluxes(const double* q, int ps, int ts, int
   if (fb != nullptr) {
     const int k = (threadIdx.x >> 5) & 3;
     double Lf, Rf;
-    weno_lane(q + ((k == 1) ? pn : (k == 2) ? pt : k) * ps, st, k == 0 || k == 3, inner, Lf, Rf);
+    weno_lane(q + ((k == 1) ? pn : (k == 2) ? pt : k) * ps, st, inner, Lf, Rf);
     fb[32 * k + lane] = Lf;
     fb[32 * (4 + k) + lane] = Rf;
     __syncthreads();
@@ -71,7 +71,7 @@ __device__ __forceinline__ bool line_fluxes(const double* q, int ps, int ts, int
     for (int k = 0; k < 4; ++k) {
       const int c = (k == 1) ? pn : (k == 2) ? pt : k;
       double Lf, Rf;
-      weno_lane(q + c * ps, st, k == 0 || k == 3, inner, Lf, Rf);
+      weno_lane(q + c * ps, st, inner, Lf, Rf);
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         L[m] = (k == m) ? Lf : L[m];
@@ -174,9 +174,10 @@ __device__ __forceinline__ void stage_lines(const StageArgs& a, int dir, int ite
     // consecutive threads along x in both directions
     const int ln = dir == 0 ? e / SB : e % SL, pos = dir == 0 ? e % SB : e / SL;
     if (!VISC && (ln == 0 || ln == SL - 1)) continue;  // lines beside the block's own serve the viscous terms
-    const int line = line0 - 1 + ln, cell = i0 - 3 + pos;
-    // cells past the array get a uniform state (they feed only cells that are not written)
-    const bool in = line >= -gyl && line < nline + gyl && cell < ncell + gyc;
+    const int line = line0 - 1 + ln, cell = imin(i0 - 3 + pos, ncell + gyc - 1);
+    // past the array a line goes on with its last cell's state and the lines beyond hold a uniform one (they
+    // feed only cells that are not written; a jump there would part the warp in weno_faces)
+    const bool in = line >= -gyl && line < nline + gyl;
     double r = 1.0, u = 0.0, v = 0.0, p = 1.0, T = 1.0;
     if (in) {
       const long long t = dir == 0 ? L.idx(cell, line) : L.idx(line, cell);
