@@ -170,9 +170,10 @@ JS_HD void weno_faces(const Qx& q0, const Fx& dm2, const Fx& dm1, const Fx& dp1,
 // Z_k is formed from the pairs, Z_0 = om_0 om_1 (e_0 - e_1) + om_0 om_2 (e_0 - e_2) and so on,
 // which keeps it accurate where one weight is nearly 1 and e_k - c nearly 0; the differences of
 // candidates are multiples of the third differences T_0 = a - 2 b + c, T_1 = b - 2 c + d.  Every
-// factor carries its own exponent to the end; the eight results are rounded from a common scale
-// of 2^-56 (they stay below 2^4).  Errors against 128-bit arithmetic: 1e-16 rms, 4 to 6 times below
-// those of the FP64 formulas.
+// factor carries its own exponent to the end and each result is rounded from the scale of its own
+// weights, so that the derivatives of 1e-12 and less beside a jump are as accurate as the large ones.
+// Errors against 128-bit arithmetic: 1e-16 rms, 4 to 6 times below those of the FP64 formulas; in units
+// of 2^-53 of the terms' sum at most 12, FP64 16 (jumps, noise, scattered and smooth stencils).
 // ---------------------------------------------------------------------------------------
 // half the logarithmic derivatives of one indicator with respect to its pair: V = m 2^(960 + k)
 struct Lv {
@@ -232,15 +233,10 @@ JS_HD GradCell grad_cell(const Fx& dm2, const Fx& dm1, const Fx& dp1, const Fx& 
 // o[0..3] = dc/d(a, b, c, d) of the right-biased (right) or left-biased side.  One code copy for both
 // (inlined twice and interleaved they take more registers than two blocks an SM leave).
 JS_HD void weno_grad_side(const GradCell& q, bool right, double o[4]) {
-  constexpr int CF = 56;
   const Wgt& g = q.g;
-  const s64 c0 = (right ? 3 : 1) * g.w0, c1 = 6 * g.w1, c2 = (right ? 1 : 3) * g.w2;
-  const u64 den = (u64)(c0 + c1 + c2);
+  const u64 den = (u64)((right ? 3 : 1) * g.w0 + 6 * g.w1 + (right ? 1 : 3) * g.w2);
   const int lz = clz32(hi32(den));
   const u64 r = recip_top(den << lz);
-  const Limb rl = limbs((s64)r);
-  // om_k 2^CF
-  const s64 o0 = sar(mul62(limbs(c0), rl), 7 - lz), o1 = sar(mul62(limbs(c1), rl), 7 - lz), o2 = sar(mul62(limbs(c2), rl), 7 - lz);
   // products of two weights, with their linear weights' product as 3 or 9 times a power of two
   const u64 r4 = r << 2;
   const u64 q0 = mul_top(q.N0.m, r4), q1 = mul_top(q.N1.m, r4), q2 = mul_top(q.N2.m, r4);
@@ -253,21 +249,27 @@ JS_HD void weno_grad_side(const GradCell& q, bool right, double o[4]) {
   const int m0 = 2 * g.n0 - q.N0.x, m1 = 2 * g.n1 - q.N1.x, m2 = 2 * g.n2 - q.N2.x;  // n_k + lz_k
   const int f = right ? 1 : 0;
   const int h01 = m0 + m1 + q.t0.l - (2 + f), h02 = m0 + m2 + t02.l, h12 = m1 + m2 + q.t1.l - (3 - f);
-  const int nu = imin(imin(h01, h02), h12);
-  const s64 z01 = sar(mul62(limbs(K01), limbs(E01)), h01 - nu), z02 = sar(mul62(limbs(K02), limbs(t02.m)), h02 - nu),
-            z12 = sar(mul62(limbs(K12), limbs(E12)), h12 - nu);
-  const Limb Z0 = limbs(z01 + z02), Z1 = limbs(z12 - z01), Z2 = limbs(-z02 - z12);
-  // 4 Z V on the scale 2^-CF: Z 2^(4 + 2 lz - 2 up - nu + F - 1081), V 2^(960 + k), product >> 62
-  const int sh = -(4 + 2 * lz - 2 * g.up - nu + q.F - 1081) - 1024 - CF;
-  const s64 x0a = scale_down(mul62(Z0, q.v0a), sh - q.k0), x0b = scale_down(mul62(Z0, q.v0b), sh - q.k0);
-  const s64 x1b = scale_down(mul62(Z1, q.v1b), sh - q.k1), x1c = scale_down(mul62(Z1, q.v1c), sh - q.k1);
-  const s64 x2c = scale_down(mul62(Z2, q.v2c), sh - q.k2), x2d = scale_down(mul62(Z2, q.v2d), sh - q.k2);
-  const s64 ga = right ? o0 : -2 * o0, gb = right ? -4 * o0 - 2 * o1 : 5 * o0 + o1,
-            gc = right ? -o1 - 5 * o2 : 2 * o1 + 4 * o2, gd = right ? 2 * o2 : -o2;
-  o[0] = fix_to_double(ga - x0a, 1086 - CF);
-  o[1] = fix_to_double(gb - x0b - x1b, 1086 - CF);
-  o[2] = fix_to_double(gc - x1c - x2c, 1086 - CF);
-  o[3] = fix_to_double(gd - x2d, 1086 - CF);
+  // each Z_k on the scale of its own larger part
+  const int nu0 = imin(h01, h02), nu1 = imin(h01, h12), nu2 = imin(h02, h12);
+  const s64 z01 = mul62(limbs(K01), limbs(E01)), z02 = mul62(limbs(K02), limbs(t02.m)), z12 = mul62(limbs(K12), limbs(E12));
+  const Limb Z0 = limbs(sar(z01, h01 - nu0) + sar(z02, h02 - nu0)), Z1 = limbs(sar(z12, h12 - nu1) - sar(z01, h01 - nu1)),
+             Z2 = limbs(-sar(z02, h02 - nu2) - sar(z12, h12 - nu2));
+  // om_k = O_k 2^e_k, 2^55 <= O_k < 2^56 (c_k q_k = c_k W_k r / 2^62 on the scale 2^(lz - up - 63 - m_k))
+  const int L = lz - g.up - 55;
+  const Sm u0 = sm_norm(right ? 3 * (q0 >> 2) : q0, L - m0 + (right ? 2 : 0)), u1 = sm_norm(3 * (q1 >> 2), L - m1 + 3),
+           u2 = sm_norm(right ? q2 : 3 * (q2 >> 2), L - m2 + (right ? 0 : 2));
+  const s64 O0 = (s64)(u0.m >> 8), O1 = (s64)(u1.m >> 8), O2 = (s64)(u2.m >> 8);
+  // 4 Z_k V: Z_k on 2^(4 + 2 lz - 2 up - nu_k + F - 1081), V on 2^(960 + k), the product >> 62
+  const int x = 2 * lz - 2 * g.up + q.F - 53, x0 = x - nu0 + q.k0, x1 = x - nu1 + q.k1, x2 = x - nu2 + q.k2;
+  // an output's scale is that of its larger weight: |4 Z_k V| stays below 34 om_k, so the sums below 2^63
+  const int eb = imax(u0.x, u1.x), ec = imax(u1.x, u2.x);
+  const s64 b0 = sar(O0, eb - u0.x), b1 = sar(O1, eb - u1.x), c1 = sar(O1, ec - u1.x), c2 = sar(O2, ec - u2.x);
+  o[0] = fix_to_double((right ? O0 : -2 * O0) - scale_down(mul62(Z0, q.v0a), u0.x - x0), u0.x + 1086);
+  o[1] = fix_to_double((right ? -4 * b0 - 2 * b1 : 5 * b0 + b1) - scale_down(mul62(Z0, q.v0b), eb - x0) -
+                           scale_down(mul62(Z1, q.v1b), eb - x1), eb + 1086);
+  o[2] = fix_to_double((right ? -c1 - 5 * c2 : 2 * c1 + 4 * c2) - scale_down(mul62(Z1, q.v1c), ec - x1) -
+                           scale_down(mul62(Z2, q.v2c), ec - x2), ec + 1086);
+  o[3] = fix_to_double((right ? 2 * O2 : -O2) - scale_down(mul62(Z2, q.v2d), u2.x - x2), u2.x + 1086);
 }
 
 }  // namespace js
