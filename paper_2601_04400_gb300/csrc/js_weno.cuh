@@ -23,7 +23,7 @@
 
 namespace js {
 
-// a cell value as m 2^(e - 1080): |m| in [2^57, 2^58), or 0
+// a cell value as m 2^(e - 1080): |m| in [2^57, 2^58), smaller below the normal range (e = 1 there)
 struct Qx {
   s64 m;
   s32 e;
@@ -31,11 +31,11 @@ struct Qx {
 JS_HD Qx qx_of(double q) {
   const u64 b = dbits(q);
   const s32 e = expo(q);
-  const u64 M = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 5;
+  const u64 M = ((b & 0x000fffffffffffffull) | (e == 0 ? 0 : 0x0010000000000000ull)) << 5;
   const u64 s = (u64)(s64)((s32)hi32(b) >> 31);
-  return Qx{e == 0 ? 0 : (s64)((M ^ s) - s), e};
+  return Qx{(s64)((M ^ s) - s), imax(e, 1)};
 }
-// a first difference as m 2^(e - 1081): |m| in [2^58, 2^59), or 0 with e = 0; e = 2047 where a value
+// a first difference as m 2^(e - 1081): |m| in [2^58, 2^59) (e may be negative), or 0 with e = 0; e = 2047 where a value
 // is not finite or above 2^477
 struct Fx {
   s64 m;

@@ -206,7 +206,7 @@ JS_HD double sound_wide(double g, double p, double r) {
 }
 
 // a signed fixed-point value c 2^(e - 1086) as a double (rounded at 53 bits):
-// c / 2^63 in [1/2, 1) has the biased exponent e.  Values below the normal range give 0.
+// c / 2^63 in [1/2, 1) has the biased exponent e.  Results below the normal range are subnormal.
 // c is the floor of the value meant (right shifts brought it there), so a negative one's magnitude is
 // -c - 1 and a fraction: the complement rounds it as a positive value's floor does.
 JS_HD double fix_to_double(s64 c, int e) {
@@ -215,8 +215,10 @@ JS_HD double fix_to_double(s64 c, int e) {
   const int lz = clz64(m);
   m <<= (lz & 63);
   const int be = e - lz;  // biased exponent of the leading bit
-  const u64 v = ((u64)(u32)(be - 1) << 52) + (m >> 11) + ((m >> 10) & 1u);  // the leading bit adds 1 to the exponent
-  return (c == 0 || be < 1) ? 0.0 : bitsd(v | ((u64)sg & 0x8000000000000000ull));
+  m = shr(m, imax(1 - be, 0));
+  // the leading bit adds 1 to the exponent
+  const u64 v = ((u64)(u32)imax(be - 1, 0) << 52) + (m >> 11) + ((m >> 10) & 1u);
+  return c == 0 ? 0.0 : bitsd(v | ((u64)sg & 0x8000000000000000ull));
 }
 
 }  // namespace js
