@@ -55,6 +55,14 @@ __device__ __forceinline__ double recip(double x) {
 }
 // a/b as a * (1/b) (1 FP64 instruction; within 1 ulp)
 __device__ __forceinline__ double quot(double a, double b) { return a * recip(b); }
+// a/b within 0.53 ulp in integer arithmetic, rb = recip_top(mant64(b)) (formed ahead of a); IEEE division
+// outside that routine's range
+__device__ __forceinline__ double quot_near(double a, double b, u64 rb) {
+  const int ea = expo(a), eb = expo(b);
+  const bool out = (u32)(ea - 1) >= 2046u || (u32)(ea - eb + 1020) > 2040u;
+  if ((u32)(eb - 1) >= 2046u || (out && (dbits(a) << 1) != 0)) return a / b;
+  return quot_wide(a, b, rb);
+}
 // 1/sqrt(x) likewise (0 instead of 5 FP64 instructions)
 __device__ __forceinline__ double rsqrt_nr(double x) {
   const s32 h = (s32)hi32(dbits(x));

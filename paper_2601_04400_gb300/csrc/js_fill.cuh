@@ -93,7 +93,8 @@ __device__ __forceinline__ void ib_image(const double* __restrict__ U, const Lay
   q[0] = q[1] = q[2] = q[3] = 0.0;
   if (w != 0.0) {
     const double r = U[s], mx = U[lay.plane + s], my = U[2 * lay.plane + s], E = U[3 * lay.plane + s];
-    const double ir = recip(r), u = mx * ir, v = my * ir;
+    const u64 rr = recip_top(mant64(r));
+    const double u = quot_near(mx, r, rr), v = quot_near(my, r, rr);
     q[0] = w * r;
     q[1] = w * u;
     q[2] = w * v;
@@ -118,8 +119,9 @@ __device__ __forceinline__ void ib_fill_one(double* __restrict__ U, const Lay& l
   const int k = t >> 2, m = t & 3;
   const double gm1 = gamma - 1.0;
   double q[4], nx, ny, ug, vg;
+  const u64 rg = recip_top(mant64(gm1));
   ib_image(U, lay, ib, gm1, wall, k, m, q, nx, ny, ug, vg);
-  const double e = fma(q[3], recip(gm1), 0.5 * q[0] * fma(ug, ug, vg * vg));
+  const double e = fma(0.5 * q[0], fma(ug, ug, vg * vg), quot_near(q[3], gm1, rg));
   U[m * lay.plane + ib.dst[k]] = pick4(m, q[0], q[0] * ug, q[0] * vg, e);
 }
 

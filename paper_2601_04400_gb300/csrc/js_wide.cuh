@@ -183,6 +183,16 @@ JS_HD double recip_wide(double x) {
   const double r = pack62(recip_top(mant64(x)), 2045 - expo(x));
   return bitsd(dbits(r) | (dbits(x) & 0x8000000000000000ull));
 }
+// a/b (rounded from about 57 bits, so within 0.53 ulp) for a normal or zero a and a normal b, rb =
+// recip_top(mant64(b)), their quotient normal: biased exponents ea - eb in -1020 .. 1020
+JS_HD double quot_wide(double a, double b, u64 rb) {
+  const u64 q = mul_top(mant64(a), rb);  // a/b = q 2^(ea - eb - 61), 2^60 <= q < 2^62
+  const int lz = clz32(hi32(q));
+  const u64 m = q << lz;
+  const u64 v = ((u64)(u32)(expo(a) - expo(b) + 1024 - lz) << 52) + (m >> 11) + ((m >> 10) & 1u);
+  const u64 sign = (dbits(a) ^ dbits(b)) & 0x8000000000000000ull;
+  return bitsd(expo(a) == 0 ? sign : v | sign);
+}
 // 1/sqrt(x) (rounded from about 57 bits) for a positive normal x
 JS_HD double rsqrt_wide(double x) {
   // x = (n / 2^64) 2^(2h), n / 2^64 in [1/4, 1)
