@@ -2,19 +2,37 @@
 
 Every variant computes identical results; only speed differs.  `autotune` times a few
 js_step calls per variant with CUDA events on the solver's stream, selects the fastest and
-caches the choice in a JSON file keyed by grid size, physics and immersed body, so later
-solvers with the same key start tuned.
+caches the choice in a JSON file keyed by the kernels' sources, grid size, physics and immersed
+body, so later solvers with the same key start tuned.  What a variant or a number of blocks
+means is the kernels' business: a choice made for other sources is not applied.
 """
+import functools
+import hashlib
 import json
 import os
 
-_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "tuning.json")
+_HERE = os.path.dirname(os.path.abspath(__file__))
+_CACHE = os.path.join(_HERE, "_build", "tuning.json")
+# variants of the line kernel that differ (3 and 4 run variant 0's)
+_VARIANTS = (0, 1, 2)
+
+
+@functools.lru_cache(maxsize=None)
+def _sources():
+    """Short hash of the kernels' sources."""
+    h = hashlib.sha1()
+    d = os.path.join(_HERE, "csrc")
+    for name in sorted(os.listdir(d)):
+        if name.endswith((".cu", ".cuh", ".h")):
+            with open(os.path.join(d, name), "rb") as f:
+                h.update(name.encode() + b"\0" + f.read())
+    return h.hexdigest()[:12]
 
 
 def _key(solver):
     sp = solver._spec
-    return "%dx%d|visc=%d|av=%d|ib=%d" % (sp["nx"], sp["ny"], int(sp["mu"] > 0), int(sp["nu"] > 0),
-                                          int(getattr(solver, "has_ib", False)))
+    return "%s|%dx%d|visc=%d|av=%d|ib=%d" % (_sources(), sp["nx"], sp["ny"], int(sp["mu"] > 0), int(sp["nu"] > 0),
+                                             int(getattr(solver, "has_ib", False)))
 
 
 def _load():
@@ -34,7 +52,9 @@ def _save(cache):
 
 
 def cached_variant(solver):
-    return _load().get(_key(solver), {}).get("variant")
+    """The saved variant of this solver's key, or None."""
+    v = _load().get(_key(solver), {}).get("variant")
+    return v if v in _VARIANTS else None
 
 
 def apply_cached(solver):
@@ -45,17 +65,16 @@ def apply_cached(solver):
 
 
 def autotune(solver, U, reps=3, use_cache=True):
-    """Time every stage-kernel variant on state U (not modified) and select the fastest.
-    Returns {variant: ms per step}."""
+    """Time the line kernel's variants that differ on state U (not modified) and select the fastest.
+    Returns {variant: ms per step} ({} when the cache had the choice)."""
     import torch
     if use_cache and apply_cached(solver) is not None:
         return {}
     dt = 0.5 * solver.max_dt(U, 0.5)
-    _, n = solver.tuning()
     stream = torch.cuda.current_stream()
     times = {}
     work = U.clone()
-    for v in range(n):
+    for v in _VARIANTS:
         solver.set_tuning(v)
         solver.step(work, dt, 1)  # warm-up (first launch sets kernel attributes)
         t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -81,11 +100,19 @@ def autotune(solver, U, reps=3, use_cache=True):
 # batched path: blocks per SM and schedule of the forward's line kernels
 # ---------------------------------------------------------------------------------------
 def batch_key(problems):
-    """The instance mix: grid sizes, physics and immersed bodies of all instances (order-free)."""
-    import hashlib
+    """The kernels' sources and the instance mix: grid sizes, physics and immersed bodies of all
+    instances (order-free)."""
     items = sorted("%dx%d|visc=%d|av=%d|ib=%d" % (p.nx, p.ny, int(p.mu > 0), int(p.nu > 0), int(p.sdf is not None))
                    for p in problems)
-    return "batch|%d|%s" % (len(items), hashlib.sha1("\n".join(items).encode()).hexdigest()[:16])
+    return "batch|%s|%d|%s" % (_sources(), len(items), hashlib.sha1("\n".join(items).encode()).hexdigest()[:16])
+
+
+def cached_batch_choice(batch, problems):
+    """The saved (blocks per SM, schedule) of this mix, or None; one out of the batch's range is not taken."""
+    c = _load().get(batch_key(problems), {}).get("choice")
+    _, most, _, nsched = batch.tuning()
+    ok = isinstance(c, list) and len(c) == 2 and c[0] in range(most + 1) and c[1] in range(nsched)
+    return tuple(c) if ok else None
 
 
 def autotune_batch(batch, problems, states, steps=2, use_cache=True):
@@ -94,10 +121,9 @@ def autotune_batch(batch, problems, states, steps=2, use_cache=True):
     identical for every choice.  The batch's registered states are `states` afterwards.
     Returns {(blocks_per_sm, schedule): ms per step} ({} when the cache had the choice)."""
     import torch
-    key = batch_key(problems)
-    cache = _load()
-    if use_cache and key in cache:
-        batch.set_tuning(*cache[key]["choice"])
+    choice = cached_batch_choice(batch, problems) if use_cache else None
+    if choice is not None:
+        batch.set_tuning(*choice)
         batch.set_states(states)
         return {}
     _, most, _, nsched = batch.tuning()
@@ -123,44 +149,17 @@ def autotune_batch(batch, problems, states, steps=2, use_cache=True):
     best = min(times, key=times.get)
     if times[best] > 0.98 * times[default]:
         best = default
+    best = (best[0] % most, best[1])  # 0: the most that fit, whatever their number
     batch.set_tuning(*best)
     batch.set_states(states)
     cache = _load()
-    cache[key] = {"choice": list(best), "ms_per_step": {"%d,%d" % k: v for k, v in times.items()}}
+    cache[batch_key(problems)] = {"choice": list(best), "ms_per_step": {"%d,%d" % k: v for k, v in times.items()}}
     _save(cache)
     return times
 
 
 def autotune_batch_reverse(batch, problems, states, dts, reps=2, use_cache=True):
-    """Time js_batch_step_vjp (one reverse step of every instance from `states` with step sizes
-    `dts`) in both settings of the launch form -- they run the same launches -- and select the
-    faster; the choice is cached per instance mix.  Results are identical for both forms.
-    Returns {split: ms per reverse step} ({} when the cache had the choice)."""
-    import torch
-    key = batch_key(problems) + "|reverse"
-    cache = _load()
-    if use_cache and key in cache:
-        batch.set_reverse_launch(cache[key]["split"])
-        return {}
-    lam = [torch.randn_like(U) for U in states]
-    out = [torch.empty_like(U) for U in states]
-    stream = torch.cuda.current_stream()
-    times = {}
-    for split in (0, 1):
-        batch.set_reverse_launch(split)
-        batch.step_vjp(states, dts, lam, out)  # warm-up (the first call prepares the workspace)
-        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        t0.record(stream)
-        for _ in range(reps):
-            batch.step_vjp(states, dts, lam, out)
-        t1.record(stream)
-        t1.synchronize()
-        times[split] = t0.elapsed_time(t1) / reps
-    if batch.status() != 0:
-        raise RuntimeError("batched reverse tuning run failed")
-    best = 1 if times[1] < 0.98 * times[0] else 0
-    batch.set_reverse_launch(best)
-    cache = _load()
-    cache[key] = {"split": best, "ms_per_reverse_step": {str(k): v for k, v in times.items()}}
-    _save(cache)
-    return times
+    """Both settings of the reverse's launch form (js_batch_set_reverse_launch) run the same launches, so
+    nothing is timed or cached: sets 0 and returns {}."""
+    batch.set_reverse_launch(0)
+    return {}
