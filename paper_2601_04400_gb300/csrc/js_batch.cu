@@ -40,14 +40,10 @@ struct BatchArgs {
   unsigned long long* red;    // [2][count][4]: bits of the IEEE rate, rho_min, the fast rate
   double* tmax;               // largest fast rate of each tile
   double* dtc;                // [count][DTC_N] stage constants of the current step
-  unsigned* bar;              // [0] arrivals, [1] generation
   int* err;
   double* t;                  // accumulated time per instance or nullptr
   double* dt_log;             // [n_steps][count] step sizes used, or nullptr
   double cfl;
-  int n_steps;
-  int extra_arrivals;         // > 0 only to exercise the barrier timeout
-  long long budget;           // barrier wait budget in clock cycles
   const double* dt_in;        // [n_steps][count] given step sizes (no CFL reduction), or nullptr
   double* const* ustate;      // [count] states advanced instead of the registered ones, or nullptr
   double* const* save;        // [n_steps][count] states after each step, or nullptr
@@ -74,39 +70,6 @@ __device__ __forceinline__ int find_inst64(const long long* pre, int count, long
   return lo;
 }
 
-// grid barrier with a bounded wait; returns false when the launch must stop
-__device__ bool grid_sync_on(unsigned* bar, int* err, int extra_arrivals, long long budget) {
-  __shared__ int s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    volatile unsigned* vgen = bar + 1;
-    const unsigned g = *vgen;
-    __threadfence();
-    const unsigned target = gridDim.x + (unsigned)extra_arrivals;
-    const unsigned arrived = atomicAdd(bar, 1u) + 1u;
-    if (arrived == target) {
-      bar[0] = 0u;
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (*vgen == g) {
-        if (*(volatile int*)err & ERR_TIMEOUT_BIT) { ok = 0; break; }
-        if (clock64() - t0 > budget) {
-          atomicOr(err, ERR_TIMEOUT_BIT);
-          ok = 0;
-          break;
-        }
-        __nanosleep(128);
-      }
-    }
-    __threadfence();
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
 __device__ __forceinline__ double inst_dt(const InstDesc& d, const unsigned long long* red, double cfl) {
   const double rate = __longlong_as_double((long long)red[0]);
   const double rmin = __longlong_as_double((long long)red[1]);
@@ -252,7 +215,7 @@ __device__ __forceinline__ void fwd_phase(const BatchArgs& b, int step, int s, d
         nxt[4 * k + 1] = 0x7ff0000000000000ULL;
         const InstDesc& d = b.inst[k];
         const double dtk = b.dt_in ? b.dt_in[(long long)step * b.count + k] : inst_dt(d, red + 4 * k, b.cfl);
-        // the stage constants, read by the cell phases (grid barriers lie between)
+        // the stage constants, read by the cell phases (later launches)
         double* dtc = b.dtc + (long long)DTC_N * k;
         dtc[0] = __ddiv_rn(dtk, d.dx);
         dtc[1] = __ddiv_rn(dtk, d.dy);
@@ -370,9 +333,43 @@ __global__ void __launch_bounds__(FNT, PH == FP_LINES ? 4 : 1) batch_phase_kerne
   fwd_phase<PH, VM>(b, step, s, smem);
 }
 
-// one bounded grid barrier (js_batch_test_timeout)
-__global__ void __launch_bounds__(FNT) batch_barrier_kernel(BatchArgs b) {
-  grid_sync_on(b.bar, b.err, b.extra_arrivals, b.budget);
+// The self-test of the error status (js_batch_test_timeout): one grid barrier, extra_arrivals short of
+// completing, whose wait ends after `budget` clock cycles.  The phases need none (kernel boundaries order them).
+__device__ bool grid_sync_on(unsigned* bar, int* err, int extra_arrivals, long long budget) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    volatile unsigned* vgen = bar + 1;
+    const unsigned g = *vgen;
+    __threadfence();
+    const unsigned target = gridDim.x + (unsigned)extra_arrivals;
+    const unsigned arrived = atomicAdd(bar, 1u) + 1u;
+    if (arrived == target) {
+      bar[0] = 0u;
+      __threadfence();
+      atomicAdd(bar + 1, 1u);
+    } else {
+      const long long t0 = clock64();
+      while (*vgen == g) {
+        if (*(volatile int*)err & ERR_TIMEOUT_BIT) { ok = 0; break; }
+        if (clock64() - t0 > budget) {
+          atomicOr(err, ERR_TIMEOUT_BIT);
+          ok = 0;
+          break;
+        }
+        __nanosleep(128);
+      }
+    }
+    __threadfence();
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+__global__ void __launch_bounds__(FNT) batch_barrier_kernel(unsigned* bar, int* err, int extra_arrivals,
+                                                            long long budget) {
+  grid_sync_on(bar, err, extra_arrivals, budget);
 }
 
 // =======================================================================================
@@ -907,12 +904,11 @@ int js_batch_create(int count, const js_grid* grids, const js_params* params, co
     js_batch_destroy(b);
     return JS_ERR_CUDA;
   }
-  int dev = 0, sms = 0, per_sm = 0, coop = 0;
+  int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, js::batch_phase_kernel<js::FP_LINES, 1>, js::FNT, smem);
-  if (!coop || per_sm < 1) { js_batch_destroy(b); return JS_ERR_CUDA; }
+  if (per_sm < 1) { js_batch_destroy(b); return JS_ERR_CUDA; }
   b->sms = sms;
   b->per_sm = per_sm;
   b->blocks = sms * per_sm;
@@ -960,8 +956,8 @@ int js_batch_set_states(js_batch* b, double* const* U) {
   return JS_OK;
 }
 
-static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, double* dt_log, int extra,
-                        double budget_s, const double* dt_in = nullptr, double* const* ustate = nullptr,
+static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, double* dt_log,
+                        const double* dt_in = nullptr, double* const* ustate = nullptr,
                         double* const* save = nullptr, double* const* save1 = nullptr,
                         double* const* save2 = nullptr) {
   if (!ustate) b->ro_fwd_log = nullptr;  // the registered states move: kept checkpoints are stale
@@ -981,24 +977,10 @@ static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, dou
   a.red = b->d_red;
   a.tmax = b->d_tmax;
   a.dtc = b->d_dtc;
-  a.line0 = b->d_line0;
-  a.bar = b->d_bar;
   a.err = b->d_err;
   a.t = t_dev;
   a.dt_log = dt_log;
   a.cfl = cfl;
-  a.n_steps = n_steps;
-  a.extra_arrivals = extra;
-  if (extra > 0) {
-    int dev = 0, khz = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
-    a.budget = (long long)(budget_s * 1e3 * (khz > 0 ? khz : 2000000));
-    void* args[] = {&a};
-    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)js::batch_barrier_kernel, dim3(b->sms), dim3(js::FNT),
-                                                      args, 0, b->stream);
-    return e == cudaSuccess ? JS_OK : JS_ERR_CUDA;
-  }
   using namespace js;
   const long long nghost = b->nghost, nhalo = b->nhalo;
   // grids: the elementwise phases a few resident blocks an SM, striding over their items; the lines one
@@ -1030,7 +1012,7 @@ static int batch_launch(js_batch* b, double cfl, int n_steps, double* t_dev, dou
 
 int js_batch_step(js_batch* b, double cfl, int n_steps, double* t_dev, double* dt_log) {
   if (!b || !b->states_set || !(cfl > 0.0) || n_steps < 0) return JS_ERR_ARG;
-  return batch_launch(b, cfl, n_steps, t_dev, dt_log, 0, 2.0);
+  return batch_launch(b, cfl, n_steps, t_dev, dt_log);
 }
 
 int js_batch_step_vjp(js_batch* b, double* const* U_n, const double* dt, double* const* lam_np1,
@@ -1065,7 +1047,7 @@ int js_batch_step_vjp(js_batch* b, double* const* U_n, const double* dt, double*
 
 int js_batch_step_fixed(js_batch* b, int n_steps, const double* dt) {
   if (!b || !b->states_set || n_steps < 0 || (n_steps > 0 && !dt)) return JS_ERR_ARG;
-  return batch_launch(b, 0.5, n_steps, nullptr, nullptr, 0, 2.0, dt);
+  return batch_launch(b, 0.5, n_steps, nullptr, nullptr, dt);
 }
 
 namespace {
@@ -1192,7 +1174,7 @@ int js_batch_rollout_forward(js_batch* b, double cfl, int n_steps, int ckpt, dou
     const int len = std::min(ckpt, n_steps - c * ckpt);
     if ((rc = batch_copy(b, T, T + L.cp(c) * n))) return rc;
     // with every state kept, the step's stage states too
-    if ((rc = batch_launch(b, cfl, len, nullptr, dt_log + (size_t)c * ckpt * n, 0, 2.0, nullptr, nullptr, nullptr,
+    if ((rc = batch_launch(b, cfl, len, nullptr, dt_log + (size_t)c * ckpt * n, nullptr, nullptr, nullptr,
                            ckpt == 1 ? tab(L.segU1(c)) : nullptr, ckpt == 1 ? tab(L.segU2(c)) : nullptr)))
       return rc;
   }
@@ -1238,7 +1220,7 @@ int js_batch_rollout_vjp(js_batch* b, int n_steps, const double* dt_log, int ckp
       if ((rc = batch_copy(b, T, work))) return rc;
       for (int c = 0; c < n_steps; ++c) {
         if ((rc = batch_copy(b, work, blk(L.cp(c))))) return rc;
-        if ((rc = batch_launch(b, 0.5, 1, nullptr, nullptr, 0, 2.0, dt_log + (size_t)c * n, tab(L.work()), nullptr,
+        if ((rc = batch_launch(b, 0.5, 1, nullptr, nullptr, dt_log + (size_t)c * n, tab(L.work()), nullptr,
                                tab(L.segU1(c)), tab(L.segU2(c)))))
           return rc;
       }
@@ -1246,7 +1228,7 @@ int js_batch_rollout_vjp(js_batch* b, int n_steps, const double* dt_log, int ckp
       if ((rc = batch_copy(b, T, blk(L.cp(0))))) return rc;
       for (int c = 1; c < L.nck; ++c) {
         if ((rc = batch_copy(b, blk(L.cp(c - 1)), blk(L.cp(c))))) return rc;
-        if ((rc = batch_launch(b, 0.5, ckpt, nullptr, nullptr, 0, 2.0, dt_log + (size_t)(c - 1) * ckpt * n,
+        if ((rc = batch_launch(b, 0.5, ckpt, nullptr, nullptr, dt_log + (size_t)(c - 1) * ckpt * n,
                                tab(L.cp(c)))))
           return rc;
       }
@@ -1258,7 +1240,7 @@ int js_batch_rollout_vjp(js_batch* b, int n_steps, const double* dt_log, int ckp
     const int s0 = c * ckpt, len = std::min(ckpt, n_steps - s0);
     if (ckpt > 1) {
       if ((rc = batch_copy(b, blk(L.cp(c)), work))) return rc;
-      if ((rc = batch_launch(b, 0.5, len, nullptr, nullptr, 0, 2.0, dt_log + (size_t)s0 * n, tab(L.work()),
+      if ((rc = batch_launch(b, 0.5, len, nullptr, nullptr, dt_log + (size_t)s0 * n, tab(L.work()),
                              tab(L.segU(1)), tab(L.segU1(0)), tab(L.segU2(0)))))
         return rc;
     }
@@ -1279,7 +1261,15 @@ int js_batch_rollout_vjp(js_batch* b, int n_steps, const double* dt_log, int ckp
 
 int js_batch_test_timeout(js_batch* b, double budget_s) {
   if (!b || !b->states_set || !(budget_s > 0.0) || budget_s > 2.0) return JS_ERR_ARG;
-  return batch_launch(b, 0.5, 0, nullptr, nullptr, 1, budget_s);
+  b->ro_fwd_log = nullptr;
+  int dev = 0, khz = 0, extra = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
+  long long budget = (long long)(budget_s * 1e3 * (khz > 0 ? khz : 2000000));
+  void* args[] = {&b->d_bar, &b->d_err, &extra, &budget};
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)js::batch_barrier_kernel, dim3(b->sms), dim3(js::FNT),
+                                                    args, 0, b->stream);
+  return e == cudaSuccess ? JS_OK : JS_ERR_CUDA;
 }
 
 int js_batch_sync_status(js_batch* b) {
