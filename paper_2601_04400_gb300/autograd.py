@@ -63,7 +63,6 @@ class _Rollout(torch.autograd.Function):
             if k + 1 in want:
                 outs[want[k + 1]] = U.clone()
         ctx.solver, ctx.dts, ctx.outputs, ctx.every = solver, list(dts), list(outputs), every
-        ctx.internals = internals
         ctx.w_device = None if weights is None else weights.device
         ctx.ckpts = ckpts
         ctx.theta = theta.detach().clone()
@@ -87,11 +86,7 @@ class _Rollout(torch.autograd.Function):
             wbar = torch.zeros_like(w)
             solver.set_neural(w, cfg["norm"], w_bar=wbar, fp32=cfg.get("fp32", False))
         scratch = torch.empty_like(lam)
-        weno = ctx.internals
-        if weno is None:
-            free = torch.cuda.mem_get_info(g.device)[0]
-            weno = solver.tape_weno_bytes(every) < 0.5 * free
-        solver.tape_reserve(every, weno=bool(weno))
+        solver.tape_reserve(every)
         for seg in reversed(range(len(ctx.ckpts))):
             start = seg * every
             stop = min(start + every, n)
