@@ -91,9 +91,9 @@ constexpr int AB = 34;                   // positions of a line's box: lane l at
 constexpr int ADJ_SPLIT = ADJ_LINES / 4;  // lines a block where four warps share one
 // plane of a block's box, [line][position] in both directions: nl lines and one on either side
 __host__ __device__ constexpr int adj_plane(int nl) { return AB * (nl + 2); }
-// shared doubles of a block: the box's 8 planes; shared lines: 13 rows of a warp's lanes a line
+// shared doubles of a block: the box's 8 planes; shared lines: 12 rows of a warp's lanes a line
 __host__ __device__ constexpr int adj_smem(bool split) {
-  return 8 * adj_plane(split ? ADJ_SPLIT : ADJ_LINES) + (split ? ADJ_SPLIT * 13 * 32 : 0);
+  return 8 * adj_plane(split ? ADJ_SPLIT : ADJ_LINES) + (split ? ADJ_SPLIT * 12 * 32 : 0);
 }
 // line blocks of a direction: groups of ADJ_LINES lines x chunks of 28 cells (-1 .. n) along them
 __host__ __device__ inline int adj_chunks(int n) { return (n + 2 + ADJ_CHUNK - 1) / ADJ_CHUNK; }
@@ -173,7 +173,7 @@ __device__ __forceinline__ void adj_lines(const AdjArgs& a, const double* __rest
     const bool face = live && inner && lane < 30 && f >= 0 && f <= ncell;
     const bool own = lane >= 2;  // (with face) the warp's faces: lanes 2..29
     const bool rev = lane >= 2 && lane < 30;
-    double* const ex = smem + 8 * AP + 13 * 32 * warp + lane;  // SPLIT: [13][32] of the line
+    double* const ex = smem + 8 * AP + 12 * 32 * warp + lane;  // SPLIT: [12][32] of the line
     double bL[4], bR[4], dl[VISC ? 5 : 4], dr[VISC ? 5 : 4];
     bool fell = SPLIT;  // a face of the warp fell back to first order
     double Lq[4], Rq[4];
