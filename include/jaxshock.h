@@ -368,7 +368,7 @@ int js_batch_rollout_spacing(js_batch* b, int n_steps, int* ckpt);
  * JS_ERR_TIMEOUT. */
 int js_batch_sync_status(js_batch* b);
 
-/* Launch shape and size: resident blocks of the forward's line kernel, 32x16 tiles, cells. */
+/* Launch shape and size: resident blocks of the forward's line kernel, 32x32 tiles, cells. */
 int js_batch_info(js_batch* b, int* blocks, int* tiles, long long* cells);
 
 /* Launch shape and schedule of the forward's line kernels (js_batch_step, js_batch_step_fixed and
@@ -430,15 +430,16 @@ int js_get_arith(js_ctx* ctx, int* mode);
 
 /* Stage-kernel tuning: variant (0 .. n_variants-1) of the line kernel used by this context's
  * js_rhs / js_step / js_step_vjp: 0, 3 and 4 four blocks of eight lines an SM (small grids: four warps
- * a line), 1 three, 2 two.  Results are identical for every variant; only speed differs (the Python autotuner times them and caches the choice). */
+ * a line), 1 three, 2 two.  Results are identical for every variant; only speed differs (the Python
+ * autotuner times 0, 1 and 2 and caches the choice). */
 int js_set_tuning(js_ctx* ctx, int variant);
 int js_get_tuning(js_ctx* ctx, int* variant, int* n_variants);
 
-/* Instrumentation.  js_profile_begin(ctx, capacity) starts timing every launch of the fused
- * stage kernel (up to `capacity` launches) with CUDA events recorded on the context's stream,
+/* Instrumentation.  js_profile_begin(ctx, capacity) starts timing every stage (its lines and
+ * cells kernels together, up to `capacity` stages) with CUDA events recorded on the context's stream,
  * and counting every kernel the context launches.  js_profile_end synchronises the stream,
- * stops recording and returns the summed stage-kernel time in ms, the number of stage
- * launches timed and the number of kernels launched in between (any pointer may be NULL). */
+ * stops recording and returns the summed time of the stages in ms, the number of
+ * stages timed and the number of kernels launched in between (any pointer may be NULL). */
 int js_profile_begin(js_ctx* ctx, int capacity);
 int js_profile_end(js_ctx* ctx, double* stage_ms, int* stage_launches, long long* kernel_launches);
 

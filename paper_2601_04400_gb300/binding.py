@@ -239,7 +239,7 @@ def js_profile_begin(ctx, capacity):
 
 
 def js_profile_end(ctx):
-    """Returns (summed stage-kernel ms, stage launches timed, kernels launched)."""
+    """Returns (summed ms of the stages, stages timed, kernels launched)."""
     ms, n, k = C.c_double(0.0), C.c_int(0), C.c_longlong(0)
     _check(lib().js_profile_end(ctx, C.byref(ms), C.byref(n), C.byref(k)), "js_profile_end")
     return ms.value, n.value, k.value
@@ -351,7 +351,7 @@ class Solver:
         self._nn = (w, w_bar, nm)  # keep the device buffers alive while the library uses them
 
     def set_arith(self, mode):
-        """"fast" (default: the fused stage kernel) or "ieee" (every operation IEEE-rounded in
+        """"fast" (default: the stage kernels in integer and FP64 arithmetic) or "ieee" (every operation IEEE-rounded in
         the canonical order: bit-reproducible)."""
         code = {"fast": JS_ARITH_FAST, "ieee": JS_ARITH_IEEE}[mode]
         _check(lib().js_set_arith(self.ctx, code), "js_set_arith")

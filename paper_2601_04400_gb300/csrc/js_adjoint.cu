@@ -144,7 +144,7 @@ long long adj_strip_doubles(const Lay& L) { return strip_size(L, 0) + strip_size
 // time.  A reverse step, Euler / viscous with a body, shared and not: 64x64 165 / 200 and 238 / 258 us,
 // 128x128 249 / 311 and 278 / 341, 180x128 (227 blocks) 305 / 345 and 329 / 351; then the chip fills:
 // 250x190 (440) 449 / 527 and 391 / 425.
-constexpr int ADJ_SPLIT_BLOCKS = 228;
+constexpr int ADJ_SPLIT_BLOCKS = 3 * GB300_SMS / 2;
 namespace {
 int line_block(const Lay& L) {  // lines a block
   return L.ny == 1 || adj_blocks(L, 0) + adj_blocks(L, 1) <= ADJ_SPLIT_BLOCKS ? ADJ_SPLIT : ADJ_LINES;

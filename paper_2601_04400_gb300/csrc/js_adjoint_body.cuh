@@ -38,9 +38,8 @@ __device__ __forceinline__ void warp_partials(double* pp, long long w, double g,
   const double v = warp_sum4(g, m, pr, n);
   if ((threadIdx.x & 7) == 0) pp[4 * w + ((threadIdx.x & 31) >> 3)] = v;
 }
-// the same summed over the block's warps in order (at most 8 warps, all threads call it): one slot
-// per block, so that the final reduction stays short
-// the block's sums of the four values, value k on thread k < 4 (the other threads return nothing)
+// the block's sums of the four values over its warps in order (at most 8 warps, all threads call it): value
+// k on thread k < 4, 0 on the others
 __device__ __forceinline__ double block_sum4(double a, double b, double c, double d) {
   __shared__ double part[8][4];
   const double v = warp_sum4(a, b, c, d);
@@ -51,6 +50,7 @@ __device__ __forceinline__ double block_sum4(double a, double b, double c, doubl
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w][threadIdx.x];
   return t;
 }
+// the same into one slot a block, so that the final reduction stays short
 __device__ __forceinline__ void block_partials(double* pp, long long slot, double g, double m, double pr, double n) {
   if (pp == nullptr) return;
   const double t = block_sum4(g, m, pr, n);
@@ -103,10 +103,11 @@ __host__ __device__ inline int adj_blocks(const Lay& L, int dir, int nl = ADJ_LI
 }
 // Blocks of eight lines that three an SM hold at once.  Up to here the line kernels take 80 registers
 // (three blocks an SM), above 64 with more spills (four).  A reverse step with four and with three, Euler /
-// viscous with a body: 256x200 (450 blocks) 462 / 490 and 424 / 499 us, 300x200 (579) 475 / 499 and 483 /
-// 511, 512x512 1358 / 1545 and 1367 / 1572, 900x600 2576 / 2944 and 2589 / 3008; 16 instances 5.30 and
-// 5.42 ms.  Two blocks (128 registers, no spills): 512x512 viscous 1681.
-constexpr int ADJ_THREE_BLOCKS = 456;
+// viscous with a body: 200x150 (302 blocks) 275 / 349 and 271 / 343 us, 250x190 (440) 339 / 418 and 333 /
+// 410; 240x200 (465) 388 / 473 and 389 / 494, 256x200 (506) 398 / 480 and 402 / 502, 300x200 (579) 400 / 484
+// and 414 / 506, 512x512 1332 / 1529 and 1340 / 1563; 16 instances 5.30 and 5.42 ms.  Two blocks (128
+// registers, no spills): 512x512 viscous 1681.
+constexpr int ADJ_THREE_BLOCKS = 3 * GB300_SMS;
 // strips of a direction: [chunk][variable (5)][4 outer cells][line]
 __host__ __device__ inline long long strip_size(const Lay& L, int dir) {
   return dir == 0 ? 20LL * adj_chunks(L.nx) * L.ny : L.ny > 1 ? 20LL * adj_chunks(L.ny) * L.nx : 0;

@@ -1054,7 +1054,7 @@ namespace {
 // one launch copying the states of table src into those of table dst (device tables of count
 // pointers)
 int batch_copy(js_batch* b, void* const* src, void* const* dst) {
-  js::launch(js::batch_copy_kernel, 4 * 152, 256, 0, b->stream, reinterpret_cast<const double* const*>(src),
+  js::launch(js::batch_copy_kernel, 4 * js::GB300_SMS, 256, 0, b->stream, reinterpret_cast<const double* const*>(src),
                                                         reinterpret_cast<double* const*>(dst), b->d_spre, b->count);
   return cudaGetLastError() == cudaSuccess ? JS_OK : JS_ERR_CUDA;
 }

@@ -396,8 +396,9 @@ __global__ void __launch_bounds__(128) stage1d_kernel(StageArgs a0) {
 namespace {
 // Blocks of eight lines up to which four warps share a line: about one block an SM, where a warp's
 // chain of four reconstructions is the time.  Per step, shared and not: 96x64 47 and 61 us, 128x128 66
-// and 73; then the chip fills: 200x128 (253 blocks) 85 and 80, 250x190 115 and 100.
-constexpr int SPLIT_BLOCKS = 160;
+// and 73; then the chip fills: 200x128 (253 blocks) 85 and 80, 250x190 115 and 100.  With face images (two
+// steps, FP32 network): 64x48 249 and 288, 128x128 327 and 331, 200x128 502 and 506, 250x190 592 and 560.
+constexpr int SPLIT_BLOCKS = GB300_SMS + 8;
 // Resident blocks an SM the registers are allotted for: 4 (64 registers, 32 warps) hides the FP64
 // and integer latencies best (2048x1024 viscous step: 4 blocks 2.42 ms, 3 blocks 2.50, 2 blocks
 // 2.96).  Tuning variants 1 and 2 are 3 and 2 blocks; every variant gives the same bits.
@@ -500,9 +501,9 @@ cudaError_t launch_cfl_init(unsigned long long* red, cudaStream_t s) {
 }
 
 // Cells up to which every rate is taken in IEEE arithmetic at once: one launch in place of two, each of
-// which is latency on such grids.  A step of 128x64 cells took 89 us with one launch and 95 with two,
-// of 256x128 116 and 120; from there the FP64 pipe decides: 256x256 155 and 153, 400x320 222 and 216
-// (before the launches overlapped).
+// which is latency on such grids.  Four steps of 128x64 cells take 200 us with one launch and 210 with two,
+// of 256x128 364 and 367; from there the FP64 pipe decides: 200x200 390 and 388, 256x256 525 and 511,
+// 400x320 777 and 741.
 constexpr long long CFL_ONE_CELLS = 32768;
 
 namespace {

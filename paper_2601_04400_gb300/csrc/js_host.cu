@@ -73,7 +73,7 @@ struct js_ctx {
   void* nn_keep[2] = {nullptr, nullptr};
   bool nn_keep_failed = false;
   double* nn_partial = nullptr;
-  int variant = 0;  // stage-kernel tile shape (js_set_tuning)
+  int variant = 0;  // variant of the line kernel (js_set_tuning)
   int arith = JS_ARITH_FAST;  // js_set_arith
   js::IeeeBufs ieee = {nullptr, nullptr, nullptr};  // workspace of JS_ARITH_IEEE
   // tape: per slot the three filled stage states of one recorded step
@@ -326,8 +326,7 @@ long long saved_plane(const js_ctx* c) {
   return (m + 31) / 32 * 32;
 }
 
-// fused stage kernel, bracketed by events while profiling
-// stage update that also writes the FP32 face images of the neural flux (FP32 and BF16
+// stage update (lines and cells, bracketed by events while profiling) that also writes the FP32 face images of the neural flux (FP32 and BF16
 // networks on 2D grids), then the network and its divergence
 int stage_img(js_ctx* c, StageArgs a, bool visc) {
   a.img = static_cast<float*>(c->nn.X);
@@ -365,7 +364,7 @@ int stage(js_ctx* c, const StageArgs& a, bool visc, bool rhs) {
 }
 
 // a forward stage (or the RHS) of js_rhs / js_step / js_step_stage in the context's arithmetic
-// mode: the fused stage kernel, or the IEEE-order kernels (stage k of step size dt)
+// mode: the fast stage kernels, or the IEEE-order ones (stage k of step size dt)
 int stage_fwd(js_ctx* c, const StageArgs& a, bool rhs, double dt, int k) {
   if (c->arith != JS_ARITH_IEEE) return stage(c, a, c->p.mu > 0.0, rhs);
   if (c->nn_on) return JS_ERR_ARG;

@@ -1,6 +1,6 @@
 // IEEE-order arithmetic mode of the forward step (js_set_arith(ctx, JS_ARITH_IEEE)).
 //
-// The same finite-volume right-hand side and SSP-RK3 stage as the fused stage kernel
+// The same finite-volume right-hand side and SSP-RK3 stage as the fast stage kernels
 // (Sec. 2: WENO5 reconstruction of the primitive variables, HLLC flux with the positivity
 // fallback, viscous and heat fluxes, flux divergence, Laplacian artificial viscosity), but
 // every operation is one IEEE-rounded double operation (this file is compiled with

@@ -6,6 +6,8 @@
 
 namespace js {
 
+constexpr int GB300_SMS = 152;
+
 // A launch whose setup overlaps the end of the kernel before it on the stream, for the chains of short
 // kernels that small grids are: its blocks start as the predecessor's last ones leave and wait in
 // pdl_enter, the first statement of every kernel launched this way, until the predecessor has
@@ -252,7 +254,7 @@ struct CflStep {
 // fluid cells (red: 4 words, reset by launch_cfl_init before the first reduction and after one
 // without a step; bmax: CFL_MAX_BLOCKS doubles of scratch).
 // padded: U is a context's padded buffer, e.g. the state N between the steps of js_step_cfl.
-constexpr int CFL_MAX_BLOCKS = 152 * 8;
+constexpr int CFL_MAX_BLOCKS = GB300_SMS * 8;
 cudaError_t launch_cfl_init(unsigned long long* red, cudaStream_t s);
 cudaError_t launch_cfl(const double* U, const Lay& lay, const unsigned char* tag, double gamma, double dx, double dy,
                        unsigned long long* red, double* bmax, const CflStep& st, cudaStream_t s, bool padded);

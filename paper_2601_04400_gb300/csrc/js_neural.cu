@@ -11,7 +11,7 @@
 // flux of frame component k through that face.
 //
 // Forward per stage: primitives -> images -> three convolution launches (T3 = tanh output)
-// -> the fused stage kernel (HLLC part) -> nn_apply subtracts the neural flux divergence.
+// -> the stage (lines, then cells: HLLC part) -> nn_apply subtracts the neural flux divergence.
 // Reverse per stage: the images and activations are recomputed from the stage state; the
 // seed is the face-flux adjoint (lambda'_right - lambda'_left)/h (the same as for the HLLC
 // flux); three data-gradient launches (ReLU masks fused), three weight-gradient launches
@@ -1547,7 +1547,7 @@ __device__ __forceinline__ double nn_warp_sum(double v) {
 }
 
 // image reverse: network-input adjoint -> WENO face-state adjoints (a.fadj) and
-// d/dgamma of the face energies (added to pbar[0]); 32 x 32 pixel tiles as nn_image_kernel
+// d/dgamma of the face energies (added to pbar[0]); tiles of 32 lines x 8 faces as nn_image_kernel
 template <class T>
 __global__ void __launch_bounds__(256) nn_image_vjp_kernel(NnArgs n, AdjArgs a) {
   pdl_enter();

@@ -41,7 +41,7 @@ def rank_loads(cells, world):
 # y-slab decomposition of one grid
 # ---------------------------------------------------------------------------------------
 def _takes_internals(slab):
-    """Whether a slab solver can store stage internals (binding.Solver on a 2D grid)."""
+    """Whether a slab solver takes the internals mark (binding.Solver on a 2D grid)."""
     import inspect
     try:
         return "internals" in inspect.signature(slab.step_stage).parameters and slab.ny > 1
@@ -291,7 +291,7 @@ class SlabGroup:
         from .binding import JS_NPARAM
         X1 = {r: self._buf(("x1", r), u) for r, u in U_n.items()}
         X2 = {r: self._buf(("x2", r), u) for r, u in U_n.items()}
-        # the recomputed stages 0 and 1 store their WENO5 internals for their reverse
+        # the recomputed stages 0 and 1 are marked for their reverse
         keep = {r: _takes_internals(s) for r, s in self.slabs.items()}
         for r, u in U_n.items():
             self._stage(r, u, u, X1[r], dt, 0, keep[r])
