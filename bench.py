@@ -1,7 +1,7 @@
 """Throughput of the FP64 WENO5-HLLC-SSP-RK3 step on one GB300 (or N independent replicas).
 
 One "step" = one pass of the whole hot path over the grid: CFL reduction for dt, then three
-Runge-Kutta stages, each = immersed-boundary ghost fill + domain halo fill + fused stage
+Runge-Kutta stages, each = immersed-boundary ghost fill + domain halo fill + stage lines and cells
 kernel (WENO5, HLLC, viscous fluxes, divergence, stage combination).  The default workload is
 the largest single-GPU configuration: the viscous Mach-2 shock over the immersed cylinder,
 2048 x 1024 cells (Navier-Stokes, Re = 1000, Pr = 0.72).
@@ -16,7 +16,8 @@ Prints ONE JSON line (rank 0).  `value` is cell-updates/s with the state residen
 `e2e` is the same metric through the C ABI with the state copied from pinned host memory
 and back every step; `roofline` divides the algorithmic FP64 operation count of the stage
 kernels (lines, then cells) by their CUDA-event time and by the FP64 peak; the kernels form WENO5,
-reciprocals and square roots in integer arithmetic beside the FP64 pipe, so the fraction exceeds 1.
+reciprocals and square roots in integer arithmetic beside the FP64 pipe, so the fraction exceeds 1; `lines_busy`
+says what bounds them (issue slots and pipes, from a capture).
 """
 import argparse
 import json
@@ -41,7 +42,11 @@ NN_FLOPS_PER_CELL_STAGE = 2 * 2 * 6336
 # DRAM bytes (read + write) per stage (lines + cells kernels), mean of the three stages of one step,
 # from an ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the current kernels; None for
 # workloads or variants without one.
-STAGE_TRAFFIC_BYTES = {("shock_cylinder", 0): 500.1e6, ("riemann2d", 0): 182.0e6}
+STAGE_TRAFFIC_BYTES = {("shock_cylinder", 0): 501.2e6, ("riemann2d", 0): 184.0e6}
+# what bounds the line kernel, from the same captures (profiles/stage_lines.md): share of its cycles in
+# which issue slots, the integer pipes and the FP64 pipe were busy
+LINES_BUSY = {"shock_cylinder": {"issue_slots": 0.68, "alu": 0.64, "wide_multiply_add": 0.62, "fp64": 0.62},
+              "riemann2d": {"issue_slots": 0.70, "alu": 0.67, "wide_multiply_add": 0.64, "fp64": 0.52}}
 L2_FLUSH_BYTES = 256 << 20
 METRIC = "FP64 cell-updates/s per RK step on 1 GB300 (% roofline); adjoint/forward time ratio"
 
@@ -212,7 +217,7 @@ def run_ours(args):
     W0 = torch.tensor(prob.W0, dtype=torch.float64, device="cuda")
     U = solver.prim_to_cons(W0)
     from paper_2601_04400_gb300 import tuning
-    tuned = tuning.autotune(solver, U)  # stage-kernel tile shape (identical results)
+    tuned = tuning.autotune(solver, U)  # variant of the line kernel (identical results)
     U0 = U.clone()
     flush = torch.empty(L2_FLUSH_BYTES // 8, dtype=torch.float64, device="cuda")
     cfl = prob.cfl
@@ -289,9 +294,9 @@ def run_ours(args):
         solver.check()
         f_ms = sum(a.elapsed_time(b) for a, b in fa) / reps
         b_ms = sum(a.elapsed_time(b) for a, b in ba) / reps
-        # reverse of a step whose stage states (and WENO internals) were recorded: the
+        # reverse of a step whose stage states were recorded: the
         # checkpointed rollout's path; its backward re-runs each step taped, then reverses it
-        solver.tape_reserve(1, weno=True)
+        solver.tape_reserve(1)
         solver.step_taped(Uw, dt, 0)
         tf = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(reps)]
         ta = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(reps)]
@@ -314,7 +319,7 @@ def run_ours(args):
                "ms_per_step_taped_forward": tf_ms, "ms_per_step_vjp_taped": t_ms, "ratio_taped": t_ms / f_ms,
                "ratio_rollout_backward": (tf_ms + t_ms) / f_ms,
                "note": "ratio: js_step_vjp (recomputes the stage states, then reverses the 3 stages) / "
-                       "js_step; ratio_taped: js_step_vjp_taped (stage states and WENO5 internals recorded "
+                       "js_step; ratio_taped: js_step_vjp_taped (stage states recorded "
                        "by js_step_taped) / js_step; ratio_rollout_backward: (js_step_taped + "
                        "js_step_vjp_taped) / js_step, the backward cost per step of a checkpointed rollout"}
 
@@ -389,14 +394,14 @@ def run_ours(args):
             "config": {"workload": desc, "nx": prob.nx, "ny": prob.ny, "cells": cells,
                        "parallelism": "replicas" if world > 1 else "single",
                        "l2": "flushed between steps (256 MiB write)",
-                       "step": "CFL reduction + device step size + 3 x (IB fill, halo fill, fused stage "
-                               "kernel) (js_step_cfl)",
+                       "step": "CFL reduction + device step size + 3 x (IB fill, halo fill, lines, cells) "
+                               "(js_step_cfl)",
                        "stage_variant": solver.tuning()[0]},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": achieved / FP64_PEAK_TFLOPS,
                          "traffic": STAGE_TRAFFIC_BYTES.get((args.workload, solver.tuning()[0])),
                          "kernel": "stage_lines + stage_cells (WENO5, HLLC, viscous fluxes; Runge-Kutta stage)", "stage_ms_avg": stage_avg,
-                         "flops_per_launch": flop_launch},
+                         "flops_per_launch": flop_launch, "lines_busy": LINES_BUSY.get(args.workload)},
             "e2e": {"value": e2e_value, "unit": "cell-updates/s", "h2d_bytes_per_step": state_bytes,
                     "d2h_bytes_per_step": state_bytes},
             "adjoint_forward_ratio": None if adj is None else adj["ratio"],
@@ -516,27 +521,19 @@ def run_batched(args):
         s.set_stream(stream)
     ok = ok and all(s.status() == 0 for s in solvers)
     # reverse of one batched step (js_batch_step_vjp over all instances) against one batched
-    # forward step, in both settings of the launch form (they run the same launches); the tuner
-    # keeps the faster for the rollout below
+    # forward step
     dts = [s.max_dt(U, 0.5) for s, U in zip(solvers, states)]
     lams = [torch.randn_like(U) for U in states]
     outs = [torch.empty_like(U) for U in states]
-    rev_tuned = tuning.autotune_batch_reverse(batch, mine, states, dts)
-    t_vjp_form = {}
-    choice = batch.reverse_launch()
     reps = 3
-    for split in (0, 1):
-        batch.set_reverse_launch(split)
+    batch.step_vjp(states, dts, lams, outs)
+    torch.cuda.synchronize()
+    e0.record(stream)
+    for _ in range(reps):
         batch.step_vjp(states, dts, lams, outs)
-        torch.cuda.synchronize()
-        e0.record(stream)
-        for _ in range(reps):
-            batch.step_vjp(states, dts, lams, outs)
-        e1.record(stream)
-        e1.synchronize()
-        t_vjp_form[split] = e0.elapsed_time(e1) / reps
-    batch.set_reverse_launch(choice)
-    t_vjp = t_vjp_form[choice]
+    e1.record(stream)
+    e1.synchronize()
+    t_vjp = e0.elapsed_time(e1) / reps
     ok = ok and batch.status() == 0
     # the whole rollout: n_ro CFL steps forward (step sizes logged), then its reverse
     # (js_batch_rollout_vjp) with the library's checkpoint spacing (every state when they fit in
@@ -552,7 +549,7 @@ def run_batched(args):
         batch.rollout_forward(0.5, log)
         batch.rollout_vjp(log, lam_r)
         torch.cuda.synchronize()
-        # the plain forward run of the same steps: one launch, device CFL
+        # the plain forward run of the same steps: device CFL
         batch.set_states([U.clone() for U in states])
         e0.record(stream)
         batch.step(0.5, n_ro, dt_log=log)
@@ -579,7 +576,7 @@ def run_batched(args):
                         "states + the reverse of each step (the chosen launch form) taking the stage states as given, "
                         "from the checkpoints js_batch_rollout_forward kept; spacing 1 = every state and "
                         "stage state kept by the forward, no re-runs) / the plain batched forward run of "
-                        "the same steps (one launch, device CFL)"}
+                        "the same steps (device CFL)"}
     info = batch.info()
     if rank == 0:
         print(json.dumps({
@@ -615,10 +612,8 @@ def run_batched(args):
             "speedup_vs_graph": t_graph / t_batch,
             "adjoint": {"ms_per_step_vjp": t_vjp, "ratio": t_vjp / (t_batch / args.steps),
                         "launch": "one launch per phase",
-                        "ms_per_step_vjp_form0": t_vjp_form[0], "ms_per_step_vjp_form1": t_vjp_form[1],
-                        "tuner_timed": {str(k): v for k, v in rev_tuned.items()},
                         "note": "js_batch_step_vjp (recompute of the stage states and the reverse of the 3 "
-                                "stages of every instance; the launch form the tuner chose) / one batched "
+                                "stages of every instance) / one batched "
                                 "forward step, rank 0's instances"},
             "rollout": roll}), flush=True)
     if dist is not None:

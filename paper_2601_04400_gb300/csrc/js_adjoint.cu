@@ -30,9 +30,9 @@ namespace js {
 // =======================================================================================
 // per-grid launches
 // =======================================================================================
-// x line blocks, then y line blocks.  Bound by the FP64 pipe (221 instructions a lane, 62% busy) and by
-// latency, with the integer WENO5 forward and reverse beside it (55% of issue slots): 1024x512 viscous
-// 709 us at B = 3 blocks an SM.  B: the resident blocks the registers are allotted for (ADJ_THREE_BLOCKS).
+// x line blocks, then y line blocks.  Bound by the FP64 pipe (231 instructions a lane, 65% busy) and by
+// latency, with the integer WENO5 forward and reverse beside it (57% of issue slots): 1024x512 viscous
+// 710 us at B = 4 blocks an SM.  B: the resident blocks the registers are allotted for (ADJ_THREE_BLOCKS).
 template <bool VISC, bool SPLIT, int B>
 __global__ void __launch_bounds__(32 * ADJ_LINES, B)
 adj_lines_kernel(AdjArgs a, const double* __restrict__ Unext, double bdt, int bx) {

@@ -400,8 +400,8 @@ namespace {
 // steps, FP32 network): 64x48 249 and 288, 128x128 327 and 331, 200x128 502 and 506, 250x190 592 and 560.
 constexpr int SPLIT_BLOCKS = GB300_SMS + 8;
 // Resident blocks an SM the registers are allotted for: 4 (64 registers, 32 warps) hides the FP64
-// and integer latencies best (2048x1024 viscous step: 4 blocks 2.42 ms, 3 blocks 2.50, 2 blocks
-// 2.96).  Tuning variants 1 and 2 are 3 and 2 blocks; every variant gives the same bits.
+// and integer latencies best (2048x1024 viscous step: 4 blocks 2.24 ms, 3 blocks 2.30, 2 blocks
+// 2.29; 1024x1024 Euler 1.11, 1.14, 1.14).  Tuning variants 1 and 2 are 3 and 2 blocks; every variant gives the same bits.
 template <bool VISC, bool IMG>
 cudaError_t launch_lines(const StageArgs& a, int variant, cudaStream_t s) {
   const int bx = stage_blocks(a.lay, 0), n = bx + stage_blocks(a.lay, 1);
